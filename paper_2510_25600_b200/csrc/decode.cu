@@ -3,7 +3,7 @@
 // query head hq reads KV head hq / G of the request's kept rows.
 //
 // Split-KV, HBM bound: a CTA owns a chunk of one (request, KV head)'s kept keys and serves all G query heads of the
-// group from one read of K and one of V.  bf16 runs on tensor cores (decode_tc_kernel, further down); the kernel
+// group from one read of K and one of V.  bf16 runs on tensor cores (decode_cluster_kernel, further down); the kernel
 // described next serves fp32.  Rows are 256 bytes (bf16 d = 128 or fp32 d = 64): a half-warp covers a
 // row with one 16-byte load per lane, so a warp instruction fetches two rows.  Pass 1 forms the G logits of every
 // key (q slices in registers; the 16 lanes' partial dot products are folded by a butterfly that halves the number of
@@ -29,19 +29,6 @@ struct Row16<float> {
     f[0] = __uint_as_float(u.x); f[1] = __uint_as_float(u.y); f[2] = __uint_as_float(u.z); f[3] = __uint_as_float(u.w);
   }
 };
-template <>
-struct Row16<__nv_bfloat16> {
-  static constexpr int E = 8;
-  static __device__ __forceinline__ void unpack(uint4 u, float (&f)[8]) {
-    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      f[2 * i] = __uint_as_float(w[i] << 16);
-      f[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
-    }
-  }
-};
-
 __device__ __forceinline__ float dec_ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -220,21 +207,6 @@ __global__ void __launch_bounds__(kDecThreads) decode_partial_kernel(
 }
 
 // ---- bf16, d = 128 on tensor cores ---------------------------------------------------------------------------
-// The CUDA-core kernel above spends about 100 instructions per key at G = 8; with mma.sync the group's heads are
-// the 16 rows of an m16n8k16 tile and the arithmetic all but disappears beside the loads.  A warp takes 16 keys per
-// trip: S = Q K^T as two n8 tiles (8 k-steps each), online softmax on the accumulator registers, which then serve
-// unchanged as the A operand of O += P V (16 n8 tiles over d).  No shared-memory staging and no transposes: a dot
-// product does not care in which order its terms are taken, so each thread feeds the k (and n) slots of the
-// fragments from contiguous bytes of a row and the same order is used for the other operand --
-//   Q K^T: thread (row lane/4, t = lane%4) holds d = 32t .. 32t+31 of its Q rows and of its key's K row;
-//          k-step ks takes elements 4ks, 4ks+1 (k slots 2t, 2t+1) and 4ks+2, 4ks+3 (k slots 2t+8, 2t+9);
-//   P V:   thread (g8 = lane/4, t) holds d = 16 g8 .. 16 g8+15 of the V rows of keys 2t, 2t+1, 8+2t, 9+2t of the trip;
-//          n tile nt covers d = 16 j + nt (j = 0 .. 7), two keys' values paired per register by a byte permute.
-__device__ __forceinline__ uint4 ldg16_stream(const uint4* p) {
-  uint4 r;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
-  return r;
-}
 __device__ __forceinline__ void dec_mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
@@ -249,40 +221,105 @@ __device__ __forceinline__ uint32_t dec_pack_bf16(float lo, float hi) {
 
 constexpr float kDecRescale = 8.f;  // the reference maximum of a row moves only when a logit exceeds it by this (log2)
 
-// grid (n_splits, H_kv, n_req), 128 threads; G <= 16.  Same outputs as decode_partial_kernel.
-__global__ void __launch_bounds__(kDecThreads) decode_tc_kernel(
-    const uint4* __restrict__ q, const uint4* __restrict__ kc, const uint4* __restrict__ vc,
-    const int32_t* __restrict__ cu_kept, int32_t n_q_heads, int32_t n_kv_heads, int32_t chunk, float scale_log2,
-    __nv_bfloat16* __restrict__ o, float* __restrict__ lse, float* __restrict__ part, int32_t n_splits) {
-  constexpr int D = 128;
-  // a row's 128 columns as four runs of 32 padded to 33, rows 132 apart: the 32 lanes of a store (8 rows x 4 runs)
-  // fall into 32 different banks
-  __shared__ float s_o[kDecThreads / 32][16][4 * 33];
-  __shared__ float s_ml[kDecThreads / 32][16][2];
+// One launch.  A cluster of C CTAs (grid (C, H_kv, n_req)) owns one (request, KV head); CTA `rank` takes the rank-th share
+// of the request's rows, so ragged requests are cut evenly, and the CTAs' partial results meet in distributed shared
+// memory instead of in a workspace that a second kernel merges (chunk kernel + merge kernel before: 12.0 us for one
+// request of 1664 rows with 28 / 4 heads, now 5.5; 128 requests of 2900-5100 rows 214 us = 5.0 TB/s, now 168 us = 6.4 TB/s).
+// Bound by HBM for large batches and by a chain of latencies for small ones: launch (1 us behind a programmatic
+// predecessor), the offsets, the rows, the products, one cluster barrier.
+// A warp takes 16 keys per trip: with mma.sync the group's heads are the 16 rows of an m16n8k16 tile (M = 16 is far below a
+// tcgen05 tile's 128 rows), S = Q K^T is two n8 tiles, and the softmax on their accumulators leaves the A operand of
+// O += P V.  Each warp streams its trips through a private ring of ST stages with cp.async (rows padded to 272 bytes, so
+// that ldmatrix reads eight rows without bank conflicts): two further trips are in flight while one is multiplied, and no
+// warp waits for another before the end.
+constexpr int kClRow = 272;                     // bytes of a row in shared memory
+constexpr int kClStageBytes = 2 * 16 * kClRow;  // 16 K rows, then 16 V rows
+constexpr int kClMax = 16;                      // CTAs per cluster
 
-  const int32_t sp = blockIdx.x, g = blockIdx.y, r = blockIdx.z;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the merge kernel may be placed meanwhile
+// Dynamic shared memory of one warp: its ring, over which its partial results (rows of 128 + 8 floats) are laid at the end.
+template <int RW, int ST>
+__host__ __device__ constexpr int cl_warp_bytes() {
+  return ST * kClStageBytes > 8 * RW * (128 + 8) * 4 ? ST * kClStageBytes : 8 * RW * (128 + 8) * 4;
+}
+
+__device__ __forceinline__ void dec_ldsm(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void dec_ldsm_t(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ uint32_t dec_mapa(const void* local, uint32_t rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(local)), "r"(rank));
+  return a;
+}
+
+// RW: row groups of eight heads in use (1: G <= 8, 2: G <= 16); W warps; ST stages of each warp's ring.
+template <int RW, int W, int ST>
+__global__ void __launch_bounds__(W * 32, (ST == 1 ? 12 : 8) / W) decode_cluster_kernel(
+    const uint4* __restrict__ q, const uint4* __restrict__ kc, const uint4* __restrict__ vc,
+    const int32_t* __restrict__ cu_kept, int32_t n_q_heads, int32_t n_kv_heads, float scale_log2,
+    __nv_bfloat16* __restrict__ o, float* __restrict__ lse) {
+  constexpr int D = 128, R = 8 * RW, kThreads = W * 32, kWarpBytes = cl_warp_bytes<RW, ST>();
+  extern __shared__ __align__(16) uint8_t cl_smem[];
+  __shared__ float s_ml[W][R][2];
+  __shared__ __align__(16) float s_part[R * D];       // what the cluster's CTAs send this one: [source][head][its columns]
+  __shared__ __align__(8) float s_pml[kClMax][R][2];  // every CTA's (reference, sum) per head
+
+  const uint32_t C = gridDim.x, rank = blockIdx.x;  // the cluster spans the grid's x dimension
+  const int32_t g = blockIdx.y, r = blockIdx.z;
   const int32_t G = n_q_heads / n_kv_heads;
   const int32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g8 = lane >> 2, t = lane & 3;
-  const int64_t j0 = (int64_t)cu_kept[r] + (int64_t)sp * chunk;
-  const int32_t n = (int32_t)max((int64_t)0, min((int64_t)cu_kept[r + 1], j0 + chunk) - j0);
+  // The next kernel of the stream may be placed meanwhile (the calls of consecutive layers follow one another); what the
+  // previous one wrote is complete and visible behind the wait.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (C > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // "started": awaited before the sends
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int64_t kept0 = cu_kept[r];
+  const int32_t n_all = cu_kept[r + 1] - (int32_t)kept0;
+  const int32_t share = ((n_all + (int32_t)C - 1) / (int32_t)C + 15) & ~15;
+  const int64_t j0 = kept0 + (int64_t)rank * share;
+  const int32_t n = max(0, min(n_all - (int32_t)rank * share, share));
+
+  // 16-row trip `trip` of this warp into stage trip % ST: a warp request covers two rows; rows past the end repeat the
+  // last one (weight 0)
+  const uint32_t ring = (uint32_t)__cvta_generic_to_shared(cl_smem) + (uint32_t)warp * kWarpBytes;
+  const int64_t row_stride = (int64_t)n_kv_heads * 16;  // 16-byte words
+  const int32_t n_trips = n > warp * 16 ? (n - warp * 16 + W * 16 - 1) / (W * 16) : 0;
+  auto fetch = [&](int32_t trip) {
+    if (trip < n_trips) {
+      const int32_t k0 = warp * 16 + trip * (W * 16);
+      const uint32_t dst = ring + (uint32_t)(trip % ST) * kClStageBytes + (uint32_t)(lane >> 4) * kClRow + (lane & 15) * 16;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int64_t src = (j0 + min(k0 + 2 * i + (lane >> 4), n - 1)) * row_stride + g * 16 + (lane & 15);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 2 * i * kClRow), "l"(kc + src) : "memory");
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int64_t src = (j0 + min(k0 + 2 * i + (lane >> 4), n - 1)) * row_stride + g * 16 + (lane & 15);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (16 + 2 * i) * kClRow), "l"(vc + src) : "memory");
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");  // (empty past the end: the group count stays in step)
+  };
+#pragma unroll
+  for (int s = 0; s < (ST > 1 ? ST - 1 : 1); ++s) fetch(s);
 
   // A fragments of Q: rows g8 and g8 + 8 (heads of the group; rows past G are zero)
   uint32_t qa[8][4];
   {
-    uint4 lo[4], hi[4];
+    const uint32_t* q32 = reinterpret_cast<const uint32_t*>(q) + ((int64_t)r * n_q_heads + g * G) * 64 + t;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      lo[c] = g8 < G ? __ldg(q + ((int64_t)r * n_q_heads + g * G + g8) * 16 + t * 4 + c) : make_uint4(0, 0, 0, 0);
-      hi[c] = g8 + 8 < G ? __ldg(q + ((int64_t)r * n_q_heads + g * G + g8 + 8) * 16 + t * 4 + c) : make_uint4(0, 0, 0, 0);
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      qa[2 * c][0] = lo[c].x; qa[2 * c][1] = hi[c].x; qa[2 * c][2] = lo[c].y; qa[2 * c][3] = hi[c].y;
-      qa[2 * c + 1][0] = lo[c].z; qa[2 * c + 1][1] = hi[c].z; qa[2 * c + 1][2] = lo[c].w; qa[2 * c + 1][3] = hi[c].w;
+    for (int ks = 0; ks < 8; ++ks) {
+      qa[ks][0] = g8 < G ? __ldg(q32 + g8 * 64 + ks * 8) : 0u;
+      qa[ks][2] = g8 < G ? __ldg(q32 + g8 * 64 + ks * 8 + 4) : 0u;
+      qa[ks][1] = RW == 2 && g8 + 8 < G ? __ldg(q32 + (g8 + 8) * 64 + ks * 8) : 0u;
+      qa[ks][3] = RW == 2 && g8 + 8 < G ? __ldg(q32 + (g8 + 8) * 64 + ks * 8 + 4) : 0u;
     }
   }
-
   float oacc[16][4];
 #pragma unroll
   for (int nt = 0; nt < 16; ++nt)
@@ -290,33 +327,26 @@ __global__ void __launch_bounds__(kDecThreads) decode_tc_kernel(
     for (int x = 0; x < 4; ++x) oacc[nt][x] = 0.f;
   float m_ref[2] = {-INFINITY, -INFINITY}, l_part[2] = {0.f, 0.f};  // rows g8 and g8 + 8
 
-  for (int32_t k0 = warp * 16; k0 < n; k0 += (kDecThreads / 32) * 16) {
-    // every load of the trip is requested before the first use; rows past the end repeat the last one (weight 0)
-    uint4 kr[2][4], vr[4][2];
-#pragma unroll
-    for (int tl = 0; tl < 2; ++tl) {
-      const uint4* row = kc + ((j0 + min(k0 + 8 * tl + g8, n - 1)) * n_kv_heads + g) * 16 + t * 4;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) kr[tl][c] = ldg16_stream(row + c);
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {  // keys 2t, 2t+1, 8+2t, 9+2t of the trip
-      const int32_t key = k0 + (i >> 1) * 8 + 2 * t + (i & 1);
-      const uint4* row = vc + ((j0 + min(key, n - 1)) * n_kv_heads + g) * 16 + g8 * 2;
-      vr[i][0] = ldg16_stream(row);
-      vr[i][1] = ldg16_stream(row + 1);
-    }
-    // S for the two tiles of 8 keys
+  // ldmatrix: lane l addresses row l % 8 (+ 8 for the third and fourth matrix of K, the second and fourth of V)
+  const uint32_t k_off = (uint32_t)((lane & 7) + 8 * (lane >> 4)) * kClRow + ((lane >> 3) & 1) * 16;
+  const uint32_t v_off = (uint32_t)(16 + (lane & 7) + 8 * ((lane >> 3) & 1)) * kClRow + (lane >> 4) * 16;
+  for (int32_t trip = 0; trip < n_trips; ++trip) {
+    const int32_t k0 = warp * 16 + trip * (W * 16);
+    if constexpr (ST > 1) fetch(trip + ST - 1);
+    asm volatile("cp.async.wait_group %0;" ::"n"(ST - 1) : "memory");
+    __syncwarp();
+    const uint32_t st = ring + (uint32_t)(trip % ST) * kClStageBytes;
     float sc[2][4];
 #pragma unroll
-    for (int tl = 0; tl < 2; ++tl) {
+    for (int tl = 0; tl < 2; ++tl)
 #pragma unroll
       for (int x = 0; x < 4; ++x) sc[tl][x] = 0.f;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        dec_mma(sc[tl], qa[2 * c], kr[tl][c].x, kr[tl][c].y);
-        dec_mma(sc[tl], qa[2 * c + 1], kr[tl][c].z, kr[tl][c].w);
-      }
+    for (int ks = 0; ks < 8; ++ks) {
+      uint32_t b[4];
+      dec_ldsm(st + k_off + ks * 32, b);
+      dec_mma(sc[0], qa[ks], b[0], b[1]);
+      dec_mma(sc[1], qa[ks], b[2], b[3]);
     }
     // log2 units; keys past the end weigh nothing.  sc[tl][0..1]: row g8, keys 2t, 2t+1 of tile tl; [2..3]: row g8 + 8
 #pragma unroll
@@ -326,9 +356,9 @@ __global__ void __launch_bounds__(kDecThreads) decode_tc_kernel(
         const int32_t key = k0 + 8 * tl + 2 * t + (x & 1);
         sc[tl][x] = key < n ? sc[tl][x] * scale_log2 : -INFINITY;
       }
-    uint32_t pa[4];
+    uint32_t pa[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-    for (int rw = 0; rw < 2; ++rw) {
+    for (int rw = 0; rw < RW; ++rw) {
       float mx = fmaxf(fmaxf(sc[0][2 * rw], sc[0][2 * rw + 1]), fmaxf(sc[1][2 * rw], sc[1][2 * rw + 1]));
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
@@ -348,69 +378,116 @@ __global__ void __launch_bounds__(kDecThreads) decode_tc_kernel(
       pa[rw] = dec_pack_bf16(p00, p01);      // k slots 2t, 2t+1: keys 2t, 2t+1 of tile 0
       pa[2 + rw] = dec_pack_bf16(p10, p11);  // k slots 2t+8, 2t+9: the same keys of tile 1
     }
-    // O += P V
-    const uint32_t* x0 = reinterpret_cast<const uint32_t*>(vr[0]);
-    const uint32_t* y0 = reinterpret_cast<const uint32_t*>(vr[1]);
-    const uint32_t* x1 = reinterpret_cast<const uint32_t*>(vr[2]);
-    const uint32_t* y1 = reinterpret_cast<const uint32_t*>(vr[3]);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      dec_mma(oacc[2 * j], pa, __byte_perm(x0[j], y0[j], 0x5410), __byte_perm(x1[j], y1[j], 0x5410));
-      dec_mma(oacc[2 * j + 1], pa, __byte_perm(x0[j], y0[j], 0x7632), __byte_perm(x1[j], y1[j], 0x7632));
+    for (int nt = 0; nt < 16; nt += 2) {
+      uint32_t b[4];
+      dec_ldsm_t(st + v_off + nt * 16, b);
+      dec_mma(oacc[nt], pa, b[0], b[1]);
+      dec_mma(oacc[nt + 1], pa, b[2], b[3]);
     }
+    __syncwarp();  // every lane has read the stage before the next fetch overwrites it
+    if constexpr (ST == 1) fetch(trip + 1);
   }
-  // a row's sum over its four threads; then the warps' results side by side in shared memory
+
+  // the warps' results side by side in shared memory (a warp's over its own ring, which nobody else reads)
 #pragma unroll
-  for (int rw = 0; rw < 2; ++rw) {
+  for (int rw = 0; rw < RW; ++rw) {
     l_part[rw] += __shfl_xor_sync(0xffffffffu, l_part[rw], 1);
     l_part[rw] += __shfl_xor_sync(0xffffffffu, l_part[rw], 2);
+    if (t == 0) {
+      s_ml[warp][g8 + 8 * rw][0] = m_ref[rw];
+      s_ml[warp][g8 + 8 * rw][1] = l_part[rw];
+    }
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncwarp();
+  constexpr int LD = D + 8;  // rows start eight banks apart: the 8-byte stores of a half-warp do not collide
+  {
+    float* s_o = reinterpret_cast<float*>(cl_smem + warp * kWarpBytes);  // [R][LD]
 #pragma unroll
-  for (int nt = 0; nt < 16; ++nt)
+    for (int nt = 0; nt < 16; ++nt)
 #pragma unroll
-    for (int x = 0; x < 4; ++x) s_o[warp][g8 + 8 * (x >> 1)][t * 33 + (x & 1) * 16 + nt] = oacc[nt][x];  // d = 32t + 16(x&1) + nt
-  if (t == 0) {
-    s_ml[warp][g8][0] = m_ref[0];
-    s_ml[warp][g8][1] = l_part[0];
-    s_ml[warp][g8 + 8][0] = m_ref[1];
-    s_ml[warp][g8 + 8][1] = l_part[1];
+      for (int rw = 0; rw < RW; ++rw)
+        *reinterpret_cast<float2*>(s_o + (g8 + 8 * rw) * LD + nt * 8 + 2 * t) = make_float2(oacc[nt][2 * rw], oacc[nt][2 * rw + 1]);
   }
   __syncthreads();
-  for (int32_t x = tid; x < G * D; x += kDecThreads) {
-    const int32_t h = x / D, c = x % D;
-    float m_all = -INFINITY;
+  if (C > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  const int32_t cols = D / (int32_t)C;  // columns of every head that each CTA of the cluster finishes
+  // one thread per four columns of a head
+  for (int32_t x = tid; x < G * (D / 4); x += kThreads) {
+    const int32_t h = x / (D / 4), c = 4 * (x % (D / 4));
+    float m_w[W], m_all = -INFINITY;
 #pragma unroll
-    for (int w = 0; w < kDecThreads / 32; ++w)
-      if (s_ml[w][h][1] > 0.f) m_all = fmaxf(m_all, s_ml[w][h][0]);
+    for (int w = 0; w < W; ++w) {
+      m_w[w] = s_ml[w][h][1] > 0.f ? s_ml[w][h][0] : -INFINITY;
+      m_all = fmaxf(m_all, m_w[w]);
+    }
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    float l = 0.f;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      const float wgt = m_w[w] > -INFINITY ? dec_ex2(m_w[w] - m_all) : 0.f;
+      const float4 v4 = *reinterpret_cast<const float4*>(cl_smem + w * kWarpBytes + (h * LD + c) * 4);
+      a.x = fmaf(wgt, v4.x, a.x); a.y = fmaf(wgt, v4.y, a.y); a.z = fmaf(wgt, v4.z, a.z); a.w = fmaf(wgt, v4.w, a.w);
+      l = fmaf(wgt, s_ml[w][h][1], l);
+    }
+    if (C == 1) {
+      const int64_t hq = (int64_t)r * n_q_heads + g * G + h;
+      const float inv = l > 0.f ? 1.f / l : 0.f;
+      *reinterpret_cast<uint2*>(o + hq * D + c) = make_uint2(dec_pack_bf16(a.x * inv, a.y * inv), dec_pack_bf16(a.z * inv, a.w * inv));
+      if (c == 0 && lse) lse[hq] = l > 0.f ? (m_all + log2f(l)) * 0.6931471805599453f : -INFINITY;
+    } else {
+      const uint32_t to = (uint32_t)(c / cols);
+      asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dec_mapa(s_part + ((int32_t)rank * G + h) * cols + c % cols, to)),
+                   "f"(a.x), "f"(a.y), "f"(a.z), "f"(a.w) : "memory");
+      if (c % cols == 0)
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dec_mapa(s_pml[rank][h], to)), "f"(m_all), "f"(l) : "memory");
+    }
+  }
+  if (C == 1) return;
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  // four threads per output value, each over every fourth CTA's share (G * cols * 4 is a multiple of 32: whole warps)
+  const int32_t part = tid & 3;
+  for (int32_t x = tid; x < G * cols * 4; x += kThreads) {
+    const int32_t h = (x >> 2) / cols, c = (x >> 2) % cols;
+    float m_all = -INFINITY, mi[kClMax / 4], li[kClMax / 4];
+#pragma unroll
+    for (int k = 0; k < kClMax / 4; ++k) {
+      const int32_t i = part + 4 * k;
+      const float2 ml = i < (int32_t)C ? *reinterpret_cast<const float2*>(s_pml[i][h]) : make_float2(0.f, 0.f);
+      li[k] = ml.y;
+      mi[k] = ml.y > 0.f ? ml.x : -INFINITY;
+      m_all = fmaxf(m_all, mi[k]);
+    }
+    m_all = fmaxf(m_all, __shfl_xor_sync(0xffffffffu, m_all, 1));
+    m_all = fmaxf(m_all, __shfl_xor_sync(0xffffffffu, m_all, 2));
     float a = 0.f, l = 0.f;
 #pragma unroll
-    for (int w = 0; w < kDecThreads / 32; ++w)
-      if (s_ml[w][h][1] > 0.f) {
-        const float wgt = dec_ex2(s_ml[w][h][0] - m_all);
-        a = fmaf(wgt, s_o[w][h][(c >> 5) * 33 + (c & 31)], a);
-        l = fmaf(wgt, s_ml[w][h][1], l);
+    for (int k = 0; k < kClMax / 4; ++k) {
+      if (mi[k] > -INFINITY) {
+        const float wgt = dec_ex2(mi[k] - m_all);
+        a = fmaf(wgt, s_part[((part + 4 * k) * G + h) * cols + c], a);
+        l = fmaf(wgt, li[k], l);
       }
-    const int32_t hq = g * G + h;
-    if (n_splits == 1) {
-      o[((int64_t)r * n_q_heads + hq) * D + c] = __float2bfloat16(l > 0.f ? a / l : 0.f);
-      if (c == 0 && lse) lse[(int64_t)r * n_q_heads + hq] = l > 0.f ? (m_all + log2f(l)) * 0.6931471805599453f : -INFINITY;
-    } else {
-      float* dst = part + (((int64_t)r * n_q_heads + hq) * n_splits + sp) * (D + 2);
-      dst[c] = a;
-      if (c == 0) {
-        dst[D] = m_all;
-        dst[D + 1] = l;
-      }
+    }
+    a += __shfl_xor_sync(0xffffffffu, a, 1);
+    l += __shfl_xor_sync(0xffffffffu, l, 1);
+    a += __shfl_xor_sync(0xffffffffu, a, 2);
+    l += __shfl_xor_sync(0xffffffffu, l, 2);
+    if (part == 0) {
+      const int64_t hq = (int64_t)r * n_q_heads + g * G + h;
+      o[hq * D + (int32_t)rank * cols + c] = __float2bfloat16(l > 0.f ? a / l : 0.f);
+      if (rank == 0 && c == 0 && lse) lse[hq] = l > 0.f ? (m_all + log2f(l)) * 0.6931471805599453f : -INFINITY;
     }
   }
 }
 
-// grid (H, n_req), D threads (D = 64 or 128): merges the chunks' partial results of one (request, head).  The
+// fp32: grid (H, n_req), D threads: merges the chunks' partial results of one (request, head).  The
 // chunks' weights 2^(m_s - m) are formed once, 128 chunks at a time, in shared memory; thread c then sums column c
 // with independent loads.
-template <typename T>
 __global__ void decode_merge_kernel(const float* __restrict__ part, int32_t n_q_heads, int32_t n_splits, int32_t D,
-                                    T* __restrict__ o, float* __restrict__ lse) {
+                                    float* __restrict__ o, float* __restrict__ lse) {
   __shared__ float s_w[128];
   __shared__ float s_red[4];
   __shared__ float s_m;
@@ -462,7 +539,7 @@ __global__ void decode_merge_kernel(const float* __restrict__ part, int32_t n_q_
   __syncthreads();
   l = 0.f;
   for (int32_t w = 0; w < n_warps; ++w) l += s_red[w];
-  o[((int64_t)r * n_q_heads + hq) * D + c] = (T)(l > 0.f ? a / l : 0.f);
+  o[((int64_t)r * n_q_heads + hq) * D + c] = l > 0.f ? a / l : 0.f;
   if (c == 0 && lse) lse[(int64_t)r * n_q_heads + hq] = l > 0.f ? (m_all + log2f(l)) * 0.6931471805599453f : -INFINITY;
 }
 
@@ -476,6 +553,64 @@ static void decode_split(int32_t n_req, int32_t max_kept, int32_t n_kv_heads, in
   c = (c + 7) / 8 * 8;
   *chunk = (int32_t)c;
   *n_splits = (int32_t)((std::max(1, max_kept) + c - 1) / c);
+}
+
+template <int RW, int W, int ST>
+static purekv_status launch_cluster_as(int32_t cl, cudaStream_t sm, const void* q, const void* kc, const void* vc,
+                                       const int32_t* cu_kept, int32_t n_req, int32_t H, int32_t Hkv, float scale_log2,
+                                       void* o, float* lse) {
+  auto kernel = decode_cluster_kernel<RW, W, ST>;
+  static std::atomic<uint64_t> smem_allowed{0}, wide_allowed{0};
+  const purekv_status st = allow_max_dynamic_smem(kernel, smem_allowed);
+  if (st != PUREKV_OK) return st;
+  if (cl > 8) {  // clusters of more than eight CTAs are opt-in, once per device
+    int dev = -1;
+    PK_CUDA(cudaGetDevice(&dev));
+    if (!(wide_allowed.load(std::memory_order_acquire) & (1ull << dev))) {
+      PK_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      wide_allowed.fetch_or(1ull << dev, std::memory_order_release);
+    }
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)cl, (unsigned)Hkv, (unsigned)n_req);
+  cfg.blockDim = dim3(W * 32);
+  cfg.dynamicSmemBytes = (size_t)W * cl_warp_bytes<RW, ST>();
+  cfg.stream = sm;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see griddepcontrol in the kernel
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cl;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  PK_CUDA(cudaLaunchKernelEx(&cfg, kernel, (const uint4*)q, (const uint4*)kc, (const uint4*)vc, cu_kept, H, Hkv, scale_log2,
+                             (__nv_bfloat16*)o, lse));
+  return PUREKV_OK;
+}
+
+template <int RW>
+static purekv_status launch_cluster(int32_t max_kept, cudaStream_t sm, const void* q, const void* kc, const void* vc,
+                                    const int32_t* cu_kept, int32_t n_req, int32_t H, int32_t Hkv, float scale_log2, void* o,
+                                    float* lse) {
+  // CTAs per cluster, measured over 1-256 requests of 1-500 000 rows: shares of down to 64 rows pay (128 rows in one CTA of
+  // eight warps are a single trip, and a cluster costs 1 us), as long as every CTA finds an SM of its own -- 128 CTAs for
+  // clusters of up to four, 64 beyond (clusters of 8 or 16 CTAs with all of an SM's memory do not fill the GPCs: two
+  // requests, 4 KV heads, 1664 rows: 7.2 us as 8 clusters of 8, 11.5 as 8 of 16).
+  const int64_t base = (int64_t)n_req * Hkv;
+  int32_t cl = 1;
+  if (max_kept > 128)
+    while (cl < kClMax && base * cl * 2 <= (cl * 2 >= 8 ? 64 : 128) && max_kept > 64 * cl) cl *= 2;
+  const int32_t share = (max_kept + cl - 1) / cl;
+  // Eight warps and the SM to themselves for CTAs that are alone on it (four requests of 20 000 rows: 41 against 47 us) or
+  // stream long shares (128 x 5000 rows: 167 against 174 us); otherwise two CTAs of four warps, so that one streams while
+  // the other starts or ends (128 requests of up to 700 rows: 39 against 52 us).  One stage when a share is a single trip.
+  const bool wide = share > 64 && (base * cl <= 148 || share > 2048);
+  if (wide)
+    return share <= 128 ? launch_cluster_as<RW, 8, 1>(cl, sm, q, kc, vc, cu_kept, n_req, H, Hkv, scale_log2, o, lse)
+                        : launch_cluster_as<RW, 8, 3>(cl, sm, q, kc, vc, cu_kept, n_req, H, Hkv, scale_log2, o, lse);
+  return share <= 64 ? launch_cluster_as<RW, 4, 1>(cl, sm, q, kc, vc, cu_kept, n_req, H, Hkv, scale_log2, o, lse)
+                     : launch_cluster_as<RW, 4, 3>(cl, sm, q, kc, vc, cu_kept, n_req, H, Hkv, scale_log2, o, lse);
 }
 
 template <typename T, int GP>
@@ -524,6 +659,13 @@ purekv_status purekv_decode_attention(const void* q, const void* k_cache, const 
   PK_REQUIRE(h_cu_kept[n_req] == 0 || (k_cache && v_cache), PUREKV_ERR_INVALID_ARG, "purekv_decode_attention: null cache");
   PK_REQUIRE(((uintptr_t)q | (uintptr_t)k_cache | (uintptr_t)v_cache | (uintptr_t)o) % 16 == 0, PUREKV_ERR_INVALID_ARG,
              "purekv_decode_attention: pointers must be 16-byte aligned");
+  const float scale = softmax_scale > 0.f ? softmax_scale : 1.f / sqrtf((float)head_dim);
+  const float scale_log2 = scale * 1.4426950408889634f;
+  cudaStream_t sm = (cudaStream_t)stream;
+  PK_REQUIRE(n_kv_heads <= 65535 && n_req <= 65535, PUREKV_ERR_UNSUPPORTED, "too many heads or requests");
+  if (dtype == PUREKV_BF16)
+    return G <= 8 ? launch_cluster<1>(max_kept, sm, q, k_cache, v_cache, cu_kept, n_req, n_q_heads, n_kv_heads, scale_log2, o, lse)
+                  : launch_cluster<2>(max_kept, sm, q, k_cache, v_cache, cu_kept, n_req, n_q_heads, n_kv_heads, scale_log2, o, lse);
   int32_t chunk, n_splits;
   decode_split(n_req, max_kept, n_kv_heads, &chunk, &n_splits);
   float* part = nullptr;
@@ -532,9 +674,6 @@ purekv_status purekv_decode_attention(const void* q, const void* k_cache, const 
                "purekv_decode_attention: workspace of %zu bytes is too small", ws_bytes);
     part = (float*)(((uintptr_t)ws + 255) & ~(uintptr_t)255);
   }
-  const float scale = softmax_scale > 0.f ? softmax_scale : 1.f / sqrtf((float)head_dim);
-  const float scale_log2 = scale * 1.4426950408889634f;
-  cudaStream_t sm = (cudaStream_t)stream;
   dim3 grid((unsigned)n_splits, (unsigned)n_kv_heads, (unsigned)n_req);
   const int GP = G <= 1 ? 1 : G <= 2 ? 2 : G <= 4 ? 4 : 8;
 #define PK_DECODE(T)                                                                                                     \
@@ -544,13 +683,7 @@ purekv_status purekv_decode_attention(const void* q, const void* k_cache, const 
     case 4: launch_decode<T, 4>(grid, sm, q, k_cache, v_cache, cu_kept, n_q_heads, n_kv_heads, chunk, scale_log2, o, lse, part, n_splits); break; \
     default: launch_decode<T, 8>(grid, sm, q, k_cache, v_cache, cu_kept, n_q_heads, n_kv_heads, chunk, scale_log2, o, lse, part, n_splits); break; \
   }
-  if (dtype == PUREKV_BF16) {
-    decode_tc_kernel<<<grid, kDecThreads, 0, sm>>>((const uint4*)q, (const uint4*)k_cache, (const uint4*)v_cache, cu_kept,
-                                                  n_q_heads, n_kv_heads, chunk, scale_log2, (__nv_bfloat16*)o, lse, part,
-                                                  n_splits);
-  } else {
-    PK_DECODE(float)
-  }
+  PK_DECODE(float)
 #undef PK_DECODE
   PK_CUDA(cudaGetLastError());
   if (n_splits > 1) {
@@ -564,11 +697,7 @@ purekv_status purekv_decode_attention(const void* q, const void* k_cache, const 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const float* part_c = part;
-    if (dtype == PUREKV_BF16)
-      PK_CUDA(cudaLaunchKernelEx(&cfg, decode_merge_kernel<__nv_bfloat16>, part_c, n_q_heads, n_splits, head_dim,
-                                 (__nv_bfloat16*)o, lse));
-    else
-      PK_CUDA(cudaLaunchKernelEx(&cfg, decode_merge_kernel<float>, part_c, n_q_heads, n_splits, head_dim, (float*)o, lse));
+    PK_CUDA(cudaLaunchKernelEx(&cfg, decode_merge_kernel, part_c, n_q_heads, n_splits, head_dim, (float*)o, lse));
     PK_CUDA(cudaGetLastError());
   }
   return PUREKV_OK;
