@@ -1,8 +1,9 @@
-"""ctypes binding of libpurekv.so: argument marshalling only.
+"""Binding of libpurekv.so: argument marshalling only.
 
 Every function here has the name of the C entry point it calls and passes torch
-tensors' device pointers straight through; no step of the method runs in Python or
-in torch.  torch supplies device memory and the current CUDA stream.  Importing
+tensors' device pointers straight through, the hot ones by way of the native module
+`_marshal`, the others with ctypes; no step of the method runs in Python or in
+torch.  torch supplies device memory and the current CUDA stream.  Importing
 this module raises if the compiled library is missing: there is no fallback path.
 """
 from __future__ import annotations
@@ -19,6 +20,7 @@ LIB_PATH = os.path.join(_HERE, "libpurekv.so")
 if not os.path.exists(LIB_PATH):
     raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2510_25600_b200.build`")
 _lib = C.CDLL(LIB_PATH)
+from . import _marshal  # noqa: E402  (after the library it calls; built with it)
 
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT, ERR_BAD_PLAN = range(7)
 BF16, FP32 = 0, 1
@@ -132,7 +134,8 @@ def _check(status: int, where: str) -> None:
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    # the current stream of the current device as an integer, without building a Stream object on every call
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -254,10 +257,9 @@ def purekv_st_sparse_prefill(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, 
         out = torch.empty_like(q)
     if ws is None and plan.info.ws_bytes > 0:
         ws = torch.empty(plan.info.ws_bytes, dtype=torch.uint8, device=q.device)
-    _check(_lib.purekv_st_sparse_prefill(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), _ptr(lse),
-                                         C.byref(batch.c), plan.buf.data_ptr(), C.byref(plan.info), h, k.shape[1], d,
-                                         _dtype_code(q), softmax_scale, _ptr(ws), 0 if ws is None else ws.numel(),
-                                         _ptr(status), _stream()),
+    _check(_marshal.purekv_st_sparse_prefill(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), _ptr(lse), batch.c,
+                                             plan.buf.data_ptr(), plan.info, h, k.shape[1], d, _dtype_code(q), softmax_scale,
+                                             _ptr(ws), 0 if ws is None else ws.numel(), _ptr(status), _stream()),
            "purekv_st_sparse_prefill")
     return out
 
@@ -277,8 +279,8 @@ def purekv_lowlayer_score(q: torch.Tensor, k: torch.Tensor, batch: Batch, window
         c_out = torch.empty((hkv, t), dtype=torch.float32, device=q.device)
     if ws is None:
         ws = torch.empty(purekv_score_ws_bytes(batch, window, h), dtype=torch.uint8, device=q.device)
-    _check(_lib.purekv_lowlayer_score(q.data_ptr(), k.data_ptr(), c_out.data_ptr(), C.byref(batch.c), window, h, hkv,
-                                      d, _dtype_code(q), softmax_scale, ws.data_ptr(), ws.numel(), _stream()),
+    _check(_marshal.purekv_lowlayer_score(q.data_ptr(), k.data_ptr(), c_out.data_ptr(), batch.c, window, h, hkv, d,
+                                          _dtype_code(q), softmax_scale, ws.data_ptr(), ws.numel(), _stream()),
            "purekv_lowlayer_score")
     return c_out
 
@@ -292,8 +294,8 @@ def purekv_lowlayer_score_lse(q: torch.Tensor, k: torch.Tensor, lse: torch.Tenso
     hkv = k.shape[1]
     if c_out is None:
         c_out = torch.empty((hkv, t), dtype=torch.float32, device=q.device)
-    _check(_lib.purekv_lowlayer_score_lse(q.data_ptr(), k.data_ptr(), lse.data_ptr(), c_out.data_ptr(), C.byref(batch.c),
-                                          window, h, hkv, d, _dtype_code(q), softmax_scale, _ptr(status), _stream()),
+    _check(_marshal.purekv_lowlayer_score_lse(q.data_ptr(), k.data_ptr(), lse.data_ptr(), c_out.data_ptr(), batch.c, window, h,
+                                              hkv, d, _dtype_code(q), softmax_scale, _ptr(status), _stream()),
            "purekv_lowlayer_score_lse")
     return c_out
 
@@ -314,9 +316,9 @@ def purekv_lowlayer_score_ex(q: torch.Tensor, k: torch.Tensor, batch: Batch, win
         c_out = torch.empty((hkv, t), dtype=torch.float32, device=q.device)
     if ws is None:
         ws = torch.empty(purekv_score_ex_ws_bytes(batch, obs_rows, pool, h, hkv), dtype=torch.uint8, device=q.device)
-    _check(_lib.purekv_lowlayer_score_ex(q.data_ptr(), k.data_ptr(), c_out.data_ptr(), C.byref(batch.c), window, obs_rows,
-                                         pool, h, hkv, d, _dtype_code(q), softmax_scale, ws.data_ptr(), ws.numel(),
-                                         _stream()), "purekv_lowlayer_score_ex")
+    _check(_marshal.purekv_lowlayer_score_ex(q.data_ptr(), k.data_ptr(), c_out.data_ptr(), batch.c, window, obs_rows, pool, h, hkv,
+                                             d, _dtype_code(q), softmax_scale, ws.data_ptr(), ws.numel(), _stream()),
+           "purekv_lowlayer_score_ex")
     return c_out
 
 
@@ -363,11 +365,10 @@ def purekv_select_topk(c: torch.Tensor, v: torch.Tensor, batch: Batch, budget: B
         idx_out = torch.empty((n_layers, hkv, budget.total_kept), dtype=torch.int32, device=v.device)
     if s_out is None and ws is None:
         ws = torch.empty(purekv_select_ws_bytes(batch, n_layers, hkv), dtype=torch.uint8, device=v.device)
-    _check(_lib.purekv_select_topk(c.data_ptr(), v.data_ptr(), v.stride(0), n_layers, C.byref(batch.c), budget.window,
-                                   budget.keep.data_ptr(), budget.h_keep.ctypes.data_as(_i32p),
-                                   budget.cu_kept.data_ptr(), budget.h_cu_kept.ctypes.data_as(_i32p), hkv, d,
-                                   _dtype_code(v), idx_out.data_ptr(), _ptr(s_out), _ptr(ws),
-                                   0 if ws is None else ws.numel(), _stream()), "purekv_select_topk")
+    _check(_marshal.purekv_select_topk(c.data_ptr(), v.data_ptr(), v.stride(0), n_layers, batch.c, budget.window,
+                                       budget.keep.data_ptr(), budget.h_keep, budget.cu_kept.data_ptr(), budget.h_cu_kept, hkv,
+                                       d, _dtype_code(v), idx_out.data_ptr(), _ptr(s_out), _ptr(ws),
+                                       0 if ws is None else ws.numel(), _stream()), "purekv_select_topk")
     return idx_out
 
 
@@ -404,10 +405,9 @@ def purekv_compact_kv(k: torch.Tensor, v: torch.Tensor, idx: torch.Tensor, batch
         k_out = torch.empty((n_layers, budget.total_kept, hkv, d), dtype=k.dtype, device=k.device)
     if v_out is None:
         v_out = torch.empty_like(k_out)
-    _check(_lib.purekv_compact_kv(k.data_ptr(), v.data_ptr(), k.stride(0), n_layers, idx.data_ptr(), C.byref(batch.c),
-                                  budget.cu_kept.data_ptr(), budget.h_cu_kept.ctypes.data_as(_i32p), hkv, d,
-                                  _dtype_code(k), k_out.data_ptr(), v_out.data_ptr(), k_out.stride(0), _stream()),
-           "purekv_compact_kv")
+    _check(_marshal.purekv_compact_kv(k.data_ptr(), v.data_ptr(), k.stride(0), n_layers, idx.data_ptr(), batch.c,
+                                      budget.cu_kept.data_ptr(), budget.h_cu_kept, hkv, d, _dtype_code(k), k_out.data_ptr(),
+                                      v_out.data_ptr(), k_out.stride(0), _stream()), "purekv_compact_kv")
     return k_out, v_out
 
 
@@ -424,15 +424,16 @@ def purekv_decode_attention(q: torch.Tensor, k_cache: torch.Tensor, v_cache: tor
     hkv = k_cache.shape[1]
     if out is None:
         out = torch.empty_like(q)
-    kept = np.diff(budget.h_cu_kept)
-    need = purekv_decode_ws_bytes(b, int(kept.max()) if len(kept) else 0, h, hkv, d)
-    if need and (ws is None or ws.numel() * ws.element_size() < need):
-        ws = torch.empty(need, dtype=torch.uint8, device=q.device)
-    _check(_lib.purekv_decode_attention(q.data_ptr(), k_cache.data_ptr(), v_cache.data_ptr(), out.data_ptr(), _ptr(lse),
-                                        budget.cu_kept.data_ptr(), budget.h_cu_kept.ctypes.data_as(_i32p), b, h, hkv, d,
-                                        _dtype_code(q), softmax_scale, _ptr(ws),
-                                        ws.numel() * ws.element_size() if ws is not None else 0, _stream()),
-           "purekv_decode_attention")
+    call = lambda w: _marshal.purekv_decode_attention(
+        q.data_ptr(), k_cache.data_ptr(), v_cache.data_ptr(), out.data_ptr(), _ptr(lse), budget.cu_kept.data_ptr(), b,
+        budget.h_cu_kept, h, hkv, d, _dtype_code(q), softmax_scale, _ptr(w), 0 if w is None else w.numel() * w.element_size(),
+        _stream())
+    status = call(ws)
+    if status == ERR_WORKSPACE:  # (fp32 rows) none given, or too small
+        kept = np.diff(budget.h_cu_kept)
+        need = purekv_decode_ws_bytes(b, int(kept.max()), h, hkv, d)
+        status = call(torch.empty(need, dtype=torch.uint8, device=q.device))
+    _check(status, "purekv_decode_attention")
     return out
 
 

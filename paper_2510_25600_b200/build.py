@@ -1,4 +1,5 @@
-"""Builds libpurekv.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a.
+"""Builds libpurekv.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _marshal.so, the Python module that
+passes arguments to it.
 
     python -m paper_2510_25600_b200.build [--force] [--verbose]
 """
@@ -7,11 +8,13 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(_HERE), "include")
 LIB = os.path.join(_HERE, "libpurekv.so")
+MARSHAL = os.path.join(_HERE, "_marshal.so")
 SOURCES = ["plan.cu", "compact.cu", "decode.cu", "select.cu", "score.cu", "score_tc.cu", "prefill.cu", "prefill_simt.cu", "prefill_tc.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--use_fast_math=false"]
@@ -57,6 +60,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("nvcc failed")
     if force or procs or _stale(LIB, objs):
         subprocess.check_call([_nvcc(), "-shared", "-o", LIB, *objs, "-gencode", "arch=compute_100a,code=sm_100a"])
+    src = os.path.join(CSRC, "marshal.cpp")
+    if force or _stale(MARSHAL, [src, LIB] + headers):
+        # found beside the module at run time: one copy of the library, whether it is loaded through this or by path
+        subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", INCLUDE,
+                               src, "-o", MARSHAL, "-L", _HERE, "-l:libpurekv.so", "-Wl,-rpath,$ORIGIN"])
     return LIB
 
 
