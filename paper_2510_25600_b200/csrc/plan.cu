@@ -11,7 +11,6 @@
 #include <cstring>
 #include <mutex>
 #include <string>
-#include <queue>
 #include <vector>
 
 #include "common.cuh"
@@ -150,12 +149,11 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
   const bool odd = (G & 1) != 0;
   const int32_t overhead = 6, split_extra = 14;
   const int32_t nq = (int32_t)qtiles.size();
-  auto halves = [&](int32_t first, int32_t last) {  // cost of entries [first, last)
-    int32_t c = 0;
-    for (int32_t i = first; i < last; ++i)
-      c += ((((entries[i].x >> 2) & 3) == 3) ? 2 : 1) * ((entries[i].x & 3) == kTileGeneral ? 5 : 4);
-    return c;
-  };
+  // running cost of the entries: a run's cost is a difference
+  std::vector<int32_t> pre(entries.size() + 1, 0);
+  for (size_t i = 0; i < entries.size(); ++i)
+    pre[i + 1] = pre[i] + ((((entries[i].x >> 2) & 3) == 3) ? 2 : 1) * ((entries[i].x & 3) == kTileGeneral ? 5 : 4);
+  auto halves = [&](int32_t first, int32_t last) { return pre[last] - pre[first]; };  // cost of entries [first, last)
   // The union of two runs of entries (of two query tiles' lists) in key-tile order: its cost and length; the entry
   // pairs go to `out` if given.
   auto merge_lists = [&](int32_t ia, int32_t ea, int32_t ib, int32_t eb, std::vector<int2>* out, int32_t* count) {
@@ -182,39 +180,51 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
   };
   // partner[i]: the tile that shares tile i's odd-head units (i leads the twin), -2 if tile i is the second of a
   // twin, -1 if it stays alone.  Twins have the same number of chunks, and a merged chunk may be a quarter longer
-  // than the cap on a chunk.
-  std::vector<int32_t> partner;
+  // than the cap on a chunk.  twin_cost: the merged chunks' costs, leader by leader, chunk by chunk.
+  std::vector<int32_t> partner, twin_cost;
+  struct Merged { int32_t n = -1, cost = 0; };
+  std::vector<Merged> whole((size_t)nq);  // tile i's whole list merged with tile i + 1's: the same under every cap that leaves both whole
+  auto merge_chunk = [&](int32_t i, int32_t c, int32_t nch) {
+    Merged m;
+    if (nch == 1 && whole[i].n >= 0) return whole[i];
+    int32_t a0, a1, b0, b1;
+    chunk_range(qtiles[i], c, nch, &a0, &a1);
+    chunk_range(qtiles[i + 1], c, nch, &b0, &b1);
+    m.cost = merge_lists(a0, a1, b0, b1, nullptr, &m.n);
+    if (nch == 1) whole[i] = m;
+    return m;
+  };
   auto find_twins = [&](int32_t l_max) {
     partner.assign((size_t)nq, -1);
+    twin_cost.clear();
     if (!odd) return;
     for (int32_t i = 0; i + 1 < nq; ++i) {
       const QTile &a = qtiles[i], &b = qtiles[i + 1];
       const int32_t nch = chunks_of(a, l_max);
       if (partner[i] != -1 || a.req_start != b.req_start || nch != chunks_of(b, l_max)) continue;
+      const size_t at = twin_cost.size();
       bool fits = true;
       for (int32_t c = 0; c < nch && fits; ++c) {
-        int32_t a0, a1, b0, b1, n = 0;
-        chunk_range(a, c, nch, &a0, &a1);
-        chunk_range(b, c, nch, &b0, &b1);
-        merge_lists(a0, a1, b0, b1, nullptr, &n);
-        fits = n <= l_max + l_max / 4;
+        const Merged m = merge_chunk(i, c, nch);
+        twin_cost.push_back(m.cost);
+        fits = m.n <= l_max + l_max / 4;
       }
-      if (!fits) continue;
+      if (!fits) {
+        twin_cost.resize(at);
+        continue;
+      }
       partner[i] = i + 1;
       partner[i + 1] = -2;
     }
   };
-  struct Item { Unit u; int32_t cost; };
-  std::vector<Item> items;
+  std::vector<Unit> items;
+  std::vector<int32_t> item_cost;
   std::vector<int2> twin_entries;
   std::vector<int32_t> part_of, counter_of;  // per query tile: first workspace slot and merge counter, -1 if unsplit
   int32_t counters = 0, mc = 1;
   int64_t slots = 0;
-  // the units when no chunk of a list may be longer than l_max entries
+  // the units when no chunk of a list may be longer than l_max entries, by decreasing cost (equal costs as they come)
   auto make_items = [&](int32_t l_max) {
-    items.clear();
-    twin_entries.clear();
-    counters = 0; mc = 1; slots = 0;
     find_twins(l_max);
     part_of.assign((size_t)nq, -1);
     counter_of.assign((size_t)nq, -1);
@@ -228,13 +238,14 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
         counters += H;
       }
     }
+    size_t twin_at = 0;
     for (int32_t qi = 0; qi < nq; ++qi) {
       const QTile& q = qtiles[qi];
       const int32_t nch = chunks_of(q, l_max);
       for (int32_t c = 0; c < nch; ++c) {
         int32_t a, e;
         chunk_range(q, c, nch, &a, &e);
-        const int32_t cost = halves(a, e) + overhead + (nch > 1 ? split_extra : 0);
+        const int32_t extra = overhead + (nch > 1 ? split_extra : 0), cost = halves(a, e) + extra;
         for (int32_t pr = 0; pr < n_pairs; ++pr) {
           if (partner[qi] != -1 && pr % ppg == ppg - 1) continue;  // the odd head goes into a twin unit
           Unit u = {};
@@ -243,14 +254,16 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
           u.pair = pr; u.chunk = c; u.n_chunks = nch;
           u.part_base = part_of[qi]; u.counter_base = counter_of[qi];
           u.part_base1 = u.counter_base1 = -1;
-          items.push_back({u, cost});
+          items.push_back(u);
+          item_cost.push_back(cost);
         }
         if (partner[qi] >= 0) {
           const QTile& q1 = qtiles[partner[qi]];
           int32_t a1, e1, n = 0;
           chunk_range(q1, c, nch, &a1, &e1);
           const int32_t at = (int32_t)(entries.size() + twin_entries.size());
-          const int32_t cost2 = merge_lists(a, e, a1, e1, &twin_entries, &n) + overhead + (nch > 1 ? split_extra : 0);
+          merge_lists(a, e, a1, e1, &twin_entries, &n);
+          const int32_t cost2 = twin_cost[twin_at++] + extra;
           for (int32_t g = 0; g < Hkv; ++g) {
             Unit u = {};
             u.q_start = q.q_start; u.q_rows = q.q_rows; u.req_start = q.req_start;
@@ -259,42 +272,63 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
             u.pair = g * ppg + ppg - 1; u.chunk = c; u.n_chunks = nch;
             u.part_base = part_of[qi]; u.counter_base = counter_of[qi];
             u.part_base1 = part_of[partner[qi]]; u.counter_base1 = counter_of[partner[qi]];
-            items.push_back({u, cost2});
+            items.push_back(u);
+            item_cost.push_back(cost2);
           }
         }
       }
     }
-    std::stable_sort(items.begin(), items.end(), [](const Item& x, const Item& y) { return x.cost > y.cost; });
+    // counting sort (costs are small numbers: at most 80 entries of 10, and the overheads)
+    int32_t top = 0;
+    for (int32_t c : item_cost) top = std::max(top, c);
+    std::vector<int32_t> at((size_t)top + 2, 0);  // at[c]: where the units of cost c begin
+    for (int32_t c : item_cost) ++at[c];
+    int32_t run = 0;
+    for (int32_t c = top; c >= 0; --c) {
+      const int32_t n = at[c];
+      at[c] = run;
+      run += n;
+    }
+    units.resize(items.size());
+    for (size_t i = 0; i < items.size(); ++i) units[at[item_cost[i]]++] = items[i];
   };
-  // the time the last CTA ends when the CTAs draw units of these costs in decreasing order, each as it becomes free
-  std::vector<int32_t> costs;
-  auto makespan = [&](int32_t l_max) {
-    costs.clear();
+  // The time the last CTA ends when the CTAs draw units in decreasing order of cost, each as it becomes free; anything
+  // above `limit` is answered as soon as it is known.  Units of one cost and CTAs free at the same time are counted, not
+  // listed: the earliest free time only grows, so one pass over the times serves all units.
+  std::vector<int32_t> n_of_cost, n_free;
+  auto makespan = [&](int32_t l_max, int64_t limit) {
     find_twins(l_max);
+    n_of_cost.clear();
+    int64_t total = 0;
+    auto add = [&](int32_t cost, int32_t n) {
+      if ((size_t)cost >= n_of_cost.size()) n_of_cost.resize((size_t)cost + 1, 0);
+      n_of_cost[cost] += n;
+      total += (int64_t)cost * n;
+    };
+    size_t twin_at = 0;
     for (int32_t qi = 0; qi < nq; ++qi) {
       const QTile& q = qtiles[qi];
-      const int32_t nch = chunks_of(q, l_max);
+      const int32_t nch = chunks_of(q, l_max), extra = overhead + (nch > 1 ? split_extra : 0);
       for (int32_t c = 0; c < nch; ++c) {
         int32_t a, e;
         chunk_range(q, c, nch, &a, &e);
-        const int32_t extra = overhead + (nch > 1 ? split_extra : 0);
-        costs.insert(costs.end(), (size_t)(partner[qi] != -1 ? n_pairs - Hkv : n_pairs), halves(a, e) + extra);
-        if (partner[qi] >= 0) {
-          int32_t a1, e1, n = 0;
-          chunk_range(qtiles[partner[qi]], c, nch, &a1, &e1);
-          costs.insert(costs.end(), (size_t)Hkv, merge_lists(a, e, a1, e1, nullptr, &n) + extra);
-        }
+        add(halves(a, e) + extra, partner[qi] != -1 ? n_pairs - Hkv : n_pairs);
+        if (partner[qi] >= 0) add(twin_cost[twin_at++] + extra, Hkv);
       }
     }
-    std::sort(costs.begin(), costs.end(), std::greater<int32_t>());
-    std::priority_queue<int64_t, std::vector<int64_t>, std::greater<int64_t>> load;
-    for (int32_t c = 0; c < n_ctas; ++c) load.push(0);
-    int64_t end = 0;
-    for (int32_t cost : costs) {
-      const int64_t t = load.top() + cost;
-      load.pop();
-      load.push(t);
-      end = std::max(end, t);
+    n_free.assign((size_t)(total / n_ctas) + n_of_cost.size() + 1, 0);  // CTAs that become free at each time
+    n_free[0] = n_ctas;
+    int64_t end = 0, now = 0;
+    for (int32_t cost = (int32_t)n_of_cost.size() - 1; cost > 0; --cost) {
+      for (int32_t m = n_of_cost[cost]; m > 0;) {
+        while (n_free[now] == 0) ++now;
+        const int32_t k = std::min(m, n_free[now]);
+        n_free[now] -= k;
+        n_free[now + cost] += k;
+        m -= k;
+        end = std::max(end, now + cost);
+        if (end > limit) return end;
+      }
     }
     return end;
   };
@@ -305,22 +339,47 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
   if ((int64_t)qtiles.size() * n_pairs < 12 * (int64_t)n_ctas) {
     int64_t t_best = -1;
     for (int32_t l_max : {64, 24, 12, 9, 7, 5}) {
-      const int64_t t = makespan(l_max);
+      const int64_t t = makespan(l_max, t_best < 0 ? INT64_MAX : t_best);
       if (t_best < 0 || t <= t_best) { t_best = t; l_best = l_max; }  // on a tie the finer cut
     }
   }
   make_items(l_best);
   entries.insert(entries.end(), twin_entries.begin(), twin_entries.end());
-  units.clear();
-  for (const Item& it : items) units.push_back(it.u);
   *n_counters = counters;
   *part_slots = slots * H;
   *max_chunks = mc;
 }
 
+// A plan on the host: its sections, and their layout in the buffer.
+struct HostPlan {
+  PlanHeader h;
+  int64_t total = 0;  // bytes
+  std::vector<QTile> qtiles;
+  std::vector<int32_t> order;
+  std::vector<int2> entries;
+  std::vector<uint32_t> masks;
+  std::vector<Unit> units;
+
+  void write(uint8_t* dst) const {  // total bytes; gaps between sections and the counters are zero
+    int64_t at = 0;
+    auto section = [&](int64_t off, const void* src, size_t bytes) {
+      memset(dst + at, 0, (size_t)(off - at));
+      if (bytes) memcpy(dst + off, src, bytes);
+      at = off + (int64_t)bytes;
+    };
+    section(0, &h, sizeof(h));
+    section(h.off_qtiles, qtiles.data(), qtiles.size() * sizeof(QTile));
+    section(h.off_order, order.data(), order.size() * 4);
+    section(h.off_entries, entries.data(), entries.size() * 8);
+    section(h.off_masks, masks.data(), masks.size() * 4);
+    section(h.off_units, units.data(), units.size() * sizeof(Unit));
+    section(total, nullptr, 0);
+  }
+};
+
 static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p, purekv_dtype dtype,
                                 int32_t head_dim, int32_t n_q_heads, int32_t n_kv_heads, int32_t n_ctas,
-                                purekv_plan_info* info, std::vector<uint8_t>& host) {
+                                purekv_plan_info* info, HostPlan& plan) {
   int tq, gk;  // rows per query tile; skip granularity in keys (the mask parameter `tile`)
   purekv_status st = check_params(b, p, dtype, head_dim, &tq, &gk);
   if (st != PUREKV_OK) return st;
@@ -339,14 +398,16 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
   const int64_t T = b->total_tokens;
   const int32_t wpr = std::max(1, tk / 32);  // mask words per row of a general tile
 
-  std::vector<QTile> qtiles;
-  std::vector<int2> entries;
-  std::vector<uint32_t> masks;
+  const int32_t gsh = 31 - __builtin_clz((unsigned)gk), tsh = 31 - __builtin_clz((unsigned)tk);  // gk and tk are powers of two
+  std::vector<QTile>& qtiles = plan.qtiles;
+  std::vector<int2>& entries = plan.entries;
+  std::vector<uint32_t>& masks = plan.masks;
   memset(info, 0, sizeof(*info));
 
   std::vector<int64_t> cnt, diff, cg;  // kept pairs per gk-key block of the current query tile
   std::vector<Span> spans, row_spans, merged;
   std::vector<char> blk_kept;
+  std::vector<int32_t> mask_of;  // per key tile of the current query tile: first word of its bit mask, or -1
   const bool coarse = (p->flags & PUREKV_FLAG_COARSE_BLOCKS) != 0 && !dense;
   std::vector<int32_t> row_off;
   for (int r = 0; r < b->n_req; ++r) {
@@ -360,6 +421,7 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
     cg.assign((size_t)nkt + 3, 0);
     const int32_t anchor_end = (int32_t)std::min<int64_t>(vis_end, npre + (int64_t)p->anchor_frames * n);  // exclusive
     // the token-level mask of row i as disjoint ascending spans of kept key positions
+    int32_t at_i = -2, at_f = 0, at_c = 0, at_y = 0, at_x = 0;  // frame, cell and its coordinates of the last visual row asked for
     auto token_spans = [&](int32_t i, std::vector<Span>& out) {
       out.clear();
       const bool visual = i >= npre && i < vis_end;
@@ -369,7 +431,14 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
       }
       spans.clear();
       if (anchor_end > 0) spans.push_back({0, std::min(i, anchor_end - 1)});  // prefix + first frame(s)
-      const int32_t f = (i - npre) / n, c = (i - npre) % n, y = c / gw, x = c % gw;
+      if (i == at_i + 1) {  // rows mostly come in order: step instead of dividing
+        if (++at_x == gw) { at_x = 0; ++at_y; }
+        if (++at_c == n) { at_c = at_y = at_x = 0; ++at_f; }
+      } else {
+        at_f = (i - npre) / n; at_c = (i - npre) % n; at_y = at_c / gw; at_x = at_c % gw;
+      }
+      at_i = i;
+      const int32_t f = at_f, y = at_y, x = at_x;
       const int32_t fs = npre + f * n;
       if (p->spatial_radius < 0) {
         spans.push_back({fs, i});  // the current frame, causal
@@ -395,7 +464,16 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
       if (p->local_window > 0) spans.push_back({std::max(npre, i - p->local_window + 1), i});  // the most recent positions
       if (p->atrous_dilation > 0)                                                             // every D-th position back
         for (int32_t j = i; j >= npre; j -= p->atrous_dilation) spans.push_back({j, j});
-      std::sort(spans.begin(), spans.end(), [](const Span& u, const Span& v) { return u.a < v.a; });
+      if (spans.size() <= 12) {  // a few spans, nearly in order: insertion
+        for (size_t x = 1; x < spans.size(); ++x) {
+          const Span sp = spans[x];
+          size_t y = x;
+          for (; y > 0 && spans[y - 1].a > sp.a; --y) spans[y] = spans[y - 1];
+          spans[y] = sp;
+        }
+      } else {
+        std::sort(spans.begin(), spans.end(), [](const Span& u, const Span& v) { return u.a < v.a; });
+      }
       int32_t ca = spans[0].a, cb = spans[0].b;
       for (size_t s = 1; s < spans.size(); ++s) {
         if (spans[s].a <= cb + 1) cb = std::max(cb, spans[s].b);
@@ -414,7 +492,7 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
       row_off.assign(1, 0);
       auto add_span = [&](int32_t a, int32_t bb) {  // inclusive, a <= bb
         row_spans.push_back({a, bb});
-        const int32_t ta = a / gk, tb = bb / gk;
+        const int32_t ta = a >> gsh, tb = bb >> gsh;
         if (ta == tb) { cnt[ta] += bb - a + 1; return; }
         cnt[ta] += (ta + 1) * gk - a;
         cnt[tb] += bb - tb * gk + 1;
@@ -422,7 +500,9 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
         diff[tb] -= gk;
       };
       // each row's kept keys as disjoint ascending spans (Sec. 3.2; App. A.3 for the local and atrous terms)
-      for (int32_t i = q0; i < q1; ++i) {
+      // (a tile of plain causal rows needs none: its counts follow from the diagonal alone)
+      const bool plain = dense || (!coarse && (q1 <= npre || q0 >= vis_end || npre == vis_end));
+      for (int32_t i = q0; i < q1 && !plain; ++i) {
         if (!coarse) {
           token_spans(i, merged);
           for (const Span& sp : merged) add_span(sp.a, sp.b);
@@ -458,10 +538,22 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
       qt.entry_begin = (int32_t)entries.size();
       qt.pad[0] = qt.pad[1] = 0;
       int64_t run = 0;
+      int32_t n_general = 0;  // tiles of this row of tiles with a bit mask
+      if (mask_of.size() < (size_t)kt_hi + 1) mask_of.resize((size_t)kt_hi + 1);
+      std::fill(mask_of.begin(), mask_of.begin() + kt_hi + 1, -1);
       for (int32_t kg = 0; kg <= kg_hi + 1; ++kg) {
         run += diff[kg];
         cg[kg] = cnt[kg] + run;
       }
+      if (plain)
+        for (int32_t kg = 0; kg <= kg_hi; ++kg) {
+          const int32_t j0 = kg * gk;
+          cg[kg] = (int64_t)(q1 - q0) * gk;
+          if (j0 + gk - 1 > q0) {
+            cg[kg] = 0;
+            for (int32_t i = std::max(q0, j0); i < q1; ++i) cg[kg] += std::min(gk, i - j0 + 1);
+          }
+        }
       info->tiles_causal += kg_hi + 1;
       for (int32_t kt = 0; kt <= kt_hi; ++kt) {
         int64_t c = 0;
@@ -483,27 +575,31 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
         if (c == full && j0 + tk <= len) cls = kTileFull;
         else if (c == causal) cls = kTileDiag;
         if (cls == kTileGeneral) {
-          // one bit per (row, key) of the tile, rows past q_rows stay zero
-          PK_REQUIRE(masks.size() + (size_t)tq * wpr < (size_t)INT32_MAX, PUREKV_ERR_UNSUPPORTED,
+          // one bit per (row, key) of the tile, rows past q_rows stay zero; the bits follow once the tile's masks are known
+          PK_REQUIRE(masks.size() + (size_t)n_general * tq * wpr + (size_t)tq * wpr < (size_t)INT32_MAX, PUREKV_ERR_UNSUPPORTED,
                      "mask table exceeds 2^31 words");
-          mask_at = (int32_t)masks.size();
-          masks.resize(masks.size() + (size_t)tq * wpr, 0u);
-          uint32_t* mw = masks.data() + mask_at;
-          for (int32_t i = q0; i < q1; ++i)
-            for (int32_t s = row_off[i - q0]; s < row_off[i - q0 + 1]; ++s) {
-              const int32_t a = std::max(row_spans[s].a, j0), bb = std::min(row_spans[s].b, j0 + tk - 1);
-              if (a > bb) continue;
-              const int32_t lo = a - j0, hi = bb - j0;  // bit range inside the tile row
-              uint32_t* rw = mw + (i - q0) * wpr;
+          mask_at = (int32_t)(masks.size() + (size_t)n_general++ * tq * wpr);
+        }
+        mask_of[kt] = mask_at;
+        entries.push_back(make_int2((kt << 4) | (half_mask << 2) | cls, mask_at));
+        info->pairs_kept += c;
+        (cls == kTileFull ? info->tiles_full : cls == kTileDiag ? info->tiles_diag : info->tiles_general)++;
+      }
+      if (n_general) {  // row by row, each span into the masks of the tiles it crosses
+        masks.resize(masks.size() + (size_t)n_general * tq * wpr, 0u);
+        for (int32_t i = q0; i < q1; ++i)
+          for (int32_t s = row_off[i - q0]; s < row_off[i - q0 + 1]; ++s) {
+            const int32_t a = row_spans[s].a, bb = row_spans[s].b;
+            for (int32_t kt = a >> tsh; kt <= bb >> tsh; ++kt) {
+              if (mask_of[kt] < 0) continue;
+              const int32_t j0 = kt << tsh, lo = std::max(a - j0, 0), hi = std::min(bb - j0, tk - 1);  // bit range inside the tile row
+              uint32_t* rw = masks.data() + mask_of[kt] + (size_t)(i - q0) * wpr;
               for (int32_t w = lo >> 5; w <= (hi >> 5); ++w) {
                 const int32_t b0 = std::max(lo - 32 * w, 0), b1 = std::min(hi - 32 * w, 31);
                 rw[w] |= (b1 - b0 == 31) ? 0xFFFFFFFFu : (((1u << (b1 - b0 + 1)) - 1u) << b0);
               }
             }
-        }
-        entries.push_back(make_int2((kt << 4) | (half_mask << 2) | cls, mask_at));
-        info->pairs_kept += c;
-        (cls == kTileFull ? info->tiles_full : cls == kTileDiag ? info->tiles_diag : info->tiles_general)++;
+          }
       }
       qt.entry_count = (int32_t)entries.size() - qt.entry_begin;
       info->max_list = std::max(info->max_list, qt.entry_count);
@@ -511,13 +607,14 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
     }
   }
   const int32_t nq = (int32_t)qtiles.size();
-  std::vector<int32_t> order((size_t)nq);
+  std::vector<int32_t>& order = plan.order;
+  order.resize((size_t)nq);
   for (int32_t i = 0; i < nq; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(),
                    [&](int32_t u, int32_t v) { return qtiles[u].entry_count > qtiles[v].entry_count; });
 
   // tensor-core plans carry the persistent kernel's schedule
-  std::vector<Unit> units;
+  std::vector<Unit>& units = plan.units;
   int32_t n_counters = 0, max_chunks = 1;
   int64_t part_slots = 0;
   if (tq == 128 && nq > 0) {
@@ -526,7 +623,7 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
     n_ctas = 0;
   }
 
-  PlanHeader h;
+  PlanHeader& h = plan.h;
   memset(&h, 0, sizeof(h));
   h.magic = kPlanMagic;
   h.tile_q = tq;
@@ -551,15 +648,7 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
   // the merge counters, then the kernel's two scheduling counters; all start at zero and the kernel leaves them so
   const int64_t total = h.off_counters + align16(((int64_t)n_counters + 2) * 4);
 
-  host.assign((size_t)total, 0);
-  memcpy(host.data(), &h, sizeof(h));
-  if (nq) memcpy(host.data() + h.off_qtiles, qtiles.data(), (size_t)nq * sizeof(QTile));
-  if (nq) memcpy(host.data() + h.off_order, order.data(), (size_t)nq * 4);
-  if (!entries.empty()) memcpy(host.data() + h.off_entries, entries.data(), entries.size() * 8);
-  if (!masks.empty()) memcpy(host.data() + h.off_masks, masks.data(), masks.size() * 4);
-  if (!units.empty()) {
-    memcpy(host.data() + h.off_units, units.data(), units.size() * sizeof(Unit));
-  }
+  plan.total = total;
 
   info->tile_q = tq;
   info->tile_k = gk;
@@ -579,21 +668,21 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
 size_t purekv_plan_bytes(const purekv_batch* b, const purekv_st_params* p, purekv_dtype dtype, int32_t head_dim,
                          int32_t n_q_heads, int32_t n_kv_heads, int32_t n_ctas) {
   purekv_plan_info info;
-  std::vector<uint8_t> host;
+  HostPlan host;
   if (build_plan(b, p, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, &info, host) != PUREKV_OK) return 0;
-  return host.size();
+  return (size_t)host.total;
 }
 
 purekv_status purekv_plan_build_host(const purekv_batch* b, const purekv_st_params* p, purekv_dtype dtype,
                                      int32_t head_dim, int32_t n_q_heads, int32_t n_kv_heads, int32_t n_ctas,
                                      void* h_plan, size_t plan_bytes, purekv_plan_info* info) {
   PK_REQUIRE(h_plan, PUREKV_ERR_INVALID_ARG, "h_plan is null");
-  std::vector<uint8_t> host;
+  HostPlan host;
   purekv_status st = build_plan(b, p, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, info, host);
   if (st != PUREKV_OK) return st;
-  PK_REQUIRE(host.size() <= plan_bytes, PUREKV_ERR_WORKSPACE, "plan needs %zu bytes, buffer has %zu", host.size(),
+  PK_REQUIRE((size_t)host.total <= plan_bytes, PUREKV_ERR_WORKSPACE, "plan needs %zu bytes, buffer has %zu", (size_t)host.total,
              plan_bytes);
-  memcpy(h_plan, host.data(), host.size());
+  host.write((uint8_t*)h_plan);
   return PUREKV_OK;
 }
 
@@ -601,11 +690,13 @@ purekv_status purekv_plan_build(const purekv_batch* b, const purekv_st_params* p
                                 int32_t head_dim, int32_t n_q_heads, int32_t n_kv_heads, int32_t n_ctas, void* plan,
                                 size_t plan_bytes, purekv_plan_info* info, void* stream) {
   PK_REQUIRE(plan, PUREKV_ERR_INVALID_ARG, "plan is null");
-  std::vector<uint8_t> host;
-  purekv_status st = build_plan(b, p, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, info, host);
+  HostPlan built;
+  purekv_status st = build_plan(b, p, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, info, built);
   if (st != PUREKV_OK) return st;
-  PK_REQUIRE(host.size() <= plan_bytes, PUREKV_ERR_WORKSPACE, "plan needs %zu bytes, buffer has %zu", host.size(),
+  PK_REQUIRE((size_t)built.total <= plan_bytes, PUREKV_ERR_WORKSPACE, "plan needs %zu bytes, buffer has %zu", (size_t)built.total,
              plan_bytes);
+  std::vector<uint8_t> host((size_t)built.total);
+  built.write(host.data());
   cudaStream_t s = (cudaStream_t)stream;
   PK_CUDA(cudaMemcpyAsync(plan, host.data(), host.size(), cudaMemcpyHostToDevice, s));
   PK_CUDA(cudaStreamSynchronize(s));
