@@ -16,8 +16,8 @@
 //   warps 0-7   one thread per query row of a slot (registers raised with setmaxnreg at the expense of
 //               warps 8-11): the row of S from TMEM into registers, the
 //               tile's predicate (none / causal / bit mask), online softmax in the log2 domain against a
-//               reference that moves only when exp2 would overflow (then O is rescaled), a share of the
-//               exponentials on the FMA pipe, bf16 P written over S; at the end of a unit either the normalised output
+//               reference that moves only when exp2 would overflow (then O is rescaled), bf16 P written
+//               over S; at the end of a unit either the normalised output
 //               (whole list in one unit) or an unnormalised fp32 partial result plus (max, sum) per row
 //               into the workspace.  The chunk of a split list that finishes last (a counter in the plan)
 //               combines the partial results in chunk order, so the result does not depend on timing.
@@ -366,7 +366,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
     }
   } else if (start_ok && warp == kWarpMma) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    // elect.sync tells the compiler that one thread runs this (a comparison with the lane number does not), so that
+    // descriptors live in uniform registers: 8320 tokens, dense causal 477 -> 448 us
+    if (elect_one()) {
       constexpr uint32_t idesc_qk = instr_desc(BK, false);
       constexpr uint32_t idesc_qk_half = instr_desc(BK / 2, false);
       constexpr uint32_t idesc_pv = instr_desc(kD, true);
@@ -587,26 +589,26 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
         {
           float2 ls2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
           const float2 sc2 = make_float2(scale_log2, scale_log2), mm2 = make_float2(-m_ref, -m_ref);
-          // exponentials of one 64-key half whose S values are in r
-          auto half_exp = [&](uint32_t (&r)[64], auto hh_c) {
-            constexpr int hh = decltype(hh_c)::value;
+          // Masked columns are set to -inf first, all of them, so that the exponentials behind are one straight run of
+          // code: with a branch per 32 columns the MUFU unit drained four times per tile (1650 clk for the exponentials of a
+          // tile against 1200 for the same code alone; 8320 tokens, dense causal 448 -> 420 us, paper mask 126 -> 123 us).
+          auto mask64 = [&](uint32_t (&r)[64], uint32_t k0, uint32_t k1) {
+            if (__any_sync(0xffffffffu, (k0 & k1) != 0xFFFFFFFFu)) {  // warp-uniform
 #pragma unroll
-            for (int cc = 0; cc < 2; ++cc) {
-              constexpr int c0 = 2 * hh;
-              const int c = c0 + cc;
-              if (cls != kTileFull && __any_sync(0xffffffffu, keep[c] != 0xFFFFFFFFu)) {  // warp-uniform
-#pragma unroll
-                for (int x = 0; x < 32; ++x)
-                  if (!((keep[c] >> x) & 1u)) r[32 * cc + x] = 0xFF800000u;  // -inf: exp2 gives 0
+              for (int x = 0; x < 32; ++x) {
+                if (!((k0 >> x) & 1u)) r[x] = 0xFF800000u;  // -inf: exp2 gives 0
+                if (!((k1 >> x) & 1u)) r[32 + x] = 0xFF800000u;
               }
+            }
+          };
+          auto exp64 = [&](const uint32_t (&r)[64], auto off_c) {  // -> pk[off ..]
+            constexpr int off = decltype(off_c)::value;
 #pragma unroll
-              for (int x = 0; x < 32; x += 2) {
-                const float2 a = __ffma2_rn(make_float2(__uint_as_float(r[32 * cc + x]), __uint_as_float(r[32 * cc + x + 1])), sc2, mm2);
-                // kPolyOf8 of every 8 column pairs take the polynomial on the FMA pipe, the rest the MUFU unit
-                const float2 pp = ((x >> 1) & 7) < kPolyOf8 ? exp2_poly2(a) : make_float2(ex2(a.x), ex2(a.y));
-                ls2[(x >> 1) & 1] = __fadd2_rn(ls2[(x >> 1) & 1], pp);
-                pk[16 * c + (x >> 1)] = pack_bf16(pp.x, pp.y);
-              }
+            for (int x = 0; x < 64; x += 2) {
+              const float2 a = __ffma2_rn(make_float2(__uint_as_float(r[x]), __uint_as_float(r[x + 1])), sc2, mm2);
+              const float2 pp = make_float2(ex2(a.x), ex2(a.y));
+              ls2[(x >> 1) & 1] = __fadd2_rn(ls2[(x >> 1) & 1], pp);
+              pk[off + (x >> 1)] = pack_bf16(pp.x, pp.y);
             }
           };
           if (hm == 3u) {  // both halves: all loads in flight before the one wait
@@ -616,15 +618,24 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
             tmem_ld32_at<0>(s_addr + 64, r1);
             tmem_ld32_at<32>(s_addr + 96, r1);
             tc_wait_ld();
-            half_exp(r0, std::integral_constant<int, 0>{});
-            half_exp(r1, std::integral_constant<int, 1>{});
+            if (cls != kTileFull) {
+              mask64(r0, keep[0], keep[1]);
+              mask64(r1, keep[2], keep[3]);
+            }
+            exp64(r0, std::integral_constant<int, 0>{});
+            exp64(r1, std::integral_constant<int, 32>{});
           } else {
             uint32_t r[64];
             tmem_ld32_at<0>(s_addr + (hm >> 1) * 64, r);
             tmem_ld32_at<32>(s_addr + (hm >> 1) * 64 + 32, r);
             tc_wait_ld();
-            if (hm == 1u) half_exp(r, std::integral_constant<int, 0>{});
-            else half_exp(r, std::integral_constant<int, 1>{});
+            if (hm == 1u) {
+              mask64(r, keep[0], keep[1]);
+              exp64(r, std::integral_constant<int, 0>{});
+            } else {
+              mask64(r, keep[2], keep[3]);
+              exp64(r, std::integral_constant<int, 32>{});
+            }
           }
           l_tile = (ls2[0].x + ls2[0].y) + (ls2[1].x + ls2[1].y);
           bool has_kept = cls == kTileFull;  // (a full tile has both halves)
