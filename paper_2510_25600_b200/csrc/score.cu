@@ -503,6 +503,386 @@ __global__ void __launch_bounds__(kMmaThreads) score_mma_colsum_kernel(
   }
 }
 
+// ---- bf16, both passes in one launch -------------------------------------------------------------------------------
+// A cluster of C CTAs owns one (request, KV head): each keeps MB blocks of 128 keys in shared memory and walks the stacked
+// rows in blocks of 128 like the two kernels above, but the logits are formed once: a CTA's (max, sum of exponentials) per
+// row goes to every CTA of the cluster through distributed shared memory, and after one cluster barrier each has the rows'
+// log-sum-exp and sums exp(s - lse) down the rows from the accumulators it still holds.  Pooling along the keys takes the
+// few scores it needs beyond a CTA's keys from its neighbours the same way.  No workspace, one launch instead of three or
+// four.  Requests of up to 16 x 256 keys; longer ones take the passes above, which read K twice but need no more than one
+// block of keys per CTA.  Bound by latencies at these sizes (launch, staging, a cluster barrier per block of rows): 2432
+// tokens, 32 / 8 heads, 32 voting rows, pool 7: 38 us with four kernels, now 15; window of 64
+// rows: 45 -> 23.
+constexpr int kClusterMax = 16;        // CTAs per cluster
+constexpr int kClusterRowBlocks = 16;  // blocks of 128 stacked rows
+constexpr int kPoolHalfMax = 64;       // scores taken from a neighbour on either side
+
+struct ScoreClusterShared {
+  float2 part[2][kClusterMax][kMmaRows];  // [parity of the block of rows][CTA][row]: (max, sum) in log2 units
+  float2 half[2][kMmaRows];               // the same per 64-key column of warps
+  float lse[kMmaRows];
+};
+
+// The mean over 2 * half + 1 keys of the scores in colbuf, a CTA's kKeys at j0 ..: `half` scores on either side come from the
+// neighbouring CTAs (outside the request: 0).  All threads of the cluster take part.
+template <int kKeys>
+__device__ __forceinline__ void pool_in_cluster(const float* colbuf, float (*halo)[kPoolHalfMax], int32_t half, int32_t rank,
+                                                int32_t C, int32_t j0, int32_t nr, int32_t len, float* cg) {
+  const int tid = threadIdx.x;
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (tid < 2 * half) {
+    const int32_t side = tid >= half, at = side ? tid - half : tid, from = rank + (side ? 1 : -1);
+    float v = 0.f;
+    if (from >= 0 && from < C) {
+      uint32_t src;
+      asm("mapa.shared::cluster.u32 %0, %1, %2;"
+          : "=r"(src) : "r"((uint32_t)__cvta_generic_to_shared(colbuf + (side ? at : kKeys - half + at))), "r"(from));
+      asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(src) : "memory");
+    }
+    halo[side][at] = v;
+  }
+  __syncthreads();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");  // done with the neighbours' memory
+  if (tid < kKeys && j0 + tid < len) {
+    float sum = 0.f;
+    if (j0 + tid < nr)
+      for (int32_t x = tid - half; x <= tid + half; ++x)
+        sum += x < 0 ? halo[0][half + x] : x >= kKeys ? halo[1][x - kKeys] : colbuf[x];
+    cg[j0 + tid] = sum / (float)(2 * half + 1);
+  }
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // a CTA's memory outlives its neighbours' reads
+}
+
+template <int MB>
+__global__ void __launch_bounds__(kMmaThreads, 1) score_cluster_kernel(
+    const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, const int32_t* __restrict__ cu_seqlens,
+    int32_t window, int32_t obs, int32_t pool, int32_t n_q_heads, int32_t n_kv_heads, int32_t d, float scale_log2,
+    int64_t n_tokens, float* __restrict__ c_out) {
+  constexpr int kKeys = MB * kCtaKeys;
+  extern __shared__ __align__(16) uint8_t smem_mma[];
+  __shared__ ScoreClusterShared sh;
+  __shared__ float red[4][kKeys];                      // per row group of warps
+  __shared__ float colbuf[kKeys];                      // the CTA's scores before pooling, read by its neighbours too
+  __shared__ float halo[2][kPoolHalfMax];
+  __nv_bfloat16* ks = reinterpret_cast<__nv_bfloat16*>(smem_mma);
+  __nv_bfloat16* qs = ks + kKeys * (d + 8);
+  const int32_t C = gridDim.x, rank = blockIdx.x, r = blockIdx.z, g = blockIdx.y, j0 = rank * kKeys;
+  const int32_t G = n_q_heads / n_kv_heads;
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // "started": awaited before the first exchange
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (launched with programmatic stream serialization)
+  const int32_t base = cu_seqlens[r], len = cu_seqlens[r + 1] - base;
+  const int32_t w = min(window, len), nr = len - w, wo = min(obs, len), n_rows = G * wo;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wr = warp >> 1, wc = warp & 1;
+  auto q_row = [&](int32_t row) -> int64_t {
+    return row < n_rows ? ((int64_t)(base + len - wo + row % wo) * n_q_heads + g * G + row / wo) * d : -1;
+  };
+  stage_rows_bf16_async(ks, k, kKeys, d, [&](int rr) -> int64_t {
+    return j0 + rr < len ? ((int64_t)(base + j0 + rr) * n_kv_heads + g) * d : -1;
+  });
+  __nv_bfloat16* qbuf[2] = {qs, qs + kMmaRows * (d + 8)};
+  stage_rows_bf16_async(qbuf[0], q, kMmaRows, d, [&](int rr) { return q_row(rr); });
+  float col[MB][8][2];
+#pragma unroll
+  for (int m = 0; m < MB; ++m)
+#pragma unroll
+    for (int nb = 0; nb < 8; ++nb) col[m][nb][0] = col[m][nb][1] = 0.f;
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  for (int32_t row0 = 0, it = 0; row0 < n_rows; row0 += kMmaRows, ++it) {
+    __syncthreads();  // everyone is done with the buffer the next copy overwrites
+    if (row0 + kMmaRows < n_rows) {
+      stage_rows_bf16_async(qbuf[(it + 1) & 1], q, kMmaRows, d, [&](int rr) { return q_row(row0 + kMmaRows + rr); });
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
+    }
+    __syncthreads();
+    float acc[MB][2][8][4];
+#pragma unroll
+    for (int m = 0; m < MB; ++m) logits_32x64(qbuf[it & 1], ks + m * kCtaKeys * (d + 8), d, acc[m]);
+    // scaled logits, causal; the warp's (max, sum) per row over its keys
+#pragma unroll
+    for (int mb = 0; mb < 2; ++mb)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int32_t rl = 32 * wr + 16 * mb + (lane >> 2) + 8 * h, row = row0 + rl;
+        const int32_t i = row < n_rows ? len - wo + row % wo : -1;  // causal limit of the row (-1: no row)
+        float mx = -INFINITY;
+#pragma unroll
+        for (int m = 0; m < MB; ++m)
+#pragma unroll
+          for (int nb = 0; nb < 8; ++nb)
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+              const int32_t j = j0 + m * kCtaKeys + 64 * wc + 8 * nb + 2 * (lane & 3) + x;
+              const float sv = j <= i ? acc[m][mb][nb][2 * h + x] * scale_log2 : -INFINITY;
+              acc[m][mb][nb][2 * h + x] = sv;
+              mx = fmaxf(mx, sv);
+            }
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+        float l = 0.f;
+        if (mx > -INFINITY) {
+#pragma unroll
+          for (int m = 0; m < MB; ++m)
+#pragma unroll
+            for (int nb = 0; nb < 8; ++nb) l += exp2f(acc[m][mb][nb][2 * h] - mx) + exp2f(acc[m][mb][nb][2 * h + 1] - mx);
+        }
+        l += __shfl_xor_sync(0xffffffffu, l, 1);
+        l += __shfl_xor_sync(0xffffffffu, l, 2);
+        if ((lane & 3) == 0) sh.half[wc][rl] = make_float2(mx, l);
+      }
+    __syncthreads();
+    // the CTA's pair per row, to every CTA of the cluster (two threads per row, each serves every other CTA)
+    {
+      const int32_t rl = tid >> 1;
+      const float2 a = sh.half[0][rl], b = sh.half[1][rl];
+      const float mx = fmaxf(a.x, b.x);
+      float l = 0.f;
+      if (a.y > 0.f) l += a.y * exp2f(a.x - mx);
+      if (b.y > 0.f) l += b.y * exp2f(b.x - mx);
+      const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&sh.part[it & 1][rank][rl]);
+      for (int32_t to = tid & 1; to < C; to += 2) {
+        uint32_t dst;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(mine), "r"(to));
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(mx), "f"(l) : "memory");
+      }
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    // the rows' log-sum-exp: two threads per row, each over every other CTA.  (The pairs of this parity are overwritten two
+    // blocks of rows later, behind the next block's barrier, which everybody reaches after this read.)
+    {
+      const int32_t rl = tid >> 1;
+      float mx = -INFINITY;
+      for (int32_t x = tid & 1; x < C; x += 2) mx = fmaxf(mx, sh.part[it & 1][x][rl].x);
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+      float l = 0.f;
+      for (int32_t x = tid & 1; x < C; x += 2) {
+        const float2 p = sh.part[it & 1][x][rl];
+        if (p.y > 0.f) l += p.y * exp2f(p.x - mx);
+      }
+      l += __shfl_xor_sync(0xffffffffu, l, 1);
+      if ((tid & 1) == 0) sh.lse[rl] = row0 + rl < n_rows ? mx + log2f(l) : INFINITY;  // (+inf: an absent row adds nothing)
+    }
+    __syncthreads();
+#pragma unroll
+    for (int mb = 0; mb < 2; ++mb)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float lse = sh.lse[32 * wr + 16 * mb + (lane >> 2) + 8 * h];
+#pragma unroll
+        for (int m = 0; m < MB; ++m)
+#pragma unroll
+          for (int nb = 0; nb < 8; ++nb) {  // keys the row does not see are -inf and add nothing
+            col[m][nb][0] += exp2f(acc[m][mb][nb][2 * h] - lse);
+            col[m][nb][1] += exp2f(acc[m][mb][nb][2 * h + 1] - lse);
+          }
+      }
+  }
+  // sum over the 8 row groups of the warp (lanes with equal lane % 4 hold the same columns), then over the 4 row warps
+#pragma unroll
+  for (int m = 0; m < MB; ++m)
+#pragma unroll
+    for (int nb = 0; nb < 8; ++nb)
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        float v = col[m][nb][x];
+        v += __shfl_xor_sync(0xffffffffu, v, 4);
+        v += __shfl_xor_sync(0xffffffffu, v, 8);
+        v += __shfl_xor_sync(0xffffffffu, v, 16);
+        if (lane < 4) red[wr][m * kCtaKeys + 64 * wc + 8 * nb + 2 * lane + x] = v;
+      }
+  __syncthreads();
+  float* cg = c_out + (int64_t)g * n_tokens + base;
+  const int32_t half = pool / 2;
+  if (tid < kKeys) {
+    const float sum = (red[0][tid] + red[1][tid]) + (red[2][tid] + red[3][tid]);
+    const int32_t j = j0 + tid;
+    const float v = j < nr ? sum / (float)G : 0.f;  // (the window, and keys past the end: 0)
+    if (half == 0 && j < len) cg[j] = v;
+    colbuf[tid] = v;
+  }
+  if (half == 0) return;  // (no CTA reads another's shared memory behind the last barrier)
+  pool_in_cluster<kKeys>(colbuf, halo, half, rank, C, j0, nr, len, cg);
+}
+
+// grid (C, Hkv, n_req) in clusters of C CTAs, behind the previous kernel by programmatic stream serialization.  `wide`: devices
+// on which the kernel's clusters of more than eight CTAs have been allowed (they are opt-in).
+template <typename... Params, typename... Args>
+static purekv_status launch_cluster(void (*kernel)(Params...), std::atomic<uint64_t>& wide, int32_t C, int32_t Hkv, int32_t n_req,
+                                    int threads, size_t smem, cudaStream_t sm, Args... args) {
+  int dev = -1;
+  PK_CUDA(cudaGetDevice(&dev));
+  if (!(wide.load(std::memory_order_acquire) & (1ull << dev))) {
+    PK_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    wide.fetch_or(1ull << dev, std::memory_order_release);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)C, (unsigned)Hkv, (unsigned)n_req);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = sm;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)C;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  PK_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
+  return PUREKV_OK;
+}
+
+template <int MB>
+static purekv_status launch_score_cluster(const void* q, const void* k, float* c_out, const purekv_batch* b, int32_t window,
+                                          int32_t obs, int32_t pool, int32_t H, int32_t Hkv, int32_t d, float scale,
+                                          cudaStream_t sm) {
+  auto kernel = score_cluster_kernel<MB>;
+  static std::atomic<uint64_t> smem_allowed{0}, wide_allowed{0};
+  const purekv_status st = allow_max_dynamic_smem(kernel, smem_allowed);
+  if (st != PUREKV_OK) return st;
+  const int32_t C = std::max(1, (max_len(b) + MB * kCtaKeys - 1) / (MB * kCtaKeys));
+  return launch_cluster(kernel, wide_allowed, C, Hkv, b->n_req, kMmaThreads,
+                        (size_t)(MB * kCtaKeys + 2 * kMmaRows) * (d + 8) * sizeof(__nv_bfloat16), sm, (const __nv_bfloat16*)q,
+                        (const __nv_bfloat16*)k, b->cu_seqlens, window, obs, pool, H, Hkv, d, scale * 1.4426950408889634f,
+                        b->total_tokens, c_out);
+}
+
+// ---- fp32, both passes in one launch -------------------------------------------------------------------------------
+// The cluster scheme above with fp32 products on CUDA cores: a CTA keeps 64 keys, a block is 32 stacked rows.  Requests of
+// up to 16 x 64 keys; for a short prompt the two-kernel form spends its time in one CTA that walks all keys (288 tokens,
+// 2 heads, window 16: 28 us for the two kernels, now 6).
+struct ScoreClusterSharedF32 {
+  float2 part[2][kClusterMax][kRB];
+  float lse[kRB];
+  float red[kThreads / 16][kKB];
+  float colbuf[kKB];
+  float halo[2][kPoolHalfMax];
+};
+
+template <typename RowOf>
+__device__ __forceinline__ void stage_rows_f32_async(float* dst, const float* src, int rows, int d, RowOf row_of) {
+  const int cpr = d / 4;
+  for (int x = threadIdx.x; x < rows * cpr; x += kThreads) {
+    const int r = x / cpr, c = 4 * (x % cpr);
+    const int64_t off = row_of(r);
+    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(dst + r * (d + 4) + c);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sa), "l"(off >= 0 ? src + off + c : src), "r"(off >= 0 ? 16u : 0u)
+                 : "memory");
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(kThreads, 1) score_cluster_f32_kernel(
+    const float* __restrict__ q, const float* __restrict__ k, const int32_t* __restrict__ cu_seqlens, int32_t window, int32_t obs,
+    int32_t pool, int32_t n_q_heads, int32_t n_kv_heads, int32_t d, float scale_log2, int64_t n_tokens,
+    float* __restrict__ c_out) {
+  extern __shared__ __align__(16) float smem[];
+  __shared__ ScoreClusterSharedF32 sh;
+  const int ld = d + 4;
+  float* ks = smem;             // [kKB][ld]
+  float* qs = ks + kKB * ld;    // [2][kRB][ld]
+  const int32_t C = gridDim.x, rank = blockIdx.x, r = blockIdx.z, g = blockIdx.y, j0 = rank * kKB;
+  const int32_t G = n_q_heads / n_kv_heads;
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // "started": awaited before the first exchange
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int32_t base = cu_seqlens[r], len = cu_seqlens[r + 1] - base;
+  const int32_t w = min(window, len), nr = len - w, wo = min(obs, len), n_rows = G * wo;
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  auto q_row = [&](int32_t row) -> int64_t {
+    return row < n_rows ? ((int64_t)(base + len - wo + row % wo) * n_q_heads + g * G + row / wo) * d : -1;
+  };
+  stage_rows_f32_async(ks, k, kKB, d, [&](int rr) -> int64_t {
+    return j0 + rr < len ? ((int64_t)(base + j0 + rr) * n_kv_heads + g) * d : -1;
+  });
+  stage_rows_f32_async(qs, q, kRB, d, q_row);
+  float col[4] = {0.f, 0.f, 0.f, 0.f};
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  for (int32_t row0 = 0, it = 0; row0 < n_rows; row0 += kRB, ++it) {
+    __syncthreads();  // everyone is done with the buffer the next copy overwrites
+    if (row0 + kRB < n_rows) {
+      stage_rows_f32_async(qs + ((it + 1) & 1) * kRB * ld, q, kRB, d, [&](int rr) { return q_row(row0 + kRB + rr); });
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
+    }
+    __syncthreads();
+    float s[2][4];
+    tile_dots(qs + (it & 1) * kRB * ld, ks, d, ld, ty, tx, s);
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      const int32_t rl = 2 * ty + a, row = row0 + rl, i = row < n_rows ? len - wo + row % wo : -1;
+      float mx = -INFINITY;
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        s[a][b] = j0 + tx + 16 * b <= i ? s[a][b] * scale_log2 : -INFINITY;
+        mx = fmaxf(mx, s[a][b]);
+      }
+#pragma unroll
+      for (int off = 8; off >= 1; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+      float l = 0.f;
+      if (mx > -INFINITY)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) l += exp2f(s[a][b] - mx);
+#pragma unroll
+      for (int off = 8; off >= 1; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+      // lane tx of the row's sixteen threads serves CTA tx of the cluster
+      if (tx < C) {
+        uint32_t dst;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;"
+            : "=r"(dst) : "r"((uint32_t)__cvta_generic_to_shared(&sh.part[it & 1][rank][rl])), "r"(tx));
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(mx), "f"(l) : "memory");
+      }
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      const int32_t rl = 2 * ty + a;
+      const float2 p = tx < C ? sh.part[it & 1][tx][rl] : make_float2(-INFINITY, 0.f);
+      float mx = p.x;
+#pragma unroll
+      for (int off = 8; off >= 1; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+      float l = p.y > 0.f ? p.y * exp2f(p.x - mx) : 0.f;
+#pragma unroll
+      for (int off = 8; off >= 1; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+      const float lse = row0 + rl < n_rows ? mx + log2f(l) : INFINITY;  // (+inf: an absent row adds nothing)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) col[b] += exp2f(s[a][b] - lse);
+    }
+  }
+#pragma unroll
+  for (int b = 0; b < 4; ++b) sh.red[ty][tx + 16 * b] = col[b];
+  __syncthreads();
+  float* cg = c_out + (int64_t)g * n_tokens + base;
+  const int32_t half = pool / 2;
+  if (tid < kKB) {
+    float sum = 0.f;
+#pragma unroll
+    for (int t = 0; t < kThreads / 16; ++t) sum += sh.red[t][tid];
+    const int32_t j = j0 + tid;
+    const float v = j < nr ? sum / (float)G : 0.f;
+    if (half == 0 && j < len) cg[j] = v;
+    sh.colbuf[tid] = v;
+  }
+  if (half == 0) return;  // (no CTA reads another's shared memory behind the last barrier)
+  pool_in_cluster<kKB>(sh.colbuf, sh.halo, half, rank, C, j0, nr, len, cg);
+}
+
+static purekv_status launch_score_cluster_f32(const float* q, const float* k, float* c_out, const purekv_batch* b,
+                                              int32_t window, int32_t obs, int32_t pool, int32_t H, int32_t Hkv, int32_t d,
+                                              float scale, cudaStream_t sm) {
+  static std::atomic<uint64_t> smem_allowed{0}, wide_allowed{0};
+  const purekv_status st = allow_max_dynamic_smem(score_cluster_f32_kernel, smem_allowed);
+  if (st != PUREKV_OK) return st;
+  const int32_t C = std::max(1, (max_len(b) + kKB - 1) / kKB);
+  return launch_cluster(score_cluster_f32_kernel, wide_allowed, C, Hkv, b->n_req, kThreads,
+                        (size_t)(kKB + 2 * kRB) * (d + 4) * sizeof(float), sm, q, k, b->cu_seqlens, window, obs, pool, H, Hkv, d,
+                        scale * 1.4426950408889634f, b->total_tokens, c_out);
+}
+
 // `obs` = accumulated rows per request and head (Eq. 2: the window itself); the first pass and the merge see only
 // rows, so they take it in place of the window.
 static purekv_status launch_score_mma(const void* q, const void* k, float* c_out, const purekv_batch* b, int32_t window,
@@ -641,6 +1021,22 @@ static purekv_status score_impl(const char* who, const void* q, const void* k, f
   float* c_raw = pool > 1 ? lse2 + score_ws_floats(batch, obs, n_q_heads) : c_out;  // scores before pooling
   const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)head_dim);
   cudaStream_t sm = (cudaStream_t)stream;
+  // One launch when a cluster holds the longest request (and the accumulated rows are not the whole of a long one: every
+  // block of rows costs a cluster barrier, and rows before a CTA's keys are multiplied for nothing).
+  const int32_t ml = max_len(batch), row_blocks = ((n_q_heads / n_kv_heads) * obs + kMmaRows - 1) / kMmaRows;
+  // With more CTAs than SMs (one fits an SM) a single block or two of rows is still faster this way (4 requests of 2432
+  // tokens, 32 rows: 42 against 72 us), more are not: nothing runs beside a CTA that waits at a barrier (8 requests, 100-row
+  // window, 6 blocks: 180 against 170 us).
+  const int64_t ctas = (int64_t)batch->n_req * n_kv_heads * ((ml + 2 * kCtaKeys - 1) / (2 * kCtaKeys)) * (ml <= kClusterMax * kCtaKeys ? 2 : 1);
+  if (dtype == PUREKV_BF16 && head_dim % 16 == 0 && head_dim <= 128 && ml <= kClusterMax * 2 * kCtaKeys &&
+      row_blocks <= kClusterRowBlocks && pool / 2 <= kPoolHalfMax && (ctas <= 148 || row_blocks <= 2))
+    return ml <= kClusterMax * kCtaKeys
+               ? launch_score_cluster<1>(q, k, c_out, batch, window, obs, pool, n_q_heads, n_kv_heads, head_dim, scale, sm)
+               : launch_score_cluster<2>(q, k, c_out, batch, window, obs, pool, n_q_heads, n_kv_heads, head_dim, scale, sm);
+  if (dtype == PUREKV_FP32 && ml <= kClusterMax * kKB && row_blocks <= kClusterRowBlocks && pool / 2 <= kKB / 2 &&
+      ((uintptr_t)q | (uintptr_t)k) % 16 == 0)
+    return launch_score_cluster_f32((const float*)q, (const float*)k, c_out, batch, window, obs, pool, n_q_heads, n_kv_heads,
+                                    head_dim, scale, sm);
   if (dtype == PUREKV_BF16 && head_dim % 16 == 0)
     st = launch_score_mma(q, k, c_raw, batch, window, obs, n_q_heads, n_kv_heads, head_dim, scale, lse2, sm);
   else if (dtype == PUREKV_BF16)
