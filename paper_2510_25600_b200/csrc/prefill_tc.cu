@@ -57,7 +57,8 @@ struct __align__(8) Barriers {
   uint64_t k_full[ST], k_empty[ST], v_full[ST], v_empty[ST];
   uint64_t m_full[MR];     // producer -> softmax: class word (and bit mask) of a tile are in place
   uint64_t s_full[2][SB];  // MMA -> softmax: S of (slot, buffer) is complete
-  uint64_t p_full[2][SB];  // softmax -> MMA: P written (and O rescaled) by the slot's four row warps
+  uint64_t p_part[2];      // softmax -> MMA: P of the first 96 keys written (and O rescaled) by the slot's four row warps
+  uint64_t p_full[2][SB];  // softmax -> MMA: all of P written
   uint64_t o_done[2];      // one completion per P.V product of the slot
   uint64_t o_final[2];     // one completion per unit, after the slot's last P.V product
   uint64_t rows_sync[2];   // the 128 row threads of a slot meet here around the merge-counter update
@@ -116,6 +117,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
         mbar_init(smem_u32(&bars.s_full[sl][b]), 1);
         mbar_init(smem_u32(&bars.p_full[sl][b]), 4);
       }
+      mbar_init(smem_u32(&bars.p_part[sl]), 4);
       mbar_init(smem_u32(&bars.o_done[sl]), 1);
       mbar_init(smem_u32(&bars.o_final[sl]), 1);
       mbar_init(smem_u32(&bars.rows_sync[sl]), 128);
@@ -429,19 +431,26 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
         const uint32_t it = it_base + (uint32_t)n;
         const uint32_t s = it % ST, b = tp[sl] % SB;
         if (sl == 0 && !mbar_wait(smem_u32(&bars.v_full[s]), (it / ST) & 1u, abort_flag, wait_ns)) return false;
-        // P of the unit's first tile also implies that the previous unit's output has left TMEM
-        if (!mbar_wait(smem_u32(&bars.p_full[sl][b]), (tp[sl] / SB) & 1u, abort_flag, wait_ns)) return false;
-        tc_fence_after();
         const uint32_t p_addr = tmem + sl * 128 + b * BK, o_addr = tmem + kColO + sl * 128;
         // B = V tile, MN-major: per K step 16 key rows (2 groups of 8, 1024 B apart) x 128 dims (2 panels)
         const uint32_t v_lo = v_lo0 + s * (kTileKV >> 4);
         const uint32_t hm = (uint32_t)((meta_s[it % MR][0].x | meta_s[it % MR][1].x) >> 2) & 3u;
         const uint32_t acc0 = n > 0 ? 1u : 0u;  // the unit's first product overwrites O
-        if (hm == 3u) {
+        // P of the unit's first tile also implies that the previous unit's output has left TMEM
+        if (hm == 3u) {  // six of the eight K steps run while the rows are still in the last quarter's exponentials
+          if (!mbar_wait(smem_u32(&bars.p_part[sl]), tp[sl] & 1u, abort_flag, wait_ns)) return false;
+          tc_fence_after();
 #pragma unroll
-          for (int ks = 0; ks < BK / 16; ++ks)
+          for (int ks = 0; ks < 6; ++ks)
             mma_ts_lh(o_addr, p_addr + ks * 8, v_lo + ks * (2048 >> 4), kDescHi, idesc_pv, ks > 0 ? 1u : acc0);
+          if (!mbar_wait(smem_u32(&bars.p_full[sl][b]), (tp[sl] / SB) & 1u, abort_flag, wait_ns)) return false;
+          tc_fence_after();
+#pragma unroll
+          for (int ks = 6; ks < 8; ++ks)
+            mma_ts_lh(o_addr, p_addr + ks * 8, v_lo + ks * (2048 >> 4), kDescHi, idesc_pv, 1u);
         } else {  // the K steps of the present half only
+          if (!mbar_wait(smem_u32(&bars.p_full[sl][b]), (tp[sl] / SB) & 1u, abort_flag, wait_ns)) return false;
+          tc_fence_after();
           const uint32_t k0 = (hm >> 1) * (BK / 32);
 #pragma unroll
           for (int ks = 0; ks < BK / 32; ++ks)
@@ -582,9 +591,19 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
         // Fast path: exponentials against the row's standing reference m_ref, no maximum taken.  Softmax does not depend
         // on the reference, and fp32 / bf16 carry 8 exponent bits, so the reference (0 at the start of a unit) only has
         // to keep exp2 in range: it moves when a tile overflows, or when everything kept so far has underflowed; those
-        // tiles take the exact path below.
+        // tiles take the exact path below.  P goes to the tensor cores in two parts, 96 keys and 32: six of the eight K steps
+        // of P V run during the last quarter's exponentials instead of behind them (8320 tokens: dense causal 421 -> 406 us,
+        // paper mask 122 -> 116 us; handing over half of P instead was measured slower, the wait between the parts then
+        // holds the MMA thread up for the other slot).
         uint32_t pk[BK / 2];
         float l_tile = 0.f;
+        auto hand_over = [&](uint32_t bar) {
+          tc_wait_st();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar);  // one arrival per warp: 4 per slot
+        };
+        const uint32_t part_bar = smem_u32(&bars.p_part[sl]), full_bar = smem_u32(&bars.p_full[sl][b]);
         bool exact = false;
         {
           float2 ls2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -601,15 +620,29 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
               }
             }
           };
-          auto exp64 = [&](const uint32_t (&r)[64], auto off_c) {  // -> pk[off ..]
-            constexpr int off = decltype(off_c)::value;
+          auto exps = [&](const uint32_t (&r)[64], auto x0_c, auto x1_c, auto off_c) {  // columns x0 .. x1 - 1 -> pk[off ..]
+            constexpr int x0 = decltype(x0_c)::value, x1 = decltype(x1_c)::value, off = decltype(off_c)::value;
 #pragma unroll
-            for (int x = 0; x < 64; x += 2) {
+            for (int x = x0; x < x1; x += 2) {
               const float2 a = __ffma2_rn(make_float2(__uint_as_float(r[x]), __uint_as_float(r[x + 1])), sc2, mm2);
               const float2 pp = make_float2(ex2(a.x), ex2(a.y));
               ls2[(x >> 1) & 1] = __fadd2_rn(ls2[(x >> 1) & 1], pp);
-              pk[off + (x >> 1)] = pack_bf16(pp.x, pp.y);
+              pk[off + ((x - x0) >> 1)] = pack_bf16(pp.x, pp.y);
             }
+          };
+          constexpr std::integral_constant<int, 0> i0{};
+          constexpr std::integral_constant<int, 32> i32{};
+          constexpr std::integral_constant<int, 48> i48{};
+          constexpr std::integral_constant<int, 64> i64{};
+          bool has_kept = cls == kTileFull;  // (a full tile has both halves)
+#pragma unroll
+          for (int c = 0; c < BK / 32; ++c) has_kept |= keep[c] != 0u;
+          // overflow (inf or NaN), or kept keys and still nothing representable: redo against the true maximum.  Settled
+          // before P of the first 96 keys goes out, from its sum and the largest logit of the last 32 keys (32 terms below
+          // 2^94 stay below 1e30; one of 2^-96 or more is representable).
+          auto bad = [&](float top) {
+            return __any_sync(0xffffffffu, !(l_tile <= 1.0e30f) || !(top < 94.f) ||
+                                               (has_kept && l_sum + l_tile < 1.0e-30f && top < -96.f));
           };
           if (hm == 3u) {  // both halves: all loads in flight before the one wait
             uint32_t r0[64], r1[64];
@@ -622,27 +655,33 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
               mask64(r0, keep[0], keep[1]);
               mask64(r1, keep[2], keep[3]);
             }
-            exp64(r0, std::integral_constant<int, 0>{});
-            exp64(r1, std::integral_constant<int, 32>{});
+            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+            for (int x = 32; x < 64; x += 2) mx[(x >> 1) & 3] = max3(mx[(x >> 1) & 3], __uint_as_float(r1[x]), __uint_as_float(r1[x + 1]));
+            exps(r0, i0, i64, i0);
+            exps(r1, i0, i32, i32);
+            l_tile = (ls2[0].x + ls2[0].y) + (ls2[1].x + ls2[1].y);
+            exact = bad(fmaf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])), scale_log2, -m_ref));  // scale > 0
+            if (!exact) {
+              tmem_st32(s_addr, reinterpret_cast<const uint32_t(&)[32]>(pk[0]));  // over columns of S that have been read
+              tmem_st16(s_addr + 32, reinterpret_cast<const uint32_t(&)[16]>(pk[32]));
+              hand_over(part_bar);
+              exps(r1, i32, i64, i48);
+              l_tile = (ls2[0].x + ls2[0].y) + (ls2[1].x + ls2[1].y);
+              tmem_st16(s_addr + 48, reinterpret_cast<const uint32_t(&)[16]>(pk[48]));
+            }
           } else {
             uint32_t r[64];
             tmem_ld32_at<0>(s_addr + (hm >> 1) * 64, r);
             tmem_ld32_at<32>(s_addr + (hm >> 1) * 64 + 32, r);
             tc_wait_ld();
-            if (hm == 1u) {
-              mask64(r, keep[0], keep[1]);
-              exp64(r, std::integral_constant<int, 0>{});
-            } else {
-              mask64(r, keep[2], keep[3]);
-              exp64(r, std::integral_constant<int, 32>{});
-            }
+            if (hm == 1u) mask64(r, keep[0], keep[1]);
+            else mask64(r, keep[2], keep[3]);
+            exps(r, i0, i64, i0);  // (the half's P, wherever it belongs)
+            l_tile = (ls2[0].x + ls2[0].y) + (ls2[1].x + ls2[1].y);
+            exact = bad(-INFINITY);
+            if (!exact) tmem_st32(s_addr + (hm >> 1) * 32, reinterpret_cast<const uint32_t(&)[32]>(pk[0]));
           }
-          l_tile = (ls2[0].x + ls2[0].y) + (ls2[1].x + ls2[1].y);
-          bool has_kept = cls == kTileFull;  // (a full tile has both halves)
-#pragma unroll
-          for (int c = 0; c < BK / 32; ++c) has_kept |= keep[c] != 0u;
-          // overflow (inf or NaN), or kept keys and still nothing representable: redo against the true maximum
-          exact = __any_sync(0xffffffffu, !(l_tile <= 1.0e30f) || (has_kept && l_sum + l_tile < 1.0e-30f));
         }
         if (exact) {
           // Exact path (rare): re-reference the row; O and the running sum are rescaled.  S is still intact in TMEM
@@ -682,7 +721,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
           float ls[2] = {0.f, 0.f};
 #pragma unroll
           for (int c = 0; c < BK / 32; ++c) {
-            uint32_t r[32];
+            uint32_t r[32], pc[16];
             tmem_ld32(s_addr + 32 * c, r);
             tc_wait_ld();
 #pragma unroll
@@ -690,22 +729,18 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
               const float p0 = ((keep[c] >> x) & 1u) ? ex2(fmaf(__uint_as_float(r[x]), scale_log2, -m_sub)) : 0.f;
               const float p1 = ((keep[c] >> (x + 1)) & 1u) ? ex2(fmaf(__uint_as_float(r[x + 1]), scale_log2, -m_sub)) : 0.f;
               ls[(x >> 1) & 1] += p0 + p1;
-              pk[16 * c + (x >> 1)] = pack_bf16(p0, p1);
+              pc[x >> 1] = pack_bf16(p0, p1);
             }
+            // (over columns of S that have been read: chunk c of P lies inside chunk c / 2 of S)
+            if ((hm >> (c >> 1)) & 1u) tmem_st16(s_addr + 16 * c, pc);
           }
           l_tile = ls[0] + ls[1];
           l_sum *= alpha;
           m_ref = m_new;
         }
         l_sum += l_tile;
-        // bf16 P over the first BK/2 columns of S, which this thread has consumed
-#pragma unroll
-        for (int c = 0; c < BK / 32; ++c)
-          if ((hm >> (c >> 1)) & 1u) tmem_st16(s_addr + 16 * c, reinterpret_cast<const uint32_t(&)[16]>(pk[16 * c]));
-        tc_wait_st();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&bars.p_full[sl][b]));  // one arrival per warp: 4 per slot
+        hand_over(full_bar);
+        if ((exact || hm != 3u) && lane == 0) mbar_arrive(part_bar);  // (counted in every tile)
         ++t;
       }
       if (!ok) break;
