@@ -802,17 +802,21 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
         if (merge_s[sl]) {
           const float* p0 = ws + ((int64_t)part_base * n_q_heads + hq) * kPartFloats;
           const int64_t cstride = (int64_t)n_q_heads * kPartFloats;
-          float m_all = -INFINITY;
-          for (int32_t c = 0; c < u.n_chunks; ++c) {
-            const float lc = __ldcg(p0 + c * cstride + 128 * 128 + 128 + row);
-            const float mc = __ldcg(p0 + c * cstride + 128 * 128 + row);
-            if (lc > 0.f) m_all = fmaxf(m_all, mc);
-          }
-          float l_all = 0.f;
-          for (int32_t c = 0; c < u.n_chunks; ++c) {
-            const float lc = __ldcg(p0 + c * cstride + 128 * 128 + 128 + row);
-            const float mc = __ldcg(p0 + c * cstride + 128 * 128 + row);
-            if (lc > 0.f) l_all += lc * ex2(mc - m_all);
+          // Two chunks at a time, their loads in flight together: the merge is a chain of L2 round trips (with one chunk at a
+          // time, weights first, it took 20 000 clk for three chunks, as long as six key tiles).
+          float m_all = -INFINITY, l_all = 0.f;
+          for (int32_t c = 0; c < u.n_chunks; c += 2) {
+            const float* pa = p0 + c * cstride + 128 * 128 + row;
+            const float* pb = p0 + (int64_t)min(c + 1, u.n_chunks - 1) * cstride + 128 * 128 + row;
+            const float ma = __ldcg(pa), la = __ldcg(pa + 128), mb = __ldcg(pb), lb_ = __ldcg(pb + 128);
+            const float lb = c + 1 < u.n_chunks ? lb_ : 0.f;
+            const float m_new = fmaxf(m_all, fmaxf(la > 0.f ? ma : -INFINITY, lb > 0.f ? mb : -INFINITY));
+            if (m_new > m_all) {
+              l_all *= ex2(m_all - m_new);  // (l_all is 0 while m_all is -inf)
+              m_all = m_new;
+            }
+            if (la > 0.f) l_all += la * ex2(ma - m_all);
+            if (lb > 0.f) l_all += lb * ex2(mb - m_all);
           }
           const float inv = 1.f / l_all;
           __nv_bfloat16* dst = o + ((int64_t)(q_first + row) * n_q_heads + hq) * kD;
@@ -821,29 +825,33 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
             float acc[32];
 #pragma unroll
             for (int x = 0; x < 32; ++x) acc[x] = 0.f;
-            for (int32_t c = 0; c < u.n_chunks; ++c) {
-              const float lc = __ldcg(p0 + c * cstride + 128 * 128 + 128 + row);
-              const float mc = __ldcg(p0 + c * cstride + 128 * 128 + row);
-              const float wgt = lc > 0.f ? ex2(mc - m_all) : 0.f;
-              const float* pc = p0 + c * cstride;
+#pragma unroll 1
+            for (int32_t c = 0; c < u.n_chunks; c += 2) {
+              const float* pa = p0 + c * cstride;
+              const float* pb = p0 + (int64_t)min(c + 1, u.n_chunks - 1) * cstride;
+              float4 va[8], vb[8];
+              const float ma = __ldcg(pa + 128 * 128 + row), la = __ldcg(pa + 128 * 128 + 128 + row);
+              const float mb = __ldcg(pb + 128 * 128 + row), lb = __ldcg(pb + 128 * 128 + 128 + row);
 #pragma unroll
-              for (int x = 0; x < 32; x += 4) {
-                const float4 v4 = __ldcg(reinterpret_cast<const float4*>(pc + ((cc * 8 + (x >> 2)) * 128 + row) * 4));
-                acc[x] = fmaf(wgt, v4.x, acc[x]);
-                acc[x + 1] = fmaf(wgt, v4.y, acc[x + 1]);
-                acc[x + 2] = fmaf(wgt, v4.z, acc[x + 2]);
-                acc[x + 3] = fmaf(wgt, v4.w, acc[x + 3]);
+              for (int x = 0; x < 8; ++x) va[x] = __ldcg(reinterpret_cast<const float4*>(pa + ((cc * 8 + x) * 128 + row) * 4));
+#pragma unroll
+              for (int x = 0; x < 8; ++x) vb[x] = __ldcg(reinterpret_cast<const float4*>(pb + ((cc * 8 + x) * 128 + row) * 4));
+              const float wa = la > 0.f ? ex2(ma - m_all) : 0.f, wb = c + 1 < u.n_chunks && lb > 0.f ? ex2(mb - m_all) : 0.f;
+#pragma unroll
+              for (int x = 0; x < 8; ++x) {  // in chunk order
+                acc[4 * x] = fmaf(wb, vb[x].x, fmaf(wa, va[x].x, acc[4 * x]));
+                acc[4 * x + 1] = fmaf(wb, vb[x].y, fmaf(wa, va[x].y, acc[4 * x + 1]));
+                acc[4 * x + 2] = fmaf(wb, vb[x].z, fmaf(wa, va[x].z, acc[4 * x + 2]));
+                acc[4 * x + 3] = fmaf(wb, vb[x].w, fmaf(wa, va[x].w, acc[4 * x + 3]));
               }
             }
             if (row_valid) {
 #pragma unroll
-              for (int x = 0; x < 32; x += 8) {
-                uint4 w;
-                w.x = pack_bf16(acc[x + 0] * inv, acc[x + 1] * inv);
-                w.y = pack_bf16(acc[x + 2] * inv, acc[x + 3] * inv);
-                w.z = pack_bf16(acc[x + 4] * inv, acc[x + 5] * inv);
-                w.w = pack_bf16(acc[x + 6] * inv, acc[x + 7] * inv);
-                *reinterpret_cast<uint4*>(dst + 32 * cc + x) = w;
+              for (int x = 0; x < 32; x += 16) {
+                uint32_t w[8];
+#pragma unroll
+                for (int y = 0; y < 8; ++y) w[y] = pack_bf16(acc[x + 2 * y] * inv, acc[x + 2 * y + 1] * inv);
+                st_global_v8(dst + 32 * cc + x, w);
               }
             }
           }
