@@ -16,6 +16,7 @@ __global__ void __launch_bounds__(256) compact_kernel(
   // one-dimensional grid of at most one full wave; the threads stride over the chunks of all layers
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t total = total_chunks_per_layer * n_layers;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // launched with programmatic stream serialization, see select_kernel
   for (int64_t xf = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; xf < total; xf += stride) {
     const int32_t layer = (int32_t)(xf / total_chunks_per_layer);
     const int64_t x = xf - layer * total_chunks_per_layer;
@@ -84,9 +85,17 @@ extern "C" purekv_status purekv_compact_kv(const void* k, const void* v, int64_t
   const int64_t blocks = (per_layer * n_layers + 255) / 256;
   // one wave: 148 SMs x 8 resident CTAs of 256 threads; fewer blocks when the job is small
   dim3 grid((unsigned)std::min<int64_t>(blocks, 148 * 8));
-  compact_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(
-      (const uint4*)k, (const uint4*)v, layer_stride * esz / 16, idx, batch->cu_seqlens, cu_kept, batch->n_req, k_tot,
-      n_kv_heads, cpr, (uint4*)k_out, (uint4*)v_out, out_layer_stride * esz / 16, per_layer, n_layers);
-  PK_CUDA(cudaGetLastError());
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(256);
+  cfg.stream = (cudaStream_t)stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  PK_CUDA(cudaLaunchKernelEx(&cfg, compact_kernel, (const uint4*)k, (const uint4*)v, layer_stride * esz / 16, idx,
+                             batch->cu_seqlens, cu_kept, batch->n_req, k_tot, n_kv_heads, cpr, (uint4*)k_out, (uint4*)v_out,
+                             out_layer_stride * esz / 16, per_layer, n_layers));
   return PUREKV_OK;
 }

@@ -1,9 +1,10 @@
 // purekv_select_topk: V-norm weighting (Eq. 3 / Eq. 4) and budgeted top-h selection (Sec. 3.1).
 //
-// Two paths.  With few (request, head, layer) segments, vnorm_score_kernel streams V once over the whole GPU (the
-// only large traffic of this step): a warp owns 32 consecutive (token, head) rows, each half-warp reads one
-// 16-byte-chunked row per step and reduces the squared norm with shuffles; select_kernel then handles one segment
-// per CTA.  With many segments one CTA does both for its segment and the scores never leave the SM.  The selection
+// vnorm_score_kernel streams V once over the whole GPU (the only large traffic of this step) and writes S; select_kernel
+// then handles one (request, KV head, layer) segment per CTA, launched so that its start-up hides behind the tail of the
+// first.  (One CTA that streamed its own segment's V and selected from shared memory, without S in memory, was the choice for
+// 296 segments and more: 8 requests of 2000 to 16 000 tokens x 4 heads x 27 layers, selection and compaction, took 552 us that
+// way and take 505 with two kernels -- the segments differ in length and no CTA keeps loads in flight while it selects.)  The selection
 // is a 4 x 8-bit MSB-first radix select over the fp32 bit patterns (keys staged in shared memory) that finds the
 // h-th largest score, then a block-scan compaction that emits the chosen positions in ascending order; among
 // scores equal to the threshold the lowest positions win, so the result is deterministic.
@@ -38,65 +39,94 @@ struct Chunk<__nv_bfloat16> {
   }
 };
 
-// grid: one dimension, at most 3 CTAs per SM (a single full wave whatever the number of layers and heads); the warps
-// stride over blocks of 32 consecutive (token, head) rows of a layer, i.e. over contiguous memory.
-// block: 256 threads = 8 warps.
+// S = C * ||V|| of every (token, head) row of every layer, rows of 256 bytes.  HBM bound: V is the only large traffic.
+// One CTA of 16 warps per SM takes a contiguous run of blocks of 16 rows (the runs differ by at most one block, so the last
+// wave is full); a warp streams its blocks through a private ring of kVnStages x 4 KB with cp.async, which keeps about 160 KB
+// per SM in flight whatever the warps are doing.  Two lanes share a row, each with every other 16-byte chunk: the sums of
+// squares meet in the order of a butterfly over 16 lanes (chunks 8 apart, then 4, 2, 1), which does not depend on the chunk
+// a lane starts at, so the lanes start at different ones and read shared memory without bank conflicts.
+// 26 layers of 8320 tokens x 4 heads (221 MB): 40 us = 5.5 TB/s when each warp loaded 16 rows to registers and reduced them
+// with 16-lane shuffles before asking for more, 38 us = 5.8 TB/s now.
+constexpr int kVnWarps = 16, kVnStages = 3, kVnRows = 16;
+constexpr int kVnSmem = kVnWarps * kVnStages * kVnRows * 256;
+
 template <typename T>
-__global__ void __launch_bounds__(256, 3) vnorm_score_kernel(const uint4* __restrict__ v, int64_t layer_stride_c,
-                                                          const float* __restrict__ c, int64_t n_tokens,
-                                                          int32_t n_kv_heads, int32_t n_layers, int32_t chunks_per_row,
-                                                          float* __restrict__ s_out) {
+__global__ void __launch_bounds__(kVnWarps * 32, 1) vnorm_score_kernel(const uint4* __restrict__ v, int64_t layer_stride_c,
+                                                                       const float* __restrict__ c, int64_t n_tokens,
+                                                                       int32_t n_kv_heads, int32_t n_layers,
+                                                                       float* __restrict__ s_out) {
+  extern __shared__ __align__(16) uint8_t vn_smem[];
   const int32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t n_rows = n_tokens * n_kv_heads;  // rows of one layer, row = token * n_kv_heads + head
-  const int64_t n_blocks = (n_rows + 31) / 32;
-  const int64_t n_items = n_blocks * n_layers;
-  for (int64_t item = (int64_t)blockIdx.x * 8 + warp; item < n_items; item += (int64_t)gridDim.x * 8) {
-    const int64_t blk = item % n_blocks;
-    const int32_t layer = (int32_t)(item / n_blocks);
-    const uint4* vl = v + layer * layer_stride_c;
-    const int64_t r0 = blk * 32;
-    float mine = 0.f;
-    if (chunks_per_row == 16) {
-      // 256-byte rows: a half-warp covers one row per step, 16 steps cover 32 rows (8 KB of contiguous memory).
-      const int32_t half = lane >> 4, ch = lane & 15;
-      float part[16];
-      // all 16 loads are issued before the first use (volatile asm keeps them ahead of the arithmetic): with the 8 KB
-      // of a warp in flight at once, three CTAs per SM keep enough bytes outstanding to stream V near the DRAM rate
-      uint4 buf[16];
+  const int64_t n_blocks = (n_rows + kVnRows - 1) / kVnRows, n_items = n_blocks * n_layers;
+  const int64_t first = n_items * blockIdx.x / gridDim.x, last = n_items * (blockIdx.x + 1) / gridDim.x;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (launched with programmatic stream serialization)
+  const uint32_t ring = (uint32_t)__cvta_generic_to_shared(vn_smem) + (uint32_t)warp * (kVnStages * kVnRows * 256);
+  // the block to load next, and the block to sum next
+  int64_t f_item = first + warp, item = f_item;
+  int32_t f_layer = (int32_t)(f_item / n_blocks), layer = f_layer;
+  int64_t f_blk = f_item - f_layer * n_blocks, blk = f_blk;
+  auto advance = [&](int64_t& it, int32_t& l, int64_t& b) {
+    it += kVnWarps;
+    for (b += kVnWarps; b >= n_blocks; b -= n_blocks) ++l;
+  };
+  auto fetch = [&](int32_t stage) {
+    if (f_item < last) {
+      const uint4* src = v + f_layer * layer_stride_c;
+      const int64_t r0 = f_blk * kVnRows;
+      const uint32_t dst = ring + (uint32_t)stage * (kVnRows * 256) + (uint32_t)lane * 16;
 #pragma unroll
-      for (int it = 0; it < 16; ++it) {
-        const int64_t r = min(r0 + it * 2 + half, n_rows - 1);  // rows past the end re-read the last one; never stored
-        const uint4* p = vl + r * 16 + ch;
-        asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(buf[it].x), "=r"(buf[it].y), "=r"(buf[it].z), "=r"(buf[it].w) : "l"(p));
+      for (int i = 0; i < 8; ++i) {  // two rows per request; rows past the end repeat the last one, never stored
+        const int64_t r = min(r0 + 2 * i + (lane >> 4), n_rows - 1);
+        asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16;" ::"r"(dst + i * 512), "l"(src + r * 16 + (lane & 15)) : "memory");
       }
-#pragma unroll
-      for (int it = 0; it < 16; ++it) part[it] = Chunk<T>::sumsq(buf[it]);
-#pragma unroll
-      for (int it = 0; it < 16; ++it) {
-        float p = part[it];
-        p += __shfl_xor_sync(0xffffffffu, p, 8);
-        p += __shfl_xor_sync(0xffffffffu, p, 4);
-        p += __shfl_xor_sync(0xffffffffu, p, 2);
-        p += __shfl_xor_sync(0xffffffffu, p, 1);
-        // lanes 0..15 now hold row 2*it's sum, lanes 16..31 row 2*it+1's; lane L keeps row L
-        const float v0 = __shfl_sync(0xffffffffu, p, 0), v1 = __shfl_sync(0xffffffffu, p, 16);
-        if (lane == it * 2) mine = v0;
-        if (lane == it * 2 + 1) mine = v1;
-      }
-    } else {
-      // generic row length: one row per lane, sequential chunks
-      const int64_t r = r0 + lane;
-      if (r < n_rows) {
-        const uint4* row = vl + r * chunks_per_row;
-        for (int32_t ch = 0; ch < chunks_per_row; ++ch) mine += Chunk<T>::sumsq(__ldg(row + ch));
-      }
+      advance(f_item, f_layer, f_blk);
     }
-    const int64_t r = r0 + lane;
-    if (r < n_rows) {
+    asm volatile("cp.async.commit_group;" ::: "memory");  // (empty past the end: the group count stays in step)
+  };
+#pragma unroll
+  for (int s = 0; s < kVnStages - 1; ++s) fetch(s);
+  const int32_t row = lane >> 1;
+  int32_t stage = 0;
+  for (; item < last; advance(item, layer, blk)) {
+    fetch(stage == 0 ? kVnStages - 1 : stage - 1);  // the stage before this one
+    asm volatile("cp.async.wait_group %0;" ::"n"(kVnStages - 1) : "memory");
+    __syncwarp();
+    const uint4* p = reinterpret_cast<const uint4*>(vn_smem + warp * (kVnStages * kVnRows * 256) + stage * (kVnRows * 256)) +
+                     row * 16 + (lane & 1);
+    float e[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) e[j] = Chunk<T>::sumsq(p[2 * ((j + row) & 7)]);
+    float sum = ((e[0] + e[4]) + (e[2] + e[6])) + ((e[1] + e[5]) + (e[3] + e[7]));
+    sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+    const int64_t r = blk * kVnRows + row;
+    if ((lane & 1) == 0 && r < n_rows) {
       const int64_t t = r / n_kv_heads;
-      const int32_t g = (int32_t)(r % n_kv_heads);
-      s_out[((int64_t)layer * n_kv_heads + g) * n_tokens + t] = __ldg(c + (int64_t)g * n_tokens + t) * sqrtf(mine);
+      const int32_t g = (int32_t)(r - t * n_kv_heads);
+      s_out[((int64_t)layer * n_kv_heads + g) * n_tokens + t] = __ldg(c + (int64_t)g * n_tokens + t) * sqrtf(sum);
     }
+    __syncwarp();  // every lane has read the stage before the next fetch overwrites it
+    stage = stage == kVnStages - 1 ? 0 : stage + 1;
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // see select_kernel
+}
+
+// The same for other row lengths: a lane per row.
+template <typename T>
+__global__ void __launch_bounds__(256) vnorm_score_rows_kernel(const uint4* __restrict__ v, int64_t layer_stride_c,
+                                                               const float* __restrict__ c, int64_t n_tokens,
+                                                               int32_t n_kv_heads, int32_t n_layers, int32_t chunks_per_row,
+                                                               float* __restrict__ s_out) {
+  const int64_t n_rows = n_tokens * n_kv_heads, total = n_rows * n_layers;
+  for (int64_t x = (int64_t)blockIdx.x * 256 + threadIdx.x; x < total; x += (int64_t)gridDim.x * 256) {
+    const int32_t layer = (int32_t)(x / n_rows);
+    const int64_t r = x - layer * n_rows, t = r / n_kv_heads;
+    const int32_t g = (int32_t)(r - t * n_kv_heads);
+    const uint4* row = v + layer * layer_stride_c + r * chunks_per_row;
+    float sum = 0.f;
+    for (int32_t ch = 0; ch < chunks_per_row; ++ch) sum += Chunk<T>::sumsq(__ldg(row + ch));
+    s_out[((int64_t)layer * n_kv_heads + g) * n_tokens + t] = __ldg(c + (int64_t)g * n_tokens + t) * sqrtf(sum);
   }
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // see select_kernel
 }
@@ -118,19 +148,15 @@ struct Gather {
   int32_t cpr;
 };
 
-// One CTA per (request, KV head, layer).  FUSED = false: the scores come from `s` (written by vnorm_score_kernel).
-// FUSED = true: the CTA first streams its own segment of V (256-byte rows), forms S = C * ||V|| into shared memory
-// (and into s_out if asked), and selects from there, so V is the only large read and S never makes a round trip;
-// used when there are enough segments to keep every SM streaming.
-template <bool FUSED, typename T, bool GATHER = false>
+// One CTA per (request, KV head, layer) over the scores `s` (written by vnorm_score_kernel).  `staged`: the launch has
+// room in shared memory for the segment's keys.
+template <bool GATHER>
 __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __restrict__ s, int64_t n_tokens,
                                                              const int32_t* __restrict__ cu_seqlens,
                                                              const int32_t* __restrict__ cu_kept,
                                                              const int32_t* __restrict__ keep, int32_t window,
                                                              int32_t k_tot, int32_t n_kv_heads,
-                                                             int32_t* __restrict__ idx_out, const uint4* __restrict__ v,
-                                                             int64_t layer_stride_c, const float* __restrict__ c,
-                                                             float* __restrict__ s_out, Gather ga) {
+                                                             int32_t* __restrict__ idx_out, bool staged, Gather ga) {
   extern __shared__ __align__(16) uint32_t skeys[];  // order keys of the segment's non-recent scores
   __shared__ int32_t hist[256];
   __shared__ uint32_t sh_prefix;
@@ -141,7 +167,11 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __rest
   const int32_t r = blockIdx.x, g = blockIdx.y, layer = blockIdx.z;
   // launched with programmatic stream serialization behind vnorm_score_kernel, which releases its dependents only
   // when its own work is done: the launch latency overlaps that kernel's tail, and its scores are complete and
-  // visible from here on (no effect in an ordinary launch)
+  // visible from here on (no effect in an ordinary launch).  The CTAs of a grid of at most one wave let the next kernel
+  // (the compaction) start its CTAs beside them, where they wait: 84.6 -> 82.6 us for selection and compaction of 26 layers of
+  // 8320 tokens x 4 heads.  Those of a larger grid do not: CTAs that wait would take the room of CTAs that are still to run
+  // (864 segments: 549 -> 567 us with it).
+  if (gridDim.x * gridDim.y * gridDim.z <= 148u) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int32_t base = cu_seqlens[r];
   const int32_t len = cu_seqlens[r + 1] - base;
@@ -153,53 +183,9 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __rest
   const int32_t tid = threadIdx.x;
 
   for (int32_t t = tid; t < w; t += kSelThreads) out[h + t] = nr + t;  // the recent window
-  if constexpr (FUSED) {
-    // a half-warp reads one 256-byte row per step (16 x 16 bytes), 16 rows in flight per thread
-    const uint4* vl = v + layer * layer_stride_c;
-    const float* cg = c + (int64_t)g * n_tokens + base;
-    float* so = s_out ? s_out + ((int64_t)layer * n_kv_heads + g) * n_tokens + base : nullptr;
-    const int32_t lane = tid & 31, wrp = tid >> 5, half = lane >> 4, ch = lane & 15;
-    const int32_t n_score = so ? len : nr;  // the window's scores are 0 by definition and only matter for s_out
-    for (int32_t t0 = wrp * 32; t0 < n_score; t0 += (kSelThreads / 32) * 32) {
-      // as in vnorm_score_kernel: the 16 row loads of the trip are issued before the first is used
-      float part[16];
-      uint4 buf[16];
-#pragma unroll
-      for (int it = 0; it < 16; ++it) {
-        const int32_t t = min(t0 + it * 2 + half, n_score - 1);  // rows past the end re-read the last one; never stored
-        const uint4* p = vl + ((int64_t)(base + t) * n_kv_heads + g) * 16 + ch;
-        asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(buf[it].x), "=r"(buf[it].y), "=r"(buf[it].z), "=r"(buf[it].w) : "l"(p));
-      }
-#pragma unroll
-      for (int it = 0; it < 16; ++it) part[it] = Chunk<T>::sumsq(buf[it]);
-      float mine = 0.f;
-#pragma unroll
-      for (int it = 0; it < 16; ++it) {
-        float p = part[it];
-        p += __shfl_xor_sync(0xffffffffu, p, 8);
-        p += __shfl_xor_sync(0xffffffffu, p, 4);
-        p += __shfl_xor_sync(0xffffffffu, p, 2);
-        p += __shfl_xor_sync(0xffffffffu, p, 1);
-        const float v0 = __shfl_sync(0xffffffffu, p, 0), v1 = __shfl_sync(0xffffffffu, p, 16);
-        if (lane == it * 2) mine = v0;
-        if (lane == it * 2 + 1) mine = v1;
-      }
-      const int32_t t = t0 + lane;
-      if (t < n_score) {
-        const float sc = __ldg(cg + t) * sqrtf(mine);
-        if (so) so[t] = sc;
-        if (t < nr) skeys[t] = order_key(sc);
-      }
-    }
-    __syncthreads();
-  }
-  // Not fused: the keys are copied into shared memory once when the launch provided room for them (s_out is unused
-  // in this mode and doubles as that flag), so the radix passes do not go back to L2.
-  const bool staged = FUSED || s_out != nullptr;
   // the range of the keys, taken along the way: the radix select only has to resolve the bits in which they differ
   uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
-  if (!FUSED && staged) {
+  if (staged) {  // copied into shared memory once, so the radix passes do not go back to L2
 #pragma unroll 8
     for (int32_t j = tid; j < nr; j += kSelThreads) {  // loads of a trip in flight together
       const uint32_t key = order_key(__ldg(seg + j));
@@ -212,7 +198,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __rest
   const int32_t lane = tid & 31, warp = tid >> 5;
   if (h > 0) {
 
-  if (FUSED || !staged) {
+  if (!staged) {
 #pragma unroll 4
     for (int32_t j = tid; j < nr; j += kSelThreads) {
       const uint32_t key = key_at(j);
@@ -492,51 +478,50 @@ static purekv_status select_impl(const float* c, const void* v, int64_t v_layer_
   const int32_t cpr = (int32_t)(head_dim * esz / 16);
   dim3 g2((unsigned)batch->n_req, (unsigned)n_kv_heads, (unsigned)n_layers);
   const int32_t k_tot = h_cu_kept[batch->n_req];
-  // Fused path: each (request, head, layer) segment is streamed, scored and selected by one CTA.  It needs 256-byte
-  // rows, the segment's keys in shared memory, and enough segments to occupy the SMs; otherwise V is streamed by a
-  // grid-wide kernel first and the selection reads the scores back.
   int32_t longest = 0;
   for (int r = 0; r < batch->n_req; ++r) longest = std::max(longest, batch->h_cu_seqlens[r + 1] - batch->h_cu_seqlens[r]);
   const size_t key_bytes = (size_t)longest * sizeof(uint32_t);
-  const int64_t segments = (int64_t)batch->n_req * n_kv_heads * n_layers;
-  if (cpr == 16 && key_bytes <= 200 * 1024 && segments >= 2 * 148) {
-    auto launch_fused = [&](auto kernel, std::atomic<uint64_t>& smem_allowed) -> purekv_status {
-      const purekv_status st_smem = allow_max_dynamic_smem(kernel, smem_allowed);
-      if (st_smem != PUREKV_OK) return st_smem;
-      kernel<<<g2, kSelThreads, key_bytes, sm>>>(nullptr, T, batch->cu_seqlens, cu_kept, keep, window, k_tot, n_kv_heads,
-                                                 idx_out, (const uint4*)v, v_layer_stride * esz / 16, c, s_out, ga);
-      PK_CUDA(cudaGetLastError());
-      return PUREKV_OK;
-    };
-    static std::atomic<uint64_t> allowed[4] = {{0}, {0}, {0}, {0}};
-    const bool gather = ga.k_src != nullptr;
-    if (dtype == PUREKV_BF16)
-      return gather ? launch_fused(select_kernel<true, __nv_bfloat16, true>, allowed[0])
-                    : launch_fused(select_kernel<true, __nv_bfloat16, false>, allowed[1]);
-    return gather ? launch_fused(select_kernel<true, float, true>, allowed[2])
-                  : launch_fused(select_kernel<true, float, false>, allowed[3]);
-  }
   float* s_buf = s_out;
   if (!s_buf) {
     PK_REQUIRE(ws && ws_bytes >= purekv_select_ws_bytes(batch, n_layers, n_kv_heads), PUREKV_ERR_WORKSPACE,
                "purekv_select_topk: workspace of %zu bytes is too small", ws_bytes);
     s_buf = (float*)(((uintptr_t)ws + 255) & ~(uintptr_t)255);
   }
-  const int64_t n_items = ((T * n_kv_heads + 31) / 32) * n_layers;  // blocks of 32 (token, head) rows per layer
-  dim3 g1((unsigned)std::min<int64_t>((n_items + 7) / 8, 148 * 3));   // one wave: 3 CTAs of 256 threads per SM (measured best)
-  if (dtype == PUREKV_BF16)
-    vnorm_score_kernel<__nv_bfloat16><<<g1, 256, 0, sm>>>((const uint4*)v, v_layer_stride * esz / 16, c, T, n_kv_heads,
-                                                          n_layers, cpr, s_buf);
-  else
-    vnorm_score_kernel<float><<<g1, 256, 0, sm>>>((const uint4*)v, v_layer_stride * esz / 16, c, T, n_kv_heads, n_layers,
-                                                  cpr, s_buf);
-  PK_CUDA(cudaGetLastError());
+  auto launch_vnorm = [&](auto tag) -> purekv_status {
+    using E = decltype(tag);
+    const int64_t stride_c = v_layer_stride * esz / 16;
+    if (cpr != 16) {
+      const int64_t blocks = (T * n_kv_heads * n_layers + 255) / 256;
+      vnorm_score_rows_kernel<E><<<(unsigned)std::min<int64_t>(blocks, 148 * 8), 256, 0, sm>>>((const uint4*)v, stride_c, c, T,
+                                                                                            n_kv_heads, n_layers, cpr, s_buf);
+      PK_CUDA(cudaGetLastError());
+      return PUREKV_OK;
+    }
+    static std::atomic<uint64_t> smem_allowed{0};
+    const purekv_status st_smem = allow_max_dynamic_smem(vnorm_score_kernel<E>, smem_allowed);
+    if (st_smem != PUREKV_OK) return st_smem;
+    const int64_t blocks = ((T * n_kv_heads + kVnRows - 1) / kVnRows) * n_layers;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min<int64_t>((blocks + kVnWarps - 1) / kVnWarps, 148));
+    cfg.blockDim = dim3(kVnWarps * 32);
+    cfg.dynamicSmemBytes = kVnSmem;
+    cfg.stream = sm;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    PK_CUDA(cudaLaunchKernelEx(&cfg, vnorm_score_kernel<E>, (const uint4*)v, stride_c, c, T, n_kv_heads, n_layers, s_buf));
+    return PUREKV_OK;
+  };
+  const purekv_status st_v = dtype == PUREKV_BF16 ? launch_vnorm(__nv_bfloat16{}) : launch_vnorm(float{});
+  if (st_v != PUREKV_OK) return st_v;
   const bool stage_keys = key_bytes <= 200 * 1024;
   const bool gather = ga.k_src != nullptr;
   if (stage_keys) {
     static std::atomic<uint64_t> smem_allowed{0}, smem_allowed_g{0};
-    const purekv_status st_smem = gather ? allow_max_dynamic_smem(select_kernel<false, float, true>, smem_allowed_g)
-                                         : allow_max_dynamic_smem(select_kernel<false, float, false>, smem_allowed);
+    const purekv_status st_smem = gather ? allow_max_dynamic_smem(select_kernel<true>, smem_allowed_g)
+                                         : allow_max_dynamic_smem(select_kernel<false>, smem_allowed);
     if (st_smem != PUREKV_OK) return st_smem;
   }
   cudaLaunchConfig_t cfg = {};
@@ -550,13 +535,11 @@ static purekv_status select_impl(const float* c, const void* v, int64_t v_layer_
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (gather)
-    PK_CUDA(cudaLaunchKernelEx(&cfg, select_kernel<false, float, true>, (const float*)s_buf, T, batch->cu_seqlens, cu_kept,
-                               keep, window, k_tot, n_kv_heads, idx_out, (const uint4*)nullptr, (int64_t)0,
-                               (const float*)nullptr, stage_keys ? s_buf : (float*)nullptr, ga));
+    PK_CUDA(cudaLaunchKernelEx(&cfg, select_kernel<true>, (const float*)s_buf, T, batch->cu_seqlens, cu_kept,
+                               keep, window, k_tot, n_kv_heads, idx_out, stage_keys, ga));
   else
-    PK_CUDA(cudaLaunchKernelEx(&cfg, select_kernel<false, float, false>, (const float*)s_buf, T, batch->cu_seqlens, cu_kept,
-                               keep, window, k_tot, n_kv_heads, idx_out, (const uint4*)nullptr, (int64_t)0,
-                               (const float*)nullptr, stage_keys ? s_buf : (float*)nullptr, ga));
+    PK_CUDA(cudaLaunchKernelEx(&cfg, select_kernel<false>, (const float*)s_buf, T, batch->cu_seqlens, cu_kept,
+                               keep, window, k_tot, n_kv_heads, idx_out, stage_keys, ga));
   PK_CUDA(cudaGetLastError());
   return PUREKV_OK;
 }
