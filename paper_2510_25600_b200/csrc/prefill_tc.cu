@@ -374,123 +374,123 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       constexpr uint32_t idesc_qk = instr_desc(BK, false);
       constexpr uint32_t idesc_qk_half = instr_desc(BK / 2, false);
       constexpr uint32_t idesc_pv = instr_desc(kD, true);
-      uint32_t it_base = 0;            // key tiles of earlier units
-      uint32_t tq[2] = {0, 0};         // S products issued per slot, over all units
-      uint32_t tp[2] = {0, 0};         // P.V products issued per slot, over all units
-      int32_t nt = 0, n_slots = 0;
-      int32_t pend_v = -1;             // V stage whose release is due behind the next S product
+      static_assert(SB == 1 && ST == 2, "S of a tile is issued behind P V of the tile before, which frees its columns");
+      uint32_t it = 0;          // the CTA's key tiles so far
+      uint32_t tp0 = 0, tp1 = 0;  // ... and those of each slot, P V issued
       // Descriptor words.  High word: stride between 8-row groups 1024 B, descriptor version 1, 128-byte swizzle.
       // Low word: start address / 16 and the leading-dimension offset / 16 (used by the MN-major V operand only).
       constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
       const uint32_t q_lo0 = ((sQ & 0x3FFFFu) >> 4) | (1u << 16);
       const uint32_t k_lo0 = ((sK & 0x3FFFFu) >> 4) | (1u << 16);
       const uint32_t v_lo0 = ((sV & 0x3FFFFu) >> 4) | ((kPanelKV >> 4) << 16);
-      // S(slot, n) = Q_slot K_n^T; the last slot to read K_n releases its stage
-      auto issue_qk = [&](auto sl_c, int32_t n) -> bool {
-        constexpr int sl = decltype(sl_c)::value;  // compile-time slot: the per-slot counters stay in registers
-        const uint32_t it = it_base + (uint32_t)n;
-        const uint32_t s = it % ST, b = tq[sl] % SB;
-        // the stage was already awaited for slot 0 of the same tile
-        if (sl == 0 && !mbar_wait(smem_u32(&bars.k_full[s]), (it / ST) & 1u, abort_flag, wait_ns)) return false;
-        tc_fence_after();
-        const uint32_t hm = (uint32_t)((meta_s[it % MR][0].x | meta_s[it % MR][1].x) >> 2) & 3u;  // written before the stage's barrier was armed
+      auto halves_of = [&](uint32_t i) {  // written before the stage's barrier was armed
+        return (uint32_t)((meta_s[i % MR][0].x | meta_s[i % MR][1].x) >> 2) & 3u;
+      };
+      // S = Q K^T of a tile in stage s, announced to the slot's rows.  A commit costs the issuing thread about as long as a
+      // product and the rows are waiting for S, so the releases of the stages follow behind and cover the same products.
+      auto issue_qk = [&](auto sl_c, uint32_t s, uint32_t hm) {
+        constexpr int sl = decltype(sl_c)::value;
         const uint32_t q_lo = q_lo0 + (uint32_t)sl * (kTileQ >> 4);
         if (hm == 3u) {
-          const uint32_t d_addr = tmem + sl * 128 + b * BK, k_lo = k_lo0 + s * (kTileKV >> 4);
+          const uint32_t d_addr = tmem + sl * 128, k_lo = k_lo0 + s * (kTileKV >> 4);
 #pragma unroll
           for (int ks = 0; ks < kD / 16; ++ks)
             mma_ss_lh(d_addr, q_lo + (ks >> 2) * (kPanelQ >> 4) + (ks & 3) * 2, kDescHi,
                       k_lo + (ks >> 2) * (kPanelKV >> 4) + (ks & 3) * 2, kDescHi, idesc_qk, ks > 0 ? 1u : 0u);
         } else {  // one 64-key half: N = 64, into that half's columns of S
           const uint32_t hh = hm >> 1;
-          const uint32_t d_addr = tmem + sl * 128 + b * BK + hh * 64;
+          const uint32_t d_addr = tmem + sl * 128 + hh * 64;
           const uint32_t k_lo = k_lo0 + s * (kTileKV >> 4) + hh * (kPanelKV >> 5);
 #pragma unroll
           for (int ks = 0; ks < kD / 16; ++ks)
             mma_ss_lh(d_addr, q_lo + (ks >> 2) * (kPanelQ >> 4) + (ks & 3) * 2, kDescHi,
                       k_lo + (ks >> 2) * (kPanelKV >> 4) + (ks & 3) * 2, kDescHi, idesc_qk_half, ks > 0 ? 1u : 0u);
         }
-        // A commit costs the issuing thread about as long as a product and the slot's rows are waiting for S, so S
-        // is announced first; the releases behind it (and the V release a preceding P.V left pending) cover the
-        // same products and only reach the producer a little later.
-        tc_commit(smem_u32(&bars.s_full[sl][b]));
-        if (pend_v >= 0) {
-          tc_commit(smem_u32(&bars.v_empty[pend_v]));
-          pend_v = -1;
-        }
-        if (sl == n_slots - 1) {
-          tc_commit(smem_u32(&bars.k_empty[s]));
-          if (n == nt - 1) tc_commit(smem_u32(&bars.q_empty));  // the unit's last read of Q
-        }
-        ++tq[sl];
+        tc_commit(smem_u32(&bars.s_full[sl][0]));
+      };
+      // O(slot) += P V of a tile: the part that waits for the first 96 keys' P ...
+      auto issue_pv_head = [&](auto sl_c, uint32_t s, uint32_t hm, uint32_t par, uint32_t acc0) -> bool {
+        constexpr int sl = decltype(sl_c)::value;
+        // B = V tile, MN-major: per K step 16 key rows (2 groups of 8, 1024 B apart) x 128 dims (2 panels)
+        const uint32_t p_addr = tmem + sl * 128, o_addr = tmem + kColO + sl * 128, v_lo = v_lo0 + s * (kTileKV >> 4);
+        if (hm != 3u) return true;
+        // P of the unit's first tile also implies that the previous unit's output has left TMEM
+        if (!mbar_wait(smem_u32(&bars.p_part[sl]), par, abort_flag, wait_ns)) return false;
+        tc_fence_after();
+#pragma unroll
+        for (int ks = 0; ks < 6; ++ks)
+          mma_ts_lh(o_addr, p_addr + ks * 8, v_lo + ks * (2048 >> 4), kDescHi, idesc_pv, ks > 0 ? 1u : acc0);
         return true;
       };
-      // O(slot) += P(slot, n) V_n; the last slot to read V_n releases its stage
-      auto issue_pv = [&](auto sl_c, int32_t n) -> bool {
+      // ... and the rest
+      auto issue_pv_tail = [&](auto sl_c, uint32_t s, uint32_t hm, uint32_t par, uint32_t acc0) -> bool {
         constexpr int sl = decltype(sl_c)::value;
-        const uint32_t it = it_base + (uint32_t)n;
-        const uint32_t s = it % ST, b = tp[sl] % SB;
-        if (sl == 0 && !mbar_wait(smem_u32(&bars.v_full[s]), (it / ST) & 1u, abort_flag, wait_ns)) return false;
-        const uint32_t p_addr = tmem + sl * 128 + b * BK, o_addr = tmem + kColO + sl * 128;
-        // B = V tile, MN-major: per K step 16 key rows (2 groups of 8, 1024 B apart) x 128 dims (2 panels)
-        const uint32_t v_lo = v_lo0 + s * (kTileKV >> 4);
-        const uint32_t hm = (uint32_t)((meta_s[it % MR][0].x | meta_s[it % MR][1].x) >> 2) & 3u;
-        const uint32_t acc0 = n > 0 ? 1u : 0u;  // the unit's first product overwrites O
-        // P of the unit's first tile also implies that the previous unit's output has left TMEM
-        if (hm == 3u) {  // six of the eight K steps run while the rows are still in the last quarter's exponentials
-          if (!mbar_wait(smem_u32(&bars.p_part[sl]), tp[sl] & 1u, abort_flag, wait_ns)) return false;
-          tc_fence_after();
-#pragma unroll
-          for (int ks = 0; ks < 6; ++ks)
-            mma_ts_lh(o_addr, p_addr + ks * 8, v_lo + ks * (2048 >> 4), kDescHi, idesc_pv, ks > 0 ? 1u : acc0);
-          if (!mbar_wait(smem_u32(&bars.p_full[sl][b]), (tp[sl] / SB) & 1u, abort_flag, wait_ns)) return false;
-          tc_fence_after();
+        const uint32_t p_addr = tmem + sl * 128, o_addr = tmem + kColO + sl * 128, v_lo = v_lo0 + s * (kTileKV >> 4);
+        if (!mbar_wait(smem_u32(&bars.p_full[sl][0]), par, abort_flag, wait_ns)) return false;
+        tc_fence_after();
+        if (hm == 3u) {
 #pragma unroll
           for (int ks = 6; ks < 8; ++ks)
             mma_ts_lh(o_addr, p_addr + ks * 8, v_lo + ks * (2048 >> 4), kDescHi, idesc_pv, 1u);
         } else {  // the K steps of the present half only
-          if (!mbar_wait(smem_u32(&bars.p_full[sl][b]), (tp[sl] / SB) & 1u, abort_flag, wait_ns)) return false;
-          tc_fence_after();
           const uint32_t k0 = (hm >> 1) * (BK / 32);
 #pragma unroll
           for (int ks = 0; ks < BK / 32; ++ks)
             mma_ts_lh(o_addr, p_addr + (k0 + ks) * 8, v_lo + (k0 + ks) * (2048 >> 4), kDescHi, idesc_pv, ks > 0 ? 1u : acc0);
         }
-        if (SB > 1) tc_commit(smem_u32(&bars.o_done[sl]));
-        if (n == nt - 1) tc_commit(smem_u32(&bars.o_final[sl]));
-        if (sl == n_slots - 1) {
-          // the V stage is released behind the S product that follows, if one does (see issue_qk)
-          if (n + SB < nt) pend_v = (int32_t)s;
-          else tc_commit(smem_u32(&bars.v_empty[s]));
-        }
-        ++tp[sl];
         return true;
       };
+      constexpr std::integral_constant<int, 0> s0{};
+      constexpr std::integral_constant<int, 1> s1{};
       bool ok = true;
       for (uint32_t uo = 0; ok; ++uo) {
         const uint32_t us = uo % kUnitRing;
-        if (!mbar_wait(smem_u32(&bars.u_full[us]), (uo / kUnitRing) & 1u, abort_flag, wait_ns)) { ok = false; break; }
-        const Unit u = unit_s[us];
+        ok = mbar_wait(smem_u32(&bars.u_full[us]), (uo / kUnitRing) & 1u, abort_flag, wait_ns);
+        if (!ok) break;
+        const int32_t nt = unit_s[us].ent_count;
+        const bool two = unit_s[us].q_rows1 != 0 || 2 * (unit_s[us].pair % ppg) + 1 < G;
         mbar_arrive(smem_u32(&bars.u_empty[us]));
-        if (u.ent_count == 0) break;
-        nt = u.ent_count;
-        n_slots = (u.q_rows1 != 0 || 2 * (u.pair % ppg) + 1 < G) ? 2 : 1;
-        ok = mbar_wait(smem_u32(&bars.q_full), uo & 1u, abort_flag, wait_ns);
-        constexpr std::integral_constant<int, 0> s0{};
-        constexpr std::integral_constant<int, 1> s1{};
-        for (int32_t n = 0; ok && n < SB && n < nt; ++n) {
-          ok = issue_qk(s0, n);
-          if (ok && n_slots == 2) ok = issue_qk(s1, n);
-        }
-        for (int32_t n = 0; ok && n < nt; ++n) {
-          ok = issue_pv(s0, n);
-          if (ok && n + SB < nt) ok = issue_qk(s0, n + SB);  // in order behind P.V of tile n, which frees S(slot, n % SB)
-          if (ok && n_slots == 2) {
-            ok = issue_pv(s1, n);
-            if (ok && n + SB < nt) ok = issue_qk(s1, n + SB);
+        if (nt == 0) break;
+        ok = mbar_wait(smem_u32(&bars.q_full), uo & 1u, abort_flag, wait_ns) &&
+             mbar_wait(smem_u32(&bars.k_full[it % ST]), (it / ST) & 1u, abort_flag, wait_ns);
+        if (!ok) break;
+        tc_fence_after();
+        uint32_t hm = halves_of(it);
+        issue_qk(s0, it % ST, hm);
+        if (two) issue_qk(s1, it % ST, hm);
+        tc_commit(smem_u32(&bars.k_empty[it % ST]));
+        if (nt == 1) tc_commit(smem_u32(&bars.q_empty));  // the unit's last read of Q
+        // Everything that the next S needs besides P V (its K, which halves) is awaited and read between the two parts of
+        // P V, so that nothing but products stands between the rows' last P and their next S: the slot's rows wait for this
+        // thread, and each wait or branch in between showed (8320 tokens: dense causal 406 -> 390 us, paper mask 116 -> 110 us).
+        uint32_t acc = 0u;  // the unit's first product overwrites O
+        for (int32_t n = 0; n < nt; ++n, ++it) {
+          const uint32_t s = it % ST, sn = (it + 1u) % ST;
+          const bool more = n + 1 < nt;
+          uint32_t hn = 3u;
+          ok = mbar_wait(smem_u32(&bars.v_full[s]), (it / ST) & 1u, abort_flag, wait_ns) && issue_pv_head(s0, s, hm, tp0 & 1u, acc);
+          if (ok && more) {
+            ok = mbar_wait(smem_u32(&bars.k_full[sn]), ((it + 1u) / ST) & 1u, abort_flag, wait_ns);
+            hn = halves_of(it + 1u);
           }
+          ok = ok && issue_pv_tail(s0, s, hm, tp0 & 1u, acc);
+          if (!ok) break;
+          ++tp0;
+          if (more) issue_qk(s0, sn, hn);
+          else tc_commit(smem_u32(&bars.o_final[0]));
+          if (two) {
+            ok = issue_pv_head(s1, s, hm, tp1 & 1u, acc) && issue_pv_tail(s1, s, hm, tp1 & 1u, acc);
+            if (!ok) break;
+            ++tp1;
+            if (more) issue_qk(s1, sn, hn);
+            else tc_commit(smem_u32(&bars.o_final[1]));
+          }
+          tc_commit(smem_u32(&bars.v_empty[s]));
+          if (more) tc_commit(smem_u32(&bars.k_empty[sn]));
+          if (n + 2 == nt) tc_commit(smem_u32(&bars.q_empty));
+          acc = 1u;
+          hm = hn;
         }
-        it_base += (uint32_t)nt;
       }
       if (!ok) {
         // leaving early: let every issued MMA finish before TMEM is released
