@@ -106,6 +106,8 @@ struct QTile {
 // entry.y = for a general tile, the index of its first mask word: row r of the query tile owns
 // words [entry.y + r*words_per_row, +words_per_row), bit c of word w = key 32*w + c of the tile
 // (causality already applied; rows past q_rows are zero); -1 otherwise.
+// In tensor-core plans the last n_entries words of the masks section are, one per entry, the halves of its tile that hold
+// any kept pair: those of the half mask, less the ones in which the bit mask is empty (a half mask of 3 may claim too much).
 
 // One unit of work of the tensor-core kernel: a query tile x a pair of query heads x a contiguous
 // chunk of the tile's kept-key list.  The list is sorted by decreasing estimated cost; CTA c of n_ctas starts with

@@ -402,6 +402,7 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
   std::vector<QTile>& qtiles = plan.qtiles;
   std::vector<int2>& entries = plan.entries;
   std::vector<uint32_t>& masks = plan.masks;
+  std::vector<uint32_t> mask_halves;  // per mask of a tensor-core plan: bit h set when its keys 64h .. 64h+63 hold any kept pair
   memset(info, 0, sizeof(*info));
 
   std::vector<int64_t> cnt, diff, cg;  // kept pairs per gk-key block of the current query tile
@@ -587,6 +588,7 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
       }
       if (n_general) {  // row by row, each span into the masks of the tiles it crosses
         masks.resize(masks.size() + (size_t)n_general * tq * wpr, 0u);
+        if (tq == 128) mask_halves.resize(mask_halves.size() + (size_t)n_general, 0u);
         for (int32_t i = q0; i < q1; ++i)
           for (int32_t s = row_off[i - q0]; s < row_off[i - q0 + 1]; ++s) {
             const int32_t a = row_spans[s].a, bb = row_spans[s].b;
@@ -594,6 +596,7 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
               if (mask_of[kt] < 0) continue;
               const int32_t j0 = kt << tsh, lo = std::max(a - j0, 0), hi = std::min(bb - j0, tk - 1);  // bit range inside the tile row
               uint32_t* rw = masks.data() + mask_of[kt] + (size_t)(i - q0) * wpr;
+              if (tq == 128) mask_halves[(size_t)mask_of[kt] / (128 * 4)] |= (1u << (lo >> 6)) | (1u << (hi >> 6));
               for (int32_t w = lo >> 5; w <= (hi >> 5); ++w) {
                 const int32_t b0 = std::max(lo - 32 * w, 0), b1 = std::min(hi - 32 * w, 31);
                 rw[w] |= (b1 - b0 == 31) ? 0xFFFFFFFFu : (((1u << (b1 - b0 + 1)) - 1u) << b0);
@@ -619,6 +622,13 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
   int64_t part_slots = 0;
   if (tq == 128 && nq > 0) {
     schedule_units(qtiles, entries, n_q_heads, n_kv_heads, n_ctas, units, &n_counters, &part_slots, &max_chunks);
+    const size_t n_masks = masks.size();
+    PK_REQUIRE(n_masks + entries.size() < (size_t)INT32_MAX, PUREKV_ERR_UNSUPPORTED, "mask table exceeds 2^31 words");
+    masks.resize(n_masks + entries.size());
+    for (size_t i = 0; i < entries.size(); ++i) {
+      const uint32_t listed = ((uint32_t)entries[i].x >> 2) & 3u;
+      masks[n_masks + i] = (entries[i].x & 3) == kTileGeneral ? listed & mask_halves[(size_t)entries[i].y / (128 * 4)] : listed;
+    }
   } else {
     n_ctas = 0;
   }
