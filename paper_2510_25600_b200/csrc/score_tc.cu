@@ -33,6 +33,23 @@ namespace sc {
 constexpr int kScorePoly = PUREKV_SCORE_POLY;
 using namespace tc;
 
+// Adds the exponentials of 32 columns of a key's logits to its sums; l4: minus the columns' log-sum-exp, in log2 units.
+// Everything but MUFU works on pairs: the kernel is paced by the instructions its warps issue (0.66 of the issue slots busy,
+// MUFU 0.48, FMA 0.49, tensor 0.37), not by one unit.  37 120 tokens, 1792 rows per head: 90 -> 87 us with pairs, 79 with the
+// log-sum-exp fetched once per group of warps besides; all exponentials on MUFU 98 us, 6 of 8 second pairs on FMA the best.
+__device__ __forceinline__ void add_exps(const uint32_t (&r)[32], const float4* l4, float scale_log2, float2 (&acc)[2]) {
+  const float2 sc = make_float2(scale_log2, scale_log2);
+#pragma unroll
+  for (int x = 0; x < 32; x += 4) {
+    const float4 l = l4[x >> 2];
+    const float2 a = __ffma2_rn(make_float2(__uint_as_float(r[x]), __uint_as_float(r[x + 1])), sc, make_float2(l.x, l.y));
+    const float2 b = __ffma2_rn(make_float2(__uint_as_float(r[x + 2]), __uint_as_float(r[x + 3])), sc, make_float2(l.z, l.w));
+    acc[0] = __fadd2_rn(acc[0], make_float2(ex2(a.x), ex2(a.y)));
+    // some of the other pairs' exponentials on the FMA pipe, beside the MUFU unit (one ex2 per logit otherwise)
+    acc[1] = __fadd2_rn(acc[1], (x >> 2) < kScorePoly ? exp2_poly2(b) : make_float2(ex2(b.x), ex2(b.y)));
+  }
+}
+
 constexpr int kKeys = 128, kRows = 128;
 constexpr int kThreads = 320;
 constexpr int kStages = 2;         // Q-row blocks in flight
@@ -44,6 +61,7 @@ struct __align__(8) Barriers {
   uint64_t k_full;
   uint64_t q_full[kStages], q_empty[kStages];
   uint64_t d_full[2], d_empty[2];
+  uint64_t l_full[2];  // a group's log-sum-exp values of its next block are in lse_s
   uint64_t drain;
 };
 
@@ -56,7 +74,7 @@ __global__ void __launch_bounds__(kThreads, 2) score_tc_kernel(
     int32_t box_rows) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ Barriers bars;
-  __shared__ __align__(16) float lse_s[8][2][kRows];  // per epilogue warp: the log-sum-exp values of two blocks of rows
+  __shared__ __align__(16) float lse_s[2][2][kRows];  // per epilogue group: minus the log-sum-exp of two blocks of rows
   __shared__ float comb_s[kKeys];                     // the second group's column sums, for the first to add
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s;
@@ -92,6 +110,7 @@ __global__ void __launch_bounds__(kThreads, 2) score_tc_kernel(
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&bars.d_full[b]), 1);
       mbar_init(smem_u32(&bars.d_empty[b]), 4);  // one arrival per epilogue warp
+      mbar_init(smem_u32(&bars.l_full[b]), 4);
     }
     mbar_init(smem_u32(&bars.drain), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -175,41 +194,37 @@ __global__ void __launch_bounds__(kThreads, 2) score_tc_kernel(
     const int key = quad * 32 + lane;
     const uint32_t t_lane = tmem + ((uint32_t)(quad * 32) << 16);
     const float kLog2e = 1.4426950408889634f;
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
     bool ok = true;
-    // The log-sum-exp of a block's 128 stacked rows (log2 units; +inf for absent rows): every key needs all of them.
-    // Each warp keeps its own copy in shared memory, fetched one block ahead (lane i loads rows i, i+32, i+64, i+96)
-    // and read back four at a time; no meeting between warps is needed.
-    float (*my_lse)[kRows] = lse_s[warp - 2];
+    // The log-sum-exp of a block's 128 stacked rows (log2 units, negated; -inf for absent rows): every key needs all of them.
+    // Each warp of the group fetches a quarter, one block ahead, into the group's copy in shared memory.  (All 128 by every
+    // warp, without this meeting, was a sixth of the warps' instructions.)
     const uint32_t w_inv = (uint32_t)(0x100000000ull / (uint32_t)w);  // floor(2^32 / w): the quotient estimate is low by at most 1
-    auto fetch_lse = [&](int32_t t, float (&lv)[4]) {
+    auto fetch_lse = [&](int32_t t) -> float {
       const int32_t blk = t + rot < n_blocks ? t + rot : t + rot - n_blocks;  // t and rot are both below n_blocks
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int32_t row = blk * kRows + 32 * c + lane;
-        lv[c] = INFINITY;
-        if (row < n_rows) {
-          // row / w by a multiplication (a division per row and block is a tenth of this warp's instructions)
-          int32_t head = (int32_t)__umulhi((uint32_t)row, w_inv);
-          head += (head + 1) * w <= row;
-          lv[c] = __ldg(lse + (int64_t)(g * G + head) * n_tokens + base + len - w + (row - head * w)) * kLog2e;
-        }
-      }
+      const int32_t row = blk * kRows + key;
+      if (row >= n_rows) return -INFINITY;
+      // row / w by a multiplication (a division per row and block is a tenth of this warp's instructions)
+      int32_t head = (int32_t)__umulhi((uint32_t)row, w_inv);
+      head += (head + 1) * w <= row;
+      return __ldg(lse + (int64_t)(g * G + head) * n_tokens + base + len - w + (row - head * w)) * -kLog2e;
     };
-    float lv[4];
-    if (wg < n_blocks) {
-      fetch_lse(wg, lv);
-#pragma unroll
-      for (int c = 0; c < 4; ++c) my_lse[0][32 * c + lane] = lv[c];
-    }
-    __syncwarp();
+    // (a buffer's last readers have announced their share of the block before this one, so it is free)
+    auto hand_lse = [&](int32_t n, float lv) {
+      lse_s[wg][n & 1][key] = lv;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&bars.l_full[wg]));
+    };
+    if (wg < n_blocks) hand_lse(0, fetch_lse(wg));
     for (int32_t t = wg, n = 0; ok && t < n_blocks; t += 2, ++n) {
-      const int32_t b = wg, lb = n & 1;
-      if (t + 2 < n_blocks) fetch_lse(t + 2, lv);  // in flight while this block is summed
-      ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.d_full[b]), (t >> 1) & 1, abort_flag, wait_ns) ? 1 : 0) != 0;
+      const int32_t b = wg;
+      float lv = 0.f;
+      if (t + 2 < n_blocks) lv = fetch_lse(t + 2);  // in flight while this block is summed
+      ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.l_full[wg]), n & 1, abort_flag, wait_ns) &&
+                                           mbar_wait(smem_u32(&bars.d_full[b]), (t >> 1) & 1, abort_flag, wait_ns) ? 1 : 0) != 0;
       if (!ok) break;
       tc_fence_after();
-      const float4* l4 = reinterpret_cast<const float4*>(my_lse[lb]);
+      const float4* l4 = reinterpret_cast<const float4*>(lse_s[wg][n & 1]);
       // the next 32 columns are on their way from TMEM while the current ones go through the exponentials
       uint32_t rr[2][32];
       tmem_ld32(t_lane + b * kRows, rr[0]);
@@ -217,35 +232,15 @@ __global__ void __launch_bounds__(kThreads, 2) score_tc_kernel(
       for (int c = 0; c < 4; ++c) {
         tc_wait_ld();
         if (c + 1 < 4) tmem_ld32(t_lane + b * kRows + 32 * (c + 1), rr[(c + 1) & 1]);
-#pragma unroll
-        for (int x = 0; x < 32; x += 4) {
-          const float4 l = l4[8 * c + (x >> 2)];
-          acc[0] += ex2(fmaf(__uint_as_float(rr[c & 1][x]), scale_log2, -l.x));
-          acc[1] += ex2(fmaf(__uint_as_float(rr[c & 1][x + 1]), scale_log2, -l.y));
-          if ((x >> 2) < kScorePoly) {
-            // this pair's exponentials on the FMA pipe: the kernel is paced by the MUFU unit (one ex2 per logit)
-            const float2 a = __ffma2_rn(make_float2(__uint_as_float(rr[c & 1][x + 2]), __uint_as_float(rr[c & 1][x + 3])),
-                                        make_float2(scale_log2, scale_log2), make_float2(-l.z, -l.w));
-            const float2 pp = exp2_poly2(a);
-            acc[2] += pp.x;
-            acc[3] += pp.y;
-          } else {
-            acc[2] += ex2(fmaf(__uint_as_float(rr[c & 1][x + 2]), scale_log2, -l.z));
-            acc[3] += ex2(fmaf(__uint_as_float(rr[c & 1][x + 3]), scale_log2, -l.w));
-          }
-        }
+        add_exps(rr[c & 1], l4 + 8 * c, scale_log2, acc);
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bars.d_empty[b]));
-      if (t + 2 < n_blocks) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) my_lse[lb ^ 1][32 * c + lane] = lv[c];  // last read two of this warp's blocks ago
-        __syncwarp();
-      }
+      if (t + 2 < n_blocks) hand_lse(n + 1, lv);
     }
     // the two groups' sums meet after the CTA's closing barrier
-    col_sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    col_sum = (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
     if (wg == 1) comb_s[key] = col_sum;
   }
 
@@ -485,12 +480,12 @@ __global__ void __launch_bounds__(kThreads, 2) score_tc_items_kernel(
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const int32_t row = blk * kRows + 32 * c + lane;
-        lv[c] = INFINITY;
+        lv[c] = -INFINITY;
         if (row < n_rows) {
           // row / w by a multiplication; the estimate from floor(2^32 / w) is low by at most 1
           int32_t head = (int32_t)__umulhi((uint32_t)row, it.w_inv);
           head += (head + 1) * it.w <= row;
-          lv[c] = __ldg(lse + (int64_t)(it.g * G + head) * n_tokens + it.base + it.len - it.w + (row - head * it.w)) * kLog2e;
+          lv[c] = __ldg(lse + (int64_t)(it.g * G + head) * n_tokens + it.base + it.len - it.w + (row - head * it.w)) * -kLog2e;
         }
       }
     };
@@ -514,7 +509,7 @@ __global__ void __launch_bounds__(kThreads, 2) score_tc_items_kernel(
     while (ok && cur.kind == 2) {
       const Item nxt = next_item(cur.number + stride);
       const uint32_t u1 = u0 + (uint32_t)cur.n_blocks;
-      float acc[4] = {0.f, 0.f, 0.f, 0.f};
+      float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
       for (int32_t t = (int32_t)((wg - u0) & 1u); t < cur.n_blocks; t += 2) {
         const uint32_t u = u0 + (uint32_t)t, lb = n_own & 1u;
         if (!ready) {
@@ -539,23 +534,7 @@ __global__ void __launch_bounds__(kThreads, 2) score_tc_items_kernel(
         for (int c = 0; c < 4; ++c) {
           tc_wait_ld();
           if (c + 1 < 4) tmem_ld32(t_lane + wg * kRows + 32 * (c + 1), rr[(c + 1) & 1]);
-#pragma unroll
-          for (int x = 0; x < 32; x += 4) {
-            const float4 l = l4[8 * c + (x >> 2)];
-            acc[0] += ex2(fmaf(__uint_as_float(rr[c & 1][x]), scale_log2, -l.x));
-            acc[1] += ex2(fmaf(__uint_as_float(rr[c & 1][x + 1]), scale_log2, -l.y));
-            if ((x >> 2) < kScorePoly) {
-              // this pair's exponentials on the FMA pipe: the kernel is paced by the MUFU unit (one ex2 per logit)
-              const float2 a = __ffma2_rn(make_float2(__uint_as_float(rr[c & 1][x + 2]), __uint_as_float(rr[c & 1][x + 3])),
-                                          make_float2(scale_log2, scale_log2), make_float2(-l.z, -l.w));
-              const float2 pp = exp2_poly2(a);
-              acc[2] += pp.x;
-              acc[3] += pp.y;
-            } else {
-              acc[2] += ex2(fmaf(__uint_as_float(rr[c & 1][x + 2]), scale_log2, -l.z));
-              acc[3] += ex2(fmaf(__uint_as_float(rr[c & 1][x + 3]), scale_log2, -l.w));
-            }
-          }
+          add_exps(rr[c & 1], l4 + 8 * c, scale_log2, acc);
         }
         tc_fence_before();
         __syncwarp();
@@ -569,7 +548,7 @@ __global__ void __launch_bounds__(kThreads, 2) score_tc_items_kernel(
       }
       if (!ok) break;
       // the item's column sums: the second group hands its share over, the first adds and writes
-      const float col_sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+      const float col_sum = (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
       if (wg == 1u) {
         if (nc > 0u) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.comb_empty), (nc - 1u) & 1u, abort_flag, wait_ns) ? 1 : 0) != 0;
         if (!ok) break;

@@ -197,7 +197,7 @@ __device__ __forceinline__ float2 exp2_poly2(float2 x) {
   x.x = fmaxf(x.x, -126.f);
   x.y = fmaxf(x.y, -126.f);
   const float2 r = __fadd2_rn(x, make_float2(kMagic, kMagic));
-  const float2 f = __fadd2_rn(x, __fadd2_rn(make_float2(kMagic, kMagic), make_float2(-r.x, -r.y)));  // x - n
+  const float2 f = __ffma2_rn(__fadd2_rn(r, make_float2(-kMagic, -kMagic)), make_float2(-1.f, -1.f), x);  // x - n
   float2 p = __ffma2_rn(make_float2(0.05517115443944931f, 0.05517115443944931f), f,
                         make_float2(0.2426101416349411f, 0.2426101416349411f));
   p = __ffma2_rn(p, f, make_float2(0.6932609677314758f, 0.6932609677314758f));
