@@ -133,9 +133,14 @@ def _check(status: int, where: str) -> None:
         raise PureKVError(status, where)
 
 
+# (None in a build of torch without CUDA, where nothing asks for a stream)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream() -> int:
     # the current stream of the current device as an integer, without building a Stream object on every call
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return _raw_stream(_current_device())
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -148,6 +153,12 @@ def _dtype_code(t: torch.Tensor) -> int:
     if t.dtype == torch.float32:
         return FP32
     raise TypeError(f"unsupported dtype {t.dtype}")
+
+
+def _layers_contiguous(t: torch.Tensor) -> bool:
+    # t[0].is_contiguous() without making the view where the strides say so plainly
+    _, _, h, d = t.shape
+    return t.stride()[1:] == (h * d, d, 1) or t[0].is_contiguous()
 
 
 def _i32(a) -> np.ndarray:
@@ -235,8 +246,8 @@ def purekv_plan_build_host(batch: Batch, params: StParams, dtype: int, head_dim:
     are written there in one pass and the used prefix of `out` is returned, ready for an asynchronous copy."""
     info = PlanInfo()
     if out is not None:
-        _check(_lib.purekv_plan_build_host(C.byref(batch.c), C.byref(params), dtype, head_dim, n_q_heads, n_kv_heads,
-                                           n_ctas, out.data_ptr(), out.numel(), C.byref(info)), "purekv_plan_build_host")
+        _check(_marshal.purekv_plan_build_host(batch.c, params, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, out.data_ptr(),
+                                               out.numel(), info), "purekv_plan_build_host")
         return out[:info.bytes_used], info
     n = purekv_plan_bytes(batch, params, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas)
     buf = np.zeros(max(n, 1), dtype=np.uint8)
@@ -359,7 +370,7 @@ def purekv_select_topk(c: torch.Tensor, v: torch.Tensor, batch: Batch, budget: B
                        idx_out: Optional[torch.Tensor] = None, s_out: Optional[torch.Tensor] = None,
                        ws: Optional[torch.Tensor] = None) -> torch.Tensor:
     """c [H_kv,T] fp32, v [L,T,H_kv,d]; returns idx [L,H_kv,K_tot] int32 (request-relative positions)."""
-    assert v.dim() == 4 and v.stride(3) == 1 and v[0].is_contiguous() and c.is_contiguous()
+    assert v.dim() == 4 and v.stride(3) == 1 and _layers_contiguous(v) and c.is_contiguous()
     n_layers, t, hkv, d = v.shape
     if idx_out is None:
         idx_out = torch.empty((n_layers, hkv, budget.total_kept), dtype=torch.int32, device=v.device)
@@ -399,7 +410,7 @@ def purekv_select_compact(c: torch.Tensor, k: torch.Tensor, v: torch.Tensor, bat
 def purekv_compact_kv(k: torch.Tensor, v: torch.Tensor, idx: torch.Tensor, batch: Batch, budget: Budget,
                       k_out: Optional[torch.Tensor] = None, v_out: Optional[torch.Tensor] = None):
     """k, v [L,T,H_kv,d]; idx [L,H_kv,K_tot]; returns (k_c, v_c) [L,K_tot,H_kv,d]."""
-    assert k.dim() == 4 and k[0].is_contiguous() and v[0].is_contiguous() and k.stride(0) == v.stride(0)
+    assert k.dim() == 4 and _layers_contiguous(k) and _layers_contiguous(v) and k.stride(0) == v.stride(0)
     n_layers, t, hkv, d = k.shape
     if k_out is None:
         k_out = torch.empty((n_layers, budget.total_kept, hkv, d), dtype=k.dtype, device=k.device)
@@ -421,19 +432,21 @@ def purekv_decode_attention(q: torch.Tensor, k_cache: torch.Tensor, v_cache: tor
     """q [B,H,d]; k_cache, v_cache [K_tot,H_kv,d] (one layer of the compact cache); returns o [B,H,d]."""
     assert q.is_contiguous() and k_cache.is_contiguous() and v_cache.is_contiguous()
     b, h, d = q.shape
-    hkv = k_cache.shape[1]
     if out is None:
         out = torch.empty_like(q)
-    call = lambda w: _marshal.purekv_decode_attention(
-        q.data_ptr(), k_cache.data_ptr(), v_cache.data_ptr(), out.data_ptr(), _ptr(lse), budget.cu_kept.data_ptr(), b,
-        budget.h_cu_kept, h, hkv, d, _dtype_code(q), softmax_scale, _ptr(w), 0 if w is None else w.numel() * w.element_size(),
-        _stream())
-    status = call(ws)
-    if status == ERR_WORKSPACE:  # (fp32 rows) none given, or too small
-        kept = np.diff(budget.h_cu_kept)
-        need = purekv_decode_ws_bytes(b, int(kept.max()), h, hkv, d)
-        status = call(torch.empty(need, dtype=torch.uint8, device=q.device))
-    _check(status, "purekv_decode_attention")
+    # (written out rather than through helpers: one conversation's step is a few microseconds of kernel per layer)
+    status = _marshal.purekv_decode_attention(
+        q.data_ptr(), k_cache.data_ptr(), v_cache.data_ptr(), out.data_ptr(), None if lse is None else lse.data_ptr(),
+        budget.cu_kept.data_ptr(), b, budget.h_cu_kept, h, k_cache.size(1), d,
+        BF16 if q.dtype is torch.bfloat16 else _dtype_code(q), softmax_scale, None if ws is None else ws.data_ptr(),
+        0 if ws is None else ws.nbytes, _raw_stream(_current_device()))
+    if status != OK:
+        if status == ERR_WORKSPACE:  # (fp32 rows) none given, or too small
+            kept = np.diff(budget.h_cu_kept)
+            need = purekv_decode_ws_bytes(b, int(kept.max()), h, k_cache.size(1), d)
+            return purekv_decode_attention(q, k_cache, v_cache, budget, out, lse, softmax_scale,
+                                           torch.empty(need, dtype=torch.uint8, device=q.device))
+        raise PureKVError(status, "purekv_decode_attention")
     return out
 
 

@@ -220,11 +220,24 @@ PyObject* decode(PyObject*, PyObject* const* v, Py_ssize_t n) {
   });
 }
 
+PyObject* plan_build_host(PyObject*, PyObject* const* v, Py_ssize_t n) {
+  Args a("plan_build_host", v, n, 10);
+  const purekv_batch* b = a.batch();
+  const purekv_st_params* p = (const purekv_st_params*)a.host(sizeof(purekv_st_params));
+  const int32_t dt = a.i32(), d = a.i32(), h = a.i32(), hkv = a.i32(), n_ctas = a.i32();
+  void* out = a.ptr();
+  const size_t bytes = (size_t)a.integer();
+  purekv_plan_info* info = (purekv_plan_info*)a.host(sizeof(purekv_plan_info));  // (a ctypes structure: written in place)
+  if (!a.ok) return nullptr;
+  return call([&] { return purekv_plan_build_host(b, p, (purekv_dtype)dt, d, h, hkv, n_ctas, out, bytes, info); });
+}
+
 #define PK_METHOD(name, f) {name, (PyCFunction)(void (*)(void))f, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {PK_METHOD("purekv_st_sparse_prefill", prefill), PK_METHOD("purekv_lowlayer_score", score),
                          PK_METHOD("purekv_lowlayer_score_lse", score_lse), PK_METHOD("purekv_lowlayer_score_ex", score_ex),
                          PK_METHOD("purekv_select_topk", select_topk), PK_METHOD("purekv_compact_kv", compact_kv),
-                         PK_METHOD("purekv_decode_attention", decode), {nullptr, nullptr, 0, nullptr}};
+                         PK_METHOD("purekv_decode_attention", decode),
+                         PK_METHOD("purekv_plan_build_host", plan_build_host), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace

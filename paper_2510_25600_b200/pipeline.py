@@ -42,13 +42,16 @@ class PureKVPipeline:
         params_dense.flags |= P.FLAG_DENSE_CAUSAL
         self.params_dense, self.params_st = params_dense, P.st_params(mask)
         hh = (n_q_heads, n_kv_heads)
-        self.plan_buf_dense = torch.empty(max(1, P.purekv_plan_bytes(self.batch, params_dense, self.code, head_dim, *hh)),
-                                          dtype=torch.uint8, device=dev)
-        self.plan_buf_st = torch.empty(max(1, P.purekv_plan_bytes(self.batch, self.params_st, self.code, head_dim, *hh)),
-                                       dtype=torch.uint8, device=dev)
+        # both plans in one buffer, and in one copy (a plan starts on a 256-byte boundary)
+        n_dense, n_st = (max(1, P.purekv_plan_bytes(self.batch, p, self.code, head_dim, *hh)) for p in (params_dense, self.params_st))
+        at_st = (n_dense + 255) // 256 * 256
+        self._plans = torch.empty(at_st + n_st, dtype=torch.uint8, device=dev)
+        self.plan_buf_dense, self.plan_buf_st = self._plans[:n_dense], self._plans[at_st:]
         self.prefill_ws = None
-        self._h_plans = [(torch.empty(self.plan_buf_dense.numel(), dtype=torch.uint8, pin_memory=True),
-                          torch.empty(self.plan_buf_st.numel(), dtype=torch.uint8, pin_memory=True)) for _ in range(3)]
+        self._h_plans = []
+        for _ in range(3):
+            both = torch.empty(at_st + n_st, dtype=torch.uint8, pin_memory=True)
+            self._h_plans.append((both, both[:n_dense], both[at_st:]))
         self._h_plan_events = [None] * len(self._h_plans)
         self._plan_slot = 0
         self.o = torch.empty((n_layers, t, n_q_heads, head_dim), dtype=dtype, device=dev)
@@ -75,18 +78,17 @@ class PureKVPipeline:
         alive until its copy has run."""
         slot = self._plan_slot
         self._plan_slot = (slot + 1) % len(self._h_plans)
-        if self._h_plan_events[slot] is not None:
-            self._h_plan_events[slot].synchronize()
-        plans = []
-        for params, h_buf, d_buf in ((self.params_dense, self._h_plans[slot][0], self.plan_buf_dense),
-                                     (self.params_st, self._h_plans[slot][1], self.plan_buf_st)):
-            h_used, info = P.purekv_plan_build_host(self.batch, params, self.code, self.d, self.h, self.hkv, out=h_buf)
-            d_buf[:info.bytes_used].copy_(h_used, non_blocking=True)
-            plans.append(P.Plan(d_buf, info))
-        ev = torch.cuda.Event()
+        ev = self._h_plan_events[slot]
+        if ev is not None:
+            ev.synchronize()
+        else:
+            ev = self._h_plan_events[slot] = torch.cuda.Event()
+        both, h_dense, h_st = self._h_plans[slot]
+        _, info_dense = P.purekv_plan_build_host(self.batch, self.params_dense, self.code, self.d, self.h, self.hkv, out=h_dense)
+        _, info_st = P.purekv_plan_build_host(self.batch, self.params_st, self.code, self.d, self.h, self.hkv, out=h_st)
+        self._plans.copy_(both, non_blocking=True)
         ev.record()
-        self._h_plan_events[slot] = ev
-        self.plan_dense, self.plan_st = plans
+        self.plan_dense, self.plan_st = P.Plan(self.plan_buf_dense, info_dense), P.Plan(self.plan_buf_st, info_st)
         need = max(16, self.plan_dense.info.ws_bytes, self.plan_st.info.ws_bytes)
         if self.prefill_ws is None or self.prefill_ws.numel() < need:
             self.prefill_ws = torch.empty(need, dtype=torch.uint8, device="cuda")
@@ -123,9 +125,10 @@ class PureKVPipeline:
             else:
                 P.purekv_lowlayer_score(q[layer], k[layer], self.batch, self.window, c_out=self.c[n], ws=self.score_ws)
         lo, hi = self.compacted[0], self.compacted[-1] + 1
-        P.purekv_select_topk(self.c[len(self.scored) - 1], v[lo:hi], self.batch, self.budget, idx_out=self.idx,
+        k_cmp, v_cmp = k[lo:hi], v[lo:hi]
+        P.purekv_select_topk(self.c[len(self.scored) - 1], v_cmp, self.batch, self.budget, idx_out=self.idx,
                              ws=self.select_ws)
-        P.purekv_compact_kv(k[lo:hi], v[lo:hi], self.idx, self.batch, self.budget, k_out=self.k_c, v_out=self.v_c)
+        P.purekv_compact_kv(k_cmp, v_cmp, self.idx, self.batch, self.budget, k_out=self.k_c, v_out=self.v_c)
 
     def alloc_host_io(self):
         """Pinned host buffers for run_host: (q, k, v) inputs and (k_c, v_c, o_last) outputs."""
