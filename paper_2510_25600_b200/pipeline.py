@@ -42,18 +42,15 @@ class PureKVPipeline:
         params_dense.flags |= P.FLAG_DENSE_CAUSAL
         self.params_dense, self.params_st = params_dense, P.st_params(mask)
         hh = (n_q_heads, n_kv_heads)
-        # both plans in one buffer, and in one copy (a plan starts on a 256-byte boundary)
-        n_dense, n_st = (max(1, P.purekv_plan_bytes(self.batch, p, self.code, head_dim, *hh)) for p in (params_dense, self.params_st))
-        at_st = (n_dense + 255) // 256 * 256
-        self._plans = torch.empty(at_st + n_st, dtype=torch.uint8, device=dev)
-        self.plan_buf_dense, self.plan_buf_st = self._plans[:n_dense], self._plans[at_st:]
+        self.plan_buf_dense = torch.empty(max(1, P.purekv_plan_bytes(self.batch, params_dense, self.code, head_dim, *hh)),
+                                          dtype=torch.uint8, device=dev)
+        self.plan_buf_st = torch.empty(max(1, P.purekv_plan_bytes(self.batch, self.params_st, self.code, head_dim, *hh)),
+                                       dtype=torch.uint8, device=dev)
         self.prefill_ws = None
-        self._h_plans = []
-        for _ in range(3):
-            both = torch.empty(at_st + n_st, dtype=torch.uint8, pin_memory=True)
-            self._h_plans.append((both, both[:n_dense], both[at_st:]))
-        self._h_plan_events = [None] * len(self._h_plans)
-        self._plan_slot = 0
+        # per mask a ring of pinned buffers, each with the event behind its last copy; the last one used comes first
+        self._h_dense, self._h_st = ([[torch.empty(b.numel(), dtype=torch.uint8, pin_memory=True), None] for _ in range(3)]
+                                     for b in (self.plan_buf_dense, self.plan_buf_st))
+        self._copies = torch.cuda.Stream()  # the sparse plan's copy runs beside the dense layers
         self.o = torch.empty((n_layers, t, n_q_heads, head_dim), dtype=dtype, device=dev)
         self.c = torch.empty((len(self.scored), n_kv_heads, t), dtype=torch.float32, device=dev)
         # one-pass tensor-core scores where the entry point supports the shape (bf16, head_dim 128, window and any
@@ -72,26 +69,32 @@ class PureKVPipeline:
         # prefill per layer, score (1 kernel one-pass, 3 otherwise), select (2), compact
         self.launches_per_step = n_layers + (1 if self.one_pass_scores else 3) * len(self.scored) + 2 + 1
 
-    def build_plans(self) -> None:
-        """Plans both masks on the host into pinned buffers and enqueues their copies on the current stream without
-        waiting, so planning overlaps the GPU work already in flight.  A small ring of pinned buffers keeps a plan
-        alive until its copy has run."""
-        slot = self._plan_slot
-        self._plan_slot = (slot + 1) % len(self._h_plans)
-        ev = self._h_plan_events[slot]
+    def _plan(self, params, ring: list, d_buf: torch.Tensor) -> P.Plan:
+        """Plans one mask on the host into a pinned buffer and enqueues its copy on the current stream without waiting, so
+        planning overlaps the GPU work already in flight.  A small ring of pinned buffers keeps a plan alive until its copy
+        has run."""
+        ring.append(ring.pop(0))
+        h_buf, ev = ring[0]
         if ev is not None:
             ev.synchronize()
         else:
-            ev = self._h_plan_events[slot] = torch.cuda.Event()
-        both, h_dense, h_st = self._h_plans[slot]
-        _, info_dense = P.purekv_plan_build_host(self.batch, self.params_dense, self.code, self.d, self.h, self.hkv, out=h_dense)
-        _, info_st = P.purekv_plan_build_host(self.batch, self.params_st, self.code, self.d, self.h, self.hkv, out=h_st)
-        self._plans.copy_(both, non_blocking=True)
+            ev = ring[0][1] = torch.cuda.Event()
+        _, info = P.purekv_plan_build_host(self.batch, params, self.code, self.d, self.h, self.hkv, out=h_buf)
+        d_buf.copy_(h_buf, non_blocking=True)
         ev.record()
-        self.plan_dense, self.plan_st = P.Plan(self.plan_buf_dense, info_dense), P.Plan(self.plan_buf_st, info_st)
-        need = max(16, self.plan_dense.info.ws_bytes, self.plan_st.info.ws_bytes)
+        return P.Plan(d_buf, info)
+
+    def _size_prefill_ws(self, plan: P.Plan) -> None:
+        need = max(16, plan.info.ws_bytes)
         if self.prefill_ws is None or self.prefill_ws.numel() < need:
             self.prefill_ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+
+    def build_plans(self) -> None:
+        """Both masks' plans; `run_device` builds each just ahead of the first layer that needs it."""
+        self.plan_dense = self._plan(self.params_dense, self._h_dense, self.plan_buf_dense)
+        self.plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st)
+        self._size_prefill_ws(self.plan_dense)
+        self._size_prefill_ws(self.plan_st)
 
     def prefill_layer(self, layer: int, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor) -> None:
         plan = self.plan_dense if layer <= self.clie else self.plan_st
@@ -105,10 +108,24 @@ class PureKVPipeline:
         `events`, if given, is a list of (start, end) torch.cuda.Event pairs, one per prefill launch (an event
         between two launches keeps the second from starting under the first's tail); `marks`, if given, is three
         events recorded before the first prefill launch, after the last dense-causal one and after the last one."""
-        self.build_plans()
+        # The sparse mask's plan, the longer one, is made and copied while the GPU works on the dense layers.  (The copy
+        # waits for whatever the stream held before this call, which may still read the last plan; in the stream itself,
+        # between two layers, it cost 10 us.)
+        before = torch.cuda.Event() if self.n_layers > self.clie + 1 else None
+        if before is not None:
+            before.record()
+        self.plan_dense = self._plan(self.params_dense, self._h_dense, self.plan_buf_dense)
+        self._size_prefill_ws(self.plan_dense)
         if marks is not None:
             marks[0].record()
         for layer in range(self.n_layers):
+            if layer == self.clie + 1:
+                main = torch.cuda.current_stream()
+                self._copies.wait_event(before)
+                with torch.cuda.stream(self._copies):
+                    self.plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st)
+                main.wait_event(self._h_st[0][1])
+                self._size_prefill_ws(self.plan_st)
             if events is not None:
                 events[layer][0].record()
             self.prefill_layer(layer, q[layer], k[layer], v[layer])
