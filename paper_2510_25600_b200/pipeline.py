@@ -66,8 +66,8 @@ class PureKVPipeline:
         self.v_c = torch.empty_like(self.k_c)
         self.status = torch.zeros(1, dtype=torch.int32, device=dev)
         self.plan_dense = self.plan_st = None
-        # prefill per layer, score (1 kernel one-pass, 3 otherwise), select (2), compact
-        self.launches_per_step = n_layers + (1 if self.one_pass_scores else 3) * len(self.scored) + 2 + 1
+        # prefill per layer, score (1 kernel one-pass or in one cluster, up to 3 otherwise: counted as 1), select (2), compact
+        self.launches_per_step = n_layers + len(self.scored) + 2 + 1
 
     def _plan(self, params, ring: list, d_buf: torch.Tensor) -> P.Plan:
         """Plans one mask on the host into a pinned buffer and enqueues its copy on the current stream without waiting, so
