@@ -130,7 +130,7 @@ struct __align__(16) Unit {
   int32_t pair;                  // KV head g = pair / ppg, first query head g*G + 2*(pair % ppg), ppg = (G+1)/2
   int32_t chunk, n_chunks;
   int32_t part_base;             // workspace slot of (chunk 0, head 0) = part_base; slot(chunk, hq) = (part_base + chunk) * H + hq
-  int32_t counter_base;          // merge counter of head hq = counters[counter_base + hq]
+  int32_t counter_base;          // merge counter of head hq = counters[counter_base + hq]: a byte per warp of 32 rows
   int32_t q_start1, q_rows1;     // a twin unit's second query tile (q_rows1 == 0: an ordinary unit)
   int32_t part_base1, counter_base1;  // ... and that tile's workspace slots and merge counters when the lists are split
   int32_t pad[2];

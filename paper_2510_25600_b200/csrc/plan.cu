@@ -172,7 +172,8 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
     *count = n;
     return cost;
   };
-  auto chunks_of = [&](const QTile& q, int32_t l_max) { return std::max(1, (q.entry_count + l_max - 1) / l_max); };
+  // (the kernel counts a list's chunks in a byte per warp)
+  auto chunks_of = [&](const QTile& q, int32_t l_max) { return std::min(255, std::max(1, (q.entry_count + l_max - 1) / l_max)); };
   // chunk c of nch of a tile's list, as a range of entries[]
   auto chunk_range = [&](const QTile& q, int32_t c, int32_t nch, int32_t* first, int32_t* last) {
     *first = q.entry_begin + (int32_t)((int64_t)q.entry_count * c / nch);

@@ -61,7 +61,6 @@ struct __align__(8) Barriers {
   uint64_t p_full[2][SB];  // softmax -> MMA: all of P written
   uint64_t o_done[2];      // one completion per P.V product of the slot
   uint64_t o_final[2];     // one completion per unit, after the slot's last P.V product
-  uint64_t rows_sync[2];   // the 128 row threads of a slot meet here around the merge-counter update
   uint64_t u_full[kUnitRing];   // the producer published a unit (or the end mark) in unit_s[]
   uint64_t u_empty[kUnitRing];  // the MMA thread and the eight softmax warps have copied it
   uint64_t drain;
@@ -88,7 +87,6 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s;
   __shared__ int abort_code_s;  // what the status word becomes if the CTA gives up: an expired wait unless set otherwise
-  __shared__ int merge_s[2];
 
   const uint32_t smem0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t sQ = smem0;                 // [2 slots][2 panels][128 rows x 128 B]
@@ -120,7 +118,6 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       mbar_init(smem_u32(&bars.p_part[sl]), 4);
       mbar_init(smem_u32(&bars.o_done[sl]), 1);
       mbar_init(smem_u32(&bars.o_final[sl]), 1);
-      mbar_init(smem_u32(&bars.rows_sync[sl]), 128);
     }
     for (int s = 0; s < kUnitRing; ++s) {
       mbar_init(smem_u32(&bars.u_full[s]), 1);
@@ -206,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
                           (int64_t)uu.ent_begin + (int64_t)uu.ent_count * (twin ? 2 : 1) <= n_entries &&
                           uu.q_rows >= 1 && uu.q_rows <= kBQ && uu.req_start >= 0 && uu.q_start >= uu.req_start &&
                           (int64_t)uu.q_start + uu.q_rows <= total_tokens && uu.pair >= 0 && uu.pair < n_pairs &&
-                          uu.n_chunks >= 1 && uu.chunk >= 0 && uu.chunk < uu.n_chunks &&
+                          uu.n_chunks >= 1 && uu.n_chunks <= 255 && uu.chunk >= 0 && uu.chunk < uu.n_chunks &&
                           (!twin || (uu.q_rows1 >= 1 && uu.q_rows1 <= kBQ && uu.q_start1 >= uu.req_start &&
                                      (int64_t)uu.q_start1 + uu.q_rows1 <= total_tokens && (G & 1) != 0 &&
                                      uu.pair % ppg == ppg - 1 &&
@@ -525,15 +522,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
     uint32_t it_base = 0;     // key tiles of earlier units (both slots)
     uint32_t t = 0;           // tiles this slot has processed, over all units
     uint32_t slot_units = 0;  // units this slot took part in
-    uint32_t row_syncs = 0;   // completed phases of rows_sync[sl]
     bool ok = true;
-    // bounded meeting of the slot's 128 row threads (a plain barrier could not be left on a failure)
-    auto sync_rows = [&]() -> bool {
-      mbar_arrive(smem_u32(&bars.rows_sync[sl]));
-      const bool r = wait_w(smem_u32(&bars.rows_sync[sl]), row_syncs & 1u);
-      ++row_syncs;
-      return r;
-    };
     for (uint32_t uo = 0; ok; ++uo) {
       const uint32_t us = uo % kUnitRing;
       if (!wait_w(smem_u32(&bars.u_full[us]), (uo / kUnitRing) & 1u)) { ok = false; break; }
@@ -798,63 +787,94 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
         }
         part[128 * 128 + row] = m_ref;
         part[128 * 128 + 128 + row] = l_sum;
-        // The 128 rows meet (ordering their stores before row 0 inside the CTA), then row 0 alone publishes with one
-        // release / acquire update of the merge counter at GPU scope: release is cumulative over what the meeting
-        // ordered before it, so no thread needs a fence of its own.
-        if (!sync_rows()) { ok = false; break; }
-        if (row == 0) {
+        // A row's partial results are read by the thread of the same row in another CTA, so each warp publishes and counts for
+        // itself: a byte of the head's counter per warp (one release / acquire update at GPU scope by lane 0; release is
+        // cumulative over what __syncwarp ordered before it, so no thread needs a fence of its own).  Whichever warp finds all
+        // chunks of its 32 rows there merges them.
+        __syncwarp();
+        int32_t last = 0;
+        if (lane == 0) {
           int32_t* cnt = counters + (second_tile ? u.counter_base1 : u.counter_base) + hq;
-          const int last = atom_add_acq_rel(cnt, 1) == u.n_chunks - 1;
-          if (last) *cnt = 0;  // every chunk has arrived: ready for the next launch (nobody touches it before then)
-          merge_s[sl] = last;
+          last = ((atom_add_acq_rel(cnt, 1 << (8 * quad)) >> (8 * quad)) & 255) == u.n_chunks - 1;
+          if (last) atomicSub(reinterpret_cast<uint32_t*>(cnt), (uint32_t)u.n_chunks << (8 * quad));  // ready for the next launch
         }
-        if (!sync_rows()) { ok = false; break; }
-        if (merge_s[sl]) {
+        last = __shfl_sync(0xffffffffu, last, 0);
+        __syncwarp();
+        if (last) {
           const float* p0 = ws + ((int64_t)part_base * n_q_heads + hq) * kPartFloats;
           const int64_t cstride = (int64_t)n_q_heads * kPartFloats;
-          // Two chunks at a time, their loads in flight together: the merge is a chain of L2 round trips (with one chunk at a
-          // time, weights first, it took 20 000 clk for three chunks, as long as six key tiles).
+          const int32_t own = u.chunk, n_ch = u.n_chunks;
+          // The merge is a chain of L2 round trips: row statistics four chunks at a time, then 32 columns of two chunks at a
+          // time, the CTA's own chunk from TMEM; always summed in chunk order.  (2432 tokens, lists in three chunks, one layer:
+          // two chunks at a time and the slot's warps together 45.6 us, this way 44.0.)
           float m_all = -INFINITY, l_all = 0.f;
-          for (int32_t c = 0; c < u.n_chunks; c += 2) {
-            const float* pa = p0 + c * cstride + 128 * 128 + row;
-            const float* pb = p0 + (int64_t)min(c + 1, u.n_chunks - 1) * cstride + 128 * 128 + row;
-            const float ma = __ldcg(pa), la = __ldcg(pa + 128), mb = __ldcg(pb), lb_ = __ldcg(pb + 128);
-            const float lb = c + 1 < u.n_chunks ? lb_ : 0.f;
-            const float m_new = fmaxf(m_all, fmaxf(la > 0.f ? ma : -INFINITY, lb > 0.f ? mb : -INFINITY));
-            if (m_new > m_all) {
-              l_all *= ex2(m_all - m_new);  // (l_all is 0 while m_all is -inf)
-              m_all = m_new;
+          for (int32_t c0 = 0; c0 < n_ch; c0 += 4) {
+            float mc[4], lc[4];
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+              const float* pc = p0 + (int64_t)min(c0 + y, n_ch - 1) * cstride + 128 * 128 + row;
+              mc[y] = __ldcg(pc);
+              lc[y] = __ldcg(pc + 128);
             }
-            if (la > 0.f) l_all += la * ex2(ma - m_all);
-            if (lb > 0.f) l_all += lb * ex2(mb - m_all);
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+              if (c0 + y < n_ch && lc[y] > 0.f) {
+                if (mc[y] > m_all) {
+                  l_all *= ex2(m_all - mc[y]);  // (l_all is 0 while m_all is -inf)
+                  m_all = mc[y];
+                }
+                l_all += lc[y] * ex2(mc[y] - m_all);
+              }
+            }
           }
-          const float inv = 1.f / l_all;
+          const float inv = 1.f / l_all, w_own = l_sum > 0.f ? ex2(m_ref - m_all) : 0.f;
           __nv_bfloat16* dst = o + ((int64_t)(q_first + row) * n_q_heads + hq) * kD;
 #pragma unroll 1
           for (int cc = 0; cc < kD / 32; ++cc) {
+            uint32_t tt[32];
+            tmem_ld32(t_lane + kColO + sl * 128 + 32 * cc, tt);
             float acc[32];
 #pragma unroll
             for (int x = 0; x < 32; ++x) acc[x] = 0.f;
+            bool own_in = false;
+            auto add = [&](float w, const float4 (&v)[8]) {
+#pragma unroll
+              for (int x = 0; x < 8; ++x) {
+                acc[4 * x] = fmaf(w, v[x].x, acc[4 * x]);
+                acc[4 * x + 1] = fmaf(w, v[x].y, acc[4 * x + 1]);
+                acc[4 * x + 2] = fmaf(w, v[x].z, acc[4 * x + 2]);
+                acc[4 * x + 3] = fmaf(w, v[x].w, acc[4 * x + 3]);
+              }
+            };
+            auto add_own = [&]() {
+#pragma unroll
+              for (int x = 0; x < 32; ++x) acc[x] = fmaf(w_own, __uint_as_float(tt[x]), acc[x]);
+              own_in = true;
+            };
 #pragma unroll 1
-            for (int32_t c = 0; c < u.n_chunks; c += 2) {
-              const float* pa = p0 + c * cstride;
-              const float* pb = p0 + (int64_t)min(c + 1, u.n_chunks - 1) * cstride;
+            for (int32_t k = 0; k < n_ch - 1; k += 2) {  // the others, in order
+              const int32_t ca = k + (k >= own), cb = min(k + 1 + (k + 1 >= own), n_ch - 1);
+              const bool two = k + 1 < n_ch - 1;
+              const float* pa = p0 + ca * cstride;
+              const float* pb = p0 + cb * cstride;
               float4 va[8], vb[8];
               const float ma = __ldcg(pa + 128 * 128 + row), la = __ldcg(pa + 128 * 128 + 128 + row);
               const float mb = __ldcg(pb + 128 * 128 + row), lb = __ldcg(pb + 128 * 128 + 128 + row);
 #pragma unroll
               for (int x = 0; x < 8; ++x) va[x] = __ldcg(reinterpret_cast<const float4*>(pa + ((cc * 8 + x) * 128 + row) * 4));
 #pragma unroll
-              for (int x = 0; x < 8; ++x) vb[x] = __ldcg(reinterpret_cast<const float4*>(pb + ((cc * 8 + x) * 128 + row) * 4));
-              const float wa = la > 0.f ? ex2(ma - m_all) : 0.f, wb = c + 1 < u.n_chunks && lb > 0.f ? ex2(mb - m_all) : 0.f;
-#pragma unroll
-              for (int x = 0; x < 8; ++x) {  // in chunk order
-                acc[4 * x] = fmaf(wb, vb[x].x, fmaf(wa, va[x].x, acc[4 * x]));
-                acc[4 * x + 1] = fmaf(wb, vb[x].y, fmaf(wa, va[x].y, acc[4 * x + 1]));
-                acc[4 * x + 2] = fmaf(wb, vb[x].z, fmaf(wa, va[x].z, acc[4 * x + 2]));
-                acc[4 * x + 3] = fmaf(wb, vb[x].w, fmaf(wa, va[x].w, acc[4 * x + 3]));
+              for (int x = 0; x < 8; ++x)
+                vb[x] = two ? __ldcg(reinterpret_cast<const float4*>(pb + ((cc * 8 + x) * 128 + row) * 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+              const float wa = la > 0.f ? ex2(ma - m_all) : 0.f, wb = two && lb > 0.f ? ex2(mb - m_all) : 0.f;
+              if (k == 0) tc_wait_ld();
+              if (!own_in && own < ca) add_own();
+              add(wa, va);
+              if (two) {
+                if (!own_in && own < cb) add_own();
+                add(wb, vb);
               }
             }
+            if (!own_in) add_own();
             if (row_valid) {
 #pragma unroll
               for (int x = 0; x < 32; x += 16) {
