@@ -257,7 +257,7 @@ purekv_status purekv_select_topk(const float *c, const void *v, int64_t v_layer_
  * purekv_select_topk followed by purekv_compact_kv of the same layers, in the selection's own kernels: the CTA
  * that has chosen a (request, KV head, layer) segment's positions copies those K and V rows (k and v share
  * layer_stride) into k_out / v_out [n_layers][K_tot, H_kv, d] (out_layer_stride) -- one launch fewer, and the
- * indices do not travel through memory between two kernels.  idx_out (and s_out, if given) are written as by
+ * indices do not travel through memory between two kernels (few segments of many rows take both kernels all the same).  idx_out (and s_out, if given) are written as by
  * purekv_select_topk; results are bit-identical to the two separate calls. */
 purekv_status purekv_select_compact(const float *c, const void *k, const void *v, int64_t layer_stride,
                                     int32_t n_layers, const purekv_batch *batch, int32_t window,

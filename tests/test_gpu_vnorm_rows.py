@@ -15,6 +15,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("dtype,d,hkv,layers,lens", [
     ("bf16", 128, 1, 1, [1]), ("bf16", 128, 1, 5, [15]), ("bf16", 128, 3, 7, [16, 1]), ("bf16", 128, 2, 40, [17, 3, 64]),
     ("bf16", 128, 4, 3, [2500, 0, 733]), ("fp32", 64, 2, 9, [129, 31]), ("fp32", 64, 1, 160, [50]),
+    ("bf16", 128, 2, 3, [1017, 1019]), ("bf16", 128, 1, 2, [1030]),  # 1017 kept rows of two requests (gathered), 515 of one (compacted)
     ("bf16", 64, 2, 3, [77, 5]), ("fp32", 20, 3, 2, [301]), ("bf16", 256, 1, 2, [40]),
 ])
 def test_scores_selection_and_rows(dtype, d, hkv, layers, lens):
