@@ -449,7 +449,7 @@ def compression_detail(pipe, wl, d_in, peaks, timer):
                 P.purekv_decode_attention(q_dec, pipe.k_c[layer], pipe.v_c[layer], pipe.budget, out=o_dec, ws=dec_ws)
         t_decode = timer(decode_all_layers)
         bytes_decode = nc * (2 * kt * row + 2 * b.n_req * wl.n_q_heads * wl.head_dim * esz)
-        detail["decode_step_after"] = dict(hbm_rec(t_decode, bytes_decode, peaks), launches=nc * (2 if dec_need else 1),
+        detail["decode_step_after"] = dict(hbm_rec(t_decode, bytes_decode, peaks), launches=nc * (2 if dec_need and wl.dtype == "fp32" else 1),
                                            us_per_layer=1e3 * t_decode / nc,
                                            note="one new query per request over the compact cache of every compacted layer, "
                                                 "one call per layer; outside the timed step")
