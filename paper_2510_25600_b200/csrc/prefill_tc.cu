@@ -19,7 +19,7 @@
 //               reference that moves only when exp2 would overflow (then O is rescaled), bf16 P written
 //               over S; at the end of a unit either the normalised output
 //               (whole list in one unit) or an unnormalised fp32 partial result plus (max, sum) per row
-//               into the workspace.  The chunk of a split list that finishes last (a counter in the plan)
+//               into the workspace.  The warp that finishes its rows of a split list last (a counter in the plan)
 //               combines the partial results in chunk order, so the result does not depend on timing.
 // Every wait on an mbarrier is bounded in time; on expiry the CTA raises a shared abort flag,
 // sets the device status word, drains, frees TMEM and exits.
