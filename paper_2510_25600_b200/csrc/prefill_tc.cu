@@ -596,11 +596,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
         // holds the MMA thread up for the other slot).
         uint32_t pk[BK / 2];
         float l_tile = 0.f;
-        auto hand_over = [&](uint32_t bar) {
+        auto p_stored = [&]() {  // the warp's P is in TMEM; lane 0 may say so, one arrival per warp: 4 per slot
           tc_wait_st();
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(bar);  // one arrival per warp: 4 per slot
         };
         const uint32_t part_bar = smem_u32(&bars.p_part[sl]), full_bar = smem_u32(&bars.p_full[sl][b]);
         bool exact = false;
@@ -664,7 +663,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
             if (!exact) {
               tmem_st32(s_addr, reinterpret_cast<const uint32_t(&)[32]>(pk[0]));  // over columns of S that have been read
               tmem_st16(s_addr + 32, reinterpret_cast<const uint32_t(&)[16]>(pk[32]));
-              hand_over(part_bar);
+              p_stored();
+              if (lane == 0) mbar_arrive(part_bar);
               exps(r1, i32, i64, i48);
               l_tile = (ls2[0].x + ls2[0].y) + (ls2[1].x + ls2[1].y);
               tmem_st16(s_addr + 48, reinterpret_cast<const uint32_t(&)[16]>(pk[48]));
@@ -738,8 +738,14 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
           m_ref = m_new;
         }
         l_sum += l_tile;
-        hand_over(full_bar);
-        if ((exact || hm != 3u) && lane == 0) mbar_arrive(part_bar);  // (counted in every tile)
+        p_stored();
+        if (lane == 0) {
+          // Every tile counts on both barriers, and on p_part first: the MMA thread waits for p_full in every tile but for p_part
+          // only where both halves are present, so p_full has to imply p_part.  (The other way round a late arrival could leave
+          // p_part a phase behind, and the parity of the next tile's wait would match the phase before it.)
+          if (exact || hm != 3u) mbar_arrive(part_bar);
+          mbar_arrive(full_bar);
+        }
         ++t;
       }
       if (!ok) break;
