@@ -37,6 +37,11 @@ void set_error(const char* fmt, ...);
 purekv_status check_batch(const purekv_batch* b, bool need_device);
 uint64_t wait_limit_ns();  // the process-wide limit of device-side waits (purekv_set_wait_limit_ns)
 
+// purekv_compact_kv's launch, for callers that have checked its arguments (compact.cu).
+purekv_status launch_compact(const void* k, const void* v, int64_t layer_stride, int32_t n_layers, const int32_t* idx,
+                             const purekv_batch* batch, const int32_t* cu_kept, int32_t k_tot, int32_t n_kv_heads, int64_t row_bytes,
+                             int64_t elem_bytes, void* k_out, void* v_out, int64_t out_layer_stride, cudaStream_t stream);
+
 // The status word a call uses when the caller passes none: one word per device inside the library, read and
 // cleared by purekv_poll_status(NULL, ...).  Its device address is looked up once per device.
 purekv_status default_status_word(int32_t** out);

@@ -43,6 +43,31 @@ __global__ void __launch_bounds__(256) compact_kernel(
   }
 }
 
+// Gathers the rows; the arguments have been checked.
+purekv_status launch_compact(const void* k, const void* v, int64_t layer_stride, int32_t n_layers, const int32_t* idx,
+                             const purekv_batch* batch, const int32_t* cu_kept, int32_t k_tot, int32_t n_kv_heads, int64_t row_bytes,
+                             int64_t elem_bytes, void* k_out, void* v_out, int64_t out_layer_stride, cudaStream_t stream) {
+  if (n_layers == 0 || k_tot == 0) return PUREKV_OK;
+  const int32_t cpr = (int32_t)(row_bytes / 16);
+  const int64_t per_layer = (int64_t)k_tot * n_kv_heads * cpr;
+  const int64_t blocks = (per_layer * n_layers + 255) / 256;
+  // one wave: 148 SMs x 8 resident CTAs of 256 threads; fewer blocks when the job is small
+  dim3 grid((unsigned)std::min<int64_t>(blocks, 148 * 8));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(256);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  PK_CUDA(cudaLaunchKernelEx(&cfg, compact_kernel, (const uint4*)k, (const uint4*)v, layer_stride * elem_bytes / 16, idx,
+                             batch->cu_seqlens, cu_kept, batch->n_req, k_tot, n_kv_heads, cpr, (uint4*)k_out, (uint4*)v_out,
+                             out_layer_stride * elem_bytes / 16, per_layer, n_layers));
+  return PUREKV_OK;
+}
+
 }  // namespace purekv
 
 using namespace purekv;
@@ -79,23 +104,6 @@ extern "C" purekv_status purekv_compact_kv(const void* k, const void* v, int64_t
              PUREKV_ERR_INVALID_ARG, "layer_stride smaller than one layer");
   PK_REQUIRE(out_layer_stride >= (int64_t)k_tot * n_kv_heads * head_dim || n_layers <= 1,
              PUREKV_ERR_INVALID_ARG, "out_layer_stride smaller than one compacted layer");
-  if (n_layers == 0 || k_tot == 0) return PUREKV_OK;
-  const int32_t cpr = (int32_t)(row_bytes / 16);
-  const int64_t per_layer = (int64_t)k_tot * n_kv_heads * cpr;
-  const int64_t blocks = (per_layer * n_layers + 255) / 256;
-  // one wave: 148 SMs x 8 resident CTAs of 256 threads; fewer blocks when the job is small
-  dim3 grid((unsigned)std::min<int64_t>(blocks, 148 * 8));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(256);
-  cfg.stream = (cudaStream_t)stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  PK_CUDA(cudaLaunchKernelEx(&cfg, compact_kernel, (const uint4*)k, (const uint4*)v, layer_stride * esz / 16, idx,
-                             batch->cu_seqlens, cu_kept, batch->n_req, k_tot, n_kv_heads, cpr, (uint4*)k_out, (uint4*)v_out,
-                             out_layer_stride * esz / 16, per_layer, n_layers));
-  return PUREKV_OK;
+  return launch_compact(k, v, layer_stride, n_layers, idx, batch, cu_kept, k_tot, n_kv_heads, row_bytes, esz, k_out, v_out,
+                        out_layer_stride, (cudaStream_t)stream);
 }

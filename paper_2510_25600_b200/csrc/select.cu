@@ -568,15 +568,17 @@ extern "C" purekv_status purekv_select_compact(const float* c, const void* k, co
   PK_REQUIRE((layer_stride * esz) % 16 == 0 && (out_layer_stride * esz) % 16 == 0 &&
                  ((uintptr_t)k | (uintptr_t)v | (uintptr_t)k_out | (uintptr_t)v_out) % 16 == 0,
              PUREKV_ERR_INVALID_ARG, "K/V bases and layer strides must be 16-byte aligned");
+  const purekv_status st_batch = check_batch(batch, true);  // (the rule below reads through the batch)
+  if (st_batch != PUREKV_OK) return st_batch;
   // Few segments of many rows leave most of the GPU idle while one CTA copies each: the compaction's own kernel takes the rows
   // then (26 layers of 8320 tokens x 4 heads, 104 segments of 1728 rows: 95 us here, 82 with two kernels; 104 segments of 224
   // rows: 16.0 and 16.4; 1024 segments: 153 and 158).
-  if (batch && h_cu_kept && (int64_t)batch->n_req * n_kv_heads * n_layers < 148 && h_cu_kept[batch->n_req] >= 512 * (int64_t)batch->n_req) {
+  if (h_cu_kept && (int64_t)batch->n_req * n_kv_heads * n_layers < 148 && h_cu_kept[batch->n_req] >= 512 * (int64_t)batch->n_req) {
     const purekv_status st = select_impl(c, v, layer_stride, n_layers, batch, window, keep, h_keep, cu_kept, h_cu_kept, n_kv_heads,
                                          head_dim, dtype, idx_out, s_out, ws, ws_bytes, stream, Gather{});
-    if (st != PUREKV_OK) return st;
-    return purekv_compact_kv(k, v, layer_stride, n_layers, idx_out, batch, cu_kept, h_cu_kept, n_kv_heads, head_dim, dtype, k_out,
-                             v_out, out_layer_stride, stream);
+    if (st != PUREKV_OK || batch->total_tokens == 0 || batch->n_req == 0) return st;
+    return launch_compact(k, v, layer_stride, n_layers, idx_out, batch, cu_kept, h_cu_kept[batch->n_req], n_kv_heads, head_dim * esz,
+                          esz, k_out, v_out, out_layer_stride, (cudaStream_t)stream);
   }
   Gather ga;
   ga.k_src = (const uint4*)k;
