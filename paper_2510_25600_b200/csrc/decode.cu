@@ -12,6 +12,7 @@
 // writes O itself; several: it leaves (unnormalised O, max, sum) per head and a second small kernel merges them.
 #include <algorithm>
 
+#include "cluster.cuh"
 #include "common.cuh"
 
 namespace purekv {
@@ -572,7 +573,6 @@ static purekv_status launch_cluster_as(int32_t cl, cudaStream_t sm, const void* 
     }
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)cl, (unsigned)Hkv, (unsigned)n_req);
   cfg.blockDim = dim3(W * 32);
   cfg.dynamicSmemBytes = (size_t)W * cl_warp_bytes<RW, ST>();
   cfg.stream = sm;
@@ -580,10 +580,17 @@ static purekv_status launch_cluster_as(int32_t cl, cudaStream_t sm, const void* 
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see griddepcontrol in the kernel
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = (unsigned)cl;
   attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
+  auto set_size = [&](int32_t c) {
+    cfg.gridDim = dim3((unsigned)c, (unsigned)Hkv, (unsigned)n_req);
+    attr[1].val.clusterDim.x = (unsigned)c;
+  };
+  set_size(cluster_that_fits(cl, [&](int32_t c) {
+    set_size(c);
+    return clusters_at_once(kernel, cfg);
+  }));
   PK_CUDA(cudaLaunchKernelEx(&cfg, kernel, (const uint4*)q, (const uint4*)kc, (const uint4*)vc, cu_kept, H, Hkv, scale_log2,
                              (__nv_bfloat16*)o, lse));
   return PUREKV_OK;

@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "cluster.cuh"
 #include "common.cuh"
 
 namespace purekv {
@@ -707,47 +708,56 @@ __global__ void __launch_bounds__(kMmaThreads, 1) score_cluster_kernel(
   pool_in_cluster<kKeys>(colbuf, halo, half, rank, C, j0, nr, len, cg);
 }
 
-// grid (C, Hkv, n_req) in clusters of C CTAs, behind the previous kernel by programmatic stream serialization.  `wide`: devices
-// on which the kernel's clusters of more than eight CTAs have been allowed (they are opt-in).
-template <typename... Params, typename... Args>
-static purekv_status launch_cluster(void (*kernel)(Params...), std::atomic<uint64_t>& wide, int32_t C, int32_t Hkv, int32_t n_req,
-                                    int threads, size_t smem, cudaStream_t sm, Args... args) {
+// A launch of grid (C, Hkv, n_req) in clusters of C CTAs, behind the previous kernel by programmatic stream serialization.
+struct ClusterLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  ClusterLaunch(int32_t C, int32_t Hkv, int32_t n_req, int threads, size_t smem, cudaStream_t sm) {
+    cfg.gridDim = dim3((unsigned)C, (unsigned)Hkv, (unsigned)n_req);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = sm;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)C;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+  }
+  ClusterLaunch(const ClusterLaunch&) = delete;
+  ClusterLaunch& operator=(const ClusterLaunch&) = delete;
+};
+
+// Allows the kernel all of an SM's shared memory and clusters of more than eight CTAs (opt-in, once per device).
+template <typename... Params>
+static purekv_status allow_wide_clusters(void (*kernel)(Params...), std::atomic<uint64_t>& smem, std::atomic<uint64_t>& wide) {
+  const purekv_status st = allow_max_dynamic_smem(kernel, smem);
+  if (st != PUREKV_OK) return st;
   int dev = -1;
   PK_CUDA(cudaGetDevice(&dev));
   if (!(wide.load(std::memory_order_acquire) & (1ull << dev))) {
     PK_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     wide.fetch_or(1ull << dev, std::memory_order_release);
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)C, (unsigned)Hkv, (unsigned)n_req);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = sm;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = (unsigned)C;
-  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  PK_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
   return PUREKV_OK;
 }
 
 template <int MB>
 static purekv_status launch_score_cluster(const void* q, const void* k, float* c_out, const purekv_batch* b, int32_t window,
                                           int32_t obs, int32_t pool, int32_t H, int32_t Hkv, int32_t d, float scale,
-                                          cudaStream_t sm) {
+                                          cudaStream_t sm, bool* launched) {
   auto kernel = score_cluster_kernel<MB>;
   static std::atomic<uint64_t> smem_allowed{0}, wide_allowed{0};
-  const purekv_status st = allow_max_dynamic_smem(kernel, smem_allowed);
+  const purekv_status st = allow_wide_clusters(kernel, smem_allowed, wide_allowed);
   if (st != PUREKV_OK) return st;
   const int32_t C = std::max(1, (max_len(b) + MB * kCtaKeys - 1) / (MB * kCtaKeys));
-  return launch_cluster(kernel, wide_allowed, C, Hkv, b->n_req, kMmaThreads,
-                        (size_t)(MB * kCtaKeys + 2 * kMmaRows) * (d + 8) * sizeof(__nv_bfloat16), sm, (const __nv_bfloat16*)q,
-                        (const __nv_bfloat16*)k, b->cu_seqlens, window, obs, pool, H, Hkv, d, scale * 1.4426950408889634f,
-                        b->total_tokens, c_out);
+  ClusterLaunch l(C, Hkv, b->n_req, kMmaThreads, (size_t)(MB * kCtaKeys + 2 * kMmaRows) * (d + 8) * sizeof(__nv_bfloat16), sm);
+  *launched = clusters_at_once(kernel, l.cfg) >= 1;
+  if (!*launched) return PUREKV_OK;
+  PK_CUDA(cudaLaunchKernelEx(&l.cfg, kernel, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, b->cu_seqlens, window, obs, pool, H, Hkv,
+                             d, scale * 1.4426950408889634f, b->total_tokens, c_out));
+  return PUREKV_OK;
 }
 
 // ---- fp32, both passes in one launch -------------------------------------------------------------------------------
@@ -873,14 +883,17 @@ __global__ void __launch_bounds__(kThreads, 1) score_cluster_f32_kernel(
 
 static purekv_status launch_score_cluster_f32(const float* q, const float* k, float* c_out, const purekv_batch* b,
                                               int32_t window, int32_t obs, int32_t pool, int32_t H, int32_t Hkv, int32_t d,
-                                              float scale, cudaStream_t sm) {
+                                              float scale, cudaStream_t sm, bool* launched) {
   static std::atomic<uint64_t> smem_allowed{0}, wide_allowed{0};
-  const purekv_status st = allow_max_dynamic_smem(score_cluster_f32_kernel, smem_allowed);
+  const purekv_status st = allow_wide_clusters(score_cluster_f32_kernel, smem_allowed, wide_allowed);
   if (st != PUREKV_OK) return st;
   const int32_t C = std::max(1, (max_len(b) + kKB - 1) / kKB);
-  return launch_cluster(score_cluster_f32_kernel, wide_allowed, C, Hkv, b->n_req, kThreads,
-                        (size_t)(kKB + 2 * kRB) * (d + 4) * sizeof(float), sm, q, k, b->cu_seqlens, window, obs, pool, H, Hkv, d,
-                        scale * 1.4426950408889634f, b->total_tokens, c_out);
+  ClusterLaunch l(C, Hkv, b->n_req, kThreads, (size_t)(kKB + 2 * kRB) * (d + 4) * sizeof(float), sm);
+  *launched = clusters_at_once(score_cluster_f32_kernel, l.cfg) >= 1;
+  if (!*launched) return PUREKV_OK;
+  PK_CUDA(cudaLaunchKernelEx(&l.cfg, score_cluster_f32_kernel, q, k, b->cu_seqlens, window, obs, pool, H, Hkv, d,
+                             scale * 1.4426950408889634f, b->total_tokens, c_out));
+  return PUREKV_OK;
 }
 
 // `obs` = accumulated rows per request and head (Eq. 2: the window itself); the first pass and the merge see only
@@ -1028,15 +1041,17 @@ static purekv_status score_impl(const char* who, const void* q, const void* k, f
   // tokens, 32 rows: 42 against 72 us), more are not: nothing runs beside a CTA that waits at a barrier (8 requests, 100-row
   // window, 6 blocks: 180 against 170 us).
   const int64_t ctas = (int64_t)batch->n_req * n_kv_heads * ((ml + 2 * kCtaKeys - 1) / (2 * kCtaKeys)) * (ml <= kClusterMax * kCtaKeys ? 2 : 1);
+  bool launched = false;
   if (dtype == PUREKV_BF16 && head_dim % 16 == 0 && head_dim <= 128 && ml <= kClusterMax * 2 * kCtaKeys &&
       row_blocks <= kClusterRowBlocks && pool / 2 <= kPoolHalfMax && (ctas <= 148 || row_blocks <= 2))
-    return ml <= kClusterMax * kCtaKeys
-               ? launch_score_cluster<1>(q, k, c_out, batch, window, obs, pool, n_q_heads, n_kv_heads, head_dim, scale, sm)
-               : launch_score_cluster<2>(q, k, c_out, batch, window, obs, pool, n_q_heads, n_kv_heads, head_dim, scale, sm);
+    st = ml <= kClusterMax * kCtaKeys
+             ? launch_score_cluster<1>(q, k, c_out, batch, window, obs, pool, n_q_heads, n_kv_heads, head_dim, scale, sm, &launched)
+             : launch_score_cluster<2>(q, k, c_out, batch, window, obs, pool, n_q_heads, n_kv_heads, head_dim, scale, sm, &launched);
   if (dtype == PUREKV_FP32 && ml <= kClusterMax * kKB && row_blocks <= kClusterRowBlocks && pool / 2 <= kKB / 2 &&
       ((uintptr_t)q | (uintptr_t)k) % 16 == 0)
-    return launch_score_cluster_f32((const float*)q, (const float*)k, c_out, batch, window, obs, pool, n_q_heads, n_kv_heads,
-                                    head_dim, scale, sm);
+    st = launch_score_cluster_f32((const float*)q, (const float*)k, c_out, batch, window, obs, pool, n_q_heads, n_kv_heads,
+                                  head_dim, scale, sm, &launched);
+  if (st != PUREKV_OK || launched) return st;  // (a device that cannot place one such cluster takes the separate kernels)
   if (dtype == PUREKV_BF16 && head_dim % 16 == 0)
     st = launch_score_mma(q, k, c_raw, batch, window, obs, n_q_heads, n_kv_heads, head_dim, scale, lse2, sm);
   else if (dtype == PUREKV_BF16)
