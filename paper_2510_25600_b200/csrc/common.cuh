@@ -72,7 +72,8 @@ __device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162flo
 // [Unit x n_units][merge counters int32 x n_counters][scheduling counters int32 x 2]
 // all sections 16-byte aligned.  The last three sections exist only in plans for the tensor-core kernel, whose
 // entries section also holds, behind the query tiles' own lists, the merged lists of the twin units (see Unit).
-constexpr uint32_t kPlanMagic = 0x504B5636u;  // "PKV6"
+// The magic names the layout and changes with it, so that a plan kept from another build of the library is refused.
+constexpr uint32_t kPlanMagic = 0x504B5637u;  // "PKV7": the kept halves behind the masks, merge counters of a byte per warp
 
 // kTileNone appears only in the merged list of a twin unit: a key tile one of the two query tiles does not keep.
 enum TileClass : int32_t { kTileFull = 0, kTileDiag = 1, kTileGeneral = 2, kTileNone = 3 };
