@@ -20,7 +20,10 @@ LIB_PATH = os.path.join(_HERE, "libpurekv.so")
 if not os.path.exists(LIB_PATH):
     raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2510_25600_b200.build`")
 _lib = C.CDLL(LIB_PATH)
-from . import _marshal  # noqa: E402  (after the library it calls; built with it)
+try:
+    from . import _marshal  # noqa: E402  (after the library it calls; built with it, one per Python ABI)
+except ImportError as e:
+    raise ImportError(f"{_HERE} holds no _marshal module for this Python: build it with `python -m paper_2510_25600_b200.build`") from e
 
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT, ERR_BAD_PLAN = range(7)
 BF16, FP32 = 0, 1
@@ -133,14 +136,16 @@ def _check(status: int, where: str) -> None:
         raise PureKVError(status, where)
 
 
-# (None in a build of torch without CUDA, where nothing asks for a stream)
-_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-_current_device = getattr(torch._C, "_cuda_getDevice", None)
+def _stream_getter(torch_c):
+    """The function that gives the current stream of the current device as an integer: without building a Stream object on
+    every call where torch has the two functions for it, which are not part of its public interface."""
+    raw, device = getattr(torch_c, "_cuda_getCurrentRawStream", None), getattr(torch_c, "_cuda_getDevice", None)
+    if raw is None or device is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(device())
 
 
-def _stream() -> int:
-    # the current stream of the current device as an integer, without building a Stream object on every call
-    return _raw_stream(_current_device())
+_stream = _stream_getter(torch._C)
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -439,7 +444,7 @@ def purekv_decode_attention(q: torch.Tensor, k_cache: torch.Tensor, v_cache: tor
         q.data_ptr(), k_cache.data_ptr(), v_cache.data_ptr(), out.data_ptr(), None if lse is None else lse.data_ptr(),
         budget.cu_kept.data_ptr(), b, budget.h_cu_kept, h, k_cache.size(1), d,
         BF16 if q.dtype is torch.bfloat16 else _dtype_code(q), softmax_scale, None if ws is None else ws.data_ptr(),
-        0 if ws is None else ws.nbytes, _raw_stream(_current_device()))
+        0 if ws is None else ws.nbytes, _stream())
     if status != OK:
         if status == ERR_WORKSPACE:  # (fp32 rows) none given, or too small
             kept = np.diff(budget.h_cu_kept)

@@ -1,5 +1,5 @@
-"""Builds libpurekv.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _marshal.so, the Python module that
-passes arguments to it.
+"""Builds libpurekv.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _marshal, the Python module that passes
+arguments to it (its file name carries the interpreter's ABI, so another Python builds its own).
 
     python -m paper_2510_25600_b200.build [--force] [--verbose]
 """
@@ -14,7 +14,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(_HERE), "include")
 LIB = os.path.join(_HERE, "libpurekv.so")
-MARSHAL = os.path.join(_HERE, "_marshal.so")
+MARSHAL = os.path.join(_HERE, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ["plan.cu", "compact.cu", "decode.cu", "select.cu", "score.cu", "score_tc.cu", "prefill.cu", "prefill_simt.cu", "prefill_tc.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--use_fast_math=false"]
@@ -61,6 +61,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if force or procs or _stale(LIB, objs):
         subprocess.check_call([_nvcc(), "-shared", "-o", LIB, *objs, "-gencode", "arch=compute_100a,code=sm_100a"])
     src = os.path.join(CSRC, "marshal.cpp")
+    untagged = os.path.join(_HERE, "_marshal.so")  # of an earlier build: any interpreter would load it
+    if os.path.exists(untagged) and untagged != MARSHAL:
+        os.remove(untagged)
     if force or _stale(MARSHAL, [src, LIB] + headers):
         # found beside the module at run time: one copy of the library, whether it is loaded through this or by path
         subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", INCLUDE,
