@@ -445,12 +445,14 @@ def purekv_decode_attention(q: torch.Tensor, k_cache: torch.Tensor, v_cache: tor
         budget.cu_kept.data_ptr(), b, budget.h_cu_kept, h, k_cache.size(1), d,
         BF16 if q.dtype is torch.bfloat16 else _dtype_code(q), softmax_scale, None if ws is None else ws.data_ptr(),
         0 if ws is None else ws.nbytes, _stream())
+    if status == ERR_WORKSPACE:  # (fp32 rows) none given, or too small: one of the size that these b requests need, once
+        need = purekv_decode_ws_bytes(b, int(np.diff(budget.h_cu_kept[:b + 1]).max()), h, k_cache.size(1), d)
+        ws = torch.empty(need, dtype=torch.uint8, device=q.device)
+        status = _marshal.purekv_decode_attention(
+            q.data_ptr(), k_cache.data_ptr(), v_cache.data_ptr(), out.data_ptr(), None if lse is None else lse.data_ptr(),
+            budget.cu_kept.data_ptr(), b, budget.h_cu_kept, h, k_cache.size(1), d, _dtype_code(q), softmax_scale, ws.data_ptr(),
+            ws.nbytes, _stream())
     if status != OK:
-        if status == ERR_WORKSPACE:  # (fp32 rows) none given, or too small
-            kept = np.diff(budget.h_cu_kept)
-            need = purekv_decode_ws_bytes(b, int(kept.max()), h, k_cache.size(1), d)
-            return purekv_decode_attention(q, k_cache, v_cache, budget, out, lse, softmax_scale,
-                                           torch.empty(need, dtype=torch.uint8, device=q.device))
         raise PureKVError(status, "purekv_decode_attention")
     return out
 
