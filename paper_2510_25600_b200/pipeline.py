@@ -65,7 +65,7 @@ class PureKVPipeline:
         self.k_c = torch.empty((nc, self.budget.total_kept, n_kv_heads, head_dim), dtype=dtype, device=dev)
         self.v_c = torch.empty_like(self.k_c)
         self.status = torch.zeros(1, dtype=torch.int32, device=dev)
-        self.plan_dense = self.plan_st = None
+        self.plan_dense = self._plan_st = None
         # prefill per layer, score (1 kernel one-pass or in one cluster, up to 3 otherwise: counted as 1), select (2), compact
         self.launches_per_step = n_layers + len(self.scored) + 2 + 1
 
@@ -84,6 +84,14 @@ class PureKVPipeline:
         ev.record()
         return P.Plan(d_buf, info)
 
+    @property
+    def plan_st(self) -> P.Plan:
+        """The sparse mask's plan.  A pass without sparse layers does not need it: it is then made when asked for."""
+        if self._plan_st is None:
+            self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st)
+            self._size_prefill_ws(self._plan_st)
+        return self._plan_st
+
     def _size_prefill_ws(self, plan: P.Plan) -> None:
         need = max(16, plan.info.ws_bytes)
         if self.prefill_ws is None or self.prefill_ws.numel() < need:
@@ -92,7 +100,7 @@ class PureKVPipeline:
     def build_plans(self) -> None:
         """Both masks' plans; `run_device` builds each just ahead of the first layer that needs it."""
         self.plan_dense = self._plan(self.params_dense, self._h_dense, self.plan_buf_dense)
-        self.plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st)
+        self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st)
         self._size_prefill_ws(self.plan_dense)
         self._size_prefill_ws(self.plan_st)
 
@@ -123,7 +131,7 @@ class PureKVPipeline:
                 main = torch.cuda.current_stream()
                 self._copies.wait_event(before)
                 with torch.cuda.stream(self._copies):
-                    self.plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st)
+                    self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st)
                 main.wait_event(self._h_st[0][1])
                 self._size_prefill_ws(self.plan_st)
             if events is not None:
