@@ -31,6 +31,5 @@ def test_a_plan_of_the_layout_before_is_refused():
     out = torch.full_like(q, 7.0)
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     pk.purekv_st_sparse_prefill(q, k, v, b, pk.Plan(torch.from_numpy(plan).cuda(), info), out=out, status=status)
-    with pytest.raises(pk.PureKVError) as e:
-        pk.purekv_poll_status(status)
-    assert e.value.status == pk.ERR_BAD_PLAN and (out == 7.0).all()
+    # (read directly: the traceback of a raised error would keep the tensors alive past the test, until some later collection)
+    assert status.item() == pk.ERR_BAD_PLAN and (out == 7.0).all()
