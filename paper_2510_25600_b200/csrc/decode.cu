@@ -597,23 +597,45 @@ static purekv_status launch_cluster_as(int32_t cl, cudaStream_t sm, const void* 
 }
 
 template <int RW>
-static purekv_status launch_cluster(int32_t max_kept, cudaStream_t sm, const void* q, const void* kc, const void* vc,
-                                    const int32_t* cu_kept, int32_t n_req, int32_t H, int32_t Hkv, float scale_log2, void* o,
-                                    float* lse) {
-  // CTAs per cluster, measured over 1-256 requests of 1-500 000 rows: shares of down to 64 rows pay (128 rows in one CTA of
-  // eight warps are a single trip, and a cluster costs 1 us), as long as every CTA finds an SM of its own -- 128 CTAs for
-  // clusters of up to four, 64 beyond (clusters of 8 or 16 CTAs with all of an SM's memory do not fill the GPCs: two
-  // requests, 4 KV heads, 1664 rows: 7.2 us as 8 clusters of 8, 11.5 as 8 of 16).
+static purekv_status launch_cluster(int32_t max_kept, int64_t total_kept, cudaStream_t sm, const void* q, const void* kc,
+                                    const void* vc, const int32_t* cu_kept, int32_t n_req, int32_t H, int32_t Hkv,
+                                    float scale_log2, void* o, float* lse) {
   const int64_t base = (int64_t)n_req * Hkv;
-  int32_t cl = 1;
-  if (max_kept > 128)
-    while (cl < kClMax && base * cl * 2 <= (cl * 2 >= 8 ? 64 : 128) && max_kept > 64 * cl) cl *= 2;
+  const bool skewed = max_kept > 256 && 2 * (int64_t)max_kept * n_req > 3 * total_kept;
+  int32_t cl = 1;  // CTAs per cluster
+  if (skewed) {
+    // One long request among short ones: more CTAs each shorten what the last one streams, and the short requests' clusters
+    // take turns on the GPU.  Times in ns as measured with an SM per CTA: 4 us for a cluster that has little to do, 6.9 ns a
+    // row for a CTA that streams among idle ones, 6.3 TB/s for all; so many clusters fit at once.  (Chosen by this rule against
+    // the one for even batches, 28 / 4 heads: 20 000 rows among 63 x 100: 40 against 132 us; 60 000 among 7 x 100: 35 against
+    // 105; 4 x 30 000 among 60 x 1000: 81 against 202; 64 x 300-9000 at random: 106 either way.)
+    const int32_t at_once[5] = {148, 74, 33, 15, 7};
+    double best = 0.;
+    for (int32_t i = 0; i < 5; ++i) {
+      const int32_t c = 1 << i;
+      const double row = std::max(6.9, 0.0813 * (double)(std::min<int64_t>(base, at_once[i]) * c));
+      const double waves = (double)((base + at_once[i] - 1) / at_once[i]);
+      const double t = std::max(waves * (4000. + (double)total_kept / n_req / c * row), 4000. + (double)max_kept / c * 6.9);
+      if (i == 0 || t < best) { best = t; cl = c; }
+    }
+  } else if (max_kept > 256) {
+    // Even batches, measured over 1-256 requests of 1-500 000 rows: shares of down to 64 rows pay (256 rows are two trips of one
+    // CTA's eight warps, 4.9 us, and a cluster costs 1 us), as long as every CTA finds an SM of its own -- 128 CTAs for
+    // clusters of up to four, 64 beyond (clusters of 8 or 16 CTAs with all of an SM's memory do not fill the GPCs: two
+    // requests, 4 KV heads, 1664 rows: 7.2 us as 8 clusters of 8, 11.5 as 8 of 16).  Where each CTA still has thousands of rows
+    // to stream, up to the 15 or 7 such clusters that fit at once (three requests of 60 000 rows, 4 KV heads: 105 -> 65 us).
+    auto room = [&](int32_t c) {
+      if (c < 8) return base * c <= 128;
+      return base * c <= 64 || (max_kept > 4096 * (c / 2) && base <= (c == 8 ? 15 : 7));
+    };
+    while (cl < kClMax && max_kept > 64 * cl && room(2 * cl)) cl *= 2;
+  }
   const int32_t share = (max_kept + cl - 1) / cl;
-  // Eight warps and the SM to themselves for CTAs that are alone on it (four requests of 20 000 rows: 41 against 47 us) or
-  // stream long shares (128 x 5000 rows: 167 against 174 us); otherwise two CTAs of four warps, so that one streams while
-  // the other starts or ends (128 requests of up to 700 rows: 39 against 52 us).  One stage when a share is a single trip.
-  const bool wide = share > 64 && (base * cl <= 148 || share > 2048);
-  if (wide)
+  // Eight warps and the SM to themselves for CTAs that are alone on it (four requests of 20 000 rows: 41 against 47 us; one of
+  // 500, 16 heads per KV head: 6.4 against 7.7) or stream long shares (128 x 5000 rows: 167 against 174 us); otherwise two CTAs
+  // of four warps, so that one streams while the other starts or ends (128 requests of up to 700 rows: 39 against 52 us).  One
+  // stage when a share is a single trip.
+  if (skewed || base * cl <= 148 || share > 2048)
     return share <= 128 ? launch_cluster_as<RW, 8, 1>(cl, sm, q, kc, vc, cu_kept, n_req, H, Hkv, scale_log2, o, lse)
                         : launch_cluster_as<RW, 8, 3>(cl, sm, q, kc, vc, cu_kept, n_req, H, Hkv, scale_log2, o, lse);
   return share <= 64 ? launch_cluster_as<RW, 4, 1>(cl, sm, q, kc, vc, cu_kept, n_req, H, Hkv, scale_log2, o, lse)
@@ -671,8 +693,8 @@ purekv_status purekv_decode_attention(const void* q, const void* k_cache, const 
   cudaStream_t sm = (cudaStream_t)stream;
   PK_REQUIRE(n_kv_heads <= 65535 && n_req <= 65535, PUREKV_ERR_UNSUPPORTED, "too many heads or requests");
   if (dtype == PUREKV_BF16)
-    return G <= 8 ? launch_cluster<1>(max_kept, sm, q, k_cache, v_cache, cu_kept, n_req, n_q_heads, n_kv_heads, scale_log2, o, lse)
-                  : launch_cluster<2>(max_kept, sm, q, k_cache, v_cache, cu_kept, n_req, n_q_heads, n_kv_heads, scale_log2, o, lse);
+    return G <= 8 ? launch_cluster<1>(max_kept, h_cu_kept[n_req], sm, q, k_cache, v_cache, cu_kept, n_req, n_q_heads, n_kv_heads, scale_log2, o, lse)
+                  : launch_cluster<2>(max_kept, h_cu_kept[n_req], sm, q, k_cache, v_cache, cu_kept, n_req, n_q_heads, n_kv_heads, scale_log2, o, lse);
   int32_t chunk, n_splits;
   decode_split(n_req, max_kept, n_kv_heads, &chunk, &n_splits);
   float* part = nullptr;
