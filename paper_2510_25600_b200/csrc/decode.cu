@@ -220,7 +220,11 @@ __device__ __forceinline__ uint32_t dec_pack_bf16(float lo, float hi) {
   return r;
 }
 
-constexpr float kDecRescale = 8.f;  // the reference maximum of a row moves only when a logit exceeds it by this (log2)
+// A row's reference maximum moves when a logit exceeds it by this (log2).  At 0 it is the largest logit so far, and the heaviest
+// weights are powers of two, exact in bf16: error against 64 bits 1.87e-3 of the norm of the result for 8 requests of 5000 rows, 1.90
+// for 64 of 700, 1.79 for one of 3000 with 16 heads per KV head; at 8, 2.29, 2.31 and 1.97e-3.  (The chunk kernel of before, at 8 but
+// with a single trip per warp for short requests: 2.28, 2.25 and 1.77.)  Up to 5 % slower with 16 heads per KV head, otherwise equal.
+constexpr float kDecRescale = 0.f;
 
 // One launch.  A cluster of C CTAs (grid (C, H_kv, n_req)) owns one (request, KV head); CTA `rank` takes the rank-th share
 // of the request's rows, so ragged requests are cut evenly, and the CTAs' partial results meet in distributed shared
