@@ -53,7 +53,7 @@ constexpr int kVnSmem = kVnWarps * kVnStages * kVnRows * 256;
 template <typename T>
 __global__ void __launch_bounds__(kVnWarps * 32, 1) vnorm_score_kernel(const uint4* __restrict__ v, int64_t layer_stride_c,
                                                                        const float* __restrict__ c, int64_t n_tokens,
-                                                                       int32_t n_kv_heads, int32_t n_layers,
+                                                                       int32_t n_kv_heads, int32_t n_layers, bool streaming,
                                                                        float* __restrict__ s_out) {
   extern __shared__ __align__(16) uint8_t vn_smem[];
   const int32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -62,6 +62,9 @@ __global__ void __launch_bounds__(kVnWarps * 32, 1) vnorm_score_kernel(const uin
   const int64_t first = n_items * blockIdx.x / gridDim.x, last = n_items * (blockIdx.x + 1) / gridDim.x;
   asm volatile("griddepcontrol.wait;" ::: "memory");  // (launched with programmatic stream serialization)
   const uint32_t ring = (uint32_t)__cvta_generic_to_shared(vn_smem) + (uint32_t)warp * (kVnStages * kVnRows * 256);
+  uint64_t policy;  // of the loads in L2: first to be evicted when V does not stay there anyway, see the launch
+  if (streaming) asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  else asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
   // the block to load next, and the block to sum next
   int64_t f_item = first + warp, item = f_item;
   int32_t f_layer = (int32_t)(f_item / n_blocks), layer = f_layer;
@@ -78,7 +81,8 @@ __global__ void __launch_bounds__(kVnWarps * 32, 1) vnorm_score_kernel(const uin
 #pragma unroll
       for (int i = 0; i < 8; ++i) {  // two rows per request; rows past the end repeat the last one, never stored
         const int64_t r = min(r0 + 2 * i + (lane >> 4), n_rows - 1);
-        asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16;" ::"r"(dst + i * 512), "l"(src + r * 16 + (lane & 15)) : "memory");
+        asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst + i * 512),
+                     "l"(src + r * 16 + (lane & 15)), "l"(policy) : "memory");
       }
       advance(f_item, f_layer, f_blk);
     }
@@ -506,6 +510,12 @@ static purekv_status select_impl(const float* c, const void* v, int64_t v_layer_
     const purekv_status st_smem = allow_max_dynamic_smem(vnorm_score_kernel<E>, smem_allowed);
     if (st_smem != PUREKV_OK) return st_smem;
     const int64_t blocks = ((T * n_kv_heads + kVnRows - 1) / kVnRows) * n_layers;
+    // A V much larger than what the L2 (126 MB) keeps cannot be found there by what comes next, and as the first to be evicted it
+    // leaves the scores, and dirty lines that would have to be written back meanwhile, in place.  One call with a cold L2, 26
+    // layers of 8320 tokens x 4 heads: 64 -> 58 us, in a row 50 -> 48; 864 ragged segments with their compaction 865 -> 829.  A
+    // smaller V does better as it is (calls in a row, without and with the hint: 38 MB 39 and 42 us, 68 MB 20 and 24, 76 MB 44
+    // and 48, 110 MB 32 and 32).
+    const bool streaming = T * n_kv_heads * n_layers * 256 > (int64_t)96 << 20;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)std::min<int64_t>((blocks + kVnWarps - 1) / kVnWarps, 148));
     cfg.blockDim = dim3(kVnWarps * 32);
@@ -516,7 +526,7 @@ static purekv_status select_impl(const float* c, const void* v, int64_t v_layer_
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    PK_CUDA(cudaLaunchKernelEx(&cfg, vnorm_score_kernel<E>, (const uint4*)v, stride_c, c, T, n_kv_heads, n_layers, s_buf));
+    PK_CUDA(cudaLaunchKernelEx(&cfg, vnorm_score_kernel<E>, (const uint4*)v, stride_c, c, T, n_kv_heads, n_layers, streaming, s_buf));
     return PUREKV_OK;
   };
   const purekv_status st_v = dtype == PUREKV_BF16 ? launch_vnorm(__nv_bfloat16{}) : launch_vnorm(float{});
