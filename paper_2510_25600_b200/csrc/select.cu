@@ -2,13 +2,13 @@
 //
 // vnorm_score_kernel streams V once over the whole GPU (the only large traffic of this step) and writes S; select_kernel
 // then handles one (request, KV head, layer) segment per CTA, launched so that its start-up hides behind the tail of the
-// first.  (One CTA that streamed its own segment's V and selected from shared memory, without S in memory, was the choice for
-// 296 segments and more: 8 requests of 2000 to 16 000 tokens x 4 heads x 27 layers, selection and compaction, took 552 us that
-// way and take 505 with two kernels -- the segments differ in length and no CTA keeps loads in flight while it selects.)  The selection
+// first.  (A CTA that streams its own segment's V and selects from shared memory, without S in memory, is for callers without a
+// workspace: the segments differ in length and no CTA keeps loads in flight while it selects, see select_impl.)  The selection
 // is a 4 x 8-bit MSB-first radix select over the fp32 bit patterns (keys staged in shared memory) that finds the
 // h-th largest score, then a block-scan compaction that emits the chosen positions in ascending order; among
 // scores equal to the threshold the lowest positions win, so the result is deterministic.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -157,15 +157,24 @@ struct Gather {
   int32_t cpr;
 };
 
+// V of a caller who hands over no room for the scores: rows of 256 bytes, layer stride in chunks, and the C of Eq. 2.
+struct Stream {
+  const uint4* v;
+  int64_t layer_stride_c;
+  const float* c;
+};
+
 // One CTA per (request, KV head, layer) over the scores `s` (written by vnorm_score_kernel).  `staged`: the launch has
-// room in shared memory for the segment's keys.
-template <bool GATHER>
+// room in shared memory for the segment's keys.  With T the element type of V the CTA forms the scores of its segment itself,
+// from `own`, and they go no further than its shared memory (as vnorm_score_kernel sums them: bit for bit the same).
+template <typename T, bool GATHER>
 __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __restrict__ s, int64_t n_tokens,
                                                              const int32_t* __restrict__ cu_seqlens,
                                                              const int32_t* __restrict__ cu_kept,
                                                              const int32_t* __restrict__ keep, int32_t window,
                                                              int32_t k_tot, int32_t n_kv_heads,
-                                                             int32_t* __restrict__ idx_out, bool staged, Gather ga) {
+                                                             int32_t* __restrict__ idx_out, bool staged, Gather ga, Stream own) {
+  constexpr bool kOwn = !std::is_void_v<T>;
   extern __shared__ __align__(16) uint32_t skeys[];  // order keys of the segment's non-recent scores
   __shared__ int32_t hist[256];
   __shared__ uint32_t sh_prefix;
@@ -192,9 +201,37 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __rest
   const int32_t tid = threadIdx.x;
 
   for (int32_t t = tid; t < w; t += kSelThreads) out[h + t] = nr + t;  // the recent window
+  if constexpr (kOwn) {  // a half-warp per row, 16 rows of each in flight
+    const uint4* vl = own.v + layer * own.layer_stride_c;
+    const float* cg = own.c + (int64_t)g * n_tokens + base;
+    const int32_t half = (tid >> 4) & 1, ch = tid & 15;
+    for (int32_t t0 = (tid >> 5) * 32; t0 < nr; t0 += kSelThreads) {
+      uint4 buf[16];
+#pragma unroll
+      for (int it = 0; it < 16; ++it) {  // rows past the end read the last one again; never stored
+        const int32_t t = min(t0 + it * 2 + half, nr - 1);
+        buf[it] = __ldcs(vl + ((int64_t)(base + t) * n_kv_heads + g) * 16 + ch);
+      }
+      float mine = 0.f;
+#pragma unroll
+      for (int it = 0; it < 16; ++it) {
+        float p = Chunk<T>::sumsq(buf[it]);
+        p += __shfl_xor_sync(0xffffffffu, p, 8);
+        p += __shfl_xor_sync(0xffffffffu, p, 4);
+        p += __shfl_xor_sync(0xffffffffu, p, 2);
+        p += __shfl_xor_sync(0xffffffffu, p, 1);
+        const float p0 = __shfl_sync(0xffffffffu, p, 0), p1 = __shfl_sync(0xffffffffu, p, 16);
+        if ((tid & 31) == it * 2) mine = p0;
+        if ((tid & 31) == it * 2 + 1) mine = p1;
+      }
+      const int32_t t = t0 + (tid & 31);
+      if (t < nr) skeys[t] = order_key(__ldg(cg + t) * sqrtf(mine));
+    }
+    __syncthreads();
+  }
   // the range of the keys, taken along the way: the radix select only has to resolve the bits in which they differ
   uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
-  if (staged) {  // copied into shared memory once, so the radix passes do not go back to L2
+  if (!kOwn && staged) {  // copied into shared memory once, so the radix passes do not go back to L2
 #pragma unroll 8
     for (int32_t j = tid; j < nr; j += kSelThreads) {  // loads of a trip in flight together
       const uint32_t key = order_key(__ldg(seg + j));
@@ -207,7 +244,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __rest
   const int32_t lane = tid & 31, warp = tid >> 5;
   if (h > 0) {
 
-  if (!staged) {
+  if (kOwn || !staged) {
 #pragma unroll 4
     for (int32_t j = tid; j < nr; j += kSelThreads) {
       const uint32_t key = key_at(j);
@@ -491,6 +528,25 @@ static purekv_status select_impl(const float* c, const void* v, int64_t v_layer_
   for (int r = 0; r < batch->n_req; ++r) longest = std::max(longest, batch->h_cu_seqlens[r + 1] - batch->h_cu_seqlens[r]);
   const size_t key_bytes = (size_t)longest * sizeof(uint32_t);
   float* s_buf = s_out;
+  const bool gather = ga.k_src != nullptr;
+  // Two waves and more of segments with rows of 256 bytes need no workspace: without one the selecting CTAs form their segments'
+  // scores themselves (16 requests of 1500 tokens x 8 heads x 31 layers: 290 us this way, 271 with the scores in memory; 8 ragged
+  // requests x 4 x 27: 510 and 458).
+  if (!s_buf && (!ws || ws_bytes < purekv_select_ws_bytes(batch, n_layers, n_kv_heads)) && cpr == 16 && key_bytes <= 200 * 1024 &&
+      (int64_t)batch->n_req * n_kv_heads * n_layers >= 2 * 148) {
+    auto launch_own = [&](auto kernel, std::atomic<uint64_t>& smem_allowed) -> purekv_status {
+      const purekv_status st_smem = allow_max_dynamic_smem(kernel, smem_allowed);
+      if (st_smem != PUREKV_OK) return st_smem;
+      kernel<<<g2, kSelThreads, key_bytes, sm>>>(nullptr, T, batch->cu_seqlens, cu_kept, keep, window, k_tot, n_kv_heads, idx_out,
+                                                 true, ga, Stream{(const uint4*)v, v_layer_stride * esz / 16, c});
+      PK_CUDA(cudaGetLastError());
+      return PUREKV_OK;
+    };
+    static std::atomic<uint64_t> allowed[4] = {{0}, {0}, {0}, {0}};
+    if (dtype == PUREKV_BF16)
+      return gather ? launch_own(select_kernel<__nv_bfloat16, true>, allowed[0]) : launch_own(select_kernel<__nv_bfloat16, false>, allowed[1]);
+    return gather ? launch_own(select_kernel<float, true>, allowed[2]) : launch_own(select_kernel<float, false>, allowed[3]);
+  }
   if (!s_buf) {
     PK_REQUIRE(ws && ws_bytes >= purekv_select_ws_bytes(batch, n_layers, n_kv_heads), PUREKV_ERR_WORKSPACE,
                "purekv_select_topk: workspace of %zu bytes is too small", ws_bytes);
@@ -532,11 +588,10 @@ static purekv_status select_impl(const float* c, const void* v, int64_t v_layer_
   const purekv_status st_v = dtype == PUREKV_BF16 ? launch_vnorm(__nv_bfloat16{}) : launch_vnorm(float{});
   if (st_v != PUREKV_OK) return st_v;
   const bool stage_keys = key_bytes <= 200 * 1024;
-  const bool gather = ga.k_src != nullptr;
   if (stage_keys) {
     static std::atomic<uint64_t> smem_allowed{0}, smem_allowed_g{0};
-    const purekv_status st_smem = gather ? allow_max_dynamic_smem(select_kernel<true>, smem_allowed_g)
-                                         : allow_max_dynamic_smem(select_kernel<false>, smem_allowed);
+    const purekv_status st_smem = gather ? allow_max_dynamic_smem(select_kernel<void, true>, smem_allowed_g)
+                                         : allow_max_dynamic_smem(select_kernel<void, false>, smem_allowed);
     if (st_smem != PUREKV_OK) return st_smem;
   }
   cudaLaunchConfig_t cfg = {};
@@ -550,11 +605,11 @@ static purekv_status select_impl(const float* c, const void* v, int64_t v_layer_
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (gather)
-    PK_CUDA(cudaLaunchKernelEx(&cfg, select_kernel<true>, (const float*)s_buf, T, batch->cu_seqlens, cu_kept,
-                               keep, window, k_tot, n_kv_heads, idx_out, stage_keys, ga));
+    PK_CUDA(cudaLaunchKernelEx(&cfg, select_kernel<void, true>, (const float*)s_buf, T, batch->cu_seqlens, cu_kept,
+                               keep, window, k_tot, n_kv_heads, idx_out, stage_keys, ga, Stream{}));
   else
-    PK_CUDA(cudaLaunchKernelEx(&cfg, select_kernel<false>, (const float*)s_buf, T, batch->cu_seqlens, cu_kept,
-                               keep, window, k_tot, n_kv_heads, idx_out, stage_keys, ga));
+    PK_CUDA(cudaLaunchKernelEx(&cfg, select_kernel<void, false>, (const float*)s_buf, T, batch->cu_seqlens, cu_kept,
+                               keep, window, k_tot, n_kv_heads, idx_out, stage_keys, ga, Stream{}));
   PK_CUDA(cudaGetLastError());
   return PUREKV_OK;
 }
