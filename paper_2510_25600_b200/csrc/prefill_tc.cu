@@ -45,28 +45,26 @@ constexpr int kUnitRing = 4;  // units in flight between the producer's publicat
 template <int BK>
 struct Cfg {
   static constexpr int kStages = 2;                 // K/V ring depth (64 KB per stage)
-  static constexpr int kSBuf = 128 / BK;            // S buffers per slot: kSBuf * BK = 128 TMEM columns
   static constexpr int kMeta = 2 * kStages;         // ring of per-tile class words and bit masks
   static constexpr uint32_t kMaskBytes = kBQ * BK / 8;
 };
 
 template <int BK>
 struct __align__(8) Barriers {
-  static constexpr int ST = Cfg<BK>::kStages, SB = Cfg<BK>::kSBuf, MR = Cfg<BK>::kMeta;
+  static constexpr int ST = Cfg<BK>::kStages, MR = Cfg<BK>::kMeta;
   uint64_t q_full, q_empty;
   uint64_t k_full[ST], k_empty[ST], v_full[ST], v_empty[ST];
   uint64_t m_full[MR];     // producer -> softmax: class word (and bit mask) of a tile are in place
-  uint64_t s_full[2][SB];  // MMA -> softmax: S of (slot, buffer) is complete
+  uint64_t s_full[2];      // MMA -> softmax: S of the slot is complete
   uint64_t p_part[2];      // softmax -> MMA: P of the first 96 keys written (and O rescaled) by the slot's four row warps
-  uint64_t p_full[2][SB];  // softmax -> MMA: all of P written
-  uint64_t o_done[2];      // one completion per P.V product of the slot
+  uint64_t p_full[2];      // softmax -> MMA: all of P written
   uint64_t o_final[2];     // one completion per unit, after the slot's last P.V product
   uint64_t u_full[kUnitRing];   // the producer published a unit (or the end mark) in unit_s[]
   uint64_t u_empty[kUnitRing];  // the MMA thread and the eight softmax warps have copied it
   uint64_t drain;
 };
 
-// TMEM columns: S(slot, buf) at slot*128 + buf*BK (P aliases its first BK/2 columns), O(slot) at 256 + slot*128.
+// TMEM columns: S(slot) at slot*128 (P aliases its first BK/2 columns), O(slot) at 256 + slot*128.
 template <int BK>
 __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
     const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
@@ -74,7 +72,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
     const __grid_constant__ CUtensorMap tm_v64, __nv_bfloat16* __restrict__ o, float* __restrict__ lse,
     uint8_t* __restrict__ plan, float* __restrict__ ws, int32_t n_q_heads, int32_t n_kv_heads, float scale_log2,
     int32_t* __restrict__ status, uint64_t wait_ns, int64_t plan_bytes, int64_t ws_floats) {
-  constexpr int ST = Cfg<BK>::kStages, SB = Cfg<BK>::kSBuf, MR = Cfg<BK>::kMeta;
+  constexpr int ST = Cfg<BK>::kStages, MR = Cfg<BK>::kMeta;
   constexpr uint32_t kPanelQ = kBQ * 128;  // bytes of one 64-column panel of a Q tile
   constexpr uint32_t kTileQ = 2 * kPanelQ;
   constexpr uint32_t kPanelKV = BK * 128;  // bytes of one 64-column panel of a K or V tile
@@ -111,12 +109,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
     }
     for (int s = 0; s < MR; ++s) mbar_init(smem_u32(&bars.m_full[s]), 1);
     for (int sl = 0; sl < 2; ++sl) {
-      for (int b = 0; b < SB; ++b) {
-        mbar_init(smem_u32(&bars.s_full[sl][b]), 1);
-        mbar_init(smem_u32(&bars.p_full[sl][b]), 4);
-      }
+      mbar_init(smem_u32(&bars.s_full[sl]), 1);
+      mbar_init(smem_u32(&bars.p_full[sl]), 4);
       mbar_init(smem_u32(&bars.p_part[sl]), 4);
-      mbar_init(smem_u32(&bars.o_done[sl]), 1);
       mbar_init(smem_u32(&bars.o_final[sl]), 1);
     }
     for (int s = 0; s < kUnitRing; ++s) {
@@ -381,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       constexpr uint32_t idesc_qk = instr_desc(BK, false);
       constexpr uint32_t idesc_qk_half = instr_desc(BK / 2, false);
       constexpr uint32_t idesc_pv = instr_desc(kD, true);
-      static_assert(SB == 1 && ST == 2, "S of a tile is issued behind P V of the tile before, which frees its columns");
+      static_assert(BK == 128 && ST == 2, "S of a tile is issued behind P V of the tile before, which frees its columns");
       uint32_t it = 0;          // the CTA's key tiles so far
       uint32_t tp0 = 0, tp1 = 0;  // ... and those of each slot, P V issued
       // Descriptor words.  High word: stride between 8-row groups 1024 B, descriptor version 1, 128-byte swizzle.
@@ -413,7 +408,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
             mma_ss_lh(d_addr, q_lo + (ks >> 2) * (kPanelQ >> 4) + (ks & 3) * 2, kDescHi,
                       k_lo + (ks >> 2) * (kPanelKV >> 4) + (ks & 3) * 2, kDescHi, idesc_qk_half, ks > 0 ? 1u : 0u);
         }
-        tc_commit(smem_u32(&bars.s_full[sl][0]));
+        tc_commit(smem_u32(&bars.s_full[sl]));
       };
       // O(slot) += P V of a tile: the part that waits for the first 96 keys' P ...
       auto issue_pv_head = [&](auto sl_c, uint32_t s, uint32_t hm, uint32_t par, uint32_t acc0) -> bool {
@@ -433,7 +428,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       auto issue_pv_tail = [&](auto sl_c, uint32_t s, uint32_t hm, uint32_t par, uint32_t acc0) -> bool {
         constexpr int sl = decltype(sl_c)::value;
         const uint32_t p_addr = tmem + sl * 128, o_addr = tmem + kColO + sl * 128, v_lo = v_lo0 + s * (kTileKV >> 4);
-        if (!mbar_wait(smem_u32(&bars.p_full[sl][0]), par, abort_flag, wait_ns)) return false;
+        if (!mbar_wait(smem_u32(&bars.p_full[sl]), par, abort_flag, wait_ns)) return false;
         tc_fence_after();
         if (hm == 3u) {
 #pragma unroll
@@ -554,7 +549,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       const int32_t i_rel = (second ? u.q_start1 : u.q_start) - u.req_start + row;
       float m_ref = 0.f, l_sum = 0.f;
       for (int32_t n = 0; n < nt; ++n) {
-        const uint32_t it = it_base + (uint32_t)n, ms = it % MR, b = t % SB;
+        const uint32_t it = it_base + (uint32_t)n, ms = it % MR;
         if (!wait_w(smem_u32(&bars.m_full[ms]), (it / MR) & 1u)) { ok = false; break; }
         const int2 e = meta_s[ms][sl];
         const int32_t cls = e.x & 3, j0 = (e.x >> 4) * BK;
@@ -584,9 +579,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
           for (int c = 0; c < BK / 32; ++c)
             if (!((hm_own >> (c >> 1)) & 1u)) keep[c] = 0u;
         }
-        if (!wait_w(smem_u32(&bars.s_full[sl][b]), (t / SB) & 1u)) { ok = false; break; }
+        if (!wait_w(smem_u32(&bars.s_full[sl]), t & 1u)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t s_addr = t_lane + sl * 128 + b * BK;
+        const uint32_t s_addr = t_lane + sl * 128;
         // Fast path: exponentials against the row's standing reference m_ref, no maximum taken.  Softmax does not depend
         // on the reference, and fp32 / bf16 carry 8 exponent bits, so the reference (0 at the start of a unit) only has
         // to keep exp2 in range: it moves when a tile overflows, or when everything kept so far has underflowed; those
@@ -601,7 +596,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
           tc_fence_before();
           __syncwarp();
         };
-        const uint32_t part_bar = smem_u32(&bars.p_part[sl]), full_bar = smem_u32(&bars.p_full[sl][b]);
+        const uint32_t part_bar = smem_u32(&bars.p_part[sl]), full_bar = smem_u32(&bars.p_full[sl]);
         bool exact = false;
         {
           float2 ls2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -703,9 +698,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
           const float alpha = l_sum > 0.f ? ex2(m_ref - m_new) : 1.f;  // with l_sum == 0 every earlier P was 0, so O is 0
           const float m_sub = m_new;
           if (n > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
-            // O must be quiescent: with one S buffer, S of tile n was issued behind P.V of tile n-1, so it is;
-            // with two, S of tile n only implies P.V of tile n-2 (o_done is then in phase t-1 or t).
-            if (SB > 1 && !wait_w(smem_u32(&bars.o_done[sl]), (t - 1u) & 1u)) { ok = false; break; }
+            // O is quiescent: S of tile n was issued behind P V of tile n-1, and it is complete.
             tc_fence_after();
 #pragma unroll
             for (int c = 0; c < kD / 32; ++c) {
@@ -750,7 +743,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       }
       if (!ok) break;
       it_base += (uint32_t)nt;
-      // o_done may be two phases behind here, which a parity wait cannot tell apart; o_final moves once per unit.
+      // (one completion per unit, behind the slot's last P V)
       if (!wait_w(smem_u32(&bars.o_final[sl]), slot_units & 1u)) { ok = false; break; }
       ++slot_units;
       tc_fence_after();
