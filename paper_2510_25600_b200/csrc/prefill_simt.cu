@@ -46,6 +46,71 @@ struct SimtCfg {
   }
 };
 
+__device__ __forceinline__ void simt_store1(float* p, float x) { *p = x; }
+__device__ __forceinline__ void simt_store1(__nv_bfloat16* p, float x) { *p = __float2bfloat16_rn(x); }
+
+// One row by one warp, straight from the plan's list and global memory: a row takes nothing from a key tile of which it keeps
+// nothing, whatever stands there.  (The kernel below multiplies every V of a chunk of several tiles by the row's weights, zeros
+// where the row keeps nothing; an infinity or a NaN there survives that, and such rows come here.)  `tile`: the query tile's place
+// in the plan's order, `row`: the row in it, `q`: its query in shared memory.
+template <typename T, int D>
+__device__ __noinline__ void prefill_simt_row(const float* q, const T* k, const T* v, T* o, float* lse, const uint8_t* plan, int32_t tile,
+                                              int32_t row, int32_t n_q_heads, int32_t n_kv_heads, float scale_log2) {
+  const PlanHeader* hdr = reinterpret_cast<const PlanHeader*>(plan);
+  const int32_t tk = hdr->tile_k, wpr = hdr->words_per_row, hq = blockIdx.y, g = hq / (n_q_heads / n_kv_heads);
+  const QTile qt = reinterpret_cast<const QTile*>(plan + hdr->off_qtiles)[reinterpret_cast<const int32_t*>(plan + hdr->off_order)[tile]];
+  const int2* entries = reinterpret_cast<const int2*>(plan + hdr->off_entries) + qt.entry_begin;
+  const uint32_t* masks = reinterpret_cast<const uint32_t*>(plan + hdr->off_masks);
+  const int lane = threadIdx.x & 31;
+  const int32_t i = qt.q_start - qt.req_start + row;
+  float m = -INFINITY, l = 0.f, acc[D / 32];
+  for (int c = 0; c < D / 32; ++c) acc[c] = 0.f;
+  for (int32_t e = 0; e < qt.entry_count; ++e) {
+    const int2 ent = entries[e];
+    const int32_t cls = ent.x & 3, j0 = (ent.x >> 4) * tk;
+    float s[4], tmax = -INFINITY;  // (tk <= 128: at most four keys per lane)
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const int32_t c = lane + 32 * x, j = j0 + c;
+      s[x] = -INFINITY;
+      if (c < tk && j < qt.req_len) {
+        const bool keep = cls == kTileGeneral ? (masks[ent.y + row * wpr + (c >> 5)] >> (c & 31)) & 1u : cls == kTileFull || j <= i;
+        if (keep) {
+          const T* kr = k + ((int64_t)(qt.req_start + j) * n_kv_heads + g) * D;
+          float a = 0.f;
+          for (int dd = 0; dd < D; ++dd) a = fmaf(q[dd], to_f32(kr[dd]), a);
+          s[x] = a * scale_log2;
+        }
+      }
+      tmax = fmaxf(tmax, s[x]);
+    }
+    for (int off = 16; off >= 1; off >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, off));
+    if (tmax == -INFINITY) continue;
+    const float mn = fmaxf(m, tmax), alpha = exp2f(m - mn);
+    float sum = 0.f;
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      s[x] = exp2f(s[x] - mn);
+      sum += s[x];
+    }
+    for (int off = 16; off >= 1; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+    l = l * alpha + sum;
+    m = mn;
+    for (int c = 0; c < D / 32; ++c) acc[c] *= alpha;
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+      for (int c = 32 * x; c < min(tk, 32 * x + 32) && j0 + c < qt.req_len; ++c) {
+        const float p = __shfl_sync(0xffffffffu, s[x], c & 31);
+        const T* vr = v + ((int64_t)(qt.req_start + j0 + c) * n_kv_heads + g) * D + lane;
+        for (int dd = 0; dd < D / 32; ++dd) acc[dd] = fmaf(p, to_f32(vr[32 * dd]), acc[dd]);
+      }
+  }
+  const float inv = 1.f / l;
+  const int64_t token = qt.q_start + row;
+  for (int c = 0; c < D / 32; ++c) simt_store1(o + (token * n_q_heads + hq) * D + lane + 32 * c, acc[c] * inv);
+  if (lse && lane == 0) lse[(int64_t)hq * hdr->total_tokens + token] = (m + log2f(l)) * 0.6931471805599453f;
+}
+
 template <typename T, int D, int NK, int TPR, int RPT>
 __global__ void __launch_bounds__(kSimtThreads) prefill_simt_kernel(
     const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, T* __restrict__ o,
@@ -58,6 +123,7 @@ __global__ void __launch_bounds__(kSimtThreads) prefill_simt_kernel(
   constexpr int CPR = D * (int)sizeof(T) / 16;  // 16-byte copies per row
   extern __shared__ __align__(16) uint8_t smem_raw[];
   __shared__ SimtSeg segs[3][kSegs];
+  __shared__ uint32_t redo[2];  // rows with a value that is not finite
   T* kv = reinterpret_cast<T*>(smem_raw);                      // [2 stages][K, V][NK][LD]
   float* qs = reinterpret_cast<float*>(kv + 2 * 2 * NK * LD);  // [R][LDQ]
   float* ps = qs + R * LDQ;                                    // [R][LDP]
@@ -105,6 +171,7 @@ __global__ void __launch_bounds__(kSimtThreads) prefill_simt_kernel(
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
 
+  if (tid < 2) redo[tid] = 0u;
   if (tid < spc) {
     segs[0][tid] = seg_of(0);
     segs[1][tid] = seg_of(1);
@@ -225,20 +292,31 @@ __global__ void __launch_bounds__(kSimtThreads) prefill_simt_kernel(
     if (tid < spc) segs[(ch + 2) % 3][tid] = ahead;
     __syncthreads();  // the stage may be overwritten, and the runs after the next are known
   }
+  bool any = false;
 #pragma unroll
   for (int rr = 0; rr < RPT; ++rr) {
     const int32_t row = grp + kGroups * rr;
     if (row0 + row >= qt.q_rows) continue;
     const float inv = 1.f / l[rr];
     T* dst = o + ((int64_t)(qt.q_start + row0 + row) * n_q_heads + hq) * D + 4 * kx;
+    float zero = 0.f;  // 0 unless a value is infinite or NaN
 #pragma unroll
     for (int nd = 0; nd < ND; ++nd) {
-      const float4 a = acc[rr][nd];
-      simt_store4(dst + 4 * TPR * nd, make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv));
+      const float4 a = make_float4(acc[rr][nd].x * inv, acc[rr][nd].y * inv, acc[rr][nd].z * inv, acc[rr][nd].w * inv);
+      simt_store4(dst + 4 * TPR * nd, a);
+      zero = fmaf(a.x, 0.f, zero); zero = fmaf(a.y, 0.f, zero); zero = fmaf(a.z, 0.f, zero); zero = fmaf(a.w, 0.f, zero);
     }
     if (lse && kx == 0)
       lse[(int64_t)hq * hdr->total_tokens + qt.q_start + row0 + row] = (m[rr] + log2f(l[rr])) * 0.6931471805599453f;
+    if (zero != 0.f) {
+      any = true;
+      atomicOr(&redo[row >> 5], 1u << (row & 31));
+    }
   }
+  if (!__syncthreads_or(any)) return;
+  for (int32_t row = tid >> 5; row < R; row += kSimtThreads / 32)
+    if ((redo[row >> 5] >> (row & 31)) & 1u)
+      prefill_simt_row<T, D>(qs + row * LDQ, k, v, o, lse, plan, blockIdx.x / n_sub, row0 + row, n_q_heads, n_kv_heads, scale_log2);
 }
 
 template <typename T, int D, int TPR, int RPT>
