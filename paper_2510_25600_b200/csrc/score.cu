@@ -833,9 +833,13 @@ __global__ void __launch_bounds__(kThreads, 1) score_cluster_f32_kernel(
 #pragma unroll
       for (int off = 8; off >= 1; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
       float l = 0.f;
-      if (mx > -INFINITY)
+      if (mx > -INFINITY) {
 #pragma unroll
         for (int b = 0; b < 4; ++b) l += exp2f(s[a][b] - mx);
+      } else {  // nothing seen, or NaN logits alone, which the maximum has passed over: the row's sum is NaN then
+#pragma unroll
+        for (int b = 0; b < 4; ++b) l += s[a][b] != -INFINITY ? s[a][b] : 0.f;
+      }
 #pragma unroll
       for (int off = 8; off >= 1; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
       // lane tx of the row's sixteen threads serves CTA tx of the cluster
@@ -855,7 +859,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_cluster_f32_kernel(
       float mx = p.x;
 #pragma unroll
       for (int off = 8; off >= 1; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-      float l = p.y > 0.f ? p.y * exp2f(p.x - mx) : 0.f;
+      float l = p.y != 0.f ? p.y * exp2f(p.x - mx) : 0.f;
 #pragma unroll
       for (int off = 8; off >= 1; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
       const float lse = row0 + rl < n_rows ? mx + log2f(l) : INFINITY;  // (+inf: an absent row adds nothing)
