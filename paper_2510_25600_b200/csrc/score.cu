@@ -10,6 +10,7 @@
 // Logits are fp32 FMA chains over exact products; exponentials use exp2f.
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "cluster.cuh"
 #include "common.cuh"
@@ -653,6 +654,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) score_cluster_kernel(
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     // the rows' log-sum-exp: two threads per row, each over every other CTA.  (The pairs of this parity are overwritten two
     // blocks of rows later, behind the next block's barrier, which everybody reaches after this read.)
+    bool odd;  // a row of NaN logits (passed over by the maxima: -inf) or with a NaN sum
     {
       const int32_t rl = tid >> 1;
       float mx = -INFINITY;
@@ -664,22 +666,31 @@ __global__ void __launch_bounds__(kMmaThreads, 1) score_cluster_kernel(
         if (p.y > 0.f) l += p.y * exp2f(p.x - mx);
       }
       l += __shfl_xor_sync(0xffffffffu, l, 1);
-      if ((tid & 1) == 0) sh.lse[rl] = row0 + rl < n_rows ? mx + log2f(l) : INFINITY;  // (+inf: an absent row adds nothing)
+      const float lse = row0 + rl < n_rows ? mx + log2f(l) : INFINITY;  // (+inf: an absent row adds nothing)
+      if ((tid & 1) == 0) sh.lse[rl] = lse;
+      odd = !(lse > -INFINITY);
     }
-    __syncthreads();
+    const bool any_odd = __syncthreads_or(odd);
+    auto add = [&](auto check_c) {
 #pragma unroll
-    for (int mb = 0; mb < 2; ++mb)
+      for (int mb = 0; mb < 2; ++mb)
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float lse = sh.lse[32 * wr + 16 * mb + (lane >> 2) + 8 * h];
+        for (int h = 0; h < 2; ++h) {
+          const float lse = sh.lse[32 * wr + 16 * mb + (lane >> 2) + 8 * h];
 #pragma unroll
-        for (int m = 0; m < MB; ++m)
+          for (int m = 0; m < MB; ++m)
 #pragma unroll
-          for (int nb = 0; nb < 8; ++nb) {  // keys the row does not see are -inf and add nothing
-            col[m][nb][0] += exp2f(acc[m][mb][nb][2 * h] - lse);
-            col[m][nb][1] += exp2f(acc[m][mb][nb][2 * h + 1] - lse);
-          }
-      }
+            for (int nb = 0; nb < 8; ++nb)
+#pragma unroll
+              for (int x = 0; x < 2; ++x) {
+                const float sv = acc[m][mb][nb][2 * h + x];
+                // keys the row does not see are -inf and add nothing, also where the row's sum is NaN
+                if (!decltype(check_c)::value || sv != -INFINITY) col[m][nb][x] += exp2f(sv - lse);
+              }
+        }
+    };
+    if (any_odd) add(std::true_type{});
+    else add(std::false_type{});
   }
   // sum over the 8 row groups of the warp (lanes with equal lane % 4 hold the same columns), then over the 4 row warps
 #pragma unroll
@@ -863,8 +874,13 @@ __global__ void __launch_bounds__(kThreads, 1) score_cluster_f32_kernel(
 #pragma unroll
       for (int off = 8; off >= 1; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
       const float lse = row0 + rl < n_rows ? mx + log2f(l) : INFINITY;  // (+inf: an absent row adds nothing)
+      if (__any_sync(0xffffffffu, !(lse > -INFINITY))) {  // a row with a NaN sum: its NaN goes to the keys it sees alone
 #pragma unroll
-      for (int b = 0; b < 4; ++b) col[b] += exp2f(s[a][b] - lse);
+        for (int b = 0; b < 4; ++b) col[b] += s[a][b] == -INFINITY ? 0.f : exp2f(s[a][b] - lse);
+      } else {
+#pragma unroll
+        for (int b = 0; b < 4; ++b) col[b] += exp2f(s[a][b] - lse);
+      }
     }
   }
 #pragma unroll

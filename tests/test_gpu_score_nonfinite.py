@@ -28,3 +28,15 @@ def test_a_nan_key_reaches_all_scores_of_its_head(length, at):
     assert torch.equal(got[0], base[0])
     # the last key is seen by the last row alone, which is enough
     assert got[1, :length - 16].isnan().all() and (got[1, length - 16:] == 0).all()
+
+
+@pytest.mark.parametrize("dtype,d,length,row,pool", [("fp32", 64, 300, 40, 1), ("fp32", 64, 500, 70, 5), ("bf16", 64, 500, 200, 1),
+                                                     ("bf16", 128, 900, 300, 7)])
+def test_a_nan_row_reaches_the_keys_it_sees(dtype, d, length, row, pool):
+    def spoil(q, k):
+        q[row, 1, 2] = float("nan")
+
+    base, got = _scores(dtype, d, length, 16, -1, pool), _scores(dtype, d, length, 16, -1, pool, spoil)
+    assert torch.equal(got[1], base[1])  # heads 2 and 3
+    reach = row + 1 + pool // 2
+    assert got[0, :reach].isnan().all() and torch.equal(got[0, reach:], base[0, reach:])
