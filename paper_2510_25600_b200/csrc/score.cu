@@ -576,6 +576,11 @@ __global__ void __launch_bounds__(kMmaThreads, 1) score_cluster_kernel(
   const int32_t base = cu_seqlens[r], len = cu_seqlens[r + 1] - base;
   const int32_t w = min(window, len), nr = len - w, wo = min(obs, len), n_rows = G * wo;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wr = warp >> 1, wc = warp & 1;
+  if (nr == 0) {  // (the same for all CTAs of the cluster) a request within its window: no key has a score
+    for (int32_t j = j0 + tid; j < min(len, j0 + kKeys); j += kMmaThreads) c_out[(int64_t)g * n_tokens + base + j] = 0.f;
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    return;
+  }
   auto q_row = [&](int32_t row) -> int64_t {
     return row < n_rows ? ((int64_t)(base + len - wo + row % wo) * n_q_heads + g * G + row / wo) * d : -1;
   };
@@ -754,20 +759,75 @@ static purekv_status allow_wide_clusters(void (*kernel)(Params...), std::atomic<
   return PUREKV_OK;
 }
 
+// Requests with a key outside their window: each is a cluster's work per KV head, the others are none.
+static int64_t live_requests(const purekv_batch* b, int32_t window) {
+  int64_t n = 0;
+  for (int r = 0; r < b->n_req; ++r) n += b->h_cu_seqlens[r + 1] - b->h_cu_seqlens[r] > window;
+  return n;
+}
+
+// Which form the scores take is decided by what each would take, in us, from times measured over 1-128 requests of 100-4200
+// tokens, 1-8 query heads per KV head and 8-400 rows (d = 128); the estimates are within a fifth of them.  A cluster of C CTAs
+// keeps C SMs through all its blocks of rows, whatever the request's length, and few of the large ones fit at once (7 of 16 CTAs,
+// 15 of 8), so clusters run in waves: 6.4 us per block of rows and 2.5 more with 128 keys per CTA, 9.3 and 3 with 256.  The
+// separate kernels take 9.4 us per block with up to one CTA per SM, 13.5 with two and so on, and 18 for three launches.
+// In one wave the cluster is always the faster (1 x 2048, 28 / 4 heads, 64 rows: 31 against 54); in several it has to be so by a
+// tenth.  (1 x 2048, 32 / 8 heads, 100 rows: 40 as 8 clusters of 8 against 51 and, as 8 of 16, 59; 2000 + 100 + 50 tokens, 64 rows:
+// 42 against 43 and 62; 4 x 2432, 100 rows: 120 against 158; 4000 + 3 x 300, 16 rows: 58 against 46.)
+static double cluster_us(int32_t keys_per_cta, int64_t live_clusters, int32_t at_once, int32_t row_blocks, double* waves) {
+  *waves = (double)std::max<int64_t>(1, (live_clusters + at_once - 1) / at_once);
+  return live_clusters == 0 ? 3. : *waves * (keys_per_cta == kCtaKeys ? 2.5 + 6.4 * row_blocks : 3. + 9.3 * row_blocks);
+}
+static double separate_us(const purekv_batch* b, int32_t window, int32_t Hkv, int32_t row_blocks) {
+  int64_t all = 0, scored = 0;  // key blocks of the first pass, and of the second
+  for (int r = 0; r < b->n_req; ++r) {
+    const int32_t len = b->h_cu_seqlens[r + 1] - b->h_cu_seqlens[r];
+    all += (len + kCtaKeys - 1) / kCtaKeys;
+    scored += (std::max(0, len - window) + kCtaKeys - 1) / kCtaKeys;
+  }
+  const double per_sm = 0.5 * (double)((all + scored) * Hkv) / 148.;
+  return 18. + 4. * per_sm + row_blocks * (per_sm > 2. ? 6.5 * per_sm + 3. : per_sm > 1. ? 13.5 : 9.4);
+}
+
+// One form of the cluster kernel for a call: its launch, and what it would take (infinity where it cannot run).
 template <int MB>
+struct ScoreCluster {
+  int32_t C;
+  ClusterLaunch l;
+  double us = INFINITY, waves = 0.;
+  ScoreCluster(const purekv_batch* b, int32_t Hkv, int32_t d, cudaStream_t sm)
+      : C(std::max(1, (max_len(b) + MB * kCtaKeys - 1) / (MB * kCtaKeys))),
+        l(C, Hkv, b->n_req, kMmaThreads, (size_t)(MB * kCtaKeys + 2 * kMmaRows) * (d + 8) * sizeof(__nv_bfloat16), sm) {}
+  purekv_status weigh(int64_t live_clusters, int32_t row_blocks) {
+    static std::atomic<uint64_t> smem_allowed{0}, wide_allowed{0};
+    if (C > kClusterMax) return PUREKV_OK;
+    const purekv_status st = allow_wide_clusters(score_cluster_kernel<MB>, smem_allowed, wide_allowed);
+    if (st != PUREKV_OK) return st;
+    const int32_t at_once = clusters_at_once(score_cluster_kernel<MB>, l.cfg);
+    if (at_once >= 1) us = cluster_us(MB * kCtaKeys, live_clusters, at_once, row_blocks, &waves);
+    return PUREKV_OK;
+  }
+};
+
+// The bf16 scores in one cluster launch, if that is the form to take (*launched).
 static purekv_status launch_score_cluster(const void* q, const void* k, float* c_out, const purekv_batch* b, int32_t window,
                                           int32_t obs, int32_t pool, int32_t H, int32_t Hkv, int32_t d, float scale,
                                           cudaStream_t sm, bool* launched) {
-  auto kernel = score_cluster_kernel<MB>;
-  static std::atomic<uint64_t> smem_allowed{0}, wide_allowed{0};
-  const purekv_status st = allow_wide_clusters(kernel, smem_allowed, wide_allowed);
+  const int32_t row_blocks = ((H / Hkv) * obs + kMmaRows - 1) / kMmaRows;
+  const int64_t live = live_requests(b, window) * Hkv;
+  ScoreCluster<1> one(b, Hkv, d, sm);
+  ScoreCluster<2> two(b, Hkv, d, sm);
+  purekv_status st = one.weigh(live, row_blocks);
+  if (st == PUREKV_OK) st = two.weigh(live, row_blocks);
   if (st != PUREKV_OK) return st;
-  const int32_t C = std::max(1, (max_len(b) + MB * kCtaKeys - 1) / (MB * kCtaKeys));
-  ClusterLaunch l(C, Hkv, b->n_req, kMmaThreads, (size_t)(MB * kCtaKeys + 2 * kMmaRows) * (d + 8) * sizeof(__nv_bfloat16), sm);
-  *launched = clusters_at_once(kernel, l.cfg) >= 1;
+  const bool small = one.us <= two.us;
+  const double us = small ? one.us : two.us, waves = small ? one.waves : two.waves;
+  *launched = us < INFINITY && (waves <= 1. || us <= 0.9 * separate_us(b, window, Hkv, row_blocks));
   if (!*launched) return PUREKV_OK;
-  PK_CUDA(cudaLaunchKernelEx(&l.cfg, kernel, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, b->cu_seqlens, window, obs, pool, H, Hkv,
-                             d, scale * 1.4426950408889634f, b->total_tokens, c_out));
+  const float scale_log2 = scale * 1.4426950408889634f;
+  const auto *qb = (const __nv_bfloat16*)q, *kb = (const __nv_bfloat16*)k;
+  if (small) PK_CUDA(cudaLaunchKernelEx(&one.l.cfg, score_cluster_kernel<1>, qb, kb, b->cu_seqlens, window, obs, pool, H, Hkv, d, scale_log2, b->total_tokens, c_out));
+  else PK_CUDA(cudaLaunchKernelEx(&two.l.cfg, score_cluster_kernel<2>, qb, kb, b->cu_seqlens, window, obs, pool, H, Hkv, d, scale_log2, b->total_tokens, c_out));
   return PUREKV_OK;
 }
 
@@ -812,6 +872,11 @@ __global__ void __launch_bounds__(kThreads, 1) score_cluster_f32_kernel(
   const int32_t base = cu_seqlens[r], len = cu_seqlens[r + 1] - base;
   const int32_t w = min(window, len), nr = len - w, wo = min(obs, len), n_rows = G * wo;
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  if (nr == 0) {  // (the same for all CTAs of the cluster) a request within its window: no key has a score
+    for (int32_t j = j0 + tid; j < min(len, j0 + kKB); j += kThreads) c_out[(int64_t)g * n_tokens + base + j] = 0.f;
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    return;
+  }
   auto q_row = [&](int32_t row) -> int64_t {
     return row < n_rows ? ((int64_t)(base + len - wo + row % wo) * n_q_heads + g * G + row / wo) * d : -1;
   };
@@ -901,15 +966,42 @@ __global__ void __launch_bounds__(kThreads, 1) score_cluster_f32_kernel(
   pool_in_cluster<kKB>(sh.colbuf, sh.halo, half, rank, C, j0, nr, len, cg);
 }
 
+// The same choice for fp32, in us as measured over 1-64 requests of 100-1024 tokens, d = 64-256.  The cluster: a block of 32 rows
+// 3.4-4.3 us (d = 64), more where clusters share SMs.  The separate kernels: one CTA walks all key blocks in the first pass and all
+// row blocks in the second, 2.4 us (d = 64) a step, more where CTAs queue.  (288 tokens, 16 rows: 5.6 in a cluster, 25 separately;
+// 64 x 300, 256 rows: 416 and 293; 8 x 1024, 8 / 2 heads, 64 rows: 101 and 86.)
+static double cluster_f32_us(int32_t C, int32_t d, int64_t live_clusters, int32_t at_once, int32_t row_blocks) {
+  auto wave = [&](int64_t clusters) {
+    const double per_sm = (double)clusters * C / 148.;
+    return 2. + row_blocks * (1.65 + 0.0262 * d + 0.055 * C) * (per_sm > 1. ? 1. + 0.8 * (per_sm - 1.) : 1.);
+  };
+  const int64_t last = live_clusters % at_once;
+  return (double)(live_clusters / at_once) * wave(at_once) + (last ? wave(last) : 0.);
+}
+static double separate_f32_us(const purekv_batch* b, int32_t window, int32_t obs, int32_t H, int32_t Hkv, int32_t d, int32_t row_blocks) {
+  int64_t rows = 0, keys = 0, scored = 0;  // CTAs of the first pass; of the second, and those that have work
+  for (int r = 0; r < b->n_req; ++r) {
+    const int32_t len = b->h_cu_seqlens[r + 1] - b->h_cu_seqlens[r];
+    rows += ((int64_t)(H / Hkv) * std::min(obs, len) + kRB - 1) / kRB;
+    keys += (len + kKB - 1) / kKB;
+    scored += (std::max(0, len - window) + kKB - 1) / kKB;
+  }
+  const double queue1 = std::max(1., 0.8 * (double)(rows * Hkv) / 148.), queue2 = std::max(1., 0.8 * (double)(scored * Hkv) / 148.);
+  const double steps = (double)((max_len(b) + kKB - 1) / kKB) * queue1 + 1.12 * row_blocks * queue2;
+  return 9. + (0.4 + 0.031 * d) * steps + 0.8 * (double)((rows + keys) * Hkv) / 148.;
+}
+
 static purekv_status launch_score_cluster_f32(const float* q, const float* k, float* c_out, const purekv_batch* b,
                                               int32_t window, int32_t obs, int32_t pool, int32_t H, int32_t Hkv, int32_t d,
                                               float scale, cudaStream_t sm, bool* launched) {
   static std::atomic<uint64_t> smem_allowed{0}, wide_allowed{0};
   const purekv_status st = allow_wide_clusters(score_cluster_f32_kernel, smem_allowed, wide_allowed);
   if (st != PUREKV_OK) return st;
-  const int32_t C = std::max(1, (max_len(b) + kKB - 1) / kKB);
+  const int32_t C = std::max(1, (max_len(b) + kKB - 1) / kKB), row_blocks = ((H / Hkv) * obs + kRB - 1) / kRB;
   ClusterLaunch l(C, Hkv, b->n_req, kThreads, (size_t)(kKB + 2 * kRB) * (d + 4) * sizeof(float), sm);
-  *launched = clusters_at_once(score_cluster_f32_kernel, l.cfg) >= 1;
+  const int32_t at_once = clusters_at_once(score_cluster_f32_kernel, l.cfg);
+  *launched = at_once >= 1 && cluster_f32_us(C, d, live_requests(b, window) * Hkv, at_once, row_blocks) <=
+                                  separate_f32_us(b, window, obs, H, Hkv, d, row_blocks);
   if (!*launched) return PUREKV_OK;
   PK_CUDA(cudaLaunchKernelEx(&l.cfg, score_cluster_f32_kernel, q, k, b->cu_seqlens, window, obs, pool, H, Hkv, d,
                              scale * 1.4426950408889634f, b->total_tokens, c_out));
@@ -1054,19 +1146,13 @@ static purekv_status score_impl(const char* who, const void* q, const void* k, f
   float* c_raw = pool > 1 ? lse2 + score_ws_floats(batch, obs, n_q_heads) : c_out;  // scores before pooling
   const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)head_dim);
   cudaStream_t sm = (cudaStream_t)stream;
-  // One launch when a cluster holds the longest request (and the accumulated rows are not the whole of a long one: every
-  // block of rows costs a cluster barrier, and rows before a CTA's keys are multiplied for nothing).
+  // One launch when a cluster holds the longest request and the accumulated rows are not the whole of a long one (every block
+  // of rows costs a cluster barrier, and rows before a CTA's keys are multiplied for nothing), and that is the faster form.
   const int32_t ml = max_len(batch), row_blocks = ((n_q_heads / n_kv_heads) * obs + kMmaRows - 1) / kMmaRows;
-  // With more CTAs than SMs (one fits an SM) a single block or two of rows is still faster this way (4 requests of 2432
-  // tokens, 32 rows: 42 against 72 us), more are not: nothing runs beside a CTA that waits at a barrier (8 requests, 100-row
-  // window, 6 blocks: 180 against 170 us).
-  const int64_t ctas = (int64_t)batch->n_req * n_kv_heads * ((ml + 2 * kCtaKeys - 1) / (2 * kCtaKeys)) * (ml <= kClusterMax * kCtaKeys ? 2 : 1);
   bool launched = false;
   if (dtype == PUREKV_BF16 && head_dim % 16 == 0 && head_dim <= 128 && ml <= kClusterMax * 2 * kCtaKeys &&
-      row_blocks <= kClusterRowBlocks && pool / 2 <= kPoolHalfMax && (ctas <= 148 || row_blocks <= 2))
-    st = ml <= kClusterMax * kCtaKeys
-             ? launch_score_cluster<1>(q, k, c_out, batch, window, obs, pool, n_q_heads, n_kv_heads, head_dim, scale, sm, &launched)
-             : launch_score_cluster<2>(q, k, c_out, batch, window, obs, pool, n_q_heads, n_kv_heads, head_dim, scale, sm, &launched);
+      row_blocks <= kClusterRowBlocks && pool / 2 <= kPoolHalfMax)
+    st = launch_score_cluster(q, k, c_out, batch, window, obs, pool, n_q_heads, n_kv_heads, head_dim, scale, sm, &launched);
   if (dtype == PUREKV_FP32 && ml <= kClusterMax * kKB && row_blocks <= kClusterRowBlocks && pool / 2 <= kKB / 2 &&
       ((uintptr_t)q | (uintptr_t)k) % 16 == 0)
     st = launch_score_cluster_f32((const float*)q, (const float*)k, c_out, batch, window, obs, pool, n_q_heads, n_kv_heads,
