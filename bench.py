@@ -11,7 +11,8 @@ whole-pipeline one, Qwen2.5-VL-7B-shaped (28 layers, 28/4 heads, head_dim 128, 8
 Prints ONE JSON line (rank 0).  `value` = prefill tokens/s of the whole job with inputs
 resident in HBM; `e2e` = the same with inputs in pinned host memory and the compact cache read
 back; `roofline` describes the dominant kernel (tensor-core prefill); `cpu_baseline` is the
-fp64 oracle timed on this machine's host cores on a bounded sample; `configs` (one GPU only) holds
+fp64 oracle timed on this machine's host cores on a bounded sample.  The longer records go to stderr as one JSON line of
+their own, ahead of it: the roofline record in full, `steps_detail` (the step's other calls), and `configs` (one GPU only),
 compact records of the other workloads -- the VideoLLaMA2-shaped pipeline, the long-video layer
 under masks of growing block density with its compression at three keep ratios, and the ragged
 serving batch -- each with the clocks sampled while it was timed.
@@ -824,7 +825,9 @@ def main():
                 "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
                 "vs_baseline": None, "dtype": wl.dtype, "data": "synthetic", "config": config_dict(wl),
                 "clocks": clocks, "e2e": e2e, "gpu_launches": launches,
-                "roofline": roofline, "cpu_baseline": cpu, "steps_detail": steps_detail, "configs": configs}
+                "roofline": {k: roofline[k] for k in ("kernel", "bound", "achieved", "peak", "unit", "frac", "peak_kind", "traffic")},
+                "cpu_baseline": cpu}
+        print(json.dumps({"roofline": roofline, "steps_detail": steps_detail, "configs": configs}), file=sys.stderr, flush=True)
         print(json.dumps(line), flush=True)
     if world > 1:
         dist.destroy_process_group()
