@@ -244,7 +244,8 @@ purekv_status purekv_lowlayer_score_noalloc(const void *q, const void *k, float 
  * relative to the request.  v is [n_layers][T, H_kv, d] with v_layer_stride elements between
  * layers.  idx_out [n_layers, H_kv, K_tot] int32, K_tot = h_cu_kept[n_req];
  * cu_kept[r+1]-cu_kept[r] must equal h_keep[r] + min(window, l_r).
- * s_out (nullable) [n_layers, H_kv, T] fp32 receives S.  ws: purekv_select_ws_bytes. */
+ * s_out (nullable) [n_layers, H_kv, T] fp32 receives S.  ws: purekv_select_ws_bytes (may be null
+ * for 296 segments -- n_req * H_kv * n_layers -- and more of 256-byte rows and at most 51200 tokens; slower). */
 size_t purekv_select_ws_bytes(const purekv_batch *batch, int32_t n_layers, int32_t n_kv_heads);
 purekv_status purekv_select_topk(const float *c, const void *v, int64_t v_layer_stride, int32_t n_layers,
                                  const purekv_batch *batch, int32_t window, const int32_t *keep /* device [n_req] */,
@@ -257,8 +258,8 @@ purekv_status purekv_select_topk(const float *c, const void *v, int64_t v_layer_
  * purekv_select_topk followed by purekv_compact_kv of the same layers, in the selection's own kernels: the CTA
  * that has chosen a (request, KV head, layer) segment's positions copies those K and V rows (k and v share
  * layer_stride) into k_out / v_out [n_layers][K_tot, H_kv, d] (out_layer_stride) -- one launch fewer, and the
- * indices do not travel through memory between two kernels (few segments of many rows take both kernels all the same).  idx_out (and s_out, if given) are written as by
- * purekv_select_topk; results are bit-identical to the two separate calls. */
+ * indices do not travel through memory between two kernels (few segments of many rows take both kernels all the
+ * same).  idx_out (and s_out, if given) are written as by purekv_select_topk; results are bit-identical to the two separate calls. */
 purekv_status purekv_select_compact(const float *c, const void *k, const void *v, int64_t layer_stride,
                                     int32_t n_layers, const purekv_batch *batch, int32_t window,
                                     const int32_t *keep /* device [n_req] */, const int32_t *h_keep,

@@ -229,7 +229,8 @@ constexpr float kDecRescale = 0.f;
 // One launch.  A cluster of C CTAs (grid (C, H_kv, n_req)) owns one (request, KV head); CTA `rank` takes the rank-th share
 // of the request's rows, so ragged requests are cut evenly, and the CTAs' partial results meet in distributed shared
 // memory instead of in a workspace that a second kernel merges (chunk kernel + merge kernel before: 12.0 us for one
-// request of 1664 rows with 28 / 4 heads, now 5.5; 128 requests of 2900-5100 rows 214 us = 5.0 TB/s, now 168 us = 6.4 TB/s).
+// request of 1664 rows with 28 / 4 heads, now 5.5; 128 requests of 2900-5100 rows 214 us = 5.0 TB/s, now 167 us = 6.4 TB/s in a row
+// and 5.6 TB/s with a cold L2).
 // Bound by HBM for large batches and by a chain of latencies for small ones: launch (1 us behind a programmatic
 // predecessor), the offsets, the rows, the products, one cluster barrier.
 // A warp takes 16 keys per trip: with mma.sync the group's heads are the 16 rows of an m16n8k16 tile (M = 16 is far below a

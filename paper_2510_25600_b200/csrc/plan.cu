@@ -134,9 +134,11 @@ purekv_status purekv_budget(int32_t len, int32_t window, double keep_ratio, int3
 // Splits long kept-key lists into chunks and orders the (query tile, head pair, chunk) units by decreasing cost:
 // the kernel's n_ctas persistent CTAs start with the first n_ctas units and draw the rest from a counter as they
 // finish, so the order is longest-first list scheduling carried out at run time.  The costs also decide how finely
-// long lists are cut.  They are in quarters of a 64-key half of a list entry, fitted
-// to measured unit times: 4 per present half (5 when the entry carries a bit mask), 6 per unit (query load, pipeline
-// fill, epilogue) and 14 more for a chunk of a split list (fp32 partial result written out, and the merge).
+// long lists are cut.  They are in quarters of a 64-key half of a list entry: 4 per
+// half that the entry lists (5 when it carries a bit mask), 6 per unit (query load, pipeline fill, epilogue) and 14 more for a
+// chunk of a split list (fp32 partial result written out, and the merge).  The constants were fitted to unit times of an
+// earlier form of the kernel, which also loaded the listed halves that hold no pair; today a half costs 0.78 of a whole entry
+// rather than half of it, and a chunk's merge less.  The order they give is still the one measured.
 //
 // With an odd group size the group's last head has no partner; a unit for it alone takes as long as a unit for two
 // heads.  Consecutive query tiles of a request whose lists are not split therefore share that head's unit (a twin
@@ -279,7 +281,7 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
         }
       }
     }
-    // counting sort (costs are small numbers: at most 80 entries of 10, and the overheads)
+    // counting sort (costs are small numbers: ten per entry of a chunk at most, and the overheads)
     int32_t top = 0;
     for (int32_t c : item_cost) top = std::max(top, c);
     std::vector<int32_t> at((size_t)top + 2, 0);  // at[c]: where the units of cost c begin

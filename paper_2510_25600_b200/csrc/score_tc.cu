@@ -34,9 +34,10 @@ constexpr int kScorePoly = PUREKV_SCORE_POLY;
 using namespace tc;
 
 // Adds the exponentials of 32 columns of a key's logits to its sums; l4: minus the columns' log-sum-exp, in log2 units.
-// Everything but MUFU works on pairs: the kernel is paced by the instructions its warps issue (0.66 of the issue slots busy,
-// MUFU 0.48, FMA 0.49, tensor 0.37), not by one unit.  37 120 tokens, 1792 rows per head: 90 -> 87 us with pairs, 79 with the
-// log-sum-exp fetched once per group of warps besides; all exponentials on MUFU 98 us, 6 of 8 second pairs on FMA the best.
+// Everything but MUFU works on pairs: with single values the kernel was paced by the instructions its warps issue.  37 120 tokens,
+// 1792 rows per head, calls in a row: 90 -> 87 us with pairs, 79 with the log-sum-exp fetched once per group of warps besides (86
+// with a cold L2, 91 among other work); all exponentials on MUFU 98 us, 6 of 8 second pairs on FMA the best.  As it stands no unit
+// is full (issue slots 0.59 busy, MUFU 0.55, tensor pipe 0.42): the warps wait for TMEM and for one another.
 __device__ __forceinline__ void add_exps(const uint32_t (&r)[32], const float4* l4, float scale_log2, float2 (&acc)[2]) {
   const float2 sc = make_float2(scale_log2, scale_log2);
 #pragma unroll
