@@ -384,10 +384,10 @@ def time_pipeline(pipe, wl, d_in, steps, warmup, local, world, peaks, sync_all):
                 "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "peak_kind": f"measured {which} cuBLAS bf16 ({why})" if "bf16_tflops_sustained" in peaks else f"fallback {which}",
                 **tensor_fracs(achieved, peaks), "traffic": ncu_traffic(wl.name),
-                "traffic_note": "dram read + write of one launch under the paper mask (26 of the 28 launches of a step), from the ncu capture summarised in profiles/; null when the kernel sources changed since",
-                "algorithmic_bytes_per_launch": wl.batch.total_tokens * wl.head_dim * 2 * (2 * wl.n_q_heads + 2 * wl.n_kv_heads),
-                "flops_per_step": fl_dense + fl_st, "launches_per_step": wl.n_layers,
-                "avg_launch_ms": ms_prefill / wl.n_layers,
+                "traffic_note": "dram read + write of a launch of one layer under the paper mask (a step's launches take the layers of one mask together), from the ncu capture summarised in profiles/; null when the kernel sources changed since",
+                "algorithmic_bytes_per_layer": wl.batch.total_tokens * wl.head_dim * 2 * (2 * wl.n_q_heads + 2 * wl.n_kv_heads),
+                "flops_per_step": fl_dense + fl_st, "launches_per_step": pipe.prefill_launches, "layers_per_step": wl.n_layers,
+                "avg_launch_ms": ms_prefill / pipe.prefill_launches, "avg_layer_ms": ms_prefill / wl.n_layers,
                 "st_layers": part(fl_st, ms_st), "dense_layers": part(fl_dense, ms_dense),
                 "st_layer_ms_isolated": float(k_ms[:, n_dense:].mean()) if n_st and len(k_ms) else None,
                 "dense_layer_ms_isolated": float(k_ms[:, :n_dense].mean()) if len(k_ms) else None,

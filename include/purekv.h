@@ -145,6 +145,17 @@ purekv_status purekv_plan_build_host(const purekv_batch *batch, const purekv_st_
                                      int32_t n_kv_heads, int32_t n_ctas, void *h_plan,
                                      size_t plan_bytes, purekv_plan_info *h_info);
 
+/* Same size and planning, for launches of n_layers layers at a time (purekv_st_sparse_prefill_layers; n_layers 1 is the call above):
+ * cutting long lists into chunks evens out the end of a launch, and where one launch serves several layers that end is paid
+ * for once, so lists are left whole when that ends sooner.  The plan serves launches of any number of layers. */
+size_t purekv_plan_layers_bytes(const purekv_batch *batch, const purekv_st_params *params, purekv_dtype dtype,
+                                int32_t head_dim, int32_t n_q_heads, int32_t n_kv_heads, int32_t n_ctas,
+                                int32_t n_layers);
+purekv_status purekv_plan_build_layers_host(const purekv_batch *batch, const purekv_st_params *params,
+                                            purekv_dtype dtype, int32_t head_dim, int32_t n_q_heads,
+                                            int32_t n_kv_heads, int32_t n_ctas, int32_t n_layers, void *h_plan,
+                                            size_t plan_bytes, purekv_plan_info *h_info);
+
 /* ---- ST-SpAttn prefill, one layer (Sec. 3.2; softmax of Eq. 1 over the kept keys) ------
  * O[i,hq,:] = sum_{j<=i, M(i,j)} softmax_j(scale * q_i.k_j) v_j.   lse (nullable) [H, T] fp32
  * receives log-sum-exp (natural log) of each row's kept logits.  softmax_scale 0 means
@@ -160,6 +171,20 @@ purekv_status purekv_st_sparse_prefill(const void *q, const void *k, const void 
                                        int32_t n_kv_heads, int32_t head_dim, purekv_dtype dtype,
                                        float softmax_scale, void *ws, size_t ws_bytes, int32_t *status,
                                        void *stream);
+
+/* The same for n_layers layers whose Q/K/V are all at hand: layer n reads q + n * q_layer_stride, k and v + n *
+ * kv_layer_stride, and writes o + n * o_layer_stride and, with lse, lse + n * lse_layer_stride (strides in elements).  Each
+ * layer's result is that of its own call with this plan.  Where the tensor-core kernel runs and the plan leaves every list
+ * whole (h_info->max_chunks 1), all layers are one launch, whose CTAs go from a layer's last units to the next layer's
+ * first; otherwise one launch per layer. */
+purekv_status purekv_st_sparse_prefill_layers(const void *q, const void *k, const void *v, void *o, float *lse,
+                                              int64_t q_layer_stride, int64_t kv_layer_stride,
+                                              int64_t o_layer_stride, int64_t lse_layer_stride, int32_t n_layers,
+                                              const purekv_batch *batch, void *plan,
+                                              const purekv_plan_info *h_info, int32_t n_q_heads,
+                                              int32_t n_kv_heads, int32_t head_dim, purekv_dtype dtype,
+                                              float softmax_scale, void *ws, size_t ws_bytes, int32_t *status,
+                                              void *stream);
 
 /* ---- low-layer window scores (Eq. 1-2) -------------------------------------------------
  * For request r of length l, w = min(window, l), KV head g, key j < l-w:

@@ -31,8 +31,8 @@ FLAG_DENSE_CAUSAL = 1
 FLAG_COARSE_BLOCKS = 2
 
 EXPORTS = ("purekv_version", "purekv_last_error", "purekv_budget", "purekv_plan_bytes", "purekv_plan_build",
-           "purekv_plan_build_host",
-           "purekv_st_sparse_prefill", "purekv_score_ws_bytes", "purekv_lowlayer_score", "purekv_lowlayer_score_lse", "purekv_lowlayer_score_noalloc",
+           "purekv_plan_build_host", "purekv_plan_layers_bytes", "purekv_plan_build_layers_host",
+           "purekv_st_sparse_prefill", "purekv_st_sparse_prefill_layers", "purekv_score_ws_bytes", "purekv_lowlayer_score", "purekv_lowlayer_score_lse", "purekv_lowlayer_score_noalloc",
            "purekv_select_ws_bytes",
            "purekv_select_topk", "purekv_compact_kv", "purekv_decode_ws_bytes", "purekv_decode_attention",
            "purekv_poll_status", "purekv_set_wait_limit_ns", "purekv_score_ex_ws_bytes", "purekv_lowlayer_score_ex",
@@ -83,6 +83,13 @@ _lib.purekv_score_ws_bytes.restype = C.c_size_t
 _lib.purekv_select_ws_bytes.restype = C.c_size_t
 _lib.purekv_plan_bytes.argtypes = [C.POINTER(CBatch), C.POINTER(StParams), C.c_int, C.c_int32, C.c_int32, C.c_int32,
                                    C.c_int32]
+_lib.purekv_plan_layers_bytes.restype = C.c_size_t
+_lib.purekv_plan_layers_bytes.argtypes = [C.POINTER(CBatch), C.POINTER(StParams), C.c_int] + [C.c_int32] * 5
+_lib.purekv_plan_build_layers_host.argtypes = [C.POINTER(CBatch), C.POINTER(StParams), C.c_int] + [C.c_int32] * 5 + [
+    C.c_void_p, C.c_size_t, C.POINTER(PlanInfo)]
+_lib.purekv_st_sparse_prefill_layers.argtypes = [C.c_void_p] * 5 + [C.c_int64] * 4 + [
+    C.c_int32, C.POINTER(CBatch), C.c_void_p, C.POINTER(PlanInfo), C.c_int32, C.c_int32, C.c_int32, C.c_int, C.c_float,
+    C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p]
 _lib.purekv_plan_build.argtypes = [C.POINTER(CBatch), C.POINTER(StParams), C.c_int, C.c_int32, C.c_int32, C.c_int32,
                                    C.c_int32, C.c_void_p, C.c_size_t, C.POINTER(PlanInfo), C.c_void_p]
 _lib.purekv_plan_build_host.argtypes = [C.POINTER(CBatch), C.POINTER(StParams), C.c_int, C.c_int32, C.c_int32,
@@ -226,8 +233,10 @@ class Plan:
 
 
 def purekv_plan_bytes(batch: Batch, params: StParams, dtype: int, head_dim: int, n_q_heads: int, n_kv_heads: int,
-                      n_ctas: int = 0) -> int:
-    return int(_lib.purekv_plan_bytes(C.byref(batch.c), C.byref(params), dtype, head_dim, n_q_heads, n_kv_heads, n_ctas))
+                      n_ctas: int = 0, n_layers: int = 1) -> int:
+    """With `n_layers`, purekv_plan_layers_bytes: of a plan for launches of that many layers."""
+    return int(_lib.purekv_plan_layers_bytes(C.byref(batch.c), C.byref(params), dtype, head_dim, n_q_heads, n_kv_heads, n_ctas,
+                                             n_layers))
 
 
 def purekv_plan_build(batch: Batch, params: StParams, dtype: int, head_dim: int, n_q_heads: int, n_kv_heads: int,
@@ -245,19 +254,20 @@ def purekv_plan_build(batch: Batch, params: StParams, dtype: int, head_dim: int,
 
 
 def purekv_plan_build_host(batch: Batch, params: StParams, dtype: int, head_dim: int, n_q_heads: int, n_kv_heads: int,
-                           n_ctas: int = 0, out: Optional[torch.Tensor] = None):
-    """Plan bytes in host memory + PlanInfo; makes no CUDA call.  Without `out` the bytes come back as a numpy
+                           n_ctas: int = 0, out: Optional[torch.Tensor] = None, n_layers: int = 1):
+    """Plan bytes in host memory + PlanInfo; makes no CUDA call (with `n_layers`, purekv_plan_build_layers_host: for
+    launches of that many layers).  Without `out` the bytes come back as a numpy
     uint8 array sized by a first planning pass; with `out` (a host uint8 tensor, e.g. pinned, large enough) they
     are written there in one pass and the used prefix of `out` is returned, ready for an asynchronous copy."""
     info = PlanInfo()
     if out is not None:
-        _check(_marshal.purekv_plan_build_host(batch.c, params, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, out.data_ptr(),
-                                               out.numel(), info), "purekv_plan_build_host")
+        _check(_marshal.purekv_plan_build_layers_host(batch.c, params, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, n_layers,
+                                                      out.data_ptr(), out.numel(), info), "purekv_plan_build_host")
         return out[:info.bytes_used], info
-    n = purekv_plan_bytes(batch, params, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas)
+    n = purekv_plan_bytes(batch, params, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, n_layers)
     buf = np.zeros(max(n, 1), dtype=np.uint8)
-    _check(_lib.purekv_plan_build_host(C.byref(batch.c), C.byref(params), dtype, head_dim, n_q_heads, n_kv_heads,
-                                       n_ctas, buf.ctypes.data, n, C.byref(info)), "purekv_plan_build_host")
+    _check(_lib.purekv_plan_build_layers_host(C.byref(batch.c), C.byref(params), dtype, head_dim, n_q_heads, n_kv_heads,
+                                              n_ctas, n_layers, buf.ctypes.data, n, C.byref(info)), "purekv_plan_build_host")
     return buf[:info.bytes_used], info
 
 
@@ -277,6 +287,28 @@ def purekv_st_sparse_prefill(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, 
                                              plan.buf.data_ptr(), plan.info, h, k.shape[1], d, _dtype_code(q), softmax_scale,
                                              _ptr(ws), 0 if ws is None else ws.numel(), _ptr(status), _stream()),
            "purekv_st_sparse_prefill")
+    return out
+
+
+def purekv_st_sparse_prefill_layers(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, batch: Batch, plan: Plan,
+                                    out: Optional[torch.Tensor] = None, lse: Optional[torch.Tensor] = None,
+                                    softmax_scale: float = 0.0, status: Optional[torch.Tensor] = None,
+                                    ws: Optional[torch.Tensor] = None) -> torch.Tensor:
+    """q [L,T,H,d], k,v [L,T,H_kv,d] on the GPU, each layer contiguous; returns O [L,T,H,d], every layer as
+    purekv_st_sparse_prefill gives it (`lse` [L,H,T]).  One launch where the plan leaves lists whole
+    (purekv_plan_build_host with n_layers)."""
+    assert q.dim() == 4 and _layers_contiguous(q) and _layers_contiguous(k) and _layers_contiguous(v) and k.stride(0) == v.stride(0)
+    n_layers, t, h, d = q.shape
+    assert k.size(0) == n_layers and v.size(0) == n_layers
+    if out is None:
+        out = torch.empty((n_layers, t, h, d), dtype=q.dtype, device=q.device)
+    assert _layers_contiguous(out) and (lse is None or lse[0].is_contiguous())
+    if ws is None and plan.info.ws_bytes > 0:
+        ws = torch.empty(plan.info.ws_bytes, dtype=torch.uint8, device=q.device)
+    _check(_marshal.purekv_st_sparse_prefill_layers(
+        q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), _ptr(lse), q.stride(0), k.stride(0), out.stride(0),
+        0 if lse is None else lse.stride(0), n_layers, batch.c, plan.buf.data_ptr(), plan.info, h, k.shape[2], d, _dtype_code(q),
+        softmax_scale, _ptr(ws), 0 if ws is None else ws.numel(), _ptr(status), _stream()), "purekv_st_sparse_prefill_layers")
     return out
 
 

@@ -139,7 +139,8 @@ struct __align__(16) Unit {
   int32_t counter_base;          // merge counter of head hq = counters[counter_base + hq]: a byte per warp of 32 rows
   int32_t q_start1, q_rows1;     // a twin unit's second query tile (q_rows1 == 0: an ordinary unit)
   int32_t part_base1, counter_base1;  // ... and that tile's workspace slots and merge counters when the lists are split
-  int32_t pad[2];
+  int32_t layer;                 // zero in the plan; the kernel's copy says which layer of the launch the unit is drawn for
+  int32_t pad;
 };
 static_assert(sizeof(Unit) == 64, "the plan's unit record is 16 words");
 

@@ -113,6 +113,29 @@ PyObject* prefill(PyObject*, PyObject* const* v, Py_ssize_t n) {
   });
 }
 
+PyObject* prefill_layers(PyObject*, PyObject* const* v, Py_ssize_t n) {
+  Args a("st_sparse_prefill_layers", v, n, 22);
+  const void *q = a.ptr(), *k = a.ptr(), *vv = a.ptr();
+  void* o = a.ptr();
+  float* lse = (float*)a.ptr();
+  const int64_t qs = a.integer(), ks = a.integer(), os = a.integer(), ls = a.integer();
+  const int32_t layers = a.i32();
+  const purekv_batch* b = a.batch();
+  void* plan = a.ptr();
+  const purekv_plan_info* info = (const purekv_plan_info*)a.host(sizeof(purekv_plan_info));
+  const int32_t h = a.i32(), hkv = a.i32(), d = a.i32(), dt = a.i32();
+  const float scale = a.f32();
+  void* ws = a.ptr();
+  const size_t ws_bytes = (size_t)a.integer();
+  int32_t* status = (int32_t*)a.ptr();
+  void* stream = a.ptr();
+  if (!a.ok) return nullptr;
+  return call([&] {
+    return purekv_st_sparse_prefill_layers(q, k, vv, o, lse, qs, ks, os, ls, layers, b, plan, info, h, hkv, d, (purekv_dtype)dt,
+                                           scale, ws, ws_bytes, status, stream);
+  });
+}
+
 PyObject* score(PyObject*, PyObject* const* v, Py_ssize_t n) {
   Args a("lowlayer_score", v, n, 13);
   const void *q = a.ptr(), *k = a.ptr();
@@ -221,23 +244,24 @@ PyObject* decode(PyObject*, PyObject* const* v, Py_ssize_t n) {
 }
 
 PyObject* plan_build_host(PyObject*, PyObject* const* v, Py_ssize_t n) {
-  Args a("plan_build_host", v, n, 10);
+  Args a("plan_build_layers_host", v, n, 11);
   const purekv_batch* b = a.batch();
   const purekv_st_params* p = (const purekv_st_params*)a.host(sizeof(purekv_st_params));
-  const int32_t dt = a.i32(), d = a.i32(), h = a.i32(), hkv = a.i32(), n_ctas = a.i32();
+  const int32_t dt = a.i32(), d = a.i32(), h = a.i32(), hkv = a.i32(), n_ctas = a.i32(), layers = a.i32();
   void* out = a.ptr();
   const size_t bytes = (size_t)a.integer();
   purekv_plan_info* info = (purekv_plan_info*)a.host(sizeof(purekv_plan_info));  // (a ctypes structure: written in place)
   if (!a.ok) return nullptr;
-  return call([&] { return purekv_plan_build_host(b, p, (purekv_dtype)dt, d, h, hkv, n_ctas, out, bytes, info); });
+  return call([&] { return purekv_plan_build_layers_host(b, p, (purekv_dtype)dt, d, h, hkv, n_ctas, layers, out, bytes, info); });
 }
 
 #define PK_METHOD(name, f) {name, (PyCFunction)(void (*)(void))f, METH_FASTCALL, nullptr}
-PyMethodDef methods[] = {PK_METHOD("purekv_st_sparse_prefill", prefill), PK_METHOD("purekv_lowlayer_score", score),
+PyMethodDef methods[] = {PK_METHOD("purekv_st_sparse_prefill", prefill), PK_METHOD("purekv_st_sparse_prefill_layers", prefill_layers),
+                         PK_METHOD("purekv_lowlayer_score", score),
                          PK_METHOD("purekv_lowlayer_score_lse", score_lse), PK_METHOD("purekv_lowlayer_score_ex", score_ex),
                          PK_METHOD("purekv_select_topk", select_topk), PK_METHOD("purekv_compact_kv", compact_kv),
                          PK_METHOD("purekv_decode_attention", decode),
-                         PK_METHOD("purekv_plan_build_host", plan_build_host), {nullptr, nullptr, 0, nullptr}};
+                         PK_METHOD("purekv_plan_build_layers_host", plan_build_host), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace

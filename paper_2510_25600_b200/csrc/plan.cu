@@ -144,7 +144,7 @@ purekv_status purekv_budget(int32_t len, int32_t window, double keep_ratio, int3
 // heads.  Consecutive query tiles of a request whose lists are not split therefore share that head's unit (a twin
 // unit, see Unit): the merged lists are appended to `entries`.
 static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& entries, int32_t H, int32_t Hkv,
-                           int32_t n_ctas,
+                           int32_t n_ctas, int32_t n_layers,
                            std::vector<Unit>& units, int32_t* n_counters,
                            int64_t* part_slots, int32_t* max_chunks) {
   const int32_t G = H / Hkv, ppg = (G + 1) / 2, n_pairs = Hkv * ppg;
@@ -299,10 +299,11 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
   // above `limit` is answered as soon as it is known.  Units of one cost and CTAs free at the same time are counted, not
   // listed: the earliest free time only grows, so one pass over the times serves all units.
   std::vector<int32_t> n_of_cost, n_free;
+  int64_t total = 0;  // the units' costs
   auto makespan = [&](int32_t l_max, int64_t limit) {
     find_twins(l_max);
     n_of_cost.clear();
-    int64_t total = 0;
+    total = 0;
     auto add = [&](int32_t cost, int32_t n) {
       if ((size_t)cost >= n_of_cost.size()) n_of_cost.resize((size_t)cost + 1, 0);
       n_of_cost[cost] += n;
@@ -346,6 +347,16 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
       if (t_best < 0 || t <= t_best) { t_best = t; l_best = l_max; }  // on a tie the finer cut
     }
   }
+  // Launches of several layers need whole lists, and pass from one layer to the next without waiting for its end: layers but
+  // the last cost the CTAs' share of the units.  Taken if that ends before n_layers launches of the lists as cut above would,
+  // a launch's start (8 us, of which a 128-key entry takes 1.6) counted in.  Few layers of long lists fall to the other side:
+  // one CTA would be on the longest list when the others are done.
+  if (n_layers > 1) {
+    const int32_t l_whole = 1 << 28, launch = 40;
+    const int64_t apart = n_layers * (makespan(l_best, INT64_MAX) + launch);
+    const int64_t last = makespan(l_whole, INT64_MAX);
+    if ((n_layers - 1) * (total + n_ctas - 1) / n_ctas + last + launch <= apart) l_best = l_whole;
+  }
   make_items(l_best);
   entries.insert(entries.end(), twin_entries.begin(), twin_entries.end());
   *n_counters = counters;
@@ -381,7 +392,7 @@ struct HostPlan {
 };
 
 static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p, purekv_dtype dtype,
-                                int32_t head_dim, int32_t n_q_heads, int32_t n_kv_heads, int32_t n_ctas,
+                                int32_t head_dim, int32_t n_q_heads, int32_t n_kv_heads, int32_t n_ctas, int32_t n_layers,
                                 purekv_plan_info* info, HostPlan& plan) {
   int tq, gk;  // rows per query tile; skip granularity in keys (the mask parameter `tile`)
   purekv_status st = check_params(b, p, dtype, head_dim, &tq, &gk);
@@ -395,6 +406,7 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
              PUREKV_ERR_INVALID_ARG, "n_q_heads %d must be a positive multiple of n_kv_heads %d", n_q_heads,
              n_kv_heads);
   PK_REQUIRE(n_ctas >= 0 && n_ctas <= 4096, PUREKV_ERR_INVALID_ARG, "n_ctas %d outside [0, 4096]", n_ctas);
+  PK_REQUIRE(n_layers >= 1 && n_layers <= 65535, PUREKV_ERR_INVALID_ARG, "n_layers %d outside [1, 65535]", n_layers);
   if (n_ctas == 0) n_ctas = 148;  // one persistent CTA per SM of a B200
   const bool dense = (p->flags & PUREKV_FLAG_DENSE_CAUSAL) != 0;
   const int32_t gw = p->grid_w, gh = p->grid_h, n = gw * gh;
@@ -624,7 +636,7 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
   int32_t n_counters = 0, max_chunks = 1;
   int64_t part_slots = 0;
   if (tq == 128 && nq > 0) {
-    schedule_units(qtiles, entries, n_q_heads, n_kv_heads, n_ctas, units, &n_counters, &part_slots, &max_chunks);
+    schedule_units(qtiles, entries, n_q_heads, n_kv_heads, n_ctas, n_layers, units, &n_counters, &part_slots, &max_chunks);
     const size_t n_masks = masks.size();
     PK_REQUIRE(n_masks + entries.size() < (size_t)INT32_MAX, PUREKV_ERR_UNSUPPORTED, "mask table exceeds 2^31 words");
     masks.resize(n_masks + entries.size());
@@ -680,18 +692,29 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
 
 size_t purekv_plan_bytes(const purekv_batch* b, const purekv_st_params* p, purekv_dtype dtype, int32_t head_dim,
                          int32_t n_q_heads, int32_t n_kv_heads, int32_t n_ctas) {
+  return purekv_plan_layers_bytes(b, p, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, 1);
+}
+
+size_t purekv_plan_layers_bytes(const purekv_batch* b, const purekv_st_params* p, purekv_dtype dtype, int32_t head_dim,
+                                int32_t n_q_heads, int32_t n_kv_heads, int32_t n_ctas, int32_t n_layers) {
   purekv_plan_info info;
   HostPlan host;
-  if (build_plan(b, p, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, &info, host) != PUREKV_OK) return 0;
+  if (build_plan(b, p, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, n_layers, &info, host) != PUREKV_OK) return 0;
   return (size_t)host.total;
 }
 
 purekv_status purekv_plan_build_host(const purekv_batch* b, const purekv_st_params* p, purekv_dtype dtype,
                                      int32_t head_dim, int32_t n_q_heads, int32_t n_kv_heads, int32_t n_ctas,
                                      void* h_plan, size_t plan_bytes, purekv_plan_info* info) {
+  return purekv_plan_build_layers_host(b, p, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, 1, h_plan, plan_bytes, info);
+}
+
+purekv_status purekv_plan_build_layers_host(const purekv_batch* b, const purekv_st_params* p, purekv_dtype dtype,
+                                            int32_t head_dim, int32_t n_q_heads, int32_t n_kv_heads, int32_t n_ctas,
+                                            int32_t n_layers, void* h_plan, size_t plan_bytes, purekv_plan_info* info) {
   PK_REQUIRE(h_plan, PUREKV_ERR_INVALID_ARG, "h_plan is null");
   HostPlan host;
-  purekv_status st = build_plan(b, p, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, info, host);
+  purekv_status st = build_plan(b, p, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, n_layers, info, host);
   if (st != PUREKV_OK) return st;
   PK_REQUIRE((size_t)host.total <= plan_bytes, PUREKV_ERR_WORKSPACE, "plan needs %zu bytes, buffer has %zu", (size_t)host.total,
              plan_bytes);
@@ -704,7 +727,7 @@ purekv_status purekv_plan_build(const purekv_batch* b, const purekv_st_params* p
                                 size_t plan_bytes, purekv_plan_info* info, void* stream) {
   PK_REQUIRE(plan, PUREKV_ERR_INVALID_ARG, "plan is null");
   HostPlan built;
-  purekv_status st = build_plan(b, p, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, info, built);
+  purekv_status st = build_plan(b, p, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, 1, info, built);
   if (st != PUREKV_OK) return st;
   PK_REQUIRE((size_t)built.total <= plan_bytes, PUREKV_ERR_WORKSPACE, "plan needs %zu bytes, buffer has %zu", (size_t)built.total,
              plan_bytes);

@@ -18,6 +18,8 @@ struct PrefillArgs {
   size_t ws_bytes;
   int32_t* status;
   cudaStream_t stream;
+  int32_t n_layers;                                  // of one launch
+  int64_t q_stride, kv_stride, o_stride, lse_stride;  // between layers, in elements (n_layers > 1)
 };
 
 purekv_status launch_prefill_simt(const PrefillArgs& a);  // CUDA cores: fp32, or bf16 with head_dim != 128

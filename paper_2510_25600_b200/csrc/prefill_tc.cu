@@ -71,7 +71,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_k64,
     const __grid_constant__ CUtensorMap tm_v64, __nv_bfloat16* __restrict__ o, float* __restrict__ lse,
     uint8_t* __restrict__ plan, float* __restrict__ ws, int32_t n_q_heads, int32_t n_kv_heads, float scale_log2,
-    int32_t* __restrict__ status, uint64_t wait_ns, int64_t plan_bytes, int64_t ws_floats) {
+    int32_t* __restrict__ status, uint64_t wait_ns, int64_t plan_bytes, int64_t ws_floats, int32_t n_layers, int64_t o_stride,
+    int64_t lse_stride) {
   constexpr int ST = Cfg<BK>::kStages, MR = Cfg<BK>::kMeta;
   constexpr uint32_t kPanelQ = kBQ * 128;  // bytes of one 64-column panel of a Q tile
   constexpr uint32_t kTileQ = 2 * kPanelQ;
@@ -168,7 +169,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
   // Units are handed out at run time: CTA c starts with unit c of the list (sorted by decreasing cost) and draws
   // every further one from a counter behind the merge counters, so the CTAs finish within one small unit of one
   // another whatever the units really cost.  The producer draws and publishes; the other roles follow unit_s[].
-  const int32_t n_units = plan_ok ? hdr->n_units : 0;
+  // With several layers the list is gone through once per layer, one after another: the CTAs pass from a layer's last (and
+  // smallest) units to the next layer's first without meeting, so a launch's start and its uneven end are paid for once.
+  const int32_t n_units = plan_ok ? hdr->n_units : 0, n_work = n_units * n_layers;
   int32_t* sched = counters + (plan_ok ? hdr->n_counters : 0);  // [0] units drawn beyond the first round, [1] CTAs that drew their last
   const int64_t n_entries = plan_ok ? hdr->n_entries : 0, n_mask_words = plan_ok ? hdr->n_mask_words - n_entries : 0;
   const int64_t total_tokens = plan_ok ? hdr->total_tokens : 0;
@@ -190,8 +193,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
     // published; the CTA gives up with PUREKV_ERR_BAD_PLAN instead.
     auto fetch = [&](int32_t idx) -> Unit {
       Unit uu = {};
-      if (idx < n_units) {
-        uu = units[idx];
+      if (idx < n_work) {
+        const int32_t layer = idx / n_units;
+        uu = units[idx - layer * n_units];
+        uu.layer = layer;
         const int32_t n_pairs = n_kv_heads * ppg;
         const bool split = uu.n_chunks > 1, twin = uu.q_rows1 != 0;
         const bool good = uu.ent_count >= 1 && uu.ent_begin >= 0 &&
@@ -199,6 +204,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
                           uu.q_rows >= 1 && uu.q_rows <= kBQ && uu.req_start >= 0 && uu.q_start >= uu.req_start &&
                           (int64_t)uu.q_start + uu.q_rows <= total_tokens && uu.pair >= 0 && uu.pair < n_pairs &&
                           uu.n_chunks >= 1 && uu.n_chunks <= 255 && uu.chunk >= 0 && uu.chunk < uu.n_chunks &&
+                          (!split || n_layers == 1) &&  // (the plan has merge counters and slots for one layer at a time)
                           (!twin || (uu.q_rows1 >= 1 && uu.q_rows1 <= kBQ && uu.q_start1 >= uu.req_start &&
                                      (int64_t)uu.q_start1 + uu.q_rows1 <= total_tokens && (G & 1) != 0 &&
                                      uu.pair % ppg == ppg - 1 &&
@@ -271,8 +277,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
           mbar_expect_tx(smem_u32(&bars.q_full), n_slots * kTileQ);
           for (int sl = 0; sl < n_slots; ++sl) {
             const int32_t hq = twin ? hq0 : hq0 + sl, qs = (twin && sl) ? u.q_start1 : u.q_start;
-            tma_load_3d(sQ + sl * kTileQ, &tm_q, smem_u32(&bars.q_full), 0, hq, qs);
-            tma_load_3d(sQ + sl * kTileQ + kPanelQ, &tm_q, smem_u32(&bars.q_full), 64, hq, qs);
+            tma_load_4d(sQ + sl * kTileQ, &tm_q, smem_u32(&bars.q_full), 0, hq, qs, u.layer);
+            tma_load_4d(sQ + sl * kTileQ + kPanelQ, &tm_q, smem_u32(&bars.q_full), 64, hq, qs, u.layer);
           }
         }
       }
@@ -324,14 +330,14 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
                 // test plans only: this tile's K is never asked for, so whoever waits for it runs into the limit
               } else if (hm == 3u) {
                 mbar_expect_tx(smem_u32(&bars.k_full[s]), kTileKV);
-                tma_load_3d(sK + s * kTileKV, &tm_k, smem_u32(&bars.k_full[s]), 0, g, tok);
-                tma_load_3d(sK + s * kTileKV + kPanelKV, &tm_k, smem_u32(&bars.k_full[s]), 64, g, tok);
+                tma_load_4d(sK + s * kTileKV, &tm_k, smem_u32(&bars.k_full[s]), 0, g, tok, u.layer);
+                tma_load_4d(sK + s * kTileKV + kPanelKV, &tm_k, smem_u32(&bars.k_full[s]), 64, g, tok, u.layer);
               } else {  // one half: 64 rows into their place inside each panel
                 const uint32_t hh = hm >> 1, off = hh * (kPanelKV / 2);
                 mbar_expect_tx(smem_u32(&bars.k_full[s]), kTileKV / 2);
-                tma_load_3d(sK + s * kTileKV + off, &tm_k64, smem_u32(&bars.k_full[s]), 0, g, tok + 64 * (int32_t)hh);
-                tma_load_3d(sK + s * kTileKV + kPanelKV + off, &tm_k64, smem_u32(&bars.k_full[s]), 64, g,
-                            tok + 64 * (int32_t)hh);
+                tma_load_4d(sK + s * kTileKV + off, &tm_k64, smem_u32(&bars.k_full[s]), 0, g, tok + 64 * (int32_t)hh, u.layer);
+                tma_load_4d(sK + s * kTileKV + kPanelKV + off, &tm_k64, smem_u32(&bars.k_full[s]), 64, g,
+                            tok + 64 * (int32_t)hh, u.layer);
               }
               if (!(withhold_first_k && it == 0u)) issued_k = (int32_t)it + 1;
               if (it >= (uint32_t)ST) ok = mbar_wait(smem_u32(&bars.v_empty[s]), par, abort_flag, wait_ns);
@@ -339,14 +345,14 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
             if (ok) {
               if (hm == 3u) {
                 mbar_expect_tx(smem_u32(&bars.v_full[s]), kTileKV);
-                tma_load_3d(sV + s * kTileKV, &tm_v, smem_u32(&bars.v_full[s]), 0, g, tok);
-                tma_load_3d(sV + s * kTileKV + kPanelKV, &tm_v, smem_u32(&bars.v_full[s]), 64, g, tok);
+                tma_load_4d(sV + s * kTileKV, &tm_v, smem_u32(&bars.v_full[s]), 0, g, tok, u.layer);
+                tma_load_4d(sV + s * kTileKV + kPanelKV, &tm_v, smem_u32(&bars.v_full[s]), 64, g, tok, u.layer);
               } else {
                 const uint32_t hh = hm >> 1, off = hh * (kPanelKV / 2);
                 mbar_expect_tx(smem_u32(&bars.v_full[s]), kTileKV / 2);
-                tma_load_3d(sV + s * kTileKV + off, &tm_v64, smem_u32(&bars.v_full[s]), 0, g, tok + 64 * (int32_t)hh);
-                tma_load_3d(sV + s * kTileKV + kPanelKV + off, &tm_v64, smem_u32(&bars.v_full[s]), 64, g,
-                            tok + 64 * (int32_t)hh);
+                tma_load_4d(sV + s * kTileKV + off, &tm_v64, smem_u32(&bars.v_full[s]), 0, g, tok + 64 * (int32_t)hh, u.layer);
+                tma_load_4d(sV + s * kTileKV + kPanelKV + off, &tm_v64, smem_u32(&bars.v_full[s]), 64, g,
+                            tok + 64 * (int32_t)hh, u.layer);
               }
               issued_v = (int32_t)it + 1;
             }
@@ -750,7 +756,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       const int32_t q_first = (u.q_rows1 != 0 && sl == 1) ? u.q_start1 : u.q_start;  // the slot's query tile
       if (u.n_chunks == 1) {
         const float inv = 1.f / l_sum;
-        __nv_bfloat16* dst = o + ((int64_t)(q_first + row) * n_q_heads + hq) * kD;
+        __nv_bfloat16* dst = o + u.layer * o_stride + ((int64_t)(q_first + row) * n_q_heads + hq) * kD;
 #pragma unroll
         for (int c = 0; c < kD / 32; ++c) {
           uint32_t tt[32];
@@ -768,7 +774,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
           }
         }
         if (lse && row_valid)
-          lse[(int64_t)hq * total_tokens + q_first + row] = (m_ref + log2f(l_sum)) * 0.6931471805599453f;
+          lse[u.layer * lse_stride + (int64_t)hq * total_tokens + q_first + row] = (m_ref + log2f(l_sum)) * 0.6931471805599453f;
       } else {
         // one chunk of a split list: leave the unnormalised result for whoever arrives last
         const bool second_tile = u.q_rows1 != 0 && sl == 1;  // a twin unit's second tile has slots and counters of its own
@@ -936,7 +942,7 @@ static purekv_status launch(const PrefillArgs& a, const CUtensorMap& mq, const C
   PK_CUDA(cudaLaunchKernelEx(&cfg, prefill_tc_kernel<BK>, mq, mk, mv, mk64, mv64, (__nv_bfloat16*)a.o, a.lse,
                              (uint8_t*)a.plan, (float*)a.ws, a.n_q_heads, a.n_kv_heads,
                              a.scale * 1.4426950408889634f, status, wait_limit_ns(), (int64_t)a.info->bytes_used,
-                             (int64_t)(a.ws_bytes / sizeof(float))));
+                             (int64_t)(a.ws_bytes / sizeof(float)), a.n_layers, a.o_stride, a.lse_stride));
   PK_CUDA(cudaGetLastError());
   return PUREKV_OK;
 }
@@ -952,11 +958,13 @@ purekv_status launch_prefill_tc(const PrefillArgs& a) {
   const int64_t T = a.batch->total_tokens;
   CUtensorMap mq, mk, mv, mk64, mv64;
   purekv_status st;
-  if ((st = make_map(&mq, a.q, T, a.n_q_heads, kBQ)) != PUREKV_OK) return st;
-  if ((st = make_map(&mk, a.k, T, a.n_kv_heads, 128)) != PUREKV_OK) return st;
-  if ((st = make_map(&mv, a.v, T, a.n_kv_heads, 128)) != PUREKV_OK) return st;
-  if ((st = make_map(&mk64, a.k, T, a.n_kv_heads, 64)) != PUREKV_OK) return st;
-  if ((st = make_map(&mv64, a.v, T, a.n_kv_heads, 64)) != PUREKV_OK) return st;
+  const int32_t L = a.n_layers;
+  const int64_t q_stride = L > 1 ? a.q_stride : T * a.n_q_heads * kD, kv_stride = L > 1 ? a.kv_stride : T * a.n_kv_heads * kD;
+  if ((st = make_map_layers(&mq, a.q, T, a.n_q_heads, kBQ, L, q_stride)) != PUREKV_OK) return st;
+  if ((st = make_map_layers(&mk, a.k, T, a.n_kv_heads, 128, L, kv_stride)) != PUREKV_OK) return st;
+  if ((st = make_map_layers(&mv, a.v, T, a.n_kv_heads, 128, L, kv_stride)) != PUREKV_OK) return st;
+  if ((st = make_map_layers(&mk64, a.k, T, a.n_kv_heads, 64, L, kv_stride)) != PUREKV_OK) return st;
+  if ((st = make_map_layers(&mv64, a.v, T, a.n_kv_heads, 64, L, kv_stride)) != PUREKV_OK) return st;
   int32_t* status = a.status;
   if (!status) {
     const purekv_status st_w = default_status_word(&status);

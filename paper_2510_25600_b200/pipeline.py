@@ -42,10 +42,12 @@ class PureKVPipeline:
         params_dense.flags |= P.FLAG_DENSE_CAUSAL
         self.params_dense, self.params_st = params_dense, P.st_params(mask)
         hh = (n_q_heads, n_kv_heads)
-        self.plan_buf_dense = torch.empty(max(1, P.purekv_plan_bytes(self.batch, params_dense, self.code, head_dim, *hh)),
-                                          dtype=torch.uint8, device=dev)
-        self.plan_buf_st = torch.empty(max(1, P.purekv_plan_bytes(self.batch, self.params_st, self.code, head_dim, *hh)),
-                                       dtype=torch.uint8, device=dev)
+        self.n_dense = min(n_layers, self.clie + 1)
+        self.n_sparse = n_layers - self.n_dense
+        plan_buf = lambda params, layers: torch.empty(
+            max(1, P.purekv_plan_bytes(self.batch, params, self.code, head_dim, *hh, n_layers=max(1, layers))), dtype=torch.uint8,
+            device=dev)
+        self.plan_buf_dense, self.plan_buf_st = plan_buf(params_dense, self.n_dense), plan_buf(self.params_st, self.n_sparse)
         self.prefill_ws = None
         # per mask a ring of pinned buffers, each with the event behind its last copy; the last one used comes first
         self._h_dense, self._h_st = ([[torch.empty(b.numel(), dtype=torch.uint8, pin_memory=True), None] for _ in range(3)]
@@ -57,6 +59,7 @@ class PureKVPipeline:
         # clipped window a multiple of 8); the two-pass kernels otherwise
         self.one_pass_scores = (dtype == torch.bfloat16 and head_dim == 128 and window % 8 == 0 and
                                 all(l >= window or l % 8 == 0 for l in seq_lens))
+        self.dense_runs, self.sparse_runs = self._runs(0, self.n_dense), self._runs(self.n_dense, n_layers)
         self.lse = torch.empty((len(self.scored), n_q_heads, t), dtype=torch.float32, device=dev)
         self.score_ws = torch.empty(P.purekv_score_ws_bytes(self.batch, window, n_q_heads), dtype=torch.uint8, device=dev)
         nc = len(self.compacted)
@@ -66,10 +69,37 @@ class PureKVPipeline:
         self.v_c = torch.empty_like(self.k_c)
         self.status = torch.zeros(1, dtype=torch.int32, device=dev)
         self.plan_dense = self._plan_st = None
-        # prefill per layer, score (1 kernel one-pass or in one cluster, up to 3 otherwise: counted as 1), select (2), compact
-        self.launches_per_step = n_layers + len(self.scored) + 2 + 1
 
-    def _plan(self, params, ring: list, d_buf: torch.Tensor) -> P.Plan:
+    @property
+    def launches_per_step(self) -> int:
+        """Kernels of a pass: prefill, score (1 one-pass or in one cluster, up to 3 otherwise: counted as 1), select (2),
+        compact."""
+        return self.prefill_launches + len(self.scored) + 2 + 1
+
+    @property
+    def prefill_launches(self) -> int:
+        """Prefill launches of the last pass: the layers under one mask are one, unless the plan cuts lists into chunks or the
+        CUDA-core kernel runs them."""
+        n = 0
+        for plan, runs in ((self.plan_dense, self.dense_runs), (self._plan_st, self.sparse_runs)):
+            whole = plan is not None and plan.info.n_units > 0 and plan.info.max_chunks == 1
+            n += sum(1 if whole else hi - lo for lo, hi in runs)
+        return n
+
+    def _runs(self, lo: int, hi: int) -> list:
+        """Layers lo .. hi - 1 in runs that one call can take: where a scored layer leaves its rows' log-sum-exp, those of a
+        run lie one after another in self.lse."""
+        row = lambda layer: self.scored.index(layer) if self.one_pass_scores and layer in self.scored else None
+        runs = []
+        for layer in range(lo, hi):
+            at, before = row(layer), row(layer - 1) if layer > lo else None
+            if runs and (at is None and before is None or at is not None and before is not None and at == before + 1):
+                runs[-1][1] = layer + 1
+            else:
+                runs.append([layer, layer + 1])
+        return runs
+
+    def _plan(self, params, ring: list, d_buf: torch.Tensor, layers: int) -> P.Plan:
         """Plans one mask on the host into a pinned buffer and enqueues its copy on the current stream without waiting, so
         planning overlaps the GPU work already in flight.  A small ring of pinned buffers keeps a plan alive until its copy
         has run."""
@@ -79,7 +109,8 @@ class PureKVPipeline:
             ev.synchronize()
         else:
             ev = ring[0][1] = torch.cuda.Event()
-        _, info = P.purekv_plan_build_host(self.batch, params, self.code, self.d, self.h, self.hkv, out=h_buf)
+        _, info = P.purekv_plan_build_host(self.batch, params, self.code, self.d, self.h, self.hkv, out=h_buf,
+                                           n_layers=max(1, layers))
         d_buf.copy_(h_buf, non_blocking=True)
         ev.record()
         return P.Plan(d_buf, info)
@@ -88,7 +119,7 @@ class PureKVPipeline:
     def plan_st(self) -> P.Plan:
         """The sparse mask's plan.  A pass without sparse layers does not need it: it is then made when asked for."""
         if self._plan_st is None:
-            self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st)
+            self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st, self.n_sparse)
             self._size_prefill_ws(self._plan_st)
         return self._plan_st
 
@@ -99,8 +130,8 @@ class PureKVPipeline:
 
     def build_plans(self) -> None:
         """Both masks' plans; `run_device` builds each just ahead of the first layer that needs it."""
-        self.plan_dense = self._plan(self.params_dense, self._h_dense, self.plan_buf_dense)
-        self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st)
+        self.plan_dense = self._plan(self.params_dense, self._h_dense, self.plan_buf_dense, self.n_dense)
+        self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st, self.n_sparse)
         self._size_prefill_ws(self.plan_dense)
         self._size_prefill_ws(self.plan_st)
 
@@ -111,36 +142,50 @@ class PureKVPipeline:
         P.purekv_st_sparse_prefill(q, k, v, self.batch, plan, out=self.o[layer], lse=lse, status=self.status,
                                    ws=self.prefill_ws)
 
+    def _prefill(self, plan: P.Plan, runs: list, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, events) -> None:
+        """The layers of `runs` of the stacked Q/K/V, in as few launches as the plan allows; with `events`, one per layer."""
+        for a, b in runs:
+            if b - a == 1 or events is not None or not isinstance(q, torch.Tensor):  # (or a sequence of layers: no stacked views)
+                for layer in range(a, b):
+                    if events is not None:
+                        events[layer][0].record()
+                    self.prefill_layer(layer, q[layer], k[layer], v[layer])
+                    if events is not None:
+                        events[layer][1].record()
+                continue
+            lse = None
+            if self.one_pass_scores and a in self.scored:
+                at = self.scored.index(a)
+                lse = self.lse[at:at + b - a]
+            P.purekv_st_sparse_prefill_layers(q[a:b], k[a:b], v[a:b], self.batch, plan, out=self.o[a:b], lse=lse, status=self.status,
+                                              ws=self.prefill_ws)
+
     def run_device(self, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, events=None, marks=None) -> None:
         """q [n_layers,T,H,d], k,v [kv_layers,T,H_kv,d] on the GPU.  Results in self.o / idx / k_c / v_c.
-        `events`, if given, is a list of (start, end) torch.cuda.Event pairs, one per prefill launch (an event
-        between two launches keeps the second from starting under the first's tail); `marks`, if given, is three
+        `events`, if given, is a list of (start, end) torch.cuda.Event pairs, one per layer, which is then a prefill launch
+        of its own; otherwise the layers under one mask are one launch where the plan allows it.  `marks`, if given, is three
         events recorded before the first prefill launch, after the last dense-causal one and after the last one."""
         # The sparse mask's plan, the longer one, is made and copied while the GPU works on the dense layers.  (The copy
         # waits for whatever the stream held before this call, which may still read the last plan; in the stream itself,
         # between two layers, it cost 10 us.)
-        before = torch.cuda.Event() if self.n_layers > self.clie + 1 else None
+        before = torch.cuda.Event() if self.n_sparse else None
         if before is not None:
             before.record()
-        self.plan_dense = self._plan(self.params_dense, self._h_dense, self.plan_buf_dense)
+        self.plan_dense = self._plan(self.params_dense, self._h_dense, self.plan_buf_dense, self.n_dense)
         self._size_prefill_ws(self.plan_dense)
         if marks is not None:
             marks[0].record()
-        for layer in range(self.n_layers):
-            if layer == self.clie + 1:
-                main = torch.cuda.current_stream()
-                self._copies.wait_event(before)
-                with torch.cuda.stream(self._copies):
-                    self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st)
-                main.wait_event(self._h_st[0][1])
-                self._size_prefill_ws(self.plan_st)
-            if events is not None:
-                events[layer][0].record()
-            self.prefill_layer(layer, q[layer], k[layer], v[layer])
-            if events is not None:
-                events[layer][1].record()
-            if marks is not None and layer == self.clie:
-                marks[1].record()
+        self._prefill(self.plan_dense, self.dense_runs, q, k, v, events)
+        if marks is not None:
+            marks[1].record()
+        if before is not None:
+            main = torch.cuda.current_stream()
+            self._copies.wait_event(before)
+            with torch.cuda.stream(self._copies):
+                self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st, self.n_sparse)
+            main.wait_event(self._h_st[0][1])
+            self._size_prefill_ws(self._plan_st)
+            self._prefill(self._plan_st, self.sparse_runs, q, k, v, events)
         if marks is not None:
             marks[2].record()
         for n, layer in enumerate(self.scored):
