@@ -139,8 +139,9 @@ struct __align__(16) Unit {
   int32_t counter_base;          // merge counter of head hq = counters[counter_base + hq]: a byte per warp of 32 rows
   int32_t q_start1, q_rows1;     // a twin unit's second query tile (q_rows1 == 0: an ordinary unit)
   int32_t part_base1, counter_base1;  // ... and that tile's workspace slots and merge counters when the lists are split
-  int32_t layer;                 // zero in the plan; the kernel's copy says which layer of the launch the unit is drawn for
-  int32_t pad;
+  // zero in the plan; in the kernel's copy, the layer of the launch that the unit is drawn for, and its first query head
+  // times two, plus one if both slots have work
+  int32_t layer, heads;
 };
 static_assert(sizeof(Unit) == 64, "the plan's unit record is 16 words");
 

@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
   constexpr uint32_t kMaskBytes = Cfg<BK>::kMaskBytes;
   extern __shared__ uint8_t smem_raw[];
   __shared__ Barriers<BK> bars;
-  __shared__ int2 meta_s[MR][2];  // per slot: the entry word, and the byte offset in shared memory of the slot's bit mask
+  __shared__ int2 meta_s[MR][2];  // per slot: the entry word, and the byte offset in shared memory of the slot's bit mask plus the halves loaded
   __shared__ Unit unit_s[kUnitRing];
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s;
@@ -199,6 +199,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
         uu.layer = layer;
         const int32_t n_pairs = n_kv_heads * ppg;
         const bool split = uu.n_chunks > 1, twin = uu.q_rows1 != 0;
+        const int32_t in_group = 2 * (uu.pair % ppg);
+        uu.heads = (uu.pair / ppg * G + in_group) * 2 + (twin || in_group + 1 < G ? 1 : 0);
         const bool good = uu.ent_count >= 1 && uu.ent_begin >= 0 &&
                           (int64_t)uu.ent_begin + (int64_t)uu.ent_count * (twin ? 2 : 1) <= n_entries &&
                           uu.q_rows >= 1 && uu.q_rows <= kBQ && uu.req_start >= 0 && uu.q_start >= uu.req_start &&
@@ -252,9 +254,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       // longest units would keep work from those that finish early.
       int32_t idx_next = 0;
       const int32_t nt = u.ent_count;
-      const int32_t g = u.pair / ppg, hq0 = g * G + 2 * (u.pair % ppg);
+      const int32_t g = u.pair / ppg, hq0 = u.heads >> 1;
       const bool twin = u.q_rows1 != 0;  // both slots on head hq0, slot 1 on the query tile at q_start1
-      const int32_t n_slots = (twin || 2 * (u.pair % ppg) + 1 < G) ? 2 : 1;
+      const int32_t n_slots = 1 + (u.heads & 1);
       // A tile's entry as slot 0 and as slot 1 see it, 32 tiles at a time, one per lane; of the halves an entry claims only
       // those that hold a kept pair are loaded and multiplied (with a skip granularity of 128 keys the entries claim both;
       // 64 frames of 24 x 24 under the paper's mask: 12 % fewer halves, 833 -> 780 us; a 64-key half costs 0.78 of a tile).
@@ -269,7 +271,22 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
           e_l.x &= (int32_t)(~12u | ((he & 3u) << 2));
           if (twin) f_l.x &= (int32_t)(~12u | ((hf & 3u) << 2));
           if (!twin) f_l = e_l;
+          // The entry is checked before its mask offset or key-tile index is used for a copy: a class the slot knows (none only
+          // in a twin unit, and then without halves), a bit mask inside the table.
+          auto entry_ok = [&](const int2& x) {
+            const int32_t c = x.x & 3;
+            const uint32_t h = (uint32_t)(x.x >> 2) & 3u;
+            if (x.x < 0 || (c == kTileNone ? (!twin || h != 0u) : h == 0u)) return false;
+            return c != kTileGeneral || (x.y >= 0 && (int64_t)x.y + (int64_t)(kMaskBytes / 4) <= n_mask_words && (x.y & 3) == 0);
+          };
+          if (!entry_ok(e_l) || !entry_ok(f_l) || (e_l.x >> 4) != (f_l.x >> 4) || ((e_l.x | f_l.x) & 12) == 0 ||
+              (int64_t)u.req_start + (int64_t)(e_l.x >> 4) * BK >= total_tokens) {
+            abort_code_s = (int)PUREKV_ERR_BAD_PLAN;
+            *abort_flag = 1;
+            return false;
+          }
         }
+        return true;
       };
       if (lane == 0) {
         if (uo > 0) ok = mbar_wait(smem_u32(&bars.q_empty), (uo - 1u) & 1u, abort_flag, wait_ns);
@@ -284,7 +301,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       }
       ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       for (int32_t n0 = 0; ok && n0 < nt; n0 += 32) {
-        load_entries(n0 + lane);
+        ok = __all_sync(0xffffffffu, load_entries(n0 + lane));
         const int32_t n1 = min(nt, n0 + 32);
         for (int32_t n = n0; ok && n < n1; ++n) {
           int2 e, f;
@@ -295,29 +312,18 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
           if (lane == 0) {
             if (n == nt - 1) idx_next = atomicAdd(sched, 1) + (int32_t)gridDim.x;  // used after the loop
             const uint32_t s = it % ST, par = ((it / ST) - 1u) & 1u, ms = it % MR;
-            const int32_t tok = u.req_start + (e.x >> 4) * BK;
             const uint32_t hm = (uint32_t)((e.x | f.x) >> 2) & 3u;  // which 64-key halves of the tile are present
-            // the entry is checked before its mask offset or key-tile index is used for a copy: a class the slot
-            // knows (none only in a twin unit, and then without halves), a bit mask inside the table
-            auto entry_ok = [&](const int2& x) {
-              const int32_t c = x.x & 3;
-              const uint32_t h = (uint32_t)(x.x >> 2) & 3u;
-              if (x.x < 0 || (c == kTileNone ? (!twin || h != 0u) : h == 0u)) return false;
-              return c != kTileGeneral ||
-                     (x.y >= 0 && (int64_t)x.y + (int64_t)(kMaskBytes / 4) <= n_mask_words && (x.y & 3) == 0);
-            };
-            if (!entry_ok(e) || !entry_ok(f) || (e.x >> 4) != (f.x >> 4) || hm == 0u || (int64_t)tok >= total_tokens) {
-              abort_code_s = (int)PUREKV_ERR_BAD_PLAN;
-              *abort_flag = 1;
-              ok = false;
-            }
+            // a whole tile, or one half: 64 rows into their place inside each panel
+            const int32_t hh = hm == 2u ? 1 : 0, row = u.req_start + (e.x >> 4) * BK + 64 * hh;
+            const uint32_t off = (uint32_t)hh * (kPanelKV / 2), bytes = hm == 3u ? kTileKV : kTileKV / 2;
+            const CUtensorMap *map_k = hm == 3u ? &tm_k : &tm_k64, *map_v = hm == 3u ? &tm_v : &tm_v64;
             if (ok && it >= (uint32_t)ST) ok = mbar_wait(smem_u32(&bars.k_empty[s]), par, abort_flag, wait_ns);
             if (ok) {
               // a slot's bit mask goes to its own buffer; outside twin units both slots read the first one
               const uint32_t m_off = (sM - smem_u32(smem_raw)) + ms * 2u * kMaskBytes;
               const bool mask0 = (e.x & 3) == kTileGeneral, mask1 = twin && (f.x & 3) == kTileGeneral;
-              meta_s[ms][0] = make_int2(e.x, (int32_t)m_off);
-              meta_s[ms][1] = make_int2(f.x, (int32_t)(m_off + (twin ? kMaskBytes : 0u)));
+              meta_s[ms][0] = make_int2(e.x, (int32_t)(m_off + hm));
+              meta_s[ms][1] = make_int2(f.x, (int32_t)(m_off + hm + (twin ? kMaskBytes : 0u)));
               if (mask0 || mask1) {
                 mbar_expect_tx(smem_u32(&bars.m_full[ms]), (mask0 && mask1) ? 2u * kMaskBytes : kMaskBytes);
                 if (mask0) bulk_load(sM + ms * 2u * kMaskBytes, masks + e.y, kMaskBytes, smem_u32(&bars.m_full[ms]));
@@ -326,34 +332,19 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
               } else {
                 mbar_arrive(smem_u32(&bars.m_full[ms]));
               }
-              if (withhold_first_k && it == 0u) {
-                // test plans only: this tile's K is never asked for, so whoever waits for it runs into the limit
-              } else if (hm == 3u) {
-                mbar_expect_tx(smem_u32(&bars.k_full[s]), kTileKV);
-                tma_load_4d(sK + s * kTileKV, &tm_k, smem_u32(&bars.k_full[s]), 0, g, tok, u.layer);
-                tma_load_4d(sK + s * kTileKV + kPanelKV, &tm_k, smem_u32(&bars.k_full[s]), 64, g, tok, u.layer);
-              } else {  // one half: 64 rows into their place inside each panel
-                const uint32_t hh = hm >> 1, off = hh * (kPanelKV / 2);
-                mbar_expect_tx(smem_u32(&bars.k_full[s]), kTileKV / 2);
-                tma_load_4d(sK + s * kTileKV + off, &tm_k64, smem_u32(&bars.k_full[s]), 0, g, tok + 64 * (int32_t)hh, u.layer);
-                tma_load_4d(sK + s * kTileKV + kPanelKV + off, &tm_k64, smem_u32(&bars.k_full[s]), 64, g,
-                            tok + 64 * (int32_t)hh, u.layer);
+              // (test plans withhold the first tile's K: whoever waits for it runs into the limit)
+              if (!(withhold_first_k && it == 0u)) {
+                mbar_expect_tx(smem_u32(&bars.k_full[s]), bytes);
+                tma_load_4d(sK + s * kTileKV + off, map_k, smem_u32(&bars.k_full[s]), 0, g, row, u.layer);
+                tma_load_4d(sK + s * kTileKV + kPanelKV + off, map_k, smem_u32(&bars.k_full[s]), 64, g, row, u.layer);
               }
               if (!(withhold_first_k && it == 0u)) issued_k = (int32_t)it + 1;
               if (it >= (uint32_t)ST) ok = mbar_wait(smem_u32(&bars.v_empty[s]), par, abort_flag, wait_ns);
             }
             if (ok) {
-              if (hm == 3u) {
-                mbar_expect_tx(smem_u32(&bars.v_full[s]), kTileKV);
-                tma_load_4d(sV + s * kTileKV, &tm_v, smem_u32(&bars.v_full[s]), 0, g, tok, u.layer);
-                tma_load_4d(sV + s * kTileKV + kPanelKV, &tm_v, smem_u32(&bars.v_full[s]), 64, g, tok, u.layer);
-              } else {
-                const uint32_t hh = hm >> 1, off = hh * (kPanelKV / 2);
-                mbar_expect_tx(smem_u32(&bars.v_full[s]), kTileKV / 2);
-                tma_load_4d(sV + s * kTileKV + off, &tm_v64, smem_u32(&bars.v_full[s]), 0, g, tok + 64 * (int32_t)hh, u.layer);
-                tma_load_4d(sV + s * kTileKV + kPanelKV + off, &tm_v64, smem_u32(&bars.v_full[s]), 64, g,
-                            tok + 64 * (int32_t)hh, u.layer);
-              }
+              mbar_expect_tx(smem_u32(&bars.v_full[s]), bytes);
+              tma_load_4d(sV + s * kTileKV + off, map_v, smem_u32(&bars.v_full[s]), 0, g, row, u.layer);
+              tma_load_4d(sV + s * kTileKV + kPanelKV + off, map_v, smem_u32(&bars.v_full[s]), 64, g, row, u.layer);
               issued_v = (int32_t)it + 1;
             }
           }
@@ -383,8 +374,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       constexpr uint32_t idesc_qk_half = instr_desc(BK / 2, false);
       constexpr uint32_t idesc_pv = instr_desc(kD, true);
       static_assert(BK == 128 && ST == 2, "S of a tile is issued behind P V of the tile before, which frees its columns");
-      uint32_t it = 0;          // the CTA's key tiles so far
-      uint32_t tp0 = 0, tp1 = 0;  // ... and those of each slot, P V issued
+      uint32_t it = 0;   // the CTA's key tiles so far, which are slot 0's
+      uint32_t tp1 = 0;  // slot 1's
       // Descriptor words.  High word: stride between 8-row groups 1024 B, descriptor version 1, 128-byte swizzle.
       // Low word: start address / 16 and the leading-dimension offset / 16 (used by the MN-major V operand only).
       constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
@@ -392,111 +383,92 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       const uint32_t k_lo0 = ((sK & 0x3FFFFu) >> 4) | (1u << 16);
       const uint32_t v_lo0 = ((sV & 0x3FFFFu) >> 4) | ((kPanelKV >> 4) << 16);
       auto halves_of = [&](uint32_t i) {  // written before the stage's barrier was armed
-        return (uint32_t)((meta_s[i % MR][0].x | meta_s[i % MR][1].x) >> 2) & 3u;
+        return (uint32_t)meta_s[i % MR][0].y & 3u;
       };
-      // S = Q K^T of a tile in stage s, announced to the slot's rows.  A commit costs the issuing thread about as long as a
-      // product and the rows are waiting for S, so the releases of the stages follow behind and cover the same products.
-      auto issue_qk = [&](auto sl_c, uint32_t s, uint32_t hm) {
-        constexpr int sl = decltype(sl_c)::value;
-        const uint32_t q_lo = q_lo0 + (uint32_t)sl * (kTileQ >> 4);
-        if (hm == 3u) {
-          const uint32_t d_addr = tmem + sl * 128, k_lo = k_lo0 + s * (kTileKV >> 4);
-#pragma unroll
-          for (int ks = 0; ks < kD / 16; ++ks)
-            mma_ss_lh(d_addr, q_lo + (ks >> 2) * (kPanelQ >> 4) + (ks & 3) * 2, kDescHi,
-                      k_lo + (ks >> 2) * (kPanelKV >> 4) + (ks & 3) * 2, kDescHi, idesc_qk, ks > 0 ? 1u : 0u);
-        } else {  // one 64-key half: N = 64, into that half's columns of S
-          const uint32_t hh = hm >> 1;
-          const uint32_t d_addr = tmem + sl * 128 + hh * 64;
-          const uint32_t k_lo = k_lo0 + s * (kTileKV >> 4) + hh * (kPanelKV >> 5);
-#pragma unroll
-          for (int ks = 0; ks < kD / 16; ++ks)
-            mma_ss_lh(d_addr, q_lo + (ks >> 2) * (kPanelQ >> 4) + (ks & 3) * 2, kDescHi,
-                      k_lo + (ks >> 2) * (kPanelKV >> 4) + (ks & 3) * 2, kDescHi, idesc_qk_half, ks > 0 ? 1u : 0u);
-        }
-        tc_commit(smem_u32(&bars.s_full[sl]));
-      };
-      // O(slot) += P V of a tile: the part that waits for the first 96 keys' P ...
-      auto issue_pv_head = [&](auto sl_c, uint32_t s, uint32_t hm, uint32_t par, uint32_t acc0) -> bool {
-        constexpr int sl = decltype(sl_c)::value;
-        // B = V tile, MN-major: per K step 16 key rows (2 groups of 8, 1024 B apart) x 128 dims (2 panels)
-        const uint32_t p_addr = tmem + sl * 128, o_addr = tmem + kColO + sl * 128, v_lo = v_lo0 + s * (kTileKV >> 4);
-        if (hm != 3u) return true;
-        // P of the unit's first tile also implies that the previous unit's output has left TMEM
-        if (!mbar_wait(smem_u32(&bars.p_part[sl]), par, abort_flag, wait_ns)) return false;
-        tc_fence_after();
-#pragma unroll
-        for (int ks = 0; ks < 6; ++ks)
-          mma_ts_lh(o_addr, p_addr + ks * 8, v_lo + ks * (2048 >> 4), kDescHi, idesc_pv, ks > 0 ? 1u : acc0);
-        return true;
-      };
-      // ... and the rest
-      auto issue_pv_tail = [&](auto sl_c, uint32_t s, uint32_t hm, uint32_t par, uint32_t acc0) -> bool {
-        constexpr int sl = decltype(sl_c)::value;
-        const uint32_t p_addr = tmem + sl * 128, o_addr = tmem + kColO + sl * 128, v_lo = v_lo0 + s * (kTileKV >> 4);
-        if (!mbar_wait(smem_u32(&bars.p_full[sl]), par, abort_flag, wait_ns)) return false;
-        tc_fence_after();
-        if (hm == 3u) {
-#pragma unroll
-          for (int ks = 6; ks < 8; ++ks)
-            mma_ts_lh(o_addr, p_addr + ks * 8, v_lo + ks * (2048 >> 4), kDescHi, idesc_pv, 1u);
-        } else {  // the K steps of the present half only
-          const uint32_t k0 = (hm >> 1) * (BK / 32);
-#pragma unroll
-          for (int ks = 0; ks < BK / 32; ++ks)
-            mma_ts_lh(o_addr, p_addr + (k0 + ks) * 8, v_lo + (k0 + ks) * (2048 >> 4), kDescHi, idesc_pv, ks > 0 ? 1u : acc0);
-        }
-        return true;
-      };
-      constexpr std::integral_constant<int, 0> s0{};
-      constexpr std::integral_constant<int, 1> s1{};
+      // One body of code for first and later tiles, whole tiles and halves.  What the roles run in a tile's time goes through
+      // the SM's instruction cache; what misses there comes from the cache that an SM shares with its neighbours, which was 78 %
+      // busy with it (ragged batch of 8: 3.3 M lines a launch, now 2.7 M, and 625 -> 613 us at full clock; dense causal 12.0 M,
+      // now 7.5 M, time unchanged: products by a rolled loop as well leave 2.8 M there and are 4 % slower).
       bool ok = true;
       for (uint32_t uo = 0; ok; ++uo) {
         const uint32_t us = uo % kUnitRing;
         ok = mbar_wait(smem_u32(&bars.u_full[us]), (uo / kUnitRing) & 1u, abort_flag, wait_ns);
         if (!ok) break;
         const int32_t nt = unit_s[us].ent_count;
-        const bool two = unit_s[us].q_rows1 != 0 || 2 * (unit_s[us].pair % ppg) + 1 < G;
+        const uint32_t last_slot = (uint32_t)unit_s[us].heads & 1u;
         mbar_arrive(smem_u32(&bars.u_empty[us]));
         if (nt == 0) break;
-        ok = mbar_wait(smem_u32(&bars.q_full), uo & 1u, abort_flag, wait_ns) &&
-             mbar_wait(smem_u32(&bars.k_full[it % ST]), (it / ST) & 1u, abort_flag, wait_ns);
-        if (!ok) break;
-        tc_fence_after();
-        uint32_t hm = halves_of(it);
-        issue_qk(s0, it % ST, hm);
-        if (two) issue_qk(s1, it % ST, hm);
-        tc_commit(smem_u32(&bars.k_empty[it % ST]));
-        if (nt == 1) tc_commit(smem_u32(&bars.q_empty));  // the unit's last read of Q
-        // Everything that the next S needs besides P V (its K, which halves) is awaited and read between the two parts of
-        // P V, so that nothing but products stands between the rows' last P and their next S: the slot's rows wait for this
-        // thread, and each wait or branch in between showed (8320 tokens: dense causal 406 -> 390 us, paper mask 116 -> 110 us).
-        uint32_t acc = 0u;  // the unit's first product overwrites O
-        for (int32_t n = 0; n < nt; ++n, ++it) {
-          const uint32_t s = it % ST, sn = (it + 1u) % ST;
-          const bool more = n + 1 < nt;
+        ok = mbar_wait(smem_u32(&bars.q_full), uo & 1u, abort_flag, wait_ns);
+        // Step n: P V of tile n and S of tile n + 1, slot 0 before slot 1; step -1 is the first S alone.
+        uint32_t hm = 0u;
+#pragma unroll 1
+        for (int32_t n = -1; ok && n < nt; ++n) {
+          const bool pv = n >= 0, qk = n + 1 < nt;
+          const uint32_t s = it % ST, sn = (pv ? it + 1u : it) % ST;  // stages of tile n, and of tile n + 1
           uint32_t hn = 3u;
-          ok = mbar_wait(smem_u32(&bars.v_full[s]), (it / ST) & 1u, abort_flag, wait_ns) && issue_pv_head(s0, s, hm, tp0 & 1u, acc);
-          if (ok && more) {
-            ok = mbar_wait(smem_u32(&bars.k_full[sn]), ((it + 1u) / ST) & 1u, abort_flag, wait_ns);
-            hn = halves_of(it + 1u);
+          if (pv) ok = mbar_wait(smem_u32(&bars.v_full[s]), (it / ST) & 1u, abort_flag, wait_ns);
+          if (ok && qk) {
+            ok = mbar_wait(smem_u32(&bars.k_full[sn]), ((pv ? it + 1u : it) / ST) & 1u, abort_flag, wait_ns);
+            hn = halves_of(pv ? it + 1u : it);
           }
-          ok = ok && issue_pv_tail(s0, s, hm, tp0 & 1u, acc);
+#pragma unroll
+          for (uint32_t sl = 0; sl < 2u; ++sl) {
+            if (sl > last_slot) break;
+            const uint32_t p_addr = tmem + sl * 128u;
+            if (pv) {
+              // O(slot) += P V, when P has come: the K steps of the first 96 keys as soon as those have, the others behind.  P of the
+              // unit's first tile also implies that the previous unit's output has left TMEM.
+              // B = V tile, MN-major: per K step 16 key rows (2 groups of 8, 1024 B apart) x 128 dims (2 panels)
+              const uint32_t par = (sl == 0u ? it : tp1) & 1u, v_lo = v_lo0 + s * (kTileKV >> 4);
+              bool part, full;
+              mbar_test2(smem_u32(&bars.p_part[sl]), par, smem_u32(&bars.p_full[sl]), par, &part, &full);
+              if (hm != 3u) part = full;
+              if (!part) ok = mbar_wait(smem_u32(hm == 3u ? &bars.p_part[sl] : &bars.p_full[sl]), par, abort_flag, wait_ns);
+              if (!ok) break;
+              tc_fence_after();
+              const uint32_t acc = n > 0 ? 1u : 0u;  // the unit's first product overwrites O
+              if (hm == 3u) {
+#pragma unroll
+                for (int ks = 0; ks < 6; ++ks)
+                  mma_ts_lh(p_addr + kColO, p_addr + ks * 8, v_lo + ks * (2048 >> 4), kDescHi, idesc_pv, ks > 0 ? 1u : acc);
+                if (!full) {
+                  ok = mbar_wait(smem_u32(&bars.p_full[sl]), par, abort_flag, wait_ns);
+                  if (!ok) break;
+                  tc_fence_after();
+                }
+#pragma unroll
+                for (int ks = 6; ks < 8; ++ks)
+                  mma_ts_lh(p_addr + kColO, p_addr + ks * 8, v_lo + ks * (2048 >> 4), kDescHi, idesc_pv, 1u);
+              } else {  // the K steps of the present half only
+                const uint32_t k0 = (hm >> 1) * (BK / 32);
+#pragma unroll
+                for (int ks = 0; ks < BK / 32; ++ks)
+                  mma_ts_lh(p_addr + kColO, p_addr + (k0 + ks) * 8, v_lo + (k0 + ks) * (2048 >> 4), kDescHi, idesc_pv, ks > 0 ? 1u : acc);
+              }
+            } else {
+              tc_fence_after();
+            }
+            if (qk) {
+              // S = Q K^T of tile n + 1; of one 64-key half with N = 64, into that half's columns of S
+              const uint32_t hh = hn == 2u ? 1u : 0u, q_lo = q_lo0 + sl * (kTileQ >> 4);
+              const uint32_t k_lo = k_lo0 + sn * (kTileKV >> 4) + hh * (kPanelKV >> 5);
+              const uint32_t d_addr = p_addr + hh * 64u, idesc = hn == 3u ? idesc_qk : idesc_qk_half;
+#pragma unroll
+              for (int ks = 0; ks < kD / 16; ++ks)
+                mma_ss_lh(d_addr, q_lo + (ks >> 2) * (kPanelQ >> 4) + (ks & 3) * 2, kDescHi,
+                          k_lo + (ks >> 2) * (kPanelKV >> 4) + (ks & 3) * 2, kDescHi, idesc, ks > 0 ? 1u : 0u);
+            }
+            // announced to the slot's rows first (they are waiting for it), the releases of the stages follow behind
+            tc_commit(smem_u32(qk ? &bars.s_full[sl] : &bars.o_final[sl]));
+          }
           if (!ok) break;
-          ++tp0;
-          if (more) issue_qk(s0, sn, hn);
-          else tc_commit(smem_u32(&bars.o_final[0]));
-          if (two) {
-            ok = issue_pv_head(s1, s, hm, tp1 & 1u, acc) && issue_pv_tail(s1, s, hm, tp1 & 1u, acc);
-            if (!ok) break;
-            ++tp1;
-            if (more) issue_qk(s1, sn, hn);
-            else tc_commit(smem_u32(&bars.o_final[1]));
+          if (pv) tc_commit(smem_u32(&bars.v_empty[s]));
+          if (qk) tc_commit(smem_u32(&bars.k_empty[sn]));
+          if (n + 2 == nt) tc_commit(smem_u32(&bars.q_empty));  // the unit's last read of Q
+          if (pv) {
+            ++it;
+            tp1 += last_slot;
           }
-          tc_commit(smem_u32(&bars.v_empty[s]));
-          if (more) tc_commit(smem_u32(&bars.k_empty[sn]));
-          if (n + 2 == nt) tc_commit(smem_u32(&bars.q_empty));
-          acc = 1u;
           hm = hn;
         }
       }
@@ -520,7 +492,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
     auto wait_w = [&](uint32_t bar, uint32_t parity) -> bool {
       return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, wait_ns) ? 1 : 0) != 0;
     };
-    uint32_t it_base = 0;     // key tiles of earlier units (both slots)
+    uint32_t it = 0;          // key tiles of the CTA so far (both slots)
     uint32_t t = 0;           // tiles this slot has processed, over all units
     uint32_t slot_units = 0;  // units this slot took part in
     bool ok = true;
@@ -536,36 +508,28 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       };
       const int32_t nt = u.ent_count;
       if (nt == 0) break;
-      const int32_t pr = u.pair % ppg, g = u.pair / ppg;
-      const bool twin = u.q_rows1 != 0;
-      const int32_t n_slots = (twin || 2 * pr + 1 < G) ? 2 : 1;
-      if (sl >= n_slots) {
+      if (sl > (u.heads & 1)) {
         // A single-head unit: this slot sits it out.  It takes no part in the tile ring meanwhile: a parity wait only
         // tells a barrier's current phase from the one before, and a slot with nothing to deliver is held back by
         // nobody, so it could fall (or run) a whole ring away from the producer.  The unit ring is a full handshake
         // instead, and the next unit is published only after every tile of this one has been issued, which puts the
         // slot's next tile within the ring's reach again.
-        it_base += (uint32_t)nt;
+        it += (uint32_t)nt;
         release_unit();
         continue;
       }
-      const int32_t hq = g * G + 2 * pr + (twin ? 0 : sl);
-      const bool second = twin && sl == 1;  // this slot works on the unit's second query tile
-      const bool row_valid = row < (second ? u.q_rows1 : u.q_rows);
-      const int32_t i_rel = (second ? u.q_start1 : u.q_start) - u.req_start + row;
+      const int32_t i_rel = (u.q_rows1 != 0 && sl == 1 ? u.q_start1 : u.q_start) - u.req_start + row;
       float m_ref = 0.f, l_sum = 0.f;
-      for (int32_t n = 0; n < nt; ++n) {
-        const uint32_t it = it_base + (uint32_t)n, ms = it % MR;
-        if (!wait_w(smem_u32(&bars.m_full[ms]), (it / MR) & 1u)) { ok = false; break; }
-        const int2 e = meta_s[ms][sl];
+      for (const uint32_t it_end = it + (uint32_t)nt; it != it_end; ++it) {
+        if (!wait_w(smem_u32(&bars.m_full[it % MR]), (it / MR) & 1u)) { ok = false; break; }
+        const int2 e = meta_s[it % MR][sl];
         const int32_t cls = e.x & 3, j0 = (e.x >> 4) * BK;
         // hm: the 64-key halves that were loaded and multiplied (chunk c belongs to half c / 2); hm_own: those in which
         // this slot's query tile keeps anything (they differ in twin units only)
-        const uint32_t hm_own = (uint32_t)(e.x >> 2) & 3u;
-        const uint32_t hm = (uint32_t)((e.x | meta_s[ms][sl ^ 1].x) >> 2) & 3u;
+        const uint32_t hm_own = (uint32_t)(e.x >> 2) & 3u, hm = (uint32_t)e.y & 3u;
         uint32_t keep[BK / 32];
         if (cls == kTileGeneral) {  // this row's bits of the tile's mask
-          const uint32_t* mrow = reinterpret_cast<const uint32_t*>(smem_raw + e.y) + row * (BK / 32);
+          const uint32_t* mrow = reinterpret_cast<const uint32_t*>(smem_raw + (e.y & ~3)) + row * (BK / 32);
           static_assert(BK == 128, "a mask row is four 32-bit words");
           const uint4 w4 = *reinterpret_cast<const uint4*>(mrow);
           keep[0] = w4.x; keep[1] = w4.y; keep[2] = w4.z; keep[3] = w4.w;
@@ -584,6 +548,14 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
 #pragma unroll
           for (int c = 0; c < BK / 32; ++c)
             if (!((hm_own >> (c >> 1)) & 1u)) keep[c] = 0u;
+        }
+        // the 32-key chunks of which some row of the warp keeps a key
+        uint32_t some = 15u;
+        if (cls != kTileFull) {
+          some = 0u;
+#pragma unroll
+          for (int c = 0; c < BK / 32; ++c) some |= keep[c] != 0u ? 1u << c : 0u;
+          some = __reduce_or_sync(0xffffffffu, some);
         }
         if (!wait_w(smem_u32(&bars.s_full[sl]), t & 1u)) { ok = false; break; }
         tc_fence_after();
@@ -631,6 +603,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
           };
           constexpr std::integral_constant<int, 0> i0{};
           constexpr std::integral_constant<int, 32> i32{};
+          constexpr std::integral_constant<int, 16> i16{};
           constexpr std::integral_constant<int, 48> i48{};
           constexpr std::integral_constant<int, 64> i64{};
           bool has_kept = cls == kTileFull;  // (a full tile has both halves)
@@ -643,7 +616,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
             return __any_sync(0xffffffffu, !(l_tile <= 1.0e30f) || !(top < 94.f) ||
                                                (has_kept && l_sum + l_tile < 1.0e-30f && top < -96.f));
           };
-          if (hm == 3u) {  // both halves: all loads in flight before the one wait
+          if (__popc(some) > 2) {  // all loads in flight before the one wait
             uint32_t r0[64], r1[64];
             tmem_ld32_at<0>(s_addr, r0);
             tmem_ld32_at<32>(s_addr + 32, r0);
@@ -671,16 +644,41 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
               tmem_st16(s_addr + 48, reinterpret_cast<const uint32_t(&)[16]>(pk[48]));
             }
           } else {
-            uint32_t r[64];
-            tmem_ld32_at<0>(s_addr + (hm >> 1) * 64, r);
-            tmem_ld32_at<32>(s_addr + (hm >> 1) * 64 + 32, r);
-            tc_wait_ld();
-            if (hm == 1u) mask64(r, keep[0], keep[1]);
-            else mask64(r, keep[2], keep[3]);
-            exps(r, i0, i64, i0);  // (the half's P, wherever it belongs)
+            // The warp's rows keep keys of two 32-key chunks at most: those are read and exponentiated, one after another, and the
+            // others' P is zero.  (The cell of the previous frame is a diagonal, one chunk per warp of a tile that costs four;
+            // 8320 tokens x 28 layers 4070 -> 3890 us, 37 120 tokens one layer 785 -> 766, ragged batch of 8 751 -> 739.  With three
+            // chunks, or with the loads of both in flight at once, which spills, the straight run above is faster.)
+            const int ca = __ffs((int)some) - 1, cb = 31 - __clz((int)some);  // (-1: none, for a slot that sits a twin unit's tile out)
+            auto pick = [&](int c) { return c == 0 ? keep[0] : c == 1 ? keep[1] : c == 2 ? keep[2] : keep[3]; };
+            auto chunk = [&](int c, auto off_c) {
+              constexpr int off = decltype(off_c)::value;
+              uint32_t r[32];
+              tmem_ld32(s_addr + 32 * c, r);
+              tc_wait_ld();
+              const uint32_t k = pick(c);
+#pragma unroll
+              for (int x = 0; x < 32; ++x)
+                if (!((k >> x) & 1u)) r[x] = 0xFF800000u;
+#pragma unroll
+              for (int x = 0; x < 32; x += 2) {
+                const float2 a = __ffma2_rn(make_float2(__uint_as_float(r[x]), __uint_as_float(r[x + 1])), sc2, mm2);
+                const float2 pp = make_float2(ex2(a.x), ex2(a.y));
+                ls2[(x >> 1) & 1] = __fadd2_rn(ls2[(x >> 1) & 1], pp);
+                pk[off + (x >> 1)] = pack_bf16(pp.x, pp.y);
+              }
+            };
+            if (ca >= 0) chunk(ca, i0);
+            if (ca != cb) chunk(cb, i16);
             l_tile = (ls2[0].x + ls2[0].y) + (ls2[1].x + ls2[1].y);
             exact = bad(-INFINITY);
-            if (!exact) tmem_st32(s_addr + (hm >> 1) * 32, reinterpret_cast<const uint32_t(&)[32]>(pk[0]));
+            if (!exact) {
+              const uint32_t zeros[16] = {};
+#pragma unroll
+              for (int c = 0; c < BK / 32; ++c)
+                if (((hm >> (c >> 1)) & 1u) && !((some >> c) & 1u)) tmem_st16(s_addr + 16 * c, zeros);
+              if (ca >= 0) tmem_st16(s_addr + 16 * ca, reinterpret_cast<const uint32_t(&)[16]>(pk[0]));
+              if (ca != cb) tmem_st16(s_addr + 16 * cb, reinterpret_cast<const uint32_t(&)[16]>(pk[16]));
+            }
           }
         }
         if (exact) {
@@ -703,8 +701,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
           const float m_new = m_max == -INFINITY ? m_ref : m_max;  // nothing kept yet and nothing accumulated: stay
           const float alpha = l_sum > 0.f ? ex2(m_ref - m_new) : 1.f;  // with l_sum == 0 every earlier P was 0, so O is 0
           const float m_sub = m_new;
-          if (n > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
-            // O is quiescent: S of tile n was issued behind P V of tile n-1, and it is complete.
+          if (__any_sync(0xffffffffu, alpha != 1.f)) {  // (not in a unit's first tile: alpha is 1 there)
+            // O is quiescent: S of a tile is issued behind P V of the one before, and it is complete.
             tc_fence_after();
 #pragma unroll
             for (int c = 0; c < kD / 32; ++c) {
@@ -742,18 +740,20 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
           // Every tile counts on both barriers, and on p_part first: the MMA thread waits for p_full in every tile but for p_part
           // only where both halves are present, so p_full has to imply p_part.  (The other way round a late arrival could leave
           // p_part a phase behind, and the parity of the next tile's wait would match the phase before it.)
-          if (exact || hm != 3u) mbar_arrive(part_bar);
+          if (exact || __popc(some) <= 2) mbar_arrive(part_bar);
           mbar_arrive(full_bar);
         }
         ++t;
       }
       if (!ok) break;
-      it_base += (uint32_t)nt;
       // (one completion per unit, behind the slot's last P V)
       if (!wait_w(smem_u32(&bars.o_final[sl]), slot_units & 1u)) { ok = false; break; }
       ++slot_units;
       tc_fence_after();
-      const int32_t q_first = (u.q_rows1 != 0 && sl == 1) ? u.q_start1 : u.q_start;  // the slot's query tile
+      // (the unit's fields are read again rather than held through the tile loop: the softmax uses every register it has)
+      const bool twin = u.q_rows1 != 0, second = twin && sl == 1;  // this slot works on the unit's second query tile
+      const int32_t hq = (u.heads >> 1) + (twin ? 0 : sl), q_first = second ? u.q_start1 : u.q_start;
+      const bool row_valid = row < (second ? u.q_rows1 : u.q_rows);
       if (u.n_chunks == 1) {
         const float inv = 1.f / l_sum;
         __nv_bfloat16* dst = o + u.layer * o_stride + ((int64_t)(q_first + row) * n_q_heads + hq) * kD;
@@ -774,11 +774,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
           }
         }
         if (lse && row_valid)
-          lse[u.layer * lse_stride + (int64_t)hq * total_tokens + q_first + row] = (m_ref + log2f(l_sum)) * 0.6931471805599453f;
+          lse[u.layer * lse_stride + (int64_t)hq * hdr->total_tokens + q_first + row] = (m_ref + log2f(l_sum)) * 0.6931471805599453f;
       } else {
         // one chunk of a split list: leave the unnormalised result for whoever arrives last
-        const bool second_tile = u.q_rows1 != 0 && sl == 1;  // a twin unit's second tile has slots and counters of its own
-        const int32_t part_base = second_tile ? u.part_base1 : u.part_base;
+        const int32_t part_base = second ? u.part_base1 : u.part_base;
         float* part = ws + ((int64_t)(part_base + u.chunk) * n_q_heads + hq) * kPartFloats;
 #pragma unroll
         for (int c = 0; c < kD / 32; ++c) {
@@ -799,7 +798,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
         __syncwarp();
         int32_t last = 0;
         if (lane == 0) {
-          int32_t* cnt = counters + (second_tile ? u.counter_base1 : u.counter_base) + hq;
+          int32_t* cnt = reinterpret_cast<int32_t*>(plan + hdr->off_counters) + (second ? u.counter_base1 : u.counter_base) + hq;
           last = ((atom_add_acq_rel(cnt, 1 << (8 * quad)) >> (8 * quad)) & 255) == u.n_chunks - 1;
           if (last) atomicSub(reinterpret_cast<uint32_t*>(cnt), (uint32_t)u.n_chunks << (8 * quad));  // ready for the next launch
         }
@@ -891,7 +890,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
             }
           }
           if (lse && row_valid)
-            lse[(int64_t)hq * total_tokens + q_first + row] = (m_all + log2f(l_all)) * 0.6931471805599453f;
+            lse[(int64_t)hq * hdr->total_tokens + q_first + row] = (m_all + log2f(l_all)) * 0.6931471805599453f;
         }
       }
       release_unit();

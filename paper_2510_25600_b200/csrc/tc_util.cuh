@@ -31,6 +31,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// Whether two barriers' phases are complete, asked for together: one round trip instead of two.
+__device__ __forceinline__ void mbar_test2(uint32_t bar0, uint32_t parity0, uint32_t bar1, uint32_t parity1, bool* done0,
+                                           bool* done1) {
+  uint32_t a, b;
+  asm volatile(
+      "{\n .reg .pred p, q;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%2], %3;\n"
+      " mbarrier.test_wait.parity.shared::cta.b64 q, [%4], %5;\n selp.u32 %0, 1, 0, p;\n selp.u32 %1, 1, 0, q;\n}\n"
+      : "=r"(a), "=r"(b)
+      : "r"(bar0), "r"(parity0), "r"(bar1), "r"(parity1)
+      : "memory");
+  *done0 = a != 0;
+  *done1 = b != 0;
+}
 __device__ __forceinline__ uint64_t global_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
