@@ -167,8 +167,8 @@ struct Stream {
 // One CTA per (request, KV head, layer) over the scores `s` (written by vnorm_score_kernel).  `staged`: the launch has
 // room in shared memory for the segment's keys.  With T the element type of V the CTA forms the scores of its segment itself,
 // from `own`, and they go no further than its shared memory (as vnorm_score_kernel sums them: bit for bit the same).
-template <typename T, bool GATHER>
-__global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __restrict__ s, int64_t n_tokens,
+template <typename T, bool GATHER, int kThreads = kSelThreads>
+__global__ void __launch_bounds__(kThreads) select_kernel(const float* __restrict__ s, int64_t n_tokens,
                                                              const int32_t* __restrict__ cu_seqlens,
                                                              const int32_t* __restrict__ cu_kept,
                                                              const int32_t* __restrict__ keep, int32_t window,
@@ -200,12 +200,12 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __rest
   int32_t* out = idx_out + ((int64_t)layer * n_kv_heads + g) * k_tot + cu_kept[r];
   const int32_t tid = threadIdx.x;
 
-  for (int32_t t = tid; t < w; t += kSelThreads) out[h + t] = nr + t;  // the recent window
+  for (int32_t t = tid; t < w; t += kThreads) out[h + t] = nr + t;  // the recent window
   if constexpr (kOwn) {  // a half-warp per row, 16 rows of each in flight
     const uint4* vl = own.v + layer * own.layer_stride_c;
     const float* cg = own.c + (int64_t)g * n_tokens + base;
     const int32_t half = (tid >> 4) & 1, ch = tid & 15;
-    for (int32_t t0 = (tid >> 5) * 32; t0 < nr; t0 += kSelThreads) {
+    for (int32_t t0 = (tid >> 5) * 32; t0 < nr; t0 += kThreads) {
       uint4 buf[16];
 #pragma unroll
       for (int it = 0; it < 16; ++it) {  // rows past the end read the last one again; never stored
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __rest
   uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
   if (!kOwn && staged) {  // copied into shared memory once, so the radix passes do not go back to L2
 #pragma unroll 8
-    for (int32_t j = tid; j < nr; j += kSelThreads) {  // loads of a trip in flight together
+    for (int32_t j = tid; j < nr; j += kThreads) {  // loads of a trip in flight together
       const uint32_t key = order_key(__ldg(seg + j));
       skeys[j] = key;
       kmin = min(kmin, key);
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __rest
 
   if (kOwn || !staged) {
 #pragma unroll 4
-    for (int32_t j = tid; j < nr; j += kSelThreads) {
+    for (int32_t j = tid; j < nr; j += kThreads) {
       const uint32_t key = key_at(j);
       kmin = min(kmin, key);
       kmax = max(kmax, key);
@@ -260,8 +260,8 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __rest
   if (lane == 0) { warp_gt[warp] = (int32_t)kmin; warp_eq[warp] = (int32_t)kmax; }
   __syncthreads();
   if (warp == 0) {
-    uint32_t a = lane < kSelThreads / 32 ? (uint32_t)warp_gt[lane] : 0xFFFFFFFFu;
-    uint32_t b = lane < kSelThreads / 32 ? (uint32_t)warp_eq[lane] : 0u;
+    uint32_t a = lane < kThreads / 32 ? (uint32_t)warp_gt[lane] : 0xFFFFFFFFu;
+    uint32_t b = lane < kThreads / 32 ? (uint32_t)warp_eq[lane] : 0u;
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) {
       a = min(a, __shfl_xor_sync(0xffffffffu, a, d));
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __rest
     // publishes is read by everybody before anybody can reach the next pass's first barrier
     for (int32_t shift = max(nbits - 8, 0);; shift = max(shift - 8, 0)) {
 #pragma unroll 4
-      for (int32_t j = tid; j < nr; j += kSelThreads) {
+      for (int32_t j = tid; j < nr; j += kThreads) {
         const uint32_t key = key_at(j);
         if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255], 1);
       }
@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __rest
   // ---- ordered compaction: one contiguous run of keys per thread, one block scan ---------------------------------
   // runs of a multiple of 4 keys (128-bit loads) whose number of 16-byte words is odd, so that the quarter-warps'
   // loads fall into different banks
-  const int32_t per = 4 * (((nr + kSelThreads * 4 - 1) / (kSelThreads * 4)) | 1);
+  const int32_t per = 4 * (((nr + kThreads * 4 - 1) / (kThreads * 4)) | 1);
   const int32_t j0 = min(nr, tid * per), j1 = min(nr, j0 + per);
   int32_t n_gt = 0, n_eq = 0;
   for (int32_t j = j0; j < j1; j += 4) {
@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __rest
   if (lane == 31) { warp_gt[warp] = inc_gt; warp_eq[warp] = inc_eq; }
   __syncthreads();
   if (warp == 0) {
-    int32_t a = lane < kSelThreads / 32 ? warp_gt[lane] : 0, b = lane < kSelThreads / 32 ? warp_eq[lane] : 0;
+    int32_t a = lane < kThreads / 32 ? warp_gt[lane] : 0, b = lane < kThreads / 32 ? warp_eq[lane] : 0;
     const int32_t ta = a, tb = b;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __rest
   // ---- gather (optional): the CTA copies the rows it has just chosen, K and V, into the compact cache ----------
   if constexpr (GATHER) {
     __syncthreads();  // every index of the segment (written above by this CTA's threads) is visible to all of them
-    const int32_t n_keep = h + w, cpr = ga.cpr, rows_per_step = kSelThreads / cpr;
+    const int32_t n_keep = h + w, cpr = ga.cpr, rows_per_step = kThreads / cpr;
     const int32_t ch = tid % cpr, r_in = tid / cpr;
     const uint4* ks = ga.k_src + layer * ga.src_layer_stride_c;
     const uint4* vs = ga.v_src + layer * ga.src_layer_stride_c;
@@ -588,15 +588,20 @@ static purekv_status select_impl(const float* c, const void* v, int64_t v_layer_
   const purekv_status st_v = dtype == PUREKV_BF16 ? launch_vnorm(__nv_bfloat16{}) : launch_vnorm(float{});
   if (st_v != PUREKV_OK) return st_v;
   const bool stage_keys = key_bytes <= 200 * 1024;
+  // A segment's selection is a chain of latencies; where every CTA finds an SM of its own, 1024 threads go through a long list in
+  // half the trips (104 segments, selection and compaction in a row: of 13 393 keys 130 -> 122 us, of 8320 77.9 -> 77.4; of 3977
+  // no difference, and more segments than SMs take turns).
+  const bool wide = !gather && (int64_t)batch->n_req * n_kv_heads * n_layers <= 148 && longest >= 4096;
   if (stage_keys) {
-    static std::atomic<uint64_t> smem_allowed{0}, smem_allowed_g{0};
+    static std::atomic<uint64_t> smem_allowed{0}, smem_allowed_g{0}, smem_allowed_w{0};
     const purekv_status st_smem = gather ? allow_max_dynamic_smem(select_kernel<void, true>, smem_allowed_g)
+                                  : wide ? allow_max_dynamic_smem(select_kernel<void, false, 1024>, smem_allowed_w)
                                          : allow_max_dynamic_smem(select_kernel<void, false>, smem_allowed);
     if (st_smem != PUREKV_OK) return st_smem;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = g2;
-  cfg.blockDim = dim3(kSelThreads);
+  cfg.blockDim = dim3(wide ? 1024 : kSelThreads);
   cfg.dynamicSmemBytes = stage_keys ? key_bytes : 0;
   cfg.stream = sm;
   cudaLaunchAttribute attr[1];
@@ -606,6 +611,9 @@ static purekv_status select_impl(const float* c, const void* v, int64_t v_layer_
   cfg.numAttrs = 1;
   if (gather)
     PK_CUDA(cudaLaunchKernelEx(&cfg, select_kernel<void, true>, (const float*)s_buf, T, batch->cu_seqlens, cu_kept,
+                               keep, window, k_tot, n_kv_heads, idx_out, stage_keys, ga, Stream{}));
+  else if (wide)
+    PK_CUDA(cudaLaunchKernelEx(&cfg, select_kernel<void, false, 1024>, (const float*)s_buf, T, batch->cu_seqlens, cu_kept,
                                keep, window, k_tot, n_kv_heads, idx_out, stage_keys, ga, Stream{}));
   else
     PK_CUDA(cudaLaunchKernelEx(&cfg, select_kernel<void, false>, (const float*)s_buf, T, batch->cu_seqlens, cu_kept,
