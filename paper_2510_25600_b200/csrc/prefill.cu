@@ -43,7 +43,7 @@ static purekv_status prefill(const char* name, const void* q, const void* k, con
   const bool apart = q_stride >= t * n_q_heads * head_dim && o_stride >= t * n_q_heads * head_dim &&
                      kv_stride >= t * n_kv_heads * head_dim && (lse == nullptr || lse_stride >= t * n_q_heads) &&
                      q_stride * esz % 16 == 0 && kv_stride * esz % 16 == 0 && o_stride * esz % 32 == 0 &&
-                     std::max(q_stride, kv_stride) < (1ll << 38);
+                     std::max({q_stride, kv_stride, o_stride}) < (1ll << 38);
   if (n_layers == 1 || (tc && apart && info->max_chunks == 1 && (int64_t)info->n_units * n_layers <= INT32_MAX / 2))
     return tc ? launch_prefill_tc(a) : launch_prefill_simt(a);
   a.n_layers = 1;

@@ -17,8 +17,8 @@
 //               warps 8-11): the row of S from TMEM into registers, the
 //               tile's predicate (none / causal / bit mask), online softmax in the log2 domain against a
 //               reference that moves only when exp2 would overflow (then O is rescaled), bf16 P written
-//               over S; at the end of a unit either the normalised output
-//               (whole list in one unit) or an unnormalised fp32 partial result plus (max, sum) per row
+//               over S; at the end of a unit either the normalised output (whole list in one unit; whole query
+//               tiles go to shared memory for warp 10 to copy out) or an unnormalised fp32 partial result plus (max, sum) per row
 //               into the workspace.  The warp that finishes its rows of a split list last (a counter in the plan)
 //               combines the partial results in chunk order, so the result does not depend on timing.
 // Every wait on an mbarrier is bounded in time; on expiry the CTA raises a shared abort flag,
@@ -32,8 +32,8 @@ namespace purekv {
 namespace tc {
 
 constexpr int kBQ = 128;
-constexpr int kThreads = 384;  // warps 0-3 softmax of slot 0, warps 4-7 of slot 1, warp 8 producer, warp 9 MMA, 10-11 idle
-constexpr int kWarpProducer = 8, kWarpMma = 9;
+constexpr int kThreads = 384;  // warps 0-3 softmax of slot 0, warps 4-7 of slot 1, warp 8 producer, warp 9 MMA, warp 10 output, 11 idle
+constexpr int kWarpProducer = 8, kWarpMma = 9, kWarpStore = 10;
 // Per-thread registers after the warpgroups trade them.  setmaxnreg only moves registers inside the CTA's launch
 // allocation (kThreads x the count ptxas gives the kernel, 168 at 384 threads); asking for more would block forever,
 // so the launch code checks the budget against the compiled register count.
@@ -60,7 +60,8 @@ struct __align__(8) Barriers {
   uint64_t p_full[2];      // softmax -> MMA: all of P written
   uint64_t o_final[2];     // one completion per unit, after the slot's last P.V product
   uint64_t u_full[kUnitRing];   // the producer published a unit (or the end mark) in unit_s[]
-  uint64_t u_empty[kUnitRing];  // the MMA thread and the eight softmax warps have copied it
+  uint64_t u_empty[kUnitRing];  // the MMA thread, the eight softmax warps and the storing thread have copied it
+  uint64_t o_staged[2];    // softmax -> storing thread: the slot's output tile is in shared memory
   uint64_t drain;
 };
 
@@ -69,7 +70,7 @@ template <int BK>
 __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
     const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_k64,
-    const __grid_constant__ CUtensorMap tm_v64, __nv_bfloat16* __restrict__ o, float* __restrict__ lse,
+    const __grid_constant__ CUtensorMap tm_v64, const __grid_constant__ CUtensorMap tm_o, __nv_bfloat16* __restrict__ o, float* __restrict__ lse,
     uint8_t* __restrict__ plan, float* __restrict__ ws, int32_t n_q_heads, int32_t n_kv_heads, float scale_log2,
     int32_t* __restrict__ status, uint64_t wait_ns, int64_t plan_bytes, int64_t ws_floats, int32_t n_layers, int64_t o_stride,
     int64_t lse_stride) {
@@ -114,10 +115,11 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       mbar_init(smem_u32(&bars.p_full[sl]), 4);
       mbar_init(smem_u32(&bars.p_part[sl]), 4);
       mbar_init(smem_u32(&bars.o_final[sl]), 1);
+      mbar_init(smem_u32(&bars.o_staged[sl]), 4);
     }
     for (int s = 0; s < kUnitRing; ++s) {
       mbar_init(smem_u32(&bars.u_full[s]), 1);
-      mbar_init(smem_u32(&bars.u_empty[s]), 9);
+      mbar_init(smem_u32(&bars.u_empty[s]), 10);
     }
     mbar_init(smem_u32(&bars.drain), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -179,6 +181,15 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
   const int64_t part_slots = plan_ok ? hdr->part_slots : 0;
   const bool withhold_first_k = plan_ok && (hdr->test_flags & 1u) != 0u;
   const bool start_ok = abort_s == 0 && plan_ok;
+  // Whether a unit's output leaves through shared memory: whole query tiles of whole lists.  The rows of a tile lie thousands of
+  // bytes apart; stored from registers each warp store touches 32 lines, and a unit's output took 2250-3400 clk of its rows' time.
+  // Through shared memory it is one copy per slot that the copy engine makes beside the next unit's first tile.  The room is the
+  // stages of the unit's last tile, whose next contents are not wanted before the next unit's second tile: K's for slot 0
+  // (both slots' S of that tile are long complete), V's for slot 1 (its last product is the unit's last).  Ragged batch of 8, sparse
+  // layer: 618 -> 595 us at full clock, 725 -> 701 in a row; 37 120 tokens 653 -> 643 and 762 -> 749; the copies by rolled loops,
+  // because of the instruction cache.
+  auto output_staged = [](const Unit& u) { return u.n_chunks == 1 && u.q_rows == kBQ && (u.q_rows1 == 0 || u.q_rows1 == kBQ); };
+
   // the two softmax warpgroups take registers from the warpgroup of the producer and MMA warps
 
   if (warp >= 8) {
@@ -396,6 +407,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
         if (!ok) break;
         const int32_t nt = unit_s[us].ent_count;
         const uint32_t last_slot = (uint32_t)unit_s[us].heads & 1u;
+        const bool staged = output_staged(unit_s[us]);
         mbar_arrive(smem_u32(&bars.u_empty[us]));
         if (nt == 0) break;
         ok = mbar_wait(smem_u32(&bars.q_full), uo & 1u, abort_flag, wait_ns);
@@ -462,8 +474,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
             tc_commit(smem_u32(qk ? &bars.s_full[sl] : &bars.o_final[sl]));
           }
           if (!ok) break;
-          if (pv) tc_commit(smem_u32(&bars.v_empty[s]));
-          if (qk) tc_commit(smem_u32(&bars.k_empty[sn]));
+          // (the last tile's stages: the output goes through them, see output_staged)
+          if (pv && (qk || !staged || last_slot == 0u)) tc_commit(smem_u32(&bars.v_empty[s]));
+          if (qk && (n + 2 < nt || !staged)) tc_commit(smem_u32(&bars.k_empty[sn]));
           if (n + 2 == nt) tc_commit(smem_u32(&bars.q_empty));  // the unit's last read of Q
           if (pv) {
             ++it;
@@ -478,6 +491,39 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
         const uint64_t t0 = global_ns();
         while (!mbar_try_wait(smem_u32(&bars.drain), 0) && global_ns() - t0 < wait_ns) {}
       }
+    }
+  } else if (start_ok && warp == kWarpStore) {
+    // ---------------- output: staged tiles to global memory ----------------
+    if (lane == 0) {
+      uint32_t it = 0, n_staged[2] = {0u, 0u};  // key tiles so far; tiles staged by each slot
+      bool ok = true;
+      for (uint32_t uo = 0; ok; ++uo) {
+        const uint32_t us = uo % kUnitRing;
+        ok = mbar_wait(smem_u32(&bars.u_full[us]), (uo / kUnitRing) & 1u, abort_flag, wait_ns);
+        if (!ok) break;
+        const Unit& u = unit_s[us];
+        const int32_t nt = u.ent_count;
+        if (nt == 0) break;
+        it += (uint32_t)nt;
+        if (output_staged(u)) {
+          const uint32_t s = (it - 1u) % ST;
+          const bool twin = u.q_rows1 != 0;
+#pragma unroll
+          for (int sl = 0; sl < 2; ++sl) {
+            if (sl > (u.heads & 1)) break;
+            ok = mbar_wait(smem_u32(&bars.o_staged[sl]), n_staged[sl]++ & 1u, abort_flag, wait_ns);
+            if (!ok) break;
+            const uint32_t buf = (sl == 0 ? sK : sV) + s * kTileKV;
+            const int32_t hq = (u.heads >> 1) + (twin ? 0 : sl), q_first = twin && sl == 1 ? u.q_start1 : u.q_start;
+            tma_store_4d(&tm_o, buf, 0, hq, q_first, u.layer);
+            tma_store_4d(&tm_o, buf + kPanelKV, 64, hq, q_first, u.layer);
+            asm volatile("cp.async.bulk.commit_group;\n cp.async.bulk.wait_group.read 0;" ::: "memory");
+            mbar_arrive(smem_u32(sl == 0 ? &bars.k_empty[s] : &bars.v_empty[s]));  // in the MMA thread's place
+          }
+        }
+        if (ok) mbar_arrive(smem_u32(&bars.u_empty[us]));
+      }
+      asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
   }
   } else {
@@ -754,10 +800,31 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       const bool twin = u.q_rows1 != 0, second = twin && sl == 1;  // this slot works on the unit's second query tile
       const int32_t hq = (u.heads >> 1) + (twin ? 0 : sl), q_first = second ? u.q_start1 : u.q_start;
       const bool row_valid = row < (second ? u.q_rows1 : u.q_rows);
-      if (u.n_chunks == 1) {
+      if (output_staged(u)) {
+        const float inv = 1.f / l_sum;
+        const uint32_t buf = (sl == 0 ? sK : sV) + ((it - 1u) % ST) * kTileKV + (uint32_t)row * 128u;
+#pragma unroll 1
+        for (int c = 0; c < kD / 32; ++c) {
+          uint32_t tt[32];
+          tmem_ld32(t_lane + kColO + sl * 128 + 32 * c, tt);
+          tc_wait_ld();
+#pragma unroll
+          for (int y = 0; y < 4; ++y) {  // 16 bytes each, placed as the 128-byte swizzle has them
+            uint32_t w[4];
+#pragma unroll
+            for (int z = 0; z < 4; ++z)
+              w[z] = pack_bf16(__uint_as_float(tt[8 * y + 2 * z]) * inv, __uint_as_float(tt[8 * y + 2 * z + 1]) * inv);
+            st_shared_v4(buf + (uint32_t)(c >> 1) * kPanelKV + ((uint32_t)((4 * (c & 1) + y) ^ (row & 7)) << 4), w);
+          }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the copy out reads what these stores wrote
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bars.o_staged[sl]));
+        if (lse) lse[u.layer * lse_stride + (int64_t)hq * hdr->total_tokens + q_first + row] = (m_ref + log2f(l_sum)) * 0.6931471805599453f;
+      } else if (u.n_chunks == 1) {
         const float inv = 1.f / l_sum;
         __nv_bfloat16* dst = o + u.layer * o_stride + ((int64_t)(q_first + row) * n_q_heads + hq) * kD;
-#pragma unroll
+#pragma unroll 1
         for (int c = 0; c < kD / 32; ++c) {
           uint32_t tt[32];
           tmem_ld32(t_lane + kColO + sl * 128 + 32 * c, tt);
@@ -908,7 +975,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
 }
 
 static purekv_status launch(const PrefillArgs& a, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
-                            const CUtensorMap& mk64, const CUtensorMap& mv64, int32_t* status) {
+                            const CUtensorMap& mk64, const CUtensorMap& mv64, const CUtensorMap& mo, int32_t* status) {
   constexpr int BK = 128;
   const size_t smem = 1024 + 2 * 2 * (size_t)kBQ * 128 + 2 * (size_t)Cfg<BK>::kStages * 2 * BK * 128 +
                       2 * (size_t)Cfg<BK>::kMeta * Cfg<BK>::kMaskBytes;
@@ -938,7 +1005,7 @@ static purekv_status launch(const PrefillArgs& a, const CUtensorMap& mq, const C
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  PK_CUDA(cudaLaunchKernelEx(&cfg, prefill_tc_kernel<BK>, mq, mk, mv, mk64, mv64, (__nv_bfloat16*)a.o, a.lse,
+  PK_CUDA(cudaLaunchKernelEx(&cfg, prefill_tc_kernel<BK>, mq, mk, mv, mk64, mv64, mo, (__nv_bfloat16*)a.o, a.lse,
                              (uint8_t*)a.plan, (float*)a.ws, a.n_q_heads, a.n_kv_heads,
                              a.scale * 1.4426950408889634f, status, wait_limit_ns(), (int64_t)a.info->bytes_used,
                              (int64_t)(a.ws_bytes / sizeof(float)), a.n_layers, a.o_stride, a.lse_stride));
@@ -955,7 +1022,7 @@ purekv_status launch_prefill_tc(const PrefillArgs& a) {
   PK_REQUIRE(a.info->n_ctas >= 1 && a.info->n_units >= 1, PUREKV_ERR_INVALID_ARG, "plan holds no schedule");
   PK_REQUIRE((uintptr_t)a.o % 32 == 0, PUREKV_ERR_INVALID_ARG, "O must be 32-byte aligned for the tensor-core kernel");
   const int64_t T = a.batch->total_tokens;
-  CUtensorMap mq, mk, mv, mk64, mv64;
+  CUtensorMap mq, mk, mv, mk64, mv64, mo;
   purekv_status st;
   const int32_t L = a.n_layers;
   const int64_t q_stride = L > 1 ? a.q_stride : T * a.n_q_heads * kD, kv_stride = L > 1 ? a.kv_stride : T * a.n_kv_heads * kD;
@@ -964,12 +1031,13 @@ purekv_status launch_prefill_tc(const PrefillArgs& a) {
   if ((st = make_map_layers(&mv, a.v, T, a.n_kv_heads, 128, L, kv_stride)) != PUREKV_OK) return st;
   if ((st = make_map_layers(&mk64, a.k, T, a.n_kv_heads, 64, L, kv_stride)) != PUREKV_OK) return st;
   if ((st = make_map_layers(&mv64, a.v, T, a.n_kv_heads, 64, L, kv_stride)) != PUREKV_OK) return st;
+  if ((st = make_map_layers(&mo, a.o, T, a.n_q_heads, kBQ, L, L > 1 ? a.o_stride : T * a.n_q_heads * kD)) != PUREKV_OK) return st;
   int32_t* status = a.status;
   if (!status) {
     const purekv_status st_w = default_status_word(&status);
     if (st_w != PUREKV_OK) return st_w;
   }
-  return launch(a, mq, mk, mv, mk64, mv64, status);
+  return launch(a, mq, mk, mv, mk64, mv64, mo, status);
 }
 
 }  // namespace purekv
