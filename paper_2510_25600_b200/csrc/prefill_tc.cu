@@ -187,8 +187,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
   // stages of the unit's last tile, whose next contents are not wanted before the next unit's second tile: K's for slot 0
   // (both slots' S of that tile are long complete), V's for slot 1 (its last product is the unit's last).  Ragged batch of 8, sparse
   // layer: 618 -> 595 us at full clock, 725 -> 701 in a row; 37 120 tokens 653 -> 643 and 762 -> 749; the copies by rolled loops,
-  // because of the instruction cache.
-  auto output_staged = [](const Unit& u) { return u.n_chunks == 1 && u.q_rows == kBQ && (u.q_rows1 == 0 || u.q_rows1 == kBQ); };
+  // because of the instruction cache.  Launches of few units per CTA store from registers: their last outputs are a larger share of
+  // the time, and the way through shared memory is the longer one (304 units for 148 CTAs 43.0 and 45.5 us, 672 126.1 and 125.0).
+  const bool many_units = n_work >= 4 * (int32_t)gridDim.x;
+  auto output_staged = [&](const Unit& u) { return many_units && u.n_chunks == 1 && u.q_rows == kBQ && (u.q_rows1 == 0 || u.q_rows1 == kBQ); };
 
   // the two softmax warpgroups take registers from the warpgroup of the producer and MMA warps
 

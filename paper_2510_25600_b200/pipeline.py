@@ -44,9 +44,10 @@ class PureKVPipeline:
         hh = (n_q_heads, n_kv_heads)
         self.n_dense = min(n_layers, self.clie + 1)
         self.n_sparse = n_layers - self.n_dense
+        # room for a plan of one layer at a time (build_plans, prefill_layer) and for one of all layers under the mask (run_device)
         plan_buf = lambda params, layers: torch.empty(
-            max(1, P.purekv_plan_bytes(self.batch, params, self.code, head_dim, *hh, n_layers=max(1, layers))), dtype=torch.uint8,
-            device=dev)
+            max(1, *(P.purekv_plan_bytes(self.batch, params, self.code, head_dim, *hh, n_layers=n) for n in {1, max(1, layers)})),
+            dtype=torch.uint8, device=dev)
         self.plan_buf_dense, self.plan_buf_st = plan_buf(params_dense, self.n_dense), plan_buf(self.params_st, self.n_sparse)
         self.prefill_ws = None
         # per mask a ring of pinned buffers, each with the event behind its last copy; the last one used comes first
@@ -99,10 +100,10 @@ class PureKVPipeline:
                 runs.append([layer, layer + 1])
         return runs
 
-    def _plan(self, params, ring: list, d_buf: torch.Tensor, layers: int) -> P.Plan:
-        """Plans one mask on the host into a pinned buffer and enqueues its copy on the current stream without waiting, so
-        planning overlaps the GPU work already in flight.  A small ring of pinned buffers keeps a plan alive until its copy
-        has run."""
+    def _plan(self, params, ring: list, d_buf: torch.Tensor, layers: int = 1) -> P.Plan:
+        """Plans one mask, for launches of `layers` layers, on the host into a pinned buffer and enqueues its copy on the
+        current stream without waiting, so planning overlaps the GPU work already in flight.  A small ring of pinned buffers
+        keeps a plan alive until its copy has run."""
         ring.append(ring.pop(0))
         h_buf, ev = ring[0]
         if ev is not None:
@@ -110,7 +111,7 @@ class PureKVPipeline:
         else:
             ev = ring[0][1] = torch.cuda.Event()
         _, info = P.purekv_plan_build_host(self.batch, params, self.code, self.d, self.h, self.hkv, out=h_buf,
-                                           n_layers=max(1, layers))
+                                           n_layers=layers)
         d_buf.copy_(h_buf, non_blocking=True)
         ev.record()
         return P.Plan(d_buf, info)
@@ -119,7 +120,7 @@ class PureKVPipeline:
     def plan_st(self) -> P.Plan:
         """The sparse mask's plan.  A pass without sparse layers does not need it: it is then made when asked for."""
         if self._plan_st is None:
-            self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st, self.n_sparse)
+            self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st)
             self._size_prefill_ws(self._plan_st)
         return self._plan_st
 
@@ -129,9 +130,10 @@ class PureKVPipeline:
             self.prefill_ws = torch.empty(need, dtype=torch.uint8, device="cuda")
 
     def build_plans(self) -> None:
-        """Both masks' plans; `run_device` builds each just ahead of the first layer that needs it."""
-        self.plan_dense = self._plan(self.params_dense, self._h_dense, self.plan_buf_dense, self.n_dense)
-        self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st, self.n_sparse)
+        """Both masks' plans, for `prefill_layer` calls; `run_device` builds its own, each just ahead of the first layer that
+        needs it."""
+        self.plan_dense = self._plan(self.params_dense, self._h_dense, self.plan_buf_dense)
+        self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st)
         self._size_prefill_ws(self.plan_dense)
         self._size_prefill_ws(self.plan_st)
 
@@ -171,7 +173,8 @@ class PureKVPipeline:
         before = torch.cuda.Event() if self.n_sparse else None
         if before is not None:
             before.record()
-        self.plan_dense = self._plan(self.params_dense, self._h_dense, self.plan_buf_dense, self.n_dense)
+        alone = events is not None  # each layer a launch of its own
+        self.plan_dense = self._plan(self.params_dense, self._h_dense, self.plan_buf_dense, 1 if alone else self.n_dense)
         self._size_prefill_ws(self.plan_dense)
         if marks is not None:
             marks[0].record()
@@ -182,7 +185,7 @@ class PureKVPipeline:
             main = torch.cuda.current_stream()
             self._copies.wait_event(before)
             with torch.cuda.stream(self._copies):
-                self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st, self.n_sparse)
+                self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st, 1 if alone else self.n_sparse)
             main.wait_event(self._h_st[0][1])
             self._size_prefill_ws(self._plan_st)
             self._prefill(self._plan_st, self.sparse_runs, q, k, v, events)

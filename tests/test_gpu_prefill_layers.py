@@ -84,3 +84,26 @@ def test_layers_that_cannot_share_a_launch(dtype, n_layers):
     out = pk.purekv_st_sparse_prefill_layers(q, k, v, b, plan)
     for n in range(3):
         assert torch.equal(out[n], pk.purekv_st_sparse_prefill(q[n], k[n], v[n], b, plan))
+
+
+@pytest.mark.gpu
+def test_a_pass_in_launches_of_many_layers_is_the_layers_one_by_one():
+    from paper_2510_25600_b200.pipeline import PureKVPipeline
+    batch = inputs.make_batch([10, 3], [12, 5], [20, 140], 12, 12)
+    mask = inputs.STMask(12, 12, tile=64)
+    wl = inputs.Workload("p", 3, "bf16", 4, 2, 128, 6, (0, 1), (2, 3, 4, 5), batch, mask, 16, 0.3)
+    xs = [inputs.make_qkv(wl, n) for n in range(6)]
+    q, k, v = (torch.stack([gc.upload(x, n, "bf16") for x in xs]) for n in "qkv")
+    pipe = PureKVPipeline(batch.seq_lens, batch.n_prefix, batch.n_frames, mask, 6, 4, 2, 128, q.dtype, (0, 1), (2, 3, 4, 5), 16, 0.3)
+    pipe.run_device(q, k, v)
+    assert pipe.prefill_launches == 2 and pipe.plan_st.info.max_chunks == 1
+    o, lse = pipe.o.clone(), pipe.lse.clone()
+    pipe.o.fill_(float("nan"))
+    pipe.lse.fill_(float("nan"))
+    pipe.build_plans()  # for a layer at a time: lists are cut where that ends a launch sooner
+    for n in range(6):
+        pipe.prefill_layer(n, q[n], k[n], v[n])
+    pipe.check_status()
+    # either way of summing rounds P and the output to bf16: each is within the oracle's tolerance, the two within both
+    assert (pipe.o.float() - o.float()).abs().max().item() <= 2 * gc.ATTN_TOL["bf16"]
+    assert (pipe.lse - lse).abs().max().item() <= 2 * 2e-3
