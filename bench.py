@@ -40,10 +40,10 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 NOMINAL_TFLOPS, NOMINAL_HBM_GBS = 2250.0, 8000.0   # B200 dense bf16 and HBM3e figures, for context beside the measured peaks
 
 
-# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one ST-SpAttn launch of the tensor-core prefill
+# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of an ST-SpAttn launch of one layer of the tensor-core prefill
 # kernel, from the ncu capture summarised under profiles/.  It is reported only while the kernel and planner
 # sources are the ones the capture was taken from (sha1 of their text); otherwise the roofline's traffic is null.
-NCU_TRAFFIC = {"cfg2_qwen25vl": {"bytes_per_launch": 113.0e6, "source_sha1": "3f5bace0115fe546dd4006c15381e73169a4d358"}}
+NCU_TRAFFIC = {"cfg2_qwen25vl": {"bytes_per_launch": 107.2e6, "source_sha1": "9379bbb3ca43e5e536c9403b9966053172a0ca86"}}
 KERNEL_SOURCES = ("prefill_tc.cu", "tc_util.cuh", "plan.cu", "common.cuh", "prefill.cuh")
 
 
