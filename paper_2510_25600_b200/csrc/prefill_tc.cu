@@ -61,7 +61,9 @@ struct __align__(8) Barriers {
   uint64_t o_final[2];     // one completion per unit, after the slot's last P.V product
   uint64_t u_full[kUnitRing];   // the producer published a unit (or the end mark) in unit_s[]
   uint64_t u_empty[kUnitRing];  // the MMA thread, the eight softmax warps and the storing thread have copied it
-  uint64_t o_staged[2];    // softmax -> storing thread: the slot's output tile is in shared memory
+  uint64_t o_staged[2][ST];  // softmax -> storing thread: the slot's output tile is in that stage.  A barrier per stage, because
+                             // a slot may be a unit of one tile (in the other stage) ahead of the copies; a stage is its own
+                             // again only when the storing thread has given it back, which is after its wait
   uint64_t drain;
 };
 
@@ -115,7 +117,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       mbar_init(smem_u32(&bars.p_full[sl]), 4);
       mbar_init(smem_u32(&bars.p_part[sl]), 4);
       mbar_init(smem_u32(&bars.o_final[sl]), 1);
-      mbar_init(smem_u32(&bars.o_staged[sl]), 4);
+      for (int s = 0; s < ST; ++s) mbar_init(smem_u32(&bars.o_staged[sl][s]), 4);
     }
     for (int s = 0; s < kUnitRing; ++s) {
       mbar_init(smem_u32(&bars.u_full[s]), 1);
@@ -497,7 +499,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
   } else if (start_ok && warp == kWarpStore) {
     // ---------------- output: staged tiles to global memory ----------------
     if (lane == 0) {
-      uint32_t it = 0, n_staged[2] = {0u, 0u};  // key tiles so far; tiles staged by each slot
+      uint32_t it = 0, phases = 0u;  // key tiles so far; bit sl * ST + s: the parity of the next phase of o_staged[sl][s]
       bool ok = true;
       for (uint32_t uo = 0; ok; ++uo) {
         const uint32_t us = uo % kUnitRing;
@@ -513,8 +515,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
 #pragma unroll
           for (int sl = 0; sl < 2; ++sl) {
             if (sl > (u.heads & 1)) break;
-            ok = mbar_wait(smem_u32(&bars.o_staged[sl]), n_staged[sl]++ & 1u, abort_flag, wait_ns);
+            const uint32_t bit = (uint32_t)sl * ST + s;
+            ok = mbar_wait(smem_u32(&bars.o_staged[sl][s]), (phases >> bit) & 1u, abort_flag, wait_ns);
             if (!ok) break;
+            phases ^= 1u << bit;
             const uint32_t buf = (sl == 0 ? sK : sV) + s * kTileKV;
             const int32_t hq = (u.heads >> 1) + (twin ? 0 : sl), q_first = twin && sl == 1 ? u.q_start1 : u.q_start;
             tma_store_4d(&tm_o, buf, 0, hq, q_first, u.layer);
@@ -821,7 +825,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the copy out reads what these stores wrote
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&bars.o_staged[sl]));
+        if (lane == 0) mbar_arrive(smem_u32(&bars.o_staged[sl][(it - 1u) % ST]));
         if (lse) lse[u.layer * lse_stride + (int64_t)hq * hdr->total_tokens + q_first + row] = (m_ref + log2f(l_sum)) * 0.6931471805599453f;
       } else if (u.n_chunks == 1) {
         const float inv = 1.f / l_sum;

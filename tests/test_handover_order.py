@@ -1,7 +1,8 @@
 """The two barriers over which a slot's four softmax warps hand P to the MMA thread: p_part (P of the first 96 keys; awaited in
 tiles with both 64-key halves) and p_full (all of P; awaited in every tile).  A parity wait only tells a barrier's current phase
 from the one before, so at no point may the MMA thread wait for a phase that the barrier is more than one completion away from.
-All interleavings of a slot's warps with the MMA thread are walked through, with the order of the arrivals as the kernel has it."""
+All interleavings of a slot's warps with the MMA thread are walked through, with the order of the arrivals as the kernel has it.
+The same for the barriers over which the slots hand whole output tiles to the thread that copies them out."""
 import itertools
 import os
 import re
@@ -69,3 +70,104 @@ def test_every_wait_for_p_is_for_its_own_tile(tiles):
 def test_the_walk_sees_an_arrival_that_comes_too_late():
     late = {FULL: ["part", "full"], HALF: ["full", "part"], EXACT: ["part", "full"]}
     assert first_fault((HALF, FULL), late) is not None
+
+
+# ---- the output's hand-over: a slot leaves a whole query tile in the stage of its unit's last key tile and says so; one thread
+# copies the tiles out, unit by unit and slot by slot, and gives the stages back.  K's stage is slot 0's, V's is slot 1's.
+STAGES = 2
+
+
+def staged_barriers_of_the_kernel():
+    """'stage' if every stage of a slot's has a barrier of its own, 'slot' if a slot has one barrier."""
+    text = open(KERNEL).read()
+    uses = re.findall(r"bars\.o_staged\[sl\](\[[^\]]*\])?", text)
+    declared = re.search(r"uint64_t o_staged\[2\](\[ST\])?;", text)
+    assert declared and len(uses) == 3, "the hand-over is not where it was"  # initialised, awaited, arrived on
+    if not declared.group(1):
+        return "slot"
+    init, wait, arrive = uses
+    assert init == "[s]" and wait == "[s]" and arrive == "[(it - 1u) % ST]" and "const uint32_t s = (it - 1u) % ST;" in text
+    return "stage"
+
+
+def first_staging_fault(units, barriers):
+    """`units` is a list of (key tiles, slots that work, whether the output is staged).  Walks all interleavings of the MMA thread,
+    the slots and the storing thread; loads are made as soon as their stage is free.  A description of the first wait that the
+    storing thread could enter with its barrier a phase too far, or of a standstill; None if there is neither."""
+    tiles = [(u, n == 0, n == count - 1) for u, (count, _, _) in enumerate(units) for n in range(count)]
+    end, works, staged = [sum(c for c, _, _ in units[:u + 1]) for u in range(len(units))], [w for _, w, _ in units], [s for _, _, s in units]
+    mma = []  # in program order: ("s" or "pv", tile, slot)
+    at = 0
+    for count, slots, _ in units:
+        mma += [("s", at, sl) for sl in range(slots)]
+        for i in range(at, at + count):
+            for sl in range(slots):
+                mma.append(("pv", i, sl))
+                if i + 1 < at + count:
+                    mma.append(("s", i + 1, sl))
+        at += count
+    done_at = {x: n for n, x in enumerate(mma)}  # an instruction is complete once the thread's count is beyond it
+    slot_of = [[("p", i) if kind == "p" else ("out", u) for u in range(len(units)) if works[u] > sl
+                for kind, i in [("p", i) for i in range(end[u] - units[u][0], end[u])] + ([("out", 0)] if staged[u] else [])] for sl in range(2)]
+    store = [(u, sl) for u in range(len(units)) if staged[u] for sl in range(works[u])]
+    barrier_of = lambda u, sl: (sl, (end[u] - 1) % STAGES if barriers == "stage" else 0)
+    arrivals = [{}, {}]  # per slot: unit -> its place in the slot's program
+    for sl in range(2):
+        for n, (kind, u) in enumerate(slot_of[sl]):
+            if kind == "out":
+                arrivals[sl][u] = n
+
+    def released(i, which, m, copied):
+        """Whether tile i's K (0) or V (1) stage has been given back."""
+        u, _, last = tiles[i]
+        if last and staged[u] and which < works[u]:
+            return store.index((u, which)) < copied
+        return m > max(done_at["s" if which == 0 else "pv", i, sl] for sl in range(works[u]))
+
+    def successors(state):
+        m, slots, copied = state
+        if m < len(mma):
+            kind, i, sl = mma[m]
+            free = i < STAGES or released(i - STAGES, 0 if kind == "s" else 1, m, copied)
+            if free and (kind == "s" or ("p", i) in slot_of[sl][:slots[sl]]):
+                yield m + 1, slots, copied
+        for sl in range(2):
+            if slots[sl] < len(slot_of[sl]):
+                kind, x = slot_of[sl][slots[sl]]
+                if m > done_at[("s", x, sl) if kind == "p" else ("pv", end[x] - 1, sl)]:
+                    yield m, (slots[0] + (sl == 0), slots[1] + (sl == 1)), copied
+        if copied < len(store):
+            u, sl = store[copied]
+            if slots[sl] > arrivals[sl][u]:
+                yield m, slots, copied + 1
+
+    seen, todo = set(), [(0, (0, 0), 0)]
+    while todo:
+        state = todo.pop()
+        if state in seen:
+            continue
+        seen.add(state)
+        m, slots, copied = state
+        if copied < len(store):
+            u, sl = store[copied]
+            mine = [x for x in arrivals[sl] if barrier_of(x, sl) == barrier_of(u, sl)]
+            if sum(slots[sl] > arrivals[sl][x] for x in mine) > mine.index(u) + 1:
+                return f"unit {u}: the barrier of slot {sl} has run a phase ahead of the storing thread"
+        following = list(successors(state))
+        if not following and (m < len(mma) or copied < len(store)):
+            return f"standstill after {copied} of {len(store)} copies"
+        todo += following
+    return None
+
+
+@pytest.mark.parametrize("lengths", [(3, 1, 3), (2, 1, 1, 1, 2), (1, 1, 1, 1, 1), (2, 2, 2), (1, 2, 3, 1), (3, 3, 1, 1, 3)], ids=str)
+def test_every_output_tile_is_copied_for_its_own_unit(lengths):
+    order = staged_barriers_of_the_kernel()
+    for kinds in itertools.product([(2, True), (1, True), (2, False)], repeat=len(lengths)):  # a pair, a single head, a cut tile
+        units = [(n, *kind) for n, kind in zip(lengths, kinds)]
+        assert first_staging_fault(units, order) is None, units
+
+
+def test_the_walk_sees_a_slot_that_runs_ahead_of_the_copies():
+    assert first_staging_fault([(3, 2, True), (1, 2, True), (3, 2, True)], "slot") is not None
+    assert first_staging_fault([(2, 2, True)] * 4, "slot") is None
