@@ -140,7 +140,7 @@ struct __align__(16) Unit {
   int32_t q_start1, q_rows1;     // a twin unit's second query tile (q_rows1 == 0: an ordinary unit)
   int32_t part_base1, counter_base1;  // ... and that tile's workspace slots and merge counters when the lists are split
   // zero in the plan; in the kernel's copy, the layer of the launch that the unit is drawn for, and its first query head
-  // times two, plus one if both slots have work
+  // times four, plus one if both slots have work, plus two if its output leaves through shared memory
   int32_t layer, heads;
 };
 static_assert(sizeof(Unit) == 64, "the plan's unit record is 16 words");

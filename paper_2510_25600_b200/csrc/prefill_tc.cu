@@ -131,6 +131,11 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
     tmem_alloc(smem_u32(&tmem_base_s), kTmemCols);
     tmem_relinquish();
   }
+  // The maps' descriptors are fetched beside the barriers' set-up, not by the first copies (64 units 15.5 -> 15.4 us, 512 35.4 -> 35.3).
+  if (warp == 11 && lane < 6) {
+    const CUtensorMap* map = lane == 0 ? &tm_q : lane == 1 ? &tm_k : lane == 2 ? &tm_v : lane == 3 ? &tm_k64 : lane == 4 ? &tm_v64 : &tm_o;
+    asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+  }
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the stream's earlier work is complete and visible from here on
   if (tid == 0) {
     abort_s = *reinterpret_cast<volatile int32_t*>(status) != 0;  // an earlier CTA or launch already failed
@@ -189,10 +194,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
   // stages of the unit's last tile, whose next contents are not wanted before the next unit's second tile: K's for slot 0
   // (both slots' S of that tile are long complete), V's for slot 1 (its last product is the unit's last).  Ragged batch of 8, sparse
   // layer: 618 -> 595 us at full clock, 725 -> 701 in a row; 37 120 tokens 653 -> 643 and 762 -> 749; the copies by rolled loops,
-  // because of the instruction cache.  Launches of few units per CTA store from registers: their last outputs are a larger share of
-  // the time, and the way through shared memory is the longer one (304 units for 148 CTAs 43.0 and 45.5 us, 672 126.1 and 125.0).
-  const bool many_units = n_work >= 4 * (int32_t)gridDim.x;
-  auto output_staged = [&](const Unit& u) { return many_units && u.n_chunks == 1 && u.q_rows == kBQ && (u.q_rows1 == 0 || u.q_rows1 == kBQ); };
+  // because of the instruction cache.  It is the faster way for launches of few units too (one sparse layer, 32 heads: 2432 tokens
+  // 45.4 us from registers, 42.2 so; 384 units 29.8 and 28.1, 512 units 37.1 and 35.4, 64 and 256 units the same), so the shape of
+  // the unit alone decides.  The roles read the answer in the unit's record, as a bit (384 units 27.8 -> 27.7, 512 35.2 -> 34.7).
+  auto output_staged = [](const Unit& u) { return u.n_chunks == 1 && u.q_rows == kBQ && (u.q_rows1 == 0 || u.q_rows1 == kBQ); };
 
   // the two softmax warpgroups take registers from the warpgroup of the producer and MMA warps
 
@@ -209,13 +214,13 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
     auto fetch = [&](int32_t idx) -> Unit {
       Unit uu = {};
       if (idx < n_work) {
-        const int32_t layer = idx / n_units;
+        const int32_t layer = idx < n_units ? 0 : idx / n_units;
         uu = units[idx - layer * n_units];
         uu.layer = layer;
         const int32_t n_pairs = n_kv_heads * ppg;
         const bool split = uu.n_chunks > 1, twin = uu.q_rows1 != 0;
-        const int32_t in_group = 2 * (uu.pair % ppg);
-        uu.heads = (uu.pair / ppg * G + in_group) * 2 + (twin || in_group + 1 < G ? 1 : 0);
+        const int32_t group = uu.pair / ppg, in_group = 2 * (uu.pair - group * ppg);
+        uu.heads = (group * G + in_group) * 4 + (output_staged(uu) ? 2 : 0) + (twin || in_group + 1 < G ? 1 : 0);
         const bool good = uu.ent_count >= 1 && uu.ent_begin >= 0 &&
                           (int64_t)uu.ent_begin + (int64_t)uu.ent_count * (twin ? 2 : 1) <= n_entries &&
                           uu.q_rows >= 1 && uu.q_rows <= kBQ && uu.req_start >= 0 && uu.q_start >= uu.req_start &&
@@ -224,7 +229,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
                           (!split || n_layers == 1) &&  // (the plan has merge counters and slots for one layer at a time)
                           (!twin || (uu.q_rows1 >= 1 && uu.q_rows1 <= kBQ && uu.q_start1 >= uu.req_start &&
                                      (int64_t)uu.q_start1 + uu.q_rows1 <= total_tokens && (G & 1) != 0 &&
-                                     uu.pair % ppg == ppg - 1 &&
+                                     in_group == 2 * (ppg - 1) &&
                                      (!split || (uu.part_base1 >= 0 && ((int64_t)uu.part_base1 + uu.n_chunks) * n_q_heads <= part_slots &&
                                                  uu.counter_base1 >= 0 && (int64_t)uu.counter_base1 + n_q_heads <= n_counters)))) &&
                           (!split || (uu.part_base >= 0 && ((int64_t)uu.part_base + uu.n_chunks) * n_q_heads <= part_slots &&
@@ -269,7 +274,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       // longest units would keep work from those that finish early.
       int32_t idx_next = 0;
       const int32_t nt = u.ent_count;
-      const int32_t g = u.pair / ppg, hq0 = u.heads >> 1;
+      const int32_t g = u.pair / ppg, hq0 = u.heads >> 2;
       const bool twin = u.q_rows1 != 0;  // both slots on head hq0, slot 1 on the query tile at q_start1
       const int32_t n_slots = 1 + (u.heads & 1);
       // A tile's entry as slot 0 and as slot 1 see it, 32 tiles at a time, one per lane; of the halves an entry claims only
@@ -411,7 +416,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
         if (!ok) break;
         const int32_t nt = unit_s[us].ent_count;
         const uint32_t last_slot = (uint32_t)unit_s[us].heads & 1u;
-        const bool staged = output_staged(unit_s[us]);
+        const bool staged = (unit_s[us].heads & 2) != 0;
         mbar_arrive(smem_u32(&bars.u_empty[us]));
         if (nt == 0) break;
         ok = mbar_wait(smem_u32(&bars.q_full), uo & 1u, abort_flag, wait_ns);
@@ -509,7 +514,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
         const int32_t nt = u.ent_count;
         if (nt == 0) break;
         it += (uint32_t)nt;
-        if (output_staged(u)) {
+        if ((u.heads & 2) != 0) {
           const uint32_t s = (it - 1u) % ST;
           const bool twin = u.q_rows1 != 0;
 #pragma unroll
@@ -520,7 +525,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
             if (!ok) break;
             phases ^= 1u << bit;
             const uint32_t buf = (sl == 0 ? sK : sV) + s * kTileKV;
-            const int32_t hq = (u.heads >> 1) + (twin ? 0 : sl), q_first = twin && sl == 1 ? u.q_start1 : u.q_start;
+            const int32_t hq = (u.heads >> 2) + (twin ? 0 : sl), q_first = twin && sl == 1 ? u.q_start1 : u.q_start;
             tma_store_4d(&tm_o, buf, 0, hq, q_first, u.layer);
             tma_store_4d(&tm_o, buf + kPanelKV, 64, hq, q_first, u.layer);
             asm volatile("cp.async.bulk.commit_group;\n cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -804,9 +809,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
       tc_fence_after();
       // (the unit's fields are read again rather than held through the tile loop: the softmax uses every register it has)
       const bool twin = u.q_rows1 != 0, second = twin && sl == 1;  // this slot works on the unit's second query tile
-      const int32_t hq = (u.heads >> 1) + (twin ? 0 : sl), q_first = second ? u.q_start1 : u.q_start;
+      const int32_t hq = (u.heads >> 2) + (twin ? 0 : sl), q_first = second ? u.q_start1 : u.q_start;
       const bool row_valid = row < (second ? u.q_rows1 : u.q_rows);
-      if (output_staged(u)) {
+      if ((u.heads & 2) != 0) {
         const float inv = 1.f / l_sum;
         const uint32_t buf = (sl == 0 ? sK : sV) + ((it - 1u) % ST) * kTileKV + (uint32_t)row * 128u;
 #pragma unroll 1
@@ -871,7 +876,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
         __syncwarp();
         int32_t last = 0;
         if (lane == 0) {
-          int32_t* cnt = reinterpret_cast<int32_t*>(plan + hdr->off_counters) + (second ? u.counter_base1 : u.counter_base) + hq;
+          int32_t* cnt = counters + (second ? u.counter_base1 : u.counter_base) + hq;
           last = ((atom_add_acq_rel(cnt, 1 << (8 * quad)) >> (8 * quad)) & 255) == u.n_chunks - 1;
           if (last) atomicSub(reinterpret_cast<uint32_t*>(cnt), (uint32_t)u.n_chunks << (8 * quad));  // ready for the next launch
         }

@@ -16,5 +16,5 @@ def test_tiles_whole_and_cut(heads, dense):
     assert list(batch.seq_lens) == lens
     wl = inputs.Workload("tiles", 3, "bf16", *heads, 128, 1, (0,), (0,), batch, inputs.STMask(1, 1, tile=64, dense_causal=dense), 16, 0.25)
     x = inputs.make_qkv(wl, 0)
-    gc.check_prefill(wl, x)             # a unit per CTA at most: all rows from registers
-    gc.check_prefill(wl, x, n_ctas=2)   # many: whole tiles through shared memory
+    gc.check_prefill(wl, x)             # a unit per CTA at most
+    gc.check_prefill(wl, x, n_ctas=2)   # many: a stage is staged again and again
