@@ -7,10 +7,11 @@ from oracle import purekv_oracle as po
 from paper_2510_25600_b200 import binding as pk, inputs
 from tests import gpu_common as gc
 
-# heads / kv heads, prefix, frames, text, grid, skip, layers, dense: one tile and less, odd groups (twin units), more units than
-# CTAs and fewer, last tiles cut by the layer's end (rows past it must not come from the next layer)
+# heads / kv heads, prefix, frames, text, grid, skip, layers, dense: one tile and less, odd groups (twin units), last tiles cut by
+# the layer's end (rows past it must not come from the next layer), requests of exactly one tile (units of one key tile in a row)
 CASES = [(1, 1, [0], [1], [16], 5, 7, 128, 2, False), (3, 1, [20, 0], [6, 4], [40, 200], 9, 11, 64, 3, False),
-         (4, 2, [0], [3], [33], 24, 24, 128, 5, True), (7, 1, [64], [4], [64], 16, 16, 128, 4, False)]
+         (4, 2, [0], [3], [33], 24, 24, 128, 5, True), (7, 1, [64], [4], [64], 16, 16, 128, 4, False),
+         (3, 1, [0] * 6, [1] * 6, [112] * 6, 4, 4, 64, 4, False)]
 
 
 def _case(H, Hkv, prefix, frames, text, gh, gw, tile, layers, dense):
@@ -19,9 +20,10 @@ def _case(H, Hkv, prefix, frames, text, gh, gw, tile, layers, dense):
                            16, 0.25)
 
 
-def _plan(wl, device, n_layers):
+def _plan(wl, device, n_layers, n_ctas=0):
     b = pk.Batch(wl.batch.seq_lens, wl.batch.n_prefix, wl.batch.n_frames, device=device)
-    return b, *pk.purekv_plan_build_host(b, pk.st_params(wl.mask), pk.BF16, 128, wl.n_q_heads, wl.n_kv_heads, n_layers=n_layers)
+    return b, *pk.purekv_plan_build_host(b, pk.st_params(wl.mask), pk.BF16, 128, wl.n_q_heads, wl.n_kv_heads, n_ctas=n_ctas,
+                                         n_layers=n_layers)
 
 
 @pytest.mark.parametrize("case", CASES)
@@ -43,12 +45,15 @@ def test_few_layers_of_a_long_list_keep_their_chunks():
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("n_ctas", [0, 2, 5])  # a unit or two for each CTA; few CTAs, which go through the units of layer after layer
 @pytest.mark.parametrize("case", CASES)
-def test_layers_are_their_own_calls(case):
+def test_layers_are_their_own_calls(case, n_ctas):
     wl = _case(*case)
     layers, t, pad = wl.n_layers, wl.batch.total_tokens, 3
     xs = [inputs.make_qkv(wl, n) for n in range(layers)]
-    b, buf, info = _plan(wl, "cuda", 30)
+    b, buf, info = _plan(wl, "cuda", 30, n_ctas)
+    assert info.max_chunks == 1 and (n_ctas == 0 or info.n_ctas == n_ctas)
+    assert n_ctas == 0 or info.n_units == 1 or info.n_units * layers >= 4 * n_ctas
     plan = pk.Plan(torch.from_numpy(buf.copy()).cuda(), info)
     stack = lambda n, width: torch.cat([torch.cat([gc.upload(x, n, "bf16"), torch.full((pad, width, 128), float("nan"), dtype=torch.bfloat16, device="cuda")])
                                         for x in xs]).view(layers, t + pad, width, 128)[:, :t]  # rows of NaN between the layers
@@ -69,17 +74,19 @@ def test_layers_are_their_own_calls(case):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("dtype,n_layers", [("fp32", 3), ("bf16", 1)])
-def test_layers_that_cannot_share_a_launch(dtype, n_layers):
-    """The CUDA-core kernel, and a plan with split lists; one Q for all layers (stride 0)."""
+@pytest.mark.parametrize("dtype,n_layers,one_q", [("fp32", 3, True), ("fp32", 3, False), ("bf16", 1, False), ("bf16", 30, True)])
+def test_layers_that_cannot_share_a_launch(dtype, n_layers, one_q):
+    """The CUDA-core kernel; a plan with split lists; one Q for all layers (stride 0) under a plan with whole ones."""
     batch = inputs.make_batch([10], [12], [20], 8, 8)
     d = 64 if dtype == "fp32" else 128
     wl = inputs.Workload("l", 3, dtype, 2, 1, d, 3, (0,), (0,), batch, inputs.STMask(8, 8, tile=16 if dtype == "fp32" else 64), 16, 0.3)
     xs = [inputs.make_qkv(wl, n) for n in range(3)]
-    q = gc.upload(xs[0], "q", dtype)[None].expand(3, -1, -1, -1)
-    k, v = (torch.stack([gc.upload(x, n, dtype) for x in xs]) for n in "kv")
+    q, k, v = (torch.stack([gc.upload(x, n, dtype) for x in xs]) for n in "qkv")
+    if one_q:
+        q = q[:1].expand(3, -1, -1, -1)
     b = pk.Batch(batch.seq_lens, batch.n_prefix, batch.n_frames)
     buf, info = pk.purekv_plan_build_host(b, pk.st_params(wl.mask), pk.BF16 if dtype == "bf16" else pk.FP32, d, 2, 1, n_layers=n_layers)
+    assert dtype == "fp32" or (info.max_chunks > 1) == (n_layers == 1)
     plan = pk.Plan(torch.from_numpy(buf.copy()).cuda(), info)
     out = pk.purekv_st_sparse_prefill_layers(q, k, v, b, plan)
     for n in range(3):
