@@ -589,9 +589,10 @@ static purekv_status select_impl(const float* c, const void* v, int64_t v_layer_
   if (st_v != PUREKV_OK) return st_v;
   const bool stage_keys = key_bytes <= 200 * 1024;
   // A segment's selection is a chain of latencies; where every CTA finds an SM of its own, 1024 threads go through a long list in
-  // half the trips (104 segments, selection and compaction in a row: of 13 393 keys 130 -> 122 us, of 8320 77.9 -> 77.4; of 3977
-  // no difference, and more segments than SMs take turns).
-  const bool wide = !gather && (int64_t)batch->n_req * n_kv_heads * n_layers <= 148 && longest >= 4096;
+  // half the trips (selection and compaction in a row, 512 and 1024 threads: 104 segments of 37 120 keys 331 and 324 us, of 13 393
+  // 128 and 120, of 8320 78.4 and 78.4, 120 of 6000 65.7 and 66.3, 104 of 4200 40.2 and 42.4; 4 of 37 120 44.3 and 36.4; keys
+  // that stay outside shared memory, 4 of 60 000 135 and 87, 32 of 100 000 502 and 411).  More segments than SMs take turns.
+  const bool wide = !gather && (int64_t)batch->n_req * n_kv_heads * n_layers <= 148 && longest >= 8192;
   if (stage_keys) {
     static std::atomic<uint64_t> smem_allowed{0}, smem_allowed_g{0}, smem_allowed_w{0};
     const purekv_status st_smem = gather ? allow_max_dynamic_smem(select_kernel<void, true>, smem_allowed_g)
