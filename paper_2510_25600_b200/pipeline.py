@@ -60,8 +60,8 @@ class PureKVPipeline:
         # clipped window a multiple of 8); the two-pass kernels otherwise
         self.one_pass_scores = (dtype == torch.bfloat16 and head_dim == 128 and window % 8 == 0 and
                                 all(l >= window or l % 8 == 0 for l in seq_lens))
-        self.dense_runs, self.sparse_runs = self._runs(0, self.n_dense), self._runs(self.n_dense, n_layers)
-        self.lse = torch.empty((len(self.scored), n_q_heads, t), dtype=torch.float32, device=dev)
+        # rows' log-sum-exp, a layer after the other: of every dense layer, so that one call takes them all, scored or not
+        self._lse = torch.empty((self.n_dense if self.one_pass_scores else 0, n_q_heads, t), dtype=torch.float32, device=dev)
         self.score_ws = torch.empty(P.purekv_score_ws_bytes(self.batch, window, n_q_heads), dtype=torch.uint8, device=dev)
         nc = len(self.compacted)
         self.select_ws = torch.empty(P.purekv_select_ws_bytes(self.batch, nc, n_kv_heads), dtype=torch.uint8, device=dev)
@@ -70,35 +70,19 @@ class PureKVPipeline:
         self.v_c = torch.empty_like(self.k_c)
         self.status = torch.zeros(1, dtype=torch.int32, device=dev)
         self.plan_dense = self._plan_st = None
+        self.prefill_launches = n_layers  # of the last pass (before the first: a layer at a time)
 
     @property
     def launches_per_step(self) -> int:
-        """Kernels of a pass: prefill, score (1 one-pass or in one cluster, up to 3 otherwise: counted as 1), select (2),
+        """Kernels of the last pass: prefill, score (1 one-pass or in one cluster, up to 3 otherwise: counted as 1), select (2),
         compact."""
         return self.prefill_launches + len(self.scored) + 2 + 1
 
     @property
-    def prefill_launches(self) -> int:
-        """Prefill launches of the last pass: the layers under one mask are one, unless the plan cuts lists into chunks or the
-        CUDA-core kernel runs them."""
-        n = 0
-        for plan, runs in ((self.plan_dense, self.dense_runs), (self._plan_st, self.sparse_runs)):
-            whole = plan is not None and plan.info.n_units > 0 and plan.info.max_chunks == 1
-            n += sum(1 if whole else hi - lo for lo, hi in runs)
-        return n
-
-    def _runs(self, lo: int, hi: int) -> list:
-        """Layers lo .. hi - 1 in runs that one call can take: where a scored layer leaves its rows' log-sum-exp, those of a
-        run lie one after another in self.lse."""
-        row = lambda layer: self.scored.index(layer) if self.one_pass_scores and layer in self.scored else None
-        runs = []
-        for layer in range(lo, hi):
-            at, before = row(layer), row(layer - 1) if layer > lo else None
-            if runs and (at is None and before is None or at is not None and before is not None and at == before + 1):
-                runs[-1][1] = layer + 1
-            else:
-                runs.append([layer, layer + 1])
-        return runs
+    def lse(self) -> torch.Tensor:
+        """[scored layers, H, T]: the log-sum-exp that the one-pass scores read."""
+        first, last = self.scored[0], self.scored[-1]
+        return self._lse[first:last + 1] if self.scored == tuple(range(first, last + 1)) else self._lse[list(self.scored)]
 
     def _plan(self, params, ring: list, d_buf: torch.Tensor, layers: int = 1) -> P.Plan:
         """Plans one mask, for launches of `layers` layers, on the host into a pinned buffer and enqueues its copy on the
@@ -140,60 +124,68 @@ class PureKVPipeline:
     def prefill_layer(self, layer: int, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor) -> None:
         plan = self.plan_dense if layer <= self.clie else self.plan_st
         # a scored layer is dense causal: its prefill also leaves the rows' log-sum-exp for the one-pass scores
-        lse = self.lse[self.scored.index(layer)] if (self.one_pass_scores and layer in self.scored) else None
+        lse = self._lse[layer] if (self.one_pass_scores and layer in self.scored) else None
         P.purekv_st_sparse_prefill(q, k, v, self.batch, plan, out=self.o[layer], lse=lse, status=self.status,
                                    ws=self.prefill_ws)
 
-    def _prefill(self, plan: P.Plan, runs: list, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, events) -> None:
-        """The layers of `runs` of the stacked Q/K/V, in as few launches as the plan allows; with `events`, one per layer."""
-        for a, b in runs:
-            if b - a == 1 or events is not None or not isinstance(q, torch.Tensor):  # (or a sequence of layers: no stacked views)
-                for layer in range(a, b):
-                    if events is not None:
-                        events[layer][0].record()
-                    self.prefill_layer(layer, q[layer], k[layer], v[layer])
-                    if events is not None:
-                        events[layer][1].record()
-                continue
-            lse = None
-            if self.one_pass_scores and a in self.scored:
-                at = self.scored.index(a)
-                lse = self.lse[at:at + b - a]
-            P.purekv_st_sparse_prefill_layers(q[a:b], k[a:b], v[a:b], self.batch, plan, out=self.o[a:b], lse=lse, status=self.status,
-                                              ws=self.prefill_ws)
+    def _share_launches(self, q, k, v) -> bool:
+        """Whether Q/K/V are stacked layers that one launch can take (a sequence of layers has no stacked views, and layers that
+        overlap, one for all of them, say, are launches of their own)."""
+        t = self.batch.total_tokens
+        return (isinstance(q, torch.Tensor) and isinstance(k, torch.Tensor) and isinstance(v, torch.Tensor) and
+                q.stride(0) >= t * self.h * self.d and k.stride(0) == v.stride(0) >= t * self.hkv * self.d)
+
+    def _prefill(self, plan: P.Plan, lo: int, hi: int, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, shared: bool, events) -> None:
+        """Layers lo .. hi - 1, all under one mask: in one call (`shared`), which is one launch if the plan is the tensor-core
+        kernel's and leaves lists whole, or one by one, each between its pair of `events` if those are given."""
+        if shared:
+            lse = self._lse[lo:hi] if self.one_pass_scores and lo < self.n_dense else None
+            P.purekv_st_sparse_prefill_layers(q[lo:hi], k[lo:hi], v[lo:hi], self.batch, plan, out=self.o[lo:hi], lse=lse,
+                                              status=self.status, ws=self.prefill_ws)
+            self.prefill_launches += 1 if plan.info.n_units > 0 and plan.info.max_chunks == 1 else hi - lo
+            return
+        for layer in range(lo, hi):
+            if events is not None:
+                events[layer][0].record()
+            self.prefill_layer(layer, q[layer], k[layer], v[layer])
+            if events is not None:
+                events[layer][1].record()
+        self.prefill_launches += hi - lo
 
     def run_device(self, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, events=None, marks=None) -> None:
         """q [n_layers,T,H,d], k,v [kv_layers,T,H_kv,d] on the GPU.  Results in self.o / idx / k_c / v_c.
         `events`, if given, is a list of (start, end) torch.cuda.Event pairs, one per layer, which is then a prefill launch
-        of its own; otherwise the layers under one mask are one launch where the plan allows it.  `marks`, if given, is three
-        events recorded before the first prefill launch, after the last dense-causal one and after the last one."""
+        of its own, as it is where Q is a sequence of layers; the layers of a stacked Q are one launch per mask where the plan
+        allows it.  `marks`, if given, is three events recorded before the first prefill launch, after the last dense-causal one and after the last one."""
         # The sparse mask's plan, the longer one, is made and copied while the GPU works on the dense layers.  (The copy
         # waits for whatever the stream held before this call, which may still read the last plan; in the stream itself,
         # between two layers, it cost 10 us.)
         before = torch.cuda.Event() if self.n_sparse else None
         if before is not None:
             before.record()
-        alone = events is not None  # each layer a launch of its own
-        self.plan_dense = self._plan(self.params_dense, self._h_dense, self.plan_buf_dense, 1 if alone else self.n_dense)
+        # planned for the launches that are made: lists that are left whole for one launch end unevenly in a launch per layer
+        shared = events is None and (self.n_dense > 1 or self.n_sparse > 1) and self._share_launches(q, k, v)
+        self.prefill_launches = 0
+        self.plan_dense = self._plan(self.params_dense, self._h_dense, self.plan_buf_dense, self.n_dense if shared else 1)
         self._size_prefill_ws(self.plan_dense)
         if marks is not None:
             marks[0].record()
-        self._prefill(self.plan_dense, self.dense_runs, q, k, v, events)
+        self._prefill(self.plan_dense, 0, self.n_dense, q, k, v, shared and self.n_dense > 1, events)
         if marks is not None:
             marks[1].record()
         if before is not None:
             main = torch.cuda.current_stream()
             self._copies.wait_event(before)
             with torch.cuda.stream(self._copies):
-                self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st, 1 if alone else self.n_sparse)
+                self._plan_st = self._plan(self.params_st, self._h_st, self.plan_buf_st, self.n_sparse if shared else 1)
             main.wait_event(self._h_st[0][1])
             self._size_prefill_ws(self._plan_st)
-            self._prefill(self._plan_st, self.sparse_runs, q, k, v, events)
+            self._prefill(self._plan_st, self.n_dense, self.n_layers, q, k, v, shared and self.n_sparse > 1, events)
         if marks is not None:
             marks[2].record()
         for n, layer in enumerate(self.scored):
             if self.one_pass_scores:
-                P.purekv_lowlayer_score_lse(q[layer], k[layer], self.lse[n], self.batch, self.window, c_out=self.c[n],
+                P.purekv_lowlayer_score_lse(q[layer], k[layer], self._lse[layer], self.batch, self.window, c_out=self.c[n],
                                             status=self.status)
             else:
                 P.purekv_lowlayer_score(q[layer], k[layer], self.batch, self.window, c_out=self.c[n], ws=self.score_ws)

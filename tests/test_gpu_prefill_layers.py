@@ -1,4 +1,6 @@
 """Several layers in one call: each layer comes out as its own call with the same plan gives it, and as the oracle computes it."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -64,6 +66,7 @@ def test_layers_are_their_own_calls(case, n_ctas):
     for _ in range(2):
         pk.purekv_st_sparse_prefill_layers(q, k, v, b, plan, out=out[:, :t], lse=lse, status=status)
     assert status.item() == 0 and (out[:, t:] == 7.0).all()
+    assert _launches(lambda: pk.purekv_st_sparse_prefill_layers(q, k, v, b, plan, out=out[:, :t], lse=lse, status=status)) == 1
     for n in range(layers):
         one, one_lse = torch.empty_like(out[n, :t]), torch.empty_like(lse[n])
         pk.purekv_st_sparse_prefill(q[n], k[n], v[n], b, plan, out=one, lse=one_lse, status=status)
@@ -89,19 +92,35 @@ def test_layers_that_cannot_share_a_launch(dtype, n_layers, one_q):
     assert dtype == "fp32" or (info.max_chunks > 1) == (n_layers == 1)
     plan = pk.Plan(torch.from_numpy(buf.copy()).cuda(), info)
     out = pk.purekv_st_sparse_prefill_layers(q, k, v, b, plan)
+    ws, again = torch.empty(max(16, info.ws_bytes), dtype=torch.uint8, device="cuda"), torch.empty_like(out)
+    assert _launches(lambda: pk.purekv_st_sparse_prefill_layers(q, k, v, b, plan, out=again, ws=ws)) == 3
     for n in range(3):
         assert torch.equal(out[n], pk.purekv_st_sparse_prefill(q[n], k[n], v[n], b, plan))
 
 
-@pytest.mark.gpu
-def test_a_pass_in_launches_of_many_layers_is_the_layers_one_by_one():
+def _launches(call):
+    """Kernels that `call` launches: the nodes of a graph that it is captured in."""
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+        call()
+    n = ctypes.c_size_t()
+    assert ctypes.CDLL("libcuda.so.1").cuGraphGetNodes(ctypes.c_void_p(graph.raw_cuda_graph()), None, ctypes.byref(n)) == 0
+    return n.value
+
+
+def _pass(scored):
     from paper_2510_25600_b200.pipeline import PureKVPipeline
     batch = inputs.make_batch([10, 3], [12, 5], [20, 140], 12, 12)
     mask = inputs.STMask(12, 12, tile=64)
     wl = inputs.Workload("p", 3, "bf16", 4, 2, 128, 6, (0, 1), (2, 3, 4, 5), batch, mask, 16, 0.3)
     xs = [inputs.make_qkv(wl, n) for n in range(6)]
     q, k, v = (torch.stack([gc.upload(x, n, "bf16") for x in xs]) for n in "qkv")
-    pipe = PureKVPipeline(batch.seq_lens, batch.n_prefix, batch.n_frames, mask, 6, 4, 2, 128, q.dtype, (0, 1), (2, 3, 4, 5), 16, 0.3)
+    return PureKVPipeline(batch.seq_lens, batch.n_prefix, batch.n_frames, mask, 6, 4, 2, 128, q.dtype, scored, (2, 3, 4, 5), 16, 0.3), q, k, v
+
+
+@pytest.mark.gpu
+def test_a_pass_in_launches_of_many_layers_is_the_layers_one_by_one():
+    pipe, q, k, v = _pass((0, 1))
     pipe.run_device(q, k, v)
     assert pipe.prefill_launches == 2 and pipe.plan_st.info.max_chunks == 1
     o, lse = pipe.o.clone(), pipe.lse.clone()
@@ -114,3 +133,35 @@ def test_a_pass_in_launches_of_many_layers_is_the_layers_one_by_one():
     # either way of summing rounds P and the output to bf16: each is within the oracle's tolerance, the two within both
     assert (pipe.o.float() - o.float()).abs().max().item() <= 2 * gc.ATTN_TOL["bf16"]
     assert (pipe.lse - lse).abs().max().item() <= 2 * 2e-3
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("scored", [(1,), (0, 1), (1, 0)], ids=str)
+def test_the_dense_layers_share_a_launch_whichever_are_scored(scored):
+    pipe, q, k, v = _pass(scored)
+    whole, *_ = _pass((0, 1))
+    for p in (pipe, whole):
+        p.run_device(q, k, v)
+        p.check_status()
+        assert p.prefill_launches == 2
+    assert torch.equal(pipe.o, whole.o) and pipe.lse.shape == (len(scored), 4, pipe.batch.total_tokens)
+    for n, layer in enumerate(scored):
+        assert torch.equal(pipe.lse[n], whole.lse[layer]) and torch.equal(pipe.c[n], whole.c[layer])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("form", ["sequence", "one Q for all", "events"])
+def test_layers_launched_one_by_one_are_planned_so(form):
+    pipe, q, k, v = _pass((0, 1))
+    if form == "one Q for all":
+        q = q[:1].expand(6, -1, -1, -1)
+    events = [[torch.cuda.Event() for _ in range(2)] for _ in range(6)] if form == "events" else None
+    pipe.run_device(list(q) if form == "sequence" else q, k, v, events=events)
+    pipe.check_status()
+    assert pipe.prefill_launches == 6
+    o, st, dense = pipe.o.clone(), pipe.plan_st.info.n_units, pipe.plan_dense.info.n_units
+    pipe.build_plans()
+    assert (st, dense) == (pipe.plan_st.info.n_units, pipe.plan_dense.info.n_units) and pipe.plan_st.info.max_chunks > 1
+    for n in range(6):
+        pipe.prefill_layer(n, q[n], k[n], v[n])
+    assert torch.equal(pipe.o, o)
