@@ -176,7 +176,9 @@ purekv_status purekv_st_sparse_prefill(const void *q, const void *k, const void 
  * kv_layer_stride, and writes o + n * o_layer_stride and, with lse, lse + n * lse_layer_stride (strides in elements).  Each
  * layer's result is that of its own call with this plan.  Where the tensor-core kernel runs and the plan leaves every list
  * whole (h_info->max_chunks 1), all layers are one launch, whose CTAs go from a layer's last units to the next layer's
- * first; otherwise one launch per layer. */
+ * first; otherwise, and where layers overlap (a stride below a layer's own size, such as 0 for one Q for all) or a stride has
+ * 2^38 elements or more, one launch per layer.  As the pointers, the strides of Q, K, V and O are multiples of 16 bytes, O's of
+ * 32 for the tensor-core kernel; other strides are refused before anything is launched. */
 purekv_status purekv_st_sparse_prefill_layers(const void *q, const void *k, const void *v, void *o, float *lse,
                                               int64_t q_layer_stride, int64_t kv_layer_stride,
                                               int64_t o_layer_stride, int64_t lse_layer_stride, int32_t n_layers,

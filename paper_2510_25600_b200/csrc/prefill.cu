@@ -37,12 +37,13 @@ static purekv_status prefill(const char* name, const void* q, const void* k, con
   // Several layers are one launch of the tensor-core kernel where lists are whole (the chunks of a split list meet in counters
   // and workspace slots that the plan has for one layer at a time).  31 layers of 2432 tokens: 44 us each as launches of their
   // own, a third of it start, merges and the uneven end.
-  // Layers that overlap (one Q for all of them, say) or that are not aligned as the tensor maps and the output's stores need
-  // are launches of their own too.
-  const int64_t esz = dtype == PUREKV_BF16 ? 2 : 4, t = batch->total_tokens;
+  // Layers that overlap (one Q for all of them, say) are launches of their own too, and so are strides that a tensor map cannot
+  // hold.
+  const int64_t esz = dtype == PUREKV_BF16 ? 2 : 4, t = batch->total_tokens, o_align = tc ? 32 : 16;
+  PK_REQUIRE(n_layers == 1 || (q_stride * esz % 16 == 0 && kv_stride * esz % 16 == 0 && o_stride * esz % o_align == 0),
+             PUREKV_ERR_INVALID_ARG, "layer strides must be multiples of 16 bytes, O's of %lld", (long long)o_align);
   const bool apart = q_stride >= t * n_q_heads * head_dim && o_stride >= t * n_q_heads * head_dim &&
                      kv_stride >= t * n_kv_heads * head_dim && (lse == nullptr || lse_stride >= t * n_q_heads) &&
-                     q_stride * esz % 16 == 0 && kv_stride * esz % 16 == 0 && o_stride * esz % 32 == 0 &&
                      std::max({q_stride, kv_stride, o_stride}) < (1ll << 38);
   if (n_layers == 1 || (tc && apart && info->max_chunks == 1 && (int64_t)info->n_units * n_layers <= INT32_MAX / 2))
     return tc ? launch_prefill_tc(a) : launch_prefill_simt(a);
@@ -53,8 +54,6 @@ static purekv_status prefill(const char* name, const void* q, const void* k, con
     a.v = (const char*)v + n * kv_stride * esz;
     a.o = (char*)o + n * o_stride * esz;
     a.lse = lse ? lse + n * lse_stride : nullptr;
-    PK_REQUIRE(((uintptr_t)a.q | (uintptr_t)a.k | (uintptr_t)a.v | (uintptr_t)a.o) % 16 == 0, PUREKV_ERR_INVALID_ARG,
-               "Q/K/V/O of layer %d must be 16-byte aligned", n);
     const purekv_status one = tc ? launch_prefill_tc(a) : launch_prefill_simt(a);
     if (one != PUREKV_OK) return one;
   }
