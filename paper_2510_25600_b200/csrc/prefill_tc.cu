@@ -74,8 +74,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_k64,
     const __grid_constant__ CUtensorMap tm_v64, const __grid_constant__ CUtensorMap tm_o, __nv_bfloat16* __restrict__ o, float* __restrict__ lse,
     uint8_t* __restrict__ plan, float* __restrict__ ws, int32_t n_q_heads, int32_t n_kv_heads, float scale_log2,
-    int32_t* __restrict__ status, uint64_t wait_ns, int64_t plan_bytes, int64_t ws_floats, int32_t n_layers, int64_t o_stride,
-    int64_t lse_stride) {
+    int32_t* __restrict__ status, uint64_t wait_ns, int64_t plan_bytes, int64_t ws_floats, int32_t n_units, int32_t n_layers,
+    int64_t o_stride, int64_t lse_stride) {
   constexpr int ST = Cfg<BK>::kStages, MR = Cfg<BK>::kMeta;
   constexpr uint32_t kPanelQ = kBQ * 128;  // bytes of one 64-column panel of a Q tile
   constexpr uint32_t kTileQ = 2 * kPanelQ;
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
     };
     plan_ok = hdr->magic == kPlanMagic && hdr->tile_q == kBQ && hdr->tile_k == BK && hdr->words_per_row == BK / 32 &&
               hdr->n_q_heads == n_q_heads && hdr->n_kv_heads == n_kv_heads && G_ >= 1 &&
-              hdr->n_ctas == (int32_t)gridDim.x && hdr->n_units >= 1 && hdr->n_counters >= 0 &&
+              hdr->n_ctas == (int32_t)gridDim.x && hdr->n_units == n_units && hdr->n_counters >= 0 &&
               section(hdr->off_entries, hdr->n_entries, 8) && section(hdr->off_masks, hdr->n_mask_words, 4) &&
               hdr->n_mask_words >= hdr->n_entries &&
               section(hdr->off_units, hdr->n_units, (int64_t)sizeof(Unit)) &&
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(
   // another whatever the units really cost.  The producer draws and publishes; the other roles follow unit_s[].
   // With several layers the list is gone through once per layer, one after another: the CTAs pass from a layer's last (and
   // smallest) units to the next layer's first without meeting, so a launch's start and its uneven end are paid for once.
-  const int32_t n_units = plan_ok ? hdr->n_units : 0, n_work = n_units * n_layers;
+  const int32_t n_work = n_units * n_layers;  // (the launch code knows that it is no more than an int32 holds)
   int32_t* sched = counters + (plan_ok ? hdr->n_counters : 0);  // [0] units drawn beyond the first round, [1] CTAs that drew their last
   const int64_t n_entries = plan_ok ? hdr->n_entries : 0, n_mask_words = plan_ok ? hdr->n_mask_words - n_entries : 0;
   const int64_t total_tokens = plan_ok ? hdr->total_tokens : 0;
@@ -1019,7 +1019,7 @@ static purekv_status launch(const PrefillArgs& a, const CUtensorMap& mq, const C
   PK_CUDA(cudaLaunchKernelEx(&cfg, prefill_tc_kernel<BK>, mq, mk, mv, mk64, mv64, mo, (__nv_bfloat16*)a.o, a.lse,
                              (uint8_t*)a.plan, (float*)a.ws, a.n_q_heads, a.n_kv_heads,
                              a.scale * 1.4426950408889634f, status, wait_limit_ns(), (int64_t)a.info->bytes_used,
-                             (int64_t)(a.ws_bytes / sizeof(float)), a.n_layers, a.o_stride, a.lse_stride));
+                             (int64_t)(a.ws_bytes / sizeof(float)), a.info->n_units, a.n_layers, a.o_stride, a.lse_stride));
   PK_CUDA(cudaGetLastError());
   return PUREKV_OK;
 }

@@ -51,10 +51,13 @@ def test_kernel_refuses_a_plan_whose_header_is_wrong_and_leaves_the_output_alone
     def more_units_than_there_are(h):
         _header(h).n_units = 1 << 28
 
+    def fewer_units_than_the_call_was_told(h):
+        _header(h).n_units -= 1
+
     def other_head_count(h):
         _header(h).n_q_heads += 2
 
-    for spoil in (bad_magic, entries_past_the_end, more_units_than_there_are, other_head_count):
+    for spoil in (bad_magic, entries_past_the_end, more_units_than_there_are, fewer_units_than_the_call_was_told, other_head_count):
         h = good.copy()
         spoil(h)
         status = torch.zeros(1, dtype=torch.int32, device="cuda")
