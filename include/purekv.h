@@ -145,7 +145,8 @@ purekv_status purekv_plan_build_host(const purekv_batch *batch, const purekv_st_
                                      int32_t n_kv_heads, int32_t n_ctas, void *h_plan,
                                      size_t plan_bytes, purekv_plan_info *h_info);
 
-/* Same size and planning, for launches of n_layers layers at a time (purekv_st_sparse_prefill_layers; n_layers 1 is the call above):
+/* Same size and planning, for launches of n_layers layers at a time (purekv_st_sparse_prefill_layers; n_layers 1 is the call above;
+ * the size is enough for the plan of n_layers and for that of a layer at a time):
  * cutting long lists into chunks evens out the end of a launch, and where one launch serves several layers that end is paid
  * for once, so lists are left whole when that ends sooner.  The plan serves launches of any number of layers. */
 size_t purekv_plan_layers_bytes(const purekv_batch *batch, const purekv_st_params *params, purekv_dtype dtype,

@@ -234,7 +234,7 @@ class Plan:
 
 def purekv_plan_bytes(batch: Batch, params: StParams, dtype: int, head_dim: int, n_q_heads: int, n_kv_heads: int,
                       n_ctas: int = 0, n_layers: int = 1) -> int:
-    """With `n_layers`, purekv_plan_layers_bytes: of a plan for launches of that many layers."""
+    """With `n_layers`, purekv_plan_layers_bytes: enough for a plan for launches of that many layers, and for one of a layer each."""
     return int(_lib.purekv_plan_layers_bytes(C.byref(batch.c), C.byref(params), dtype, head_dim, n_q_heads, n_kv_heads, n_ctas,
                                              n_layers))
 

@@ -131,6 +131,11 @@ purekv_status purekv_budget(int32_t len, int32_t window, double keep_ratio, int3
   return PUREKV_OK;
 }
 
+// What a schedule takes in a plan.
+struct ScheduleSize {
+  int64_t units = 0, twin_entries = 0, counters = 0;
+};
+
 // Splits long kept-key lists into chunks and orders the (query tile, head pair, chunk) units by decreasing cost:
 // the kernel's n_ctas persistent CTAs start with the first n_ctas units and draw the rest from a counter as they
 // finish, so the order is longest-first list scheduling carried out at run time.  The costs also decide how finely
@@ -143,10 +148,12 @@ purekv_status purekv_budget(int32_t len, int32_t window, double keep_ratio, int3
 // With an odd group size the group's last head has no partner; a unit for it alone takes as long as a unit for two
 // heads.  Consecutive query tiles of a request whose lists are not split therefore share that head's unit (a twin
 // unit, see Unit): the merged lists are appended to `entries`.
+//
+// `apart_size`: of the schedule that one layer a launch would get (where n_layers > 1; the plan's own otherwise).
 static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& entries, int32_t H, int32_t Hkv,
                            int32_t n_ctas, int32_t n_layers,
                            std::vector<Unit>& units, int32_t* n_counters,
-                           int64_t* part_slots, int32_t* max_chunks) {
+                           int64_t* part_slots, int32_t* max_chunks, ScheduleSize* apart_size) {
   const int32_t G = H / Hkv, ppg = (G + 1) / 2, n_pairs = Hkv * ppg;
   const bool odd = (G & 1) != 0;
   const int32_t overhead = 6, split_extra = 14;
@@ -183,8 +190,8 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
   };
   // partner[i]: the tile that shares tile i's odd-head units (i leads the twin), -2 if tile i is the second of a
   // twin, -1 if it stays alone.  Twins have the same number of chunks, and a merged chunk may be a quarter longer
-  // than the cap on a chunk.  twin_cost: the merged chunks' costs, leader by leader, chunk by chunk.
-  std::vector<int32_t> partner, twin_cost;
+  // than the cap on a chunk.  twin_cost, twin_len: the merged chunks' costs and lengths, leader by leader, chunk by chunk.
+  std::vector<int32_t> partner, twin_cost, twin_len;
   struct Merged { int32_t n = -1, cost = 0; };
   std::vector<Merged> whole((size_t)nq);  // tile i's whole list merged with tile i + 1's: the same under every cap that leaves both whole
   auto merge_chunk = [&](int32_t i, int32_t c, int32_t nch) {
@@ -200,6 +207,7 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
   auto find_twins = [&](int32_t l_max) {
     partner.assign((size_t)nq, -1);
     twin_cost.clear();
+    twin_len.clear();
     if (!odd) return;
     for (int32_t i = 0; i + 1 < nq; ++i) {
       const QTile &a = qtiles[i], &b = qtiles[i + 1];
@@ -210,10 +218,12 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
       for (int32_t c = 0; c < nch && fits; ++c) {
         const Merged m = merge_chunk(i, c, nch);
         twin_cost.push_back(m.cost);
+        twin_len.push_back(m.n);
         fits = m.n <= l_max + l_max / 4;
       }
       if (!fits) {
         twin_cost.resize(at);
+        twin_len.resize(at);
         continue;
       }
       partner[i] = i + 1;
@@ -300,11 +310,14 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
   // listed: the earliest free time only grows, so one pass over the times serves all units.
   std::vector<int32_t> n_of_cost, n_free;
   int64_t total = 0;  // the units' costs
+  ScheduleSize size;
   auto makespan = [&](int32_t l_max, int64_t limit) {
     find_twins(l_max);
     n_of_cost.clear();
     total = 0;
+    size = ScheduleSize{};
     auto add = [&](int32_t cost, int32_t n) {
+      size.units += n;
       if ((size_t)cost >= n_of_cost.size()) n_of_cost.resize((size_t)cost + 1, 0);
       n_of_cost[cost] += n;
       total += (int64_t)cost * n;
@@ -313,11 +326,15 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
     for (int32_t qi = 0; qi < nq; ++qi) {
       const QTile& q = qtiles[qi];
       const int32_t nch = chunks_of(q, l_max), extra = overhead + (nch > 1 ? split_extra : 0);
+      if (nch > 1) size.counters += H;
       for (int32_t c = 0; c < nch; ++c) {
         int32_t a, e;
         chunk_range(q, c, nch, &a, &e);
         add(halves(a, e) + extra, partner[qi] != -1 ? n_pairs - Hkv : n_pairs);
-        if (partner[qi] >= 0) add(twin_cost[twin_at++] + extra, Hkv);
+        if (partner[qi] >= 0) {
+          size.twin_entries += 2 * twin_len[twin_at];
+          add(twin_cost[twin_at++] + extra, Hkv);
+        }
       }
     }
     n_free.assign((size_t)(total / n_ctas) + n_of_cost.size() + 1, 0);  // CTAs that become free at each time
@@ -354,10 +371,12 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
   if (n_layers > 1) {
     const int32_t l_whole = 1 << 28, launch = 40;
     const int64_t apart = n_layers * (makespan(l_best, INT64_MAX) + launch);
+    *apart_size = size;
     const int64_t last = makespan(l_whole, INT64_MAX);
     if ((n_layers - 1) * (total + n_ctas - 1) / n_ctas + last + launch <= apart) l_best = l_whole;
   }
   make_items(l_best);
+  if (n_layers == 1) *apart_size = ScheduleSize{(int64_t)units.size(), (int64_t)twin_entries.size(), counters};
   entries.insert(entries.end(), twin_entries.begin(), twin_entries.end());
   *n_counters = counters;
   *part_slots = slots * H;
@@ -368,6 +387,7 @@ static void schedule_units(const std::vector<QTile>& qtiles, std::vector<int2>& 
 struct HostPlan {
   PlanHeader h;
   int64_t total = 0;  // bytes
+  int64_t room = 0;   // bytes, also for the plan of the same layers one a launch
   std::vector<QTile> qtiles;
   std::vector<int32_t> order;
   std::vector<int2> entries;
@@ -635,9 +655,11 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
   std::vector<Unit>& units = plan.units;
   int32_t n_counters = 0, max_chunks = 1;
   int64_t part_slots = 0;
+  ScheduleSize apart;
+  const int64_t n_listed = (int64_t)entries.size();
+  const size_t n_masks = masks.size();
   if (tq == 128 && nq > 0) {
-    schedule_units(qtiles, entries, n_q_heads, n_kv_heads, n_ctas, n_layers, units, &n_counters, &part_slots, &max_chunks);
-    const size_t n_masks = masks.size();
+    schedule_units(qtiles, entries, n_q_heads, n_kv_heads, n_ctas, n_layers, units, &n_counters, &part_slots, &max_chunks, &apart);
     PK_REQUIRE(n_masks + entries.size() < (size_t)INT32_MAX, PUREKV_ERR_UNSUPPORTED, "mask table exceeds 2^31 words");
     masks.resize(n_masks + entries.size());
     for (size_t i = 0; i < entries.size(); ++i) {
@@ -658,22 +680,30 @@ static purekv_status build_plan(const purekv_batch* b, const purekv_st_params* p
   h.n_entries = (int64_t)entries.size();
   h.n_mask_words = (int64_t)masks.size();
   h.words_per_row = wpr;
-  h.off_qtiles = align16(sizeof(PlanHeader));
-  h.off_order = h.off_qtiles + align16((int64_t)nq * sizeof(QTile));
-  h.off_entries = h.off_order + align16((int64_t)nq * 4);
-  h.off_masks = h.off_entries + align16(h.n_entries * 8);
   h.n_ctas = units.empty() ? 0 : n_ctas;
   h.n_units = (int32_t)units.size();
   h.n_counters = n_counters;
   h.n_q_heads = n_q_heads;
   h.n_kv_heads = n_kv_heads;
   h.part_slots = part_slots;
-  h.off_units = h.off_masks + align16(h.n_mask_words * 4);
-  h.off_counters = h.off_units + align16((int64_t)h.n_units * sizeof(Unit));
-  // the merge counters, then the kernel's two scheduling counters; all start at zero and the kernel leaves them so
-  const int64_t total = h.off_counters + align16(((int64_t)n_counters + 2) * 4);
+  // Lays the sections out and returns the bytes they take.
+  auto layout = [&](int64_t n_entries, int64_t n_mask_words, int64_t n_units, int64_t counters) {
+    h.off_qtiles = align16(sizeof(PlanHeader));
+    h.off_order = h.off_qtiles + align16((int64_t)nq * sizeof(QTile));
+    h.off_entries = h.off_order + align16((int64_t)nq * 4);
+    h.off_masks = h.off_entries + align16(n_entries * 8);
+    h.off_units = h.off_masks + align16(n_mask_words * 4);
+    h.off_counters = h.off_units + align16(n_units * (int64_t)sizeof(Unit));
+    // the merge counters, then the kernel's two scheduling counters; all start at zero and the kernel leaves them so
+    return h.off_counters + align16((counters + 2) * 4);
+  };
+  const int64_t apart_entries = n_listed + apart.twin_entries;
+  const int64_t apart_total =
+      layout(apart_entries, (int64_t)n_masks + (tq == 128 && nq > 0 ? apart_entries : 0), apart.units, apart.counters);
+  const int64_t total = layout(h.n_entries, h.n_mask_words, h.n_units, n_counters);
 
   plan.total = total;
+  plan.room = std::max(total, apart_total);
 
   info->tile_q = tq;
   info->tile_k = gk;
@@ -700,7 +730,7 @@ size_t purekv_plan_layers_bytes(const purekv_batch* b, const purekv_st_params* p
   purekv_plan_info info;
   HostPlan host;
   if (build_plan(b, p, dtype, head_dim, n_q_heads, n_kv_heads, n_ctas, n_layers, &info, host) != PUREKV_OK) return 0;
-  return (size_t)host.total;
+  return (size_t)host.room;
 }
 
 purekv_status purekv_plan_build_host(const purekv_batch* b, const purekv_st_params* p, purekv_dtype dtype,

@@ -44,10 +44,10 @@ class PureKVPipeline:
         hh = (n_q_heads, n_kv_heads)
         self.n_dense = min(n_layers, self.clie + 1)
         self.n_sparse = n_layers - self.n_dense
-        # room for a plan of one layer at a time (build_plans, prefill_layer) and for one of all layers under the mask (run_device)
+        # room for a plan of all layers under the mask (run_device) and for one of a layer at a time (build_plans, prefill_layer)
         plan_buf = lambda params, layers: torch.empty(
-            max(1, *(P.purekv_plan_bytes(self.batch, params, self.code, head_dim, *hh, n_layers=n) for n in {1, max(1, layers)})),
-            dtype=torch.uint8, device=dev)
+            max(1, P.purekv_plan_bytes(self.batch, params, self.code, head_dim, *hh, n_layers=max(1, layers))), dtype=torch.uint8,
+            device=dev)
         self.plan_buf_dense, self.plan_buf_st = plan_buf(params_dense, self.n_dense), plan_buf(self.params_st, self.n_sparse)
         self.prefill_ws = None
         # per mask a ring of pinned buffers, each with the event behind its last copy; the last one used comes first

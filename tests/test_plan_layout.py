@@ -33,3 +33,14 @@ def test_a_plan_of_the_layout_before_is_refused():
     pk.purekv_st_sparse_prefill(q, k, v, b, pk.Plan(torch.from_numpy(plan).cuda(), info), out=out, status=status)
     # (read directly: the traceback of a raised error would keep the tensors alive past the test, until some later collection)
     assert status.item() == pk.ERR_BAD_PLAN and (out == 7.0).all()
+
+
+@pytest.mark.parametrize("heads", [(1, 1), (2, 1), (7, 1), (28, 4)])
+@pytest.mark.parametrize("frames,dense", [([0], False), ([3], False), ([16], False), ([16], True), ([5, 30, 1], False), ([40], True)])
+@pytest.mark.parametrize("n_layers", [1, 2, 30])
+def test_the_size_for_many_layers_is_enough_for_a_layer_at_a_time(heads, frames, dense, n_layers):
+    batch = inputs.make_batch([5] * len(frames), frames, [40] * len(frames), 12, 13)
+    b = pk.Batch(batch.seq_lens, batch.n_prefix, batch.n_frames, device=None)
+    args = (b, pk.st_params(inputs.STMask(12, 13, tile=64, dense_causal=dense)), pk.BF16, 128, *heads)
+    one, many = (pk.purekv_plan_build_host(*args, n_layers=n)[1].bytes_used for n in (1, n_layers))
+    assert pk.purekv_plan_bytes(*args, n_layers=n_layers) == max(one, many) and pk.purekv_plan_bytes(*args) == one
