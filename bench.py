@@ -43,7 +43,7 @@ NOMINAL_TFLOPS, NOMINAL_HBM_GBS = 2250.0, 8000.0   # B200 dense bf16 and HBM3e f
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of an ST-SpAttn launch of one layer of the tensor-core prefill
 # kernel, from the ncu capture summarised under profiles/.  It is reported only while the kernel and planner
 # sources are the ones the capture was taken from (sha1 of their text); otherwise the roofline's traffic is null.
-NCU_TRAFFIC = {"cfg2_qwen25vl": {"bytes_per_launch": 107.2e6, "source_sha1": "9379bbb3ca43e5e536c9403b9966053172a0ca86"}}
+NCU_TRAFFIC = {"cfg2_qwen25vl": {"bytes_per_launch": 106.9e6, "source_sha1": "6972530a89474202cc1da308da2e63b3be672142"}}
 KERNEL_SOURCES = ("prefill_tc.cu", "tc_util.cuh", "plan.cu", "common.cuh", "prefill.cuh")
 
 

@@ -331,8 +331,10 @@ purekv_status purekv_decode_attention(const void *q, const void *k_cache, const 
 /* Failure detection (no counterpart in the paper).  Every wait inside the tensor-core kernels -- on a copy, on a
  * product, on another role of the CTA -- is bounded: when the limit passes the CTA raises the status word to
  * PUREKV_ERR_TIMEOUT, lets its copies and products in flight finish, frees its tensor memory and returns, so the
- * context stays usable.  The limit is process-wide, 1 s by default; ns == 0 restores the default.  The tensor-core
- * prefill also checks the plan before using it (header, section offsets against the plan's size, every unit's and
+ * context stays usable.  The limit is process-wide, 1 s by default; ns == 0 restores the default.  The roles of a prefill CTA
+ * also wait for one another for as long as a unit lasts: one query tile's list of key tiles at 1.6 us each, 0.5 ms for a whole
+ * causal list of 37 000 keys (purekv_plan_build_layers_host leaves lists whole), which a lower limit has to leave room for.
+ * The tensor-core prefill also checks the plan before using it (header, section offsets against the plan's size, every unit's and
  * entry's indices against the header's counts): on a mismatch nothing is read through the bad field, the status
  * word becomes PUREKV_ERR_BAD_PLAN and the output is undefined (untouched when the header itself fails).  After either code the plan's scheduling counters are
  * undefined: build the plan again before the next launch. */

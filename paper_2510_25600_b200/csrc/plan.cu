@@ -143,7 +143,8 @@ struct ScheduleSize {
 // half that the entry lists (5 when it carries a bit mask), 6 per unit (query load, pipeline fill, epilogue) and 14 more for a
 // chunk of a split list (fp32 partial result written out, and the merge).  The constants were fitted to unit times of an
 // earlier form of the kernel, which also loaded the listed halves that hold no pair; today a half costs 0.78 of a whole entry
-// rather than half of it, and a chunk's merge less.  The order they give is still the one measured.
+// rather than half of it, a chunk's merge less, and an entry with a bit mask of which a warp keeps one or two 32-key chunks less
+// than one without.  The order they give is still the one measured.
 //
 // With an odd group size the group's last head has no partner; a unit for it alone takes as long as a unit for two
 // heads.  Consecutive query tiles of a request whose lists are not split therefore share that head's unit (a twin
