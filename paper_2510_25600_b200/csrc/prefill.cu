@@ -35,7 +35,7 @@ static purekv_status prefill(const char* name, const void* q, const void* k, con
                 (cudaStream_t)stream, n_layers, q_stride, kv_stride, o_stride, lse_stride};
   const bool tc = dtype == PUREKV_BF16 && head_dim == 128 && info->tile_q == 128;
   // Several layers are one launch of the tensor-core kernel where lists are whole (the chunks of a split list meet in counters
-  // and workspace slots that the plan has for one layer at a time).  31 layers of 2432 tokens: 44 us each as launches of their
+  // and workspace slots that the plan has for one layer at a time).  31 layers of 2432 tokens: 40 us each as launches of their
   // own, a third of it start, merges and the uneven end.
   // Layers that overlap (one Q for all of them, say) are launches of their own too, and so are strides that a tensor map cannot
   // hold.
